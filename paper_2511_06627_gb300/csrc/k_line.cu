@@ -349,6 +349,10 @@ void launch_resample_adj_tiled(const float *sig, const int4 *tiles, const uint16
 
 // ----------------------------------------------------------------------------- S D F
 
+// Floats of a table that complex values follow in shared memory (their pairs start on 8
+// bytes; P W is odd when P is).
+__host__ __device__ __forceinline__ constexpr int even_floats(int n) { return (n + 1) & ~1; }
+
 // Twiddle table tw1[p][0..W): cos(2 pi d p / P) for d = 0..hw, then sin(2 pi d p / P)
 // for d = 1..hw.
 template <int HW>
@@ -360,7 +364,7 @@ __global__ void __launch_bounds__(128) k_dft_fwd(const float *__restrict__ sig,
     extern __shared__ float sm[];
     const int W = 2 * HW + 1;
     float *stw = sm;                               // P * W
-    float2 *sT = (float2 *)(sm + d.P * W);         // S * W
+    float2 *sT = (float2 *)(sm + even_floats(d.P * W));  // S * W
     const int seg = blockIdx.x;
     for (int i = threadIdx.x; i < d.P * W; i += blockDim.x) stw[i] = tw1[i];
     __syncthreads();
@@ -410,7 +414,7 @@ __global__ void __launch_bounds__(128) k_dft_adj(const float *__restrict__ data,
     extern __shared__ float sm[];
     const int W = 2 * HW + 1;
     float *stw = sm;                               // P * W
-    float2 *sy = (float2 *)(sm + d.P * W);         // nb: conj(D) y / sqrt(L)
+    float2 *sy = (float2 *)(sm + even_floats(d.P * W));  // nb: conj(D) y / sqrt(L)
     const int seg = blockIdx.x;
     for (int i = threadIdx.x; i < d.P * W; i += blockDim.x) stw[i] = tw1[i];
     for (int o = threadIdx.x; o < d.nb; o += blockDim.x) {
@@ -607,7 +611,7 @@ template <int HW>
 static void dft_fwd_hw(const float *sig, const float *tw1, const float2 *tw2_ro, const float2 *dgam,
                        float *data, const Dims &d, cudaStream_t st) {
     const int W = 2 * HW + 1;
-    const size_t smem = sizeof(float) * d.P * W + sizeof(float2) * d.S * W;
+    const size_t smem = sizeof(float) * even_floats(d.P * W) + sizeof(float2) * d.S * W;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_dft_fwd<HW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     k_dft_fwd<HW><<<d.nseg, 128, smem, st>>>(sig, tw1, tw2_ro, dgam, data, d, (float)(1.0 / sqrt((double)d.L)));
@@ -707,7 +711,7 @@ template <int HW>
 static void dft_adj_hw(const float *data, const float *tw1, const float2 *tw2_qr, const float2 *dgam,
                        float *sig, const Dims &d, cudaStream_t st) {
     const int W = 2 * HW + 1;
-    const size_t smem = sizeof(float) * d.P * W + sizeof(float2) * d.nb;
+    const size_t smem = sizeof(float) * even_floats(d.P * W) + sizeof(float2) * d.nb;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_dft_adj<HW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     k_dft_adj<HW><<<d.nseg, 128, smem, st>>>(data, tw1, tw2_qr, dgam, sig, d, (float)(1.0 / sqrt((double)d.L)));
