@@ -259,10 +259,19 @@ ALGO_BYTES = {
     "tc_adj": lambda d: 4 * (d["nfine"] + d["ndata"]),
     # the slice-interleaving pass: reads the volume, writes its interleaved copy
     "transpose": lambda d: 8 * d["nvox"],
-    # the full-GEMM path applies W H to projections, the line-GEMM path W to fine rows
-    "gemm_fwd": lambda d: 4 * ((d["nproj"] if d["path"].startswith("full_gemm") else d["nfine"]) + d["ndata"]),
-    "gemm_adj": lambda d: 4 * ((d["nproj"] if d["path"].startswith("full_gemm") else d["nfine"]) + d["ndata"]),
+    # the full-GEMM and staged paths apply W H to projections, the line-GEMM path W to fine rows
+    "gemm_fwd": lambda d: 4 * ((d["nproj"] if folds_psf(d["path"]) else d["nfine"]) + d["ndata"]),
+    "gemm_adj": lambda d: 4 * ((d["nproj"] if folds_psf(d["path"]) else d["nfine"]) + d["ndata"]),
 }
+
+
+def folds_psf(path):
+    """Whether a path's line stage takes projections (the PSF folded into its matrix)."""
+    return path.startswith("full_gemm") or path == "staged"
+
+
+# FP32 FMA rate of the CUDA cores: 152 SMs x 128 lanes x 2 flops x 2.07 GHz
+FP32_PEAK_TFLOPS = 80.5
 
 # Shared-memory bytes the projector pair reads per launch: two interpolation taps of
 # 4 bytes for every (angle, ray, march step, slice) sample, M N N N_z = M n_vox samples. Both
@@ -329,7 +338,7 @@ def kernel_rooflines(prof, d, hbm, sm_peak):
     bf16, _ = bf16_peak_tflops()
     nz = d["nvox"] // (d["N"] * d["N"])
     nseg = d["M"] * nz
-    rows_k = d["N"] if d["path"].startswith("full_gemm") else d["nfine"] // nseg
+    rows_k = d["N"] if folds_psf(d["path"]) else d["nfine"] // nseg
     # tf32 operands: the measured bf16 peak times the nominal tf32/bf16 ratio (1.1 / 2.25 PFLOP/s)
     tensor_peak = bf16 * (1.1 / 2.25) if d["path"].endswith("_tf32") else bf16
     out = {}
@@ -340,7 +349,9 @@ def kernel_rooflines(prof, d, hbm, sm_peak):
         e = {"ms_per_launch": t_ms / n, "hbm_frac": ALGO_BYTES[k](d) / sec / 1e9 / hbm}
         if k in SMEM_BYTES:
             e["smem_frac"] = SMEM_BYTES[k](d) / sec / 1e9 / sm_peak
-        if k in ("gemm_fwd", "gemm_adj"):
+        if k in ("gemm_fwd", "gemm_adj") and d["path"] == "staged":  # FP32 on CUDA cores
+            e["fp32_frac"] = 2 * nseg * (d["ndata"] // nseg) * rows_k / sec / 1e12 / FP32_PEAK_TFLOPS
+        elif k in ("gemm_fwd", "gemm_adj"):
             flops = 3 * 2 * nseg * (d["ndata"] // nseg) * rows_k
             e["tensor_tflops"] = flops / sec / 1e12
             e["tensor_frac"] = e["tensor_tflops"] / tensor_peak

@@ -63,14 +63,17 @@ extern "C" {
 #define MPI_FFL_ERR_UNSUPPORTED (-6)
 
 /* Arithmetic of the harmonic-band DFT and its transpose (the other stages are FP32). */
-#define MPI_FFL_PREC_FP32 0   /* plain: FP32 FMA on CUDA cores, stage by stage        */
+#define MPI_FFL_PREC_FP32 0   /* plain: FP32 FMA on CUDA cores                        */
 #define MPI_FFL_PREC_BF16X3 1 /* tensor cores: bf16 hi+lo split, 3 products, FP32 acc  */
 #define MPI_FFL_PREC_TF32 2   /* tensor cores: tf32 hi+lo split, 3 products, FP32 acc  */
 
 /* How A and A^T are evaluated (the operator is the same; only the order of evaluation
  * and the arithmetic differ):
- *   STAGED     P, H, E V B and S D_Gamma F as separate FP32 CUDA-core kernels; the
- *              time signal (L floats per line) passes through HBM. Precision FP32.
+ *   STAGED     P, then S D_Gamma F V E H as one matrix per trajectory, built in double
+ *              precision on the first use and applied in FP32 on CUDA cores; for short
+ *              lines with wide bands, where that matrix costs more than the stages, H,
+ *              E V B and S D_Gamma F as separate FP32 kernels with the time signal in
+ *              HBM (mpi_ffl_apply_stage runs the stages for every shape). Precision FP32.
  *   FUSED      P and H as above; E V B fused with the band DFT on tensor cores
  *              (tcgen05, BF16x3): the time signal stays on chip.
  *   LINE_GEMM  P and H as above; S D_Gamma F V E, identical for every line of one

@@ -10,6 +10,7 @@
 
 #include "internal.h"
 #include "collapsed.h"
+#include "fold.h"
 #include "tc.h"
 
 using namespace mpiffl;
@@ -147,6 +148,7 @@ double langevin_half_point() {
 
 namespace mpiffl {
 double langevin_d1_host(double x) { return langevin_d1(x); }
+double langevin_d2_host(double x) { return langevin_d2(x); }
 double langevin_half_point_host() { return langevin_half_point(); }
 // FFL sample j of a line with the given trajectory (parity): fine cell n, fraction f, velocity v
 void traj_point_host(const mpi_ffl_handle *h, int par, int j, int &n, double &f, double &v) {
@@ -414,6 +416,7 @@ void release(mpi_ffl_handle *h) {
     if (h->hs_copy) cudaStreamDestroy(h->hs_copy);
     tc_release(h);
     col_release(h);
+    fold_release(h);
 }
 
 // ------------------------------------------------------------ host buffers
@@ -637,6 +640,15 @@ void stage_pt(mpi_ffl_handle *h, const float *proj, float *x, cudaStream_t st) {
     check_launch(h, "backproject");
 }
 
+// FP32 operands of the staged path's folded line stage, built on first use
+void need_fold(mpi_ffl_handle *h, int slot, cudaStream_t st) {
+    const int rc = fold_ready(h, slot, st);
+    if (rc != MPI_FFL_OK) {
+        set_err(h, "building the folded line operator failed");
+        throw Fail{rc};
+    }
+}
+
 // blockdiag(A_DC) on projections: proj -> data
 // prepacked: the projector wrote the full stage's A operand (proj not stored)
 void line_forward_impl(mpi_ffl_handle *h, const float *proj, float *b, const float *htab, const float *gain,
@@ -657,6 +669,13 @@ void line_forward_impl(mpi_ffl_handle *h, const float *proj, float *b, const flo
     if (path == MPI_FFL_PATH_FULL_GEMM) {
         TIMED(MPI_FFL_K_GEMM_FWD, col_forward(h, proj, true, gain, b, st, prepacked));
         check_launch(h, "gemm_fwd");
+        return;
+    }
+    if (path == MPI_FFL_PATH_STAGED && fold_fits(d)) {
+        const int slot = htab == h->t_dhtab ? 1 : 0;
+        need_fold(h, slot, st);
+        TIMED(MPI_FFL_K_GEMM_FWD, fold_forward(h, slot, proj, gain, b, st));
+        check_launch(h, "fold_forward");
         return;
     }
     TIMED(MPI_FFL_K_PSF_FWD, launch_psf_fwd(proj, htab, h->w_fine, d, st));
@@ -696,6 +715,12 @@ void line_adjoint_body(mpi_ffl_handle *h, const float *b, float *proj, cudaStrea
     if (h->path == MPI_FFL_PATH_FULL_GEMM) {
         TIMED(MPI_FFL_K_GEMM_ADJ, col_adjoint(h, b, true, h->t_gain, proj, st));
         check_launch(h, "gemm_adj");
+        return;
+    }
+    if (h->path == MPI_FFL_PATH_STAGED && fold_fits(d)) {
+        need_fold(h, 0, st);
+        TIMED(MPI_FFL_K_GEMM_ADJ, fold_adjoint(h, b, h->t_gain, proj, st));
+        check_launch(h, "fold_adjoint");
         return;
     }
     if (h->path == MPI_FFL_PATH_LINE_GEMM) {
@@ -1189,6 +1214,10 @@ extern "C" int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm) {
         CK(cudaMemcpy(h->t_htab, ht.data(), sizeof(float) * ht.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->t_dhtab, dht.data(), sizeof(float) * dht.size(), cudaMemcpyHostToDevice));
         tc_tables_changed(h);
+        if (fold_psf_changed(h) != MPI_FFL_OK) {
+            h->err = "the folded line operator could not be rebuilt";
+            return MPI_FFL_ERR_CUDA;
+        }
         // W H holds the PSF: rebuild the collapsed operator if it was built and the
         // full-GEMM path is selected; otherwise W (which holds no PSF) stays and W H is
         // rebuilt when the full-GEMM path is next selected

@@ -4,9 +4,8 @@
 // same band DFT, so S D_Gamma F V E (Sec. 2.1, Eq. (13), without the per-angle
 // gain) is one fixed complex matrix W of n_bins x N_e per trajectory -- the same
 // reassociation of the operator chain that lets the paper apply one FFT instead of
-// three. W is built once on the host in double precision from the trajectory
-// (W[o][e] = D_o L^-1/2 sum_j e^{2 pi i w_o j / L} (w0_j [n_j = e] + w1_j [n_j + 1 = e])),
-// and optionally folded with H into W H (n_bins x N). A line stage then is
+// three. W, and W H with the PSF folded in (n_bins x N), are built in double precision on
+// the device (fold.cu) and split here. A line stage then is
 //     data[line] = g_m W fine[line]          (forward)
 //     fine[line] = g_m Re(W^H data[line])    (adjoint, real inner product)
 // i.e. one dense GEMM per trajectory, with W stored as a real matrix whose rows
@@ -23,10 +22,10 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <thread>
 #include <vector>
 
 #include "collapsed.h"
+#include "fold.h"
 #include "split_operands.cuh"
 #include "tc_ptx.cuh"
 
@@ -432,67 +431,47 @@ __global__ void __launch_bounds__(kGemmThreads, 2) k_gemm_batch(const GemmArgs *
     if (warp == 0) ptx::tmem_dealloc(tslot, cols);
 }
 
-uint16_t bf16_bits(double x) {
-    const float f = (float)x;
-    uint32_t u;
-    std::memcpy(&u, &f, 4);
-    const uint32_t rounding = 0x7FFFu + ((u >> 16) & 1u);
-    return (uint16_t)((u + rounding) >> 16);
+__device__ __forceinline__ uint16_t bf16_bits_dev(double x) {
+    const uint32_t u = __float_as_uint((float)x);
+    return (uint16_t)((u + 0x7FFFu + ((u >> 16) & 1u)) >> 16);
 }
-double bf16_value(uint16_t b) {
-    const uint32_t u = (uint32_t)b << 16;
-    float f;
-    std::memcpy(&f, &u, 4);
-    return f;
+__device__ __forceinline__ uint32_t tf32_bits_dev(double x) {
+    return (__float_as_uint((float)x) + 0x1000u) & 0xFFFFE000u;
 }
 
-uint32_t tf32_bits(double x) {
-    const float f = (float)x;
-    uint32_t u;
-    std::memcpy(&u, &f, 4);
-    return (u + 0x1000u) & 0xFFFFE000u;  // round to nearest (ties away), 10-bit mantissa
-}
-double tf32_value(uint32_t b) {
-    float f;
-    std::memcpy(&f, &b, 4);
-    return f;
-}
-
-// Pre-split B operand for k_gemm_split: Bm is Nv x Kv (row-major, double); padded to
-// ntile*BN x nkc*(K per chunk); blocks [tile][chunk][hi, lo] of BN rows x 128 bytes per
-// row in the canonical layout (64 bf16 or 32 tf32 elements per row and chunk).
-std::vector<uint8_t> pack_b(const std::vector<double> &Bm, int Nv, int Kv, int BN, int &ntile, int &nkc, bool tf32) {
-    ntile = (Nv + BN - 1) / BN;
+// pack_b on the device: one thread per (tile, chunk, row, K element) of the canonical
+// layout; hi = round(v), lo = round(v - hi), in bf16 or tf32.
+template <class Src>
+__global__ void k_pack_b(Src src, int Nv, long long Kv, int BN, int ntile, int nkc, int tf32, uint8_t *out) {
     const int kpc = tf32 ? kBK / 2 : kBK;
-    nkc = (Kv + kpc - 1) / kpc;
     const size_t blk = (size_t)BN * kBK * 2;
-    std::vector<uint8_t> out((size_t)ntile * nkc * 2 * blk, 0);
-    for (int t = 0; t < ntile; ++t)
-        for (int kc = 0; kc < nkc; ++kc) {
-            uint8_t *hi = out.data() + ((size_t)t * nkc + kc) * 2 * blk;
-            uint8_t *lo = hi + blk;
-            for (int nl = 0; nl < BN; ++nl) {
-                const int n = t * BN + nl;
-                for (int kl = 0; kl < kpc; ++kl) {
-                    const int k = kc * kpc + kl;
-                    const double v = (n < Nv && k < Kv) ? Bm[(size_t)n * Kv + k] : 0.0;
-                    if (tf32) {
-                        const uint32_t hb = tf32_bits(v);
-                        const uint32_t lb = tf32_bits(v - tf32_value(hb));
-                        const size_t off = (size_t)(nl / 8) * 1024 + (kl / 4) * 128 + (nl % 8) * 16 + (kl % 4) * 4;
-                        std::memcpy(hi + off, &hb, 4);
-                        std::memcpy(lo + off, &lb, 4);
-                    } else {
-                        const uint16_t hb = bf16_bits(v);
-                        const uint16_t lb = bf16_bits(v - bf16_value(hb));
-                        const size_t off = (size_t)(nl / 8) * 1024 + (kl / 8) * 128 + (nl % 8) * 16 + (kl % 8) * 2;
-                        std::memcpy(hi + off, &hb, 2);
-                        std::memcpy(lo + off, &lb, 2);
-                    }
-                }
-            }
+    const size_t total = (size_t)ntile * nkc * BN * kpc;
+    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
+         idx += (size_t)gridDim.x * blockDim.x) {
+        const int kl = (int)(idx % kpc);
+        size_t r = idx / kpc;
+        const int nl = (int)(r % BN);
+        r /= BN;
+        const int kc = (int)(r % nkc), t = (int)(r / nkc);
+        const int n = t * BN + nl;
+        const long long k = (long long)kc * kpc + kl;
+        const double v = (n < Nv && k < Kv) ? src(n, k) : 0.0;
+        uint8_t *hi = out + ((size_t)t * nkc + kc) * 2 * blk;
+        uint8_t *lo = hi + blk;
+        if (tf32) {
+            const uint32_t hb = tf32_bits_dev(v);
+            const uint32_t lb = tf32_bits_dev(v - (double)__uint_as_float(hb));
+            const size_t off = (size_t)(nl / 8) * 1024 + (kl / 4) * 128 + (nl % 8) * 16 + (kl % 4) * 4;
+            *reinterpret_cast<uint32_t *>(hi + off) = hb;
+            *reinterpret_cast<uint32_t *>(lo + off) = lb;
+        } else {
+            const uint16_t hb = bf16_bits_dev(v);
+            const uint16_t lb = bf16_bits_dev(v - (double)__uint_as_float((uint32_t)hb << 16));
+            const size_t off = (size_t)(nl / 8) * 1024 + (kl / 8) * 128 + (nl % 8) * 16 + (kl % 8) * 2;
+            *reinterpret_cast<uint16_t *>(hi + off) = hb;
+            *reinterpret_cast<uint16_t *>(lo + off) = lb;
         }
-    return out;
+    }
 }
 
 struct Packed {
@@ -501,12 +480,29 @@ struct Packed {
     int per_sm = 2;  // blocks per SM the tiling was chosen for (1: deeper pipeline, all TMEM)
 };
 
+template <class Src>
+bool pack_dev(Packed &p, Src src, int Nv, long long Kv, int BN, int tf32) {
+    const int kpc = tf32 ? kBK / 2 : kBK;
+    p.BN = BN;
+    p.ntile = (Nv + BN - 1) / BN;
+    p.nkc = (int)((Kv + kpc - 1) / kpc);
+    const size_t bytes = (size_t)p.ntile * p.nkc * 2 * BN * kBK * 2;
+    if (p.dev) dev_free(p.dev);
+    p.dev = nullptr;
+    if (dev_malloc((void **)&p.dev, bytes) != cudaSuccess) {
+        p.dev = nullptr;
+        cudaGetLastError();
+        return false;
+    }
+    k_pack_b<Src><<<4 * 152 * 8, 256>>>(src, Nv, Kv, BN, p.ntile, p.nkc, tf32, p.dev);
+    return cudaGetLastError() == cudaSuccess;
+}
+
 struct ColState {
     bool ok = false;
     // per operand format (0 bf16, 1 tf32) and trajectory: forward / adjoint operands of
     // W (line) and W H (full)
     Packed evf_f[2][2], evf_a[2][2], full_f[2][2], full_a[2][2];
-    std::vector<double> W[2];           // S D_Gamma F V E per trajectory (2 n_b x N_e, double)
     struct TensorState *ten = nullptr;  // slice-coupled operator of the tensor PSF
     int *rows[2] = {nullptr, nullptr};  // line indices of each trajectory
     int nrows[2] = {0, 0};
@@ -570,14 +566,6 @@ __global__ void __launch_bounds__(256) k_pack_lines(const float *__restrict__ in
         *reinterpret_cast<uint4 *>(p.out + ((2 * (size_t)c) * G + gq) * 1024u + off) = hi;
         *reinterpret_cast<uint4 *>(p.out + ((2 * (size_t)c + 1) * G + gq) * 1024u + off) = lo;
     }
-}
-
-bool upload_packed(Packed &p, const std::vector<uint8_t> &v) {
-    if (dev_malloc((void **)&p.dev, v.size()) != cudaSuccess) {
-        p.dev = nullptr;
-        return false;
-    }
-    return cudaMemcpy(p.dev, v.data(), v.size(), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
 // Pipeline depth: for two blocks per SM, as many stages (2..4) as leave room for both,
@@ -685,90 +673,39 @@ bool col_supported(const mpi_ffl_handle *h) {
     return s && s->ok;
 }
 
-// W per trajectory (real rows: Re then Im of each kept bin), from the double-precision
-// trajectory; then W H with the PSF taps h(u_lo + e/Q - i).
+// Value (n, k) of the GEMM operands: rows of a matrix [R][C] in double (row stride C) or of
+// its transpose.
+struct MatSrc {
+    const double *m;
+    int C;
+    bool transposed;
+    __device__ double operator()(int n, long long k) const {
+        return transposed ? m[(size_t)k * C + n] : m[(size_t)n * C + k];
+    }
+};
+
+// The split operands of W and W H (FP64 matrices built on the device, fold.cu).
 void col_init(mpi_ffl_handle *h) {
     ColState *s = new ColState();
     h->col_state = s;
     const Dims &d = h->d;
     if ((size_t)d.N * 2 * d.nb * 8 > (size_t)1 << 31) return;
     s->n_par = d.n_par;
-    const double kPi = 3.14159265358979323846;
     const int R = 2 * d.nb;
-    // PSF matrix H[e][i] in double
-    const double a = h->fwhm / (2.0 * langevin_half_point_host());
-    std::vector<double> Hm((size_t)d.Ne * d.N);
-    for (int e = 0; e < d.Ne; ++e)
-        for (int i = 0; i < d.N; ++i) {
-            const double u = (double)(e - d.D) / d.Q - i;
-            Hm[(size_t)e * d.N + i] = 3.0 * langevin_d1_host(u / a);
-        }
-    // e^{2 pi i k r / S} and e^{2 pi i delta j / L}
-    std::vector<double> ckr(d.S), skr(d.S);
-    for (int m = 0; m < d.S; ++m) {
-        ckr[m] = std::cos(2.0 * kPi * m / d.S);
-        skr[m] = std::sin(2.0 * kPi * m / d.S);
+    const double *WH = fold_wh(h, 0, nullptr), *W = fold_w_dev(h);
+    if (!WH || !W) {
+        s->oom = true;
+        return;
     }
-    const double isl = 1.0 / std::sqrt((double)d.L);
     for (int par = 0; par < d.n_par; ++par) {
-        std::vector<double> Wr((size_t)R * d.Ne, 0.0);
-        for (int j = 0; j < d.L; ++j) {
-            int n;
-            double f, v;
-            traj_point_host(h, par, j, n, f, v);
-            const int r = j % d.S;
-            for (int di = 0; di < d.W; ++di) {
-                const int64_t dl = di - d.hw;
-                const int64_t num = ((dl * j) % d.L + d.L) % d.L;
-                const double ang = 2.0 * kPi * (double)num / d.L;
-                const double cd = std::cos(ang), sd = std::sin(ang);
-                for (int k = 0; k < d.K; ++k) {
-                    const int o = k * d.W + di;
-                    const int m = (int)(((int64_t)(d.kmin + k) * r) % d.S);
-                    // e^{2 pi i (kP + delta) j / L} = e^{2 pi i k r / S} e^{2 pi i delta j / L}
-                    const double er = ckr[m] * cd - skr[m] * sd, ei = ckr[m] * sd + skr[m] * cd;
-                    const double gr = h->dgamma[2 * o], gi = h->dgamma[2 * o + 1];
-                    const double wr = (gr * er - gi * ei) * isl, wi = (gr * ei + gi * er) * isl;
-                    const double w0 = (1.0 - f) * v, w1 = f * v;
-                    Wr[(size_t)(2 * o) * d.Ne + n] += w0 * wr;
-                    Wr[(size_t)(2 * o + 1) * d.Ne + n] += w0 * wi;
-                    Wr[(size_t)(2 * o) * d.Ne + n + 1] += w1 * wr;
-                    Wr[(size_t)(2 * o + 1) * d.Ne + n + 1] += w1 * wi;
-                }
+        const MatSrc w{W + (size_t)par * R * d.Ne, d.Ne, false}, wt{w.m, d.Ne, true};
+        const MatSrc wh{WH + (size_t)par * R * d.N, d.N, false}, wht{wh.m, d.N, true};
+        auto mk = [&](Packed (&p)[2][2], const MatSrc &m, int Nv, int Kv, int BN, int per_sm) {
+            for (int tf = 0; tf < 2; ++tf) {
+                p[tf][par].per_sm = per_sm;
+                if (!pack_dev(p[tf][par], m, Nv, Kv, BN, tf)) return false;
             }
-        }
-        // transposed W (Ne x R), W H (R x N) and its transpose (N x R)
-        std::vector<double> Wt((size_t)d.Ne * R), WH((size_t)R * d.N, 0.0), WHt((size_t)d.N * R);
-        for (int o = 0; o < R; ++o)
-            for (int e = 0; e < d.Ne; ++e) Wt[(size_t)e * R + o] = Wr[(size_t)o * d.Ne + e];
-        {
-            // rows of W H on the host's cores (each row is independent)
-            const int nt = std::max(1, std::min<int>(R, (int)std::thread::hardware_concurrency()));
-            std::vector<std::thread> pool;
-            for (int t = 0; t < nt; ++t)
-                pool.emplace_back([&, t]() {
-                    for (int o = t; o < R; o += nt) {
-                        double *out = WH.data() + (size_t)o * d.N;
-                        const double *wrow = Wr.data() + (size_t)o * d.Ne;
-                        for (int e = 0; e < d.Ne; ++e) {
-                            const double w = wrow[e];
-                            if (w == 0.0) continue;
-                            const double *hrow = Hm.data() + (size_t)e * d.N;
-                            for (int i = 0; i < d.N; ++i) out[i] += w * hrow[i];
-                        }
-                    }
-                });
-            for (auto &th : pool) th.join();
-        }
-        for (int o = 0; o < R; ++o)
-            for (int i = 0; i < d.N; ++i) WHt[(size_t)i * R + o] = WH[(size_t)o * d.N + i];
-        auto mk1 = [&](Packed &p, const std::vector<double> &m, int Nv, int Kv, int BN, int per_sm, bool tf) {
-            p.BN = BN;
-            p.per_sm = per_sm;
-            return upload_packed(p, pack_b(m, Nv, Kv, BN, p.ntile, p.nkc, tf));
-        };
-        auto mk = [&](Packed (&p)[2][2], const std::vector<double> &m, int Nv, int Kv, int BN, int per_sm) {
-            return mk1(p[0][par], m, Nv, Kv, BN, per_sm, false) && mk1(p[1][par], m, Nv, Kv, BN, per_sm, true);
+            return true;
         };
         // N tile: about two blocks per SM over both trajectories' M tiles
         int n_sm = 152, dev = 0;
@@ -795,12 +732,11 @@ void col_init(mpi_ffl_handle *h) {
         int ps[4];
         const int bn_ef = pick_bn(R, ps[0]), bn_ea = pick_bn(d.Ne, ps[1]);
         const int bn_ff = pick_bn(R, ps[2]), bn_fa = pick_bn(d.N, ps[3]);
-        if (!mk(s->evf_f, Wr, R, d.Ne, bn_ef, ps[0]) || !mk(s->evf_a, Wt, d.Ne, R, bn_ea, ps[1]) ||
-            !mk(s->full_f, WH, R, d.N, bn_ff, ps[2]) || !mk(s->full_a, WHt, d.N, R, bn_fa, ps[3])) {
+        if (!mk(s->evf_f, w, R, d.Ne, bn_ef, ps[0]) || !mk(s->evf_a, wt, d.Ne, R, bn_ea, ps[1]) ||
+            !mk(s->full_f, wh, R, d.N, bn_ff, ps[2]) || !mk(s->full_a, wht, d.N, R, bn_fa, ps[3])) {
             s->oom = true;
             return;
         }
-        s->W[par] = std::move(Wr);
         // lines of this trajectory
         std::vector<int> rows;
         for (int m = 0; m < d.M; ++m)
@@ -828,6 +764,10 @@ void col_init(mpi_ffl_handle *h) {
         return;
     }
     cudaMemset(s->err, 0, sizeof(int));
+    if (cudaStreamSynchronize(nullptr) != cudaSuccess) {  // the operands are packed
+        s->oom = true;
+        return;
+    }
     for (const void *k : {(const void *)k_gemm_split<0>, (const void *)k_gemm_split<1>, (const void *)k_gemm_pair<0>,
                           (const void *)k_gemm_pair<1>, (const void *)k_gemm_pair<0, true>,
                           (const void *)k_gemm_pair<1, true>})
@@ -1068,51 +1008,6 @@ struct TensorState {
     uint32_t cols[2] = {32, 32};  // TMEM columns a block of the forward and adjoint launches holds
 };
 
-// W_{par,d}[o][i] = sum_e W_par[o][e] g_d[e - D - Q i - kmin] in FP64 (g_d[k - kmin] =
-// h_uu(k / Q, d)). A block takes 8 rows o, 128 columns i, one offset and trajectory;
-// e runs in tiles of 256 staged in shared memory with the g values they meet.
-constexpr int kWdRows = 8, kWdCols = 128, kWdTile = 256;
-
-__global__ void __launch_bounds__(kWdCols) k_tensor_wd(const double *__restrict__ W, const double *__restrict__ g,
-                                                       double *__restrict__ Wd, int R, int Ne, int N, int Nz, int D,
-                                                       int Q, int kmin, int Lk) {
-    __shared__ double sw[kWdRows][kWdTile];
-    extern __shared__ double sg[];  // kWdTile + Q (kWdCols - 1) values of g_d
-    const int ncb = (N + kWdCols - 1) / kWdCols;
-    const int o0 = (blockIdx.x / ncb) * kWdRows, i0 = (blockIdx.x % ncb) * kWdCols;
-    const int d = blockIdx.y, par = blockIdx.z;
-    const int il = threadIdx.x, i = i0 + il;
-    const double *Wp = W + (size_t)par * R * Ne;
-    const double *gd = g + (size_t)d * Lk;
-    const int span = kWdTile + Q * (kWdCols - 1);
-    double acc[kWdRows];
-#pragma unroll
-    for (int r = 0; r < kWdRows; ++r) acc[r] = 0.0;
-    for (int e0 = 0; e0 < Ne; e0 += kWdTile) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kWdRows * kWdTile; t += blockDim.x) {
-            const int r = t / kWdTile, e = e0 + t % kWdTile;
-            sw[r][t % kWdTile] = (o0 + r < R && e < Ne) ? Wp[(size_t)(o0 + r) * Ne + e] : 0.0;
-        }
-        // k = e - D - Q i runs from kb (e = e0, i = i0 + kWdCols - 1) upwards
-        const int kb = e0 - D - Q * (i0 + kWdCols - 1) - kmin;
-        for (int t = threadIdx.x; t < span; t += blockDim.x) {
-            const int k = kb + t;
-            sg[t] = (k >= 0 && k < Lk) ? gd[k] : 0.0;
-        }
-        __syncthreads();
-        const double *gl = sg + Q * (kWdCols - 1 - il);
-        for (int e = 0; e < kWdTile; ++e) {
-            const double gv = gl[e];
-#pragma unroll
-            for (int r = 0; r < kWdRows; ++r) acc[r] = fma(sw[r][e], gv, acc[r]);
-        }
-    }
-    if (i < N)
-        for (int r = 0; r < kWdRows; ++r)
-            if (o0 + r < R) Wd[(((size_t)par * Nz + d) * R + o0 + r) * N + i] = acc[r];
-}
-
 // Forward table value T_par[n = o][k = (t + Tpre) Np + i] and adjoint table value
 // Tadj_s[n = i][k = (t + Tpre) Op + o], read from W_{par,|d|} (zero past |d| = Nz - 1).
 struct TenFwdSrc {
@@ -1136,49 +1031,6 @@ struct TenAdjSrc {
         return Wd[(((size_t)par * Nz + abs(dd)) * R + o) * N + n];
     }
 };
-
-__device__ __forceinline__ uint16_t bf16_bits_dev(double x) {
-    const uint32_t u = __float_as_uint((float)x);
-    return (uint16_t)((u + 0x7FFFu + ((u >> 16) & 1u)) >> 16);
-}
-__device__ __forceinline__ uint32_t tf32_bits_dev(double x) {
-    return (__float_as_uint((float)x) + 0x1000u) & 0xFFFFE000u;
-}
-
-// pack_b on the device: one thread per (tile, chunk, row, K element) of the canonical
-// layout; hi = round(v), lo = round(v - hi), in bf16 or tf32.
-template <class Src>
-__global__ void k_pack_b(Src src, int Nv, long long Kv, int BN, int ntile, int nkc, int tf32, uint8_t *out) {
-    const int kpc = tf32 ? kBK / 2 : kBK;
-    const size_t blk = (size_t)BN * kBK * 2;
-    const size_t total = (size_t)ntile * nkc * BN * kpc;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int kl = (int)(idx % kpc);
-        size_t r = idx / kpc;
-        const int nl = (int)(r % BN);
-        r /= BN;
-        const int kc = (int)(r % nkc), t = (int)(r / nkc);
-        const int n = t * BN + nl;
-        const long long k = (long long)kc * kpc + kl;
-        const double v = (n < Nv && k < Kv) ? src(n, k) : 0.0;
-        uint8_t *hi = out + ((size_t)t * nkc + kc) * 2 * blk;
-        uint8_t *lo = hi + blk;
-        if (tf32) {
-            const uint32_t hb = tf32_bits_dev(v);
-            const uint32_t lb = tf32_bits_dev(v - (double)__uint_as_float(hb));
-            const size_t off = (size_t)(nl / 8) * 1024 + (kl / 4) * 128 + (nl % 8) * 16 + (kl % 4) * 4;
-            *reinterpret_cast<uint32_t *>(hi + off) = hb;
-            *reinterpret_cast<uint32_t *>(lo + off) = lb;
-        } else {
-            const uint16_t hb = bf16_bits_dev(v);
-            const uint16_t lb = bf16_bits_dev(v - (double)__uint_as_float((uint32_t)hb << 16));
-            const size_t off = (size_t)(nl / 8) * 1024 + (kl / 8) * 128 + (nl % 8) * 16 + (kl % 8) * 2;
-            *reinterpret_cast<uint16_t *>(hi + off) = hb;
-            *reinterpret_cast<uint16_t *>(lo + off) = lb;
-        }
-    }
-}
 
 // A operand of the tensor-PSF GEMMs, split once per call: row m (angle) of the padded
 // block holds K = Zp * per values, value (zp, c) = b[z][c] in[(m Nz + z) ncols + c] for
@@ -1226,24 +1078,6 @@ __global__ void __launch_bounds__(256) k_pack_rows(const float *__restrict__ in,
     }
 }
 
-template <class Src>
-bool pack_dev(Packed &p, Src src, int Nv, long long Kv, int BN, int tf32) {
-    const int kpc = tf32 ? kBK / 2 : kBK;
-    p.BN = BN;
-    p.ntile = (Nv + BN - 1) / BN;
-    p.nkc = (int)((Kv + kpc - 1) / kpc);
-    const size_t bytes = (size_t)p.ntile * p.nkc * 2 * BN * kBK * 2;
-    if (p.dev) dev_free(p.dev);
-    p.dev = nullptr;
-    if (dev_malloc((void **)&p.dev, bytes) != cudaSuccess) {
-        p.dev = nullptr;
-        cudaGetLastError();
-        return false;
-    }
-    k_pack_b<Src><<<4 * 152 * 8, 256>>>(src, Nv, Kv, BN, p.ntile, p.nkc, tf32, p.dev);
-    return cudaGetLastError() == cudaSuccess;
-}
-
 // h_uu at in-plane offset (u, z) voxels; a = FWHM / (2 x_h)
 double h_uu_host(double u, double z, double a) {
     const double rho2 = u * u + z * z;
@@ -1273,27 +1107,19 @@ bool talloc(T **p, size_t n) {
 bool ten_build_wd(const mpi_ffl_handle *h, ColState *s, TensorState *t) {
     const Dims &d = h->d;
     const int R = 2 * d.nb;
-    const int kmin = -d.D - d.Q * (d.N - 1), Lk = d.Ne + d.Q * (d.N - 1);
+    const int kmin = fold_kmin(d), Lk = fold_taps(d);
     const double a = h->fwhm / (2.0 * langevin_half_point_host());
     std::vector<double> g((size_t)d.Nz * Lk);
     for (int dz = 0; dz < d.Nz; ++dz)
         for (int k = 0; k < Lk; ++k) g[(size_t)dz * Lk + k] = h_uu_host((double)(k + kmin) / d.Q, dz, a);
-    double *dW = nullptr, *dg = nullptr;
-    bool ok = talloc(&dW, (size_t)s->n_par * R * d.Ne) && talloc(&dg, g.size());
+    double *dg = nullptr;
+    bool ok = fold_w_dev(h) && talloc(&dg, g.size());
     if (ok && !t->Wd) ok = talloc(&t->Wd, (size_t)s->n_par * d.Nz * R * d.N);
     if (ok) {
-        for (int par = 0; par < s->n_par; ++par)
-            cudaMemcpy(dW + (size_t)par * R * d.Ne, s->W[par].data(), (size_t)R * d.Ne * sizeof(double),
-                       cudaMemcpyHostToDevice);
         cudaMemcpy(dg, g.data(), g.size() * sizeof(double), cudaMemcpyHostToDevice);
-        const int ncb = (d.N + kWdCols - 1) / kWdCols;
-        const size_t smem = sizeof(double) * (kWdTile + d.Q * (kWdCols - 1));
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k_tensor_wd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_tensor_wd<<<dim3(((R + kWdRows - 1) / kWdRows) * ncb, d.Nz, s->n_par), kWdCols, smem>>>(
-            dW, dg, t->Wd, R, d.Ne, d.N, d.Nz, d.D, d.Q, kmin, Lk);
+        launch_fold_taps(fold_w_dev(h), dg, t->Wd, d, s->n_par, d.Nz, nullptr);
         ok = cudaDeviceSynchronize() == cudaSuccess;
     }
-    if (dW) dev_free(dW);
     if (dg) dev_free(dg);
     cudaGetLastError();
     return ok;
@@ -1441,7 +1267,7 @@ void ten_release(ColState *s) {
 
 int ten_init(mpi_ffl_handle *h) {
     ColState *s = cs(h);
-    if (!s || !s->ok || s->W[0].empty()) return MPI_FFL_ERR_UNSUPPORTED;
+    if (!s || !s->ok || !fold_w_dev(h)) return MPI_FFL_ERR_UNSUPPORTED;
     const Dims &d = h->d;
     const int R = 2 * d.nb;
     ten_release(s);

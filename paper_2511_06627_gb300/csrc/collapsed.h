@@ -6,7 +6,7 @@
 
 namespace mpiffl {
 
-void col_init(mpi_ffl_handle *h);        // builds W and W H in double precision and uploads them
+void col_init(mpi_ffl_handle *h);        // splits W and W H (fold.h) into operands
 void col_release(mpi_ffl_handle *h);
 bool col_supported(const mpi_ffl_handle *h);
 bool col_init_oom(const mpi_ffl_handle *h);  // col_init failed on a device allocation
@@ -47,7 +47,7 @@ void ten_adjoint(mpi_ffl_handle *h, const float *data, const float *coil, float 
 
 // host-side model pieces shared with the table builders (api.cu)
 double langevin_d1_host(double x);
+double langevin_d2_host(double x);
 double langevin_half_point_host();
-void traj_point_host(const mpi_ffl_handle *h, int parity, int j, int &n, double &f, double &v);
 
 }  // namespace mpiffl

@@ -1,0 +1,355 @@
+// The line operator of one trajectory folded to one matrix (Sec. 2.1, Eq. (13)).
+//
+// Every raster line of a trajectory (line parity) sees the same E, V and band DFT, so
+// W = S D_Gamma F V E is one matrix per trajectory and W H, with the PSF folded in, takes
+// a projection straight to the line's kept bins:
+//     W[o][e] = D_o L^-1/2 sum_j e^{2 pi i w_o j / L} (w0_j [n_j = e] + w1_j [n_j + 1 = e])
+//     data[line] = g_m (W H) proj[line],   proj[line] = g_m (W H)^T data[line]
+// Both are built here in FP64 on the device; the tensor-core paths split them to hi + lo
+// operands (collapsed.cu), the staged path applies W H in FP32 (sgemm.cu).
+#include <cmath>
+#include <vector>
+
+#include "collapsed.h"
+#include "fold.h"
+
+namespace mpiffl {
+
+namespace {
+
+struct FoldState {
+    double *W = nullptr;     // [n_par][2 n_b][N_e]
+    double *taps = nullptr;  // one slot's PSF taps
+    double *WH = nullptr;    // [n_par][2 n_b][N]
+    // FP32 operands of slot 0 (h) and 1 (d h / d fwhm): B of the forward [n_par][N][ldf]
+    // and of the adjoint [n_par][2 n_b][lda]
+    float *f[2] = {nullptr, nullptr}, *a[2] = {nullptr, nullptr};
+    int ldf = 0, lda = 0;
+    int *rows = nullptr;  // lines of trajectory 0, then of trajectory 1
+    int nrows[2] = {0, 0};
+};
+
+FoldState *fs(const mpi_ffl_handle *h) { return reinterpret_cast<FoldState *>(h->fold_state); }
+
+template <class T>
+bool falloc(T **p, size_t n) {
+    if (*p) return true;
+    if (dev_malloc((void **)p, n * sizeof(T)) != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
+// A block owns one fine cell of one trajectory, a thread one kept bin: the samples that
+// touch the cell (its CSR list) are taken kWBatch at a time; their weights, phases r and
+// e^{2 pi i delta j / L} are formed once per block in shared memory, and each bin adds
+// w e^{2 pi i k r / S} e^{2 pi i delta j / L} in FP64. Bound by the FP64 pipe (about two
+// FMAs a clock and SM): 0.3 ms at 65536 samples, 144 bins and two trajectories, against
+// some 0.1 s on the host's cores.
+constexpr int kWBatch = 32;
+
+struct FoldTraj {
+    const int *csr_ptr;
+    const CsrEntry *csr;
+    const int2 *tnf;           // (cell n, -) per sample
+    const double *drive;       // [S] A sin(2 pi r / S + phi0)
+    const double *vel;         // [n_par][S]
+    const double2 *unit_s;     // [S] e^{2 pi i m / S}
+    const float2 *dgam;
+    double slope;              // (N - 1) / (L - 1)
+};
+
+__global__ void __launch_bounds__(256) k_fold_w(FoldTraj T, double *__restrict__ W, Dims d) {
+    extern __shared__ double fw_sm[];  // [kWBatch][W] (cos, sin) pairs, then [kWBatch] weights
+    double2 *ph = reinterpret_cast<double2 *>(fw_sm);
+    double *wt = fw_sm + 2 * kWBatch * d.W;
+    int *rr = reinterpret_cast<int *>(wt + kWBatch);
+    const int e = blockIdx.x, par = blockIdx.y;
+    const int *ptr = T.csr_ptr + (size_t)par * (d.Ne + 1);
+    const CsrEntry *ent = T.csr + (size_t)par * 2 * d.L;
+    const int k0 = ptr[e], k1 = ptr[e + 1];
+    for (int o0 = 0; o0 < d.nb; o0 += blockDim.x) {  // uniform trip count
+        const int o = o0 + threadIdx.x;
+        const int kh = d.kmin + o / d.W, di = o % d.W;
+        double ar = 0.0, ai = 0.0;
+        for (int kb = k0; kb < k1; kb += kWBatch) {
+            const int n = min(kWBatch, k1 - kb);
+            __syncthreads();  // the previous batch has been used
+            for (int t = threadIdx.x; t < n * d.W; t += blockDim.x) {
+                const int q = t / d.W, dd = t - q * d.W;
+                const int j = ent[kb + q].j;
+                long long num = (long long)(dd - d.hw) * j % d.L;
+                if (num < 0) num += d.L;
+                double s, c;
+                sincospi(2.0 * (double)num / (double)d.L, &s, &c);
+                ph[t] = make_double2(c, s);
+                if (dd == 0) {
+                    const int r = j % d.S, cell = T.tnf[(size_t)par * d.L + j].x;
+                    const double slow = par ? (double)(d.N - 1) - T.slope * j : T.slope * j;
+                    const double f = (double)d.Q * (slow + T.drive[r]) + (double)d.D - (double)cell;
+                    wt[q] = T.vel[(size_t)par * d.S + r] * (cell == e ? 1.0 - f : f);
+                    rr[q] = r;
+                }
+            }
+            __syncthreads();
+            if (o < d.nb)
+                for (int q = 0; q < n; ++q) {
+                    const double2 u = T.unit_s[(int)((long long)kh * rr[q] % d.S)];
+                    const double2 p = ph[q * d.W + di];
+                    ar = fma(wt[q], u.x * p.x - u.y * p.y, ar);
+                    ai = fma(wt[q], u.x * p.y + u.y * p.x, ai);
+                }
+        }
+        if (o < d.nb) {
+            const double isl = 1.0 / sqrt((double)d.L);
+            const float2 g = T.dgam[o];
+            double *out = W + ((size_t)par * 2 * d.nb + 2 * o) * d.Ne + e;
+            out[0] = isl * ((double)g.x * ar - (double)g.y * ai);
+            out[d.Ne] = isl * ((double)g.x * ai + (double)g.y * ar);
+        }
+    }
+}
+
+// out[par][z][o][i] = sum_e W[par][o][e] g[z][e - D - Q i - kmin]: a block takes 8 rows o,
+// 128 columns i, one z and trajectory; e runs in tiles of 256 staged in shared memory with
+// the taps they meet.
+constexpr int kWdRows = 8, kWdCols = 128, kWdTile = 256;
+
+__global__ void __launch_bounds__(kWdCols) k_fold_taps(const double *__restrict__ W, const double *__restrict__ g,
+                                                       double *__restrict__ out, int R, int Ne, int N, int Nz, int D,
+                                                       int Q, int kmin, int Lk) {
+    __shared__ double sw[kWdRows][kWdTile];
+    extern __shared__ double sg[];  // kWdTile + Q (kWdCols - 1) taps
+    const int ncb = (N + kWdCols - 1) / kWdCols;
+    const int o0 = (blockIdx.x / ncb) * kWdRows, i0 = (blockIdx.x % ncb) * kWdCols;
+    const int d = blockIdx.y, par = blockIdx.z;
+    const int il = threadIdx.x, i = i0 + il;
+    const double *Wp = W + (size_t)par * R * Ne;
+    const double *gd = g + (size_t)d * Lk;
+    const int span = kWdTile + Q * (kWdCols - 1);
+    double acc[kWdRows];
+#pragma unroll
+    for (int r = 0; r < kWdRows; ++r) acc[r] = 0.0;
+    for (int e0 = 0; e0 < Ne; e0 += kWdTile) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < kWdRows * kWdTile; t += blockDim.x) {
+            const int r = t / kWdTile, e = e0 + t % kWdTile;
+            sw[r][t % kWdTile] = (o0 + r < R && e < Ne) ? Wp[(size_t)(o0 + r) * Ne + e] : 0.0;
+        }
+        // k = e - D - Q i runs from kb (e = e0, i = i0 + kWdCols - 1) upwards
+        const int kb = e0 - D - Q * (i0 + kWdCols - 1) - kmin;
+        for (int t = threadIdx.x; t < span; t += blockDim.x) {
+            const int k = kb + t;
+            sg[t] = (k >= 0 && k < Lk) ? gd[k] : 0.0;
+        }
+        __syncthreads();
+        const double *gl = sg + Q * (kWdCols - 1 - il);
+        for (int e = 0; e < kWdTile; ++e) {
+            const double gv = gl[e];
+#pragma unroll
+            for (int r = 0; r < kWdRows; ++r) acc[r] = fma(sw[r][e], gv, acc[r]);
+        }
+    }
+    if (i < N)
+        for (int r = 0; r < kWdRows; ++r)
+            if (o0 + r < R) out[(((size_t)par * Nz + d) * R + o0 + r) * N + i] = acc[r];
+}
+
+// FP32 operands of the staged path from W H: f[par][i][o] (columns past 2 n_b zero) and
+// a[par][o][i] (columns past N zero)
+__global__ void __launch_bounds__(256) k_fold_operands(const double *__restrict__ WH, float *__restrict__ f,
+                                                       float *__restrict__ a, int R, int N, int ldf, int lda) {
+    const int par = blockIdx.y;
+    const double *src = WH + (size_t)par * R * N;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < N * ldf; t += gridDim.x * blockDim.x) {
+        const int i = t / ldf, o = t - i * ldf;
+        f[(size_t)par * N * ldf + t] = o < R ? (float)src[(size_t)o * N + i] : 0.f;
+    }
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < R * lda; t += gridDim.x * blockDim.x) {
+        const int o = t / lda, i = t - o * lda;
+        a[(size_t)par * R * lda + t] = i < N ? (float)src[(size_t)o * N + i] : 0.f;
+    }
+}
+
+FoldState *state(mpi_ffl_handle *h) {
+    if (!h->fold_state) h->fold_state = new FoldState();
+    return fs(h);
+}
+
+// FP64 taps of slot 0 (h) or 1 (d h / d fwhm) at offsets (kmin + k) / Q
+std::vector<double> psf_taps(const mpi_ffl_handle *h, int slot) {
+    const Dims &d = h->d;
+    std::vector<double> g(fold_taps(d));
+    const double a = h->fwhm / (2.0 * langevin_half_point_host());
+    for (size_t k = 0; k < g.size(); ++k) {
+        const double x = (double)((int)k + fold_kmin(d)) / d.Q / a;
+        g[k] = slot ? -3.0 * langevin_d2_host(x) * x / h->fwhm : 3.0 * langevin_d1_host(x);
+    }
+    return g;
+}
+
+int refold(mpi_ffl_handle *h, int slot, cudaStream_t st) {
+    const Dims &d = h->d;
+    FoldState *s = fs(h);
+    const int R = 2 * d.nb;
+    const double *wh = fold_wh(h, slot, st);
+    if (!wh) return MPI_FFL_ERR_OOM;
+    const int work = std::max(d.N * s->ldf, R * s->lda);
+    k_fold_operands<<<dim3(std::min(608, (work + 255) / 256), d.n_par), 256, 0, st>>>(wh, s->f[slot], s->a[slot], R,
+                                                                                     d.N, s->ldf, s->lda);
+    // another stream may use the operands next, and the host taps may be freed
+    return cudaStreamSynchronize(st) == cudaSuccess ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
+}
+
+}  // namespace
+
+int fold_w(mpi_ffl_handle *h) {
+    FoldState *s = state(h);
+    if (s->W) return MPI_FFL_OK;
+    const Dims &d = h->d;
+    const double kPi = 3.14159265358979323846;
+    double *drive = nullptr, *vel = nullptr, *W = nullptr;
+    double2 *unit_s = nullptr;
+    const bool ok = falloc(&drive, d.S) && falloc(&vel, (size_t)d.n_par * d.S) && falloc(&unit_s, d.S) &&
+                    falloc(&W, (size_t)d.n_par * 2 * d.nb * d.Ne);
+    int rc = ok ? MPI_FFL_OK : MPI_FFL_ERR_OOM;
+    if (ok) {
+        std::vector<double> hd(d.S), hv((size_t)d.n_par * d.S);
+        std::vector<double2> hu(d.S);
+        const double slope = (double)(d.N - 1) / (double)(d.L - 1);
+        for (int r = 0; r < d.S; ++r) {
+            const double ph = 2.0 * kPi * r / d.S + h->phase;
+            hd[r] = h->amp * std::sin(ph);
+            for (int par = 0; par < d.n_par; ++par)
+                hv[(size_t)par * d.S + r] = (par ? -slope : slope) + h->amp * (2.0 * kPi / d.S) * std::cos(ph);
+            hu[r] = make_double2(std::cos(2.0 * kPi * r / d.S), std::sin(2.0 * kPi * r / d.S));
+        }
+        cudaMemcpy(drive, hd.data(), hd.size() * sizeof(double), cudaMemcpyHostToDevice);
+        cudaMemcpy(vel, hv.data(), hv.size() * sizeof(double), cudaMemcpyHostToDevice);
+        cudaMemcpy(unit_s, hu.data(), hu.size() * sizeof(double2), cudaMemcpyHostToDevice);
+        const FoldTraj T{h->t_csr_ptr, h->t_csr, h->t_tnf, drive, vel, unit_s, h->t_dgam, slope};
+        const size_t smem = sizeof(double) * (2 * kWBatch * d.W + kWBatch) + sizeof(int) * kWBatch;
+        const int threads = std::min(256, (d.nb + 31) / 32 * 32);
+        k_fold_w<<<dim3(d.Ne, d.n_par), threads, smem>>>(T, W, d);
+        if (cudaStreamSynchronize(nullptr) != cudaSuccess) rc = MPI_FFL_ERR_CUDA;
+    }
+    for (void *p : {(void *)drive, (void *)vel, (void *)unit_s})
+        if (p) dev_free(p);
+    if (rc == MPI_FFL_OK) s->W = W;
+    else if (W) dev_free(W);
+    return rc;
+}
+
+const double *fold_w_dev(const mpi_ffl_handle *h) { return fs(h) ? fs(h)->W : nullptr; }
+
+void launch_fold_taps(const double *W, const double *g, double *out, const Dims &d, int n_par, int nz,
+                      cudaStream_t st) {
+    const int R = 2 * d.nb, ncb = (d.N + kWdCols - 1) / kWdCols;
+    const size_t smem = sizeof(double) * (kWdTile + d.Q * (kWdCols - 1));
+    if (smem > 32 * 1024) cudaFuncSetAttribute(k_fold_taps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_fold_taps<<<dim3(((R + kWdRows - 1) / kWdRows) * ncb, nz, n_par), kWdCols, smem, st>>>(
+        W, g, out, R, d.Ne, d.N, nz, d.D, d.Q, fold_kmin(d), fold_taps(d));
+}
+
+const double *fold_wh(mpi_ffl_handle *h, int slot, cudaStream_t st) {
+    const Dims &d = h->d;
+    if (fold_w(h) != MPI_FFL_OK) return nullptr;
+    FoldState *s = fs(h);
+    if (!falloc(&s->taps, fold_taps(d)) || !falloc(&s->WH, (size_t)d.n_par * 2 * d.nb * d.N)) return nullptr;
+    const std::vector<double> g = psf_taps(h, slot);
+    // pageable memory: the copy has left the host vector when the call returns
+    if (cudaMemcpyAsync(s->taps, g.data(), g.size() * sizeof(double), cudaMemcpyHostToDevice, st) != cudaSuccess)
+        return nullptr;
+    launch_fold_taps(s->W, s->taps, s->WH, d, d.n_par, 1, st);
+    return s->WH;
+}
+
+// The folded stage costs 2 n_b N FMAs a line, the stage kernels N N_e (H), about
+// L (2 w + 3) (resampling and band DFT) and the signal's way through HBM: the stages are
+// cheaper only for short lines with wide bands. W is kept in FP64 (at most 512 MB). With
+// the stages an FP32 pair took 1617 us at 256^2 x 128 and 36 angles, 299 us at 128^2 x 64
+// and 24; folded 276 and 70 us, with smaller errors against 64 bits (one rounded matrix in
+// the place of rounded taps, weights and twiddles). A band of 2 n_b = 180 and lines of 256
+// samples on 20 bins (N_e = 109) is on the other side of the line.
+bool fold_fits(const Dims &d) {
+    const double folded = 2.0 * d.nb * d.N, staged = (double)d.N * d.Ne + (double)d.L * (d.W + 2);
+    return folded <= staged && (double)d.n_par * 2 * d.nb * d.Ne * sizeof(double) <= 512e6;
+}
+
+int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
+    const Dims &d = h->d;
+    FoldState *s = state(h);
+    if (s->f[slot]) return MPI_FFL_OK;
+    const int R = 2 * d.nb;
+    if (!s->rows) {
+        std::vector<int> rows;
+        for (int par = 0; par < d.n_par; ++par) {
+            for (int m = 0; m < d.M; ++m)
+                for (int z = par; z < d.Nz; z += d.n_par) rows.push_back(m * d.Nz + z);
+            s->nrows[par] = (int)rows.size() - (par ? s->nrows[0] : 0);
+        }
+        if (!falloc(&s->rows, rows.size())) return MPI_FFL_ERR_OOM;
+        cudaMemcpy(s->rows, rows.data(), rows.size() * sizeof(int), cudaMemcpyHostToDevice);
+    }
+    s->ldf = (R + 3) / 4 * 4;
+    s->lda = (d.N + 3) / 4 * 4;
+    int rc = MPI_FFL_ERR_OOM;
+    if (falloc(&s->f[slot], (size_t)d.n_par * d.N * s->ldf) && falloc(&s->a[slot], (size_t)d.n_par * R * s->lda))
+        rc = refold(h, slot, st);
+    if (rc != MPI_FFL_OK)  // nothing of a failed build is kept: the next call tries again
+        for (float **p : {&s->f[slot], &s->a[slot]})
+            if (*p) {
+                dev_free(*p);
+                *p = nullptr;
+            }
+    return rc;
+}
+
+void fold_forward(mpi_ffl_handle *h, int slot, const float *proj, const float *gain, float *data, cudaStream_t st) {
+    const Dims &d = h->d;
+    const FoldState *s = fs(h);
+    SgemmArgs g[2];
+    for (int par = 0; par < d.n_par; ++par) {
+        const int *rows = s->rows + (par ? s->nrows[0] : 0);
+        g[par] = SgemmArgs{proj, d.N,      rows, s->nrows[par], d.N,  s->f[slot] + (size_t)par * d.N * s->ldf,
+                           s->ldf, data,   2 * d.nb, rows,      2 * d.nb, gain, d.Nz};
+    }
+    launch_sgemm(g, d.n_par, st);
+}
+
+void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float *proj, cudaStream_t st) {
+    const Dims &d = h->d;
+    const FoldState *s = fs(h);
+    const int R = 2 * d.nb;
+    SgemmArgs g[2];
+    for (int par = 0; par < d.n_par; ++par) {
+        const int *rows = s->rows + (par ? s->nrows[0] : 0);
+        g[par] = SgemmArgs{data, R,    rows, s->nrows[par], R,   s->a[0] + (size_t)par * R * s->lda,
+                           s->lda, proj, d.N, rows,          d.N, gain, d.Nz};
+    }
+    launch_sgemm(g, d.n_par, st);
+}
+
+int fold_psf_changed(mpi_ffl_handle *h) {
+    FoldState *s = fs(h);
+    for (int slot = 0; s && slot < 2; ++slot)
+        if (s->f[slot]) {
+            const int rc = refold(h, slot, nullptr);
+            if (rc != MPI_FFL_OK) return rc;
+        }
+    return MPI_FFL_OK;
+}
+
+void fold_release(mpi_ffl_handle *h) {
+    FoldState *s = fs(h);
+    if (!s) return;
+    for (void *p : {(void *)s->W, (void *)s->taps, (void *)s->WH, (void *)s->f[0], (void *)s->f[1], (void *)s->a[0],
+                    (void *)s->a[1], (void *)s->rows})
+        if (p) dev_free(p);
+    delete s;
+    h->fold_state = nullptr;
+}
+
+}  // namespace mpiffl

@@ -1,0 +1,51 @@
+// The line operator of one trajectory folded to a matrix in FP64 on the device, and the
+// FP32 matrix products that apply it (fold.cu).
+#pragma once
+
+#include "internal.h"
+
+namespace mpiffl {
+
+// FP64 matrices, one per trajectory: W = S D_Gamma F V E ([2 n_b][N_e], rows alternating
+// Re and Im of the kept bins) and taps applied to it, W T ([2 n_b][N]) with
+// T[e][i] = taps[e - D - Q i - kmin].
+int fold_w(mpi_ffl_handle *h);                  // builds W on first use; MPI_FFL_OK or an error
+const double *fold_w_dev(const mpi_ffl_handle *h);  // [n_par][2 n_b][N_e], after fold_w
+// first index k = e - D - Q i of the taps and their count
+inline int fold_kmin(const Dims &d) { return -d.D - d.Q * (d.N - 1); }
+inline int fold_taps(const Dims &d) { return d.Ne + d.Q * (d.N - 1); }
+// out[par][z][o][i] = sum_e W[par][o][e] g[z][e - D - Q i - kmin], z < nz, on the stream
+void launch_fold_taps(const double *W, const double *g, double *out, const Dims &d, int n_par, int nz,
+                      cudaStream_t st);
+// W H in FP64 ([n_par][2 n_b][N]) for the handle's PSF (slot 0) or d H / d fwhm (slot 1),
+// valid until the next call; NULL when an allocation failed
+const double *fold_wh(mpi_ffl_handle *h, int slot, cudaStream_t st);
+
+// Staged path: W H in FP32, applied to the projections (forward) or to the data (adjoint).
+bool fold_fits(const Dims &d);                  // the rule by sizes
+int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st);  // operands built on first use
+void fold_forward(mpi_ffl_handle *h, int slot, const float *proj, const float *gain, float *data, cudaStream_t st);
+void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float *proj, cudaStream_t st);
+int fold_psf_changed(mpi_ffl_handle *h);        // refolds the operands that were built
+void fold_release(mpi_ffl_handle *h);
+
+// C[crow[i]][n] = scale[arow[i] / rdiv] sum_k A[arow[i]][k] B[k][n] in FP32 (arow, crow and
+// scale may be NULL: row i, row i and 1). B is K x ldb, ldb a multiple of 4, on 16 bytes.
+struct SgemmArgs {
+    const float *A;
+    int64_t lda;
+    const int *arow;
+    int M, K;
+    const float *B;
+    int ldb;
+    float *C;
+    int64_t ldc;
+    const int *crow;
+    int N;
+    const float *scale;
+    int rdiv;
+};
+// n problems (1 or 2) of one kind in one launch
+void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st);
+
+}  // namespace mpiffl

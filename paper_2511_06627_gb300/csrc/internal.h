@@ -181,6 +181,7 @@ struct mpi_ffl_handle {
     void *tc_twb = nullptr;
     void *tc_state = nullptr;
     void *col_state = nullptr;  // collapsed line operator (collapsed.cu)
+    void *fold_state = nullptr; // its FP64 matrices and the staged path's FP32 operands (fold.cu)
     int path = 0;               // MPI_FFL_PATH_*
     int64_t bytes = 0;
     // host buffers given to forward/adjoint: device staging, allocated on first use

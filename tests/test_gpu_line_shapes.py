@@ -45,3 +45,42 @@ def test_band_dft_with_an_odd_number_of_periods(S, P):
     y = (rng.standard_normal(st.data_shape) + 1j * rng.standard_normal(st.data_shape)).astype(np.complex64)
     got = _n(op.apply_stage(3, _t(to_interleaved(y)), transpose=True))
     assert rel_l2(got, operator.compress_adj(y, st)) < OP_TOL
+
+
+# the staged path's folded line stage: both tile sizes of its matrix product with ragged
+# edges, one trajectory and two, and a short line with a wide band, which keeps the stages
+STAGED = {
+    "ragged": dict(nx=33, nz=7, n_angles=5, S=12, P=40, k_max=4, half_width=2),
+    "one trajectory": dict(nx=38, nz=9, n_angles=4, zigzag=0, S=16, P=33, k_max=6, half_width=0),
+    "large tiles": dict(nx=50, nz=129, n_angles=26, S=16, P=50, k_max=6, half_width=4),
+    "stages": dict(nx=20, nz=6, n_angles=3, S=64, P=4, k_max=30, half_width=1),
+}
+
+
+@pytest.mark.parametrize("name", list(STAGED))
+def test_staged_path_against_the_oracle(name):
+    st, op = _make(**STAGED[name])
+    rng = np.random.default_rng(6)
+    gains = (1 + 0.1 * rng.standard_normal(st.n_angles)).astype(np.float32)
+    op.set_gain(gains)
+    st.gains = gains.astype(np.float64)
+    m = np.array([st.n_angles - 1])  # one angle is enough to place every line
+    x = rng.standard_normal((st.nz, st.nx, st.nx)).astype(np.float32)
+    y = np.zeros(st.data_shape, dtype=np.complex64)
+    y[m] = rng.standard_normal(y[m].shape) + 1j * rng.standard_normal(y[m].shape)
+    for fwhm in (2.5, 3.25):  # the second width refolds the operands
+        op.set_fwhm(fwhm)
+        st.fwhm = fwhm
+        ref = operator.forward_stages(x, st, angles=m)
+        assert rel_l2(_n(op.forward(_t(x)))[m], to_interleaved(ref["data"])) < OP_TOL
+        assert rel_l2(_n(op.adjoint(_t(to_interleaved(y)))), operator.adjoint_stages(y[m], st, angles=m)["vol"]) < OP_TOL
+        dfine = ref["proj"] @ operator.psf.dh_dfwhm((np.arange(st.n_fine)[:, None] - st.D) / st.Q
+                                                     - np.arange(st.nx)[None, :], fwhm).T
+        db = operator.compress_fwd(operator.resample_fwd(dfine, st, m), st)
+        gb = np.zeros(st.data_shape, dtype=np.complex64)
+        gb[m] = db  # the width gradient's inner product without cancellation
+        gg, gw = op.param_grad(_t(x), _t(to_interleaved(gb)))
+        assert abs(float(gw) / np.vdot(gb[m], db).real - 1) < 2 * OP_TOL
+        bare = np.vdot(gb[m], ref["data"] / gains[m[0]]).real
+        assert abs(float(gg[m[0]]) - bare) < OP_TOL * np.linalg.norm(gb) * np.linalg.norm(ref["data"])
+    op.close()
