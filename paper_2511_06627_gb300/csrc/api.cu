@@ -417,6 +417,7 @@ void release(mpi_ffl_handle *h) {
     tc_release(h);
     col_release(h);
     fold_release(h);
+    zfold_release(h);
 }
 
 // ------------------------------------------------------------ host buffers
@@ -1214,7 +1215,7 @@ extern "C" int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm) {
         CK(cudaMemcpy(h->t_htab, ht.data(), sizeof(float) * ht.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->t_dhtab, dht.data(), sizeof(float) * dht.size(), cudaMemcpyHostToDevice));
         tc_tables_changed(h);
-        if (fold_psf_changed(h) != MPI_FFL_OK) {
+        if (fold_psf_changed(h) != MPI_FFL_OK || zfold_psf_changed(h) != MPI_FFL_OK) {
             h->err = "the folded line operator could not be rebuilt";
             return MPI_FFL_ERR_CUDA;
         }
@@ -1392,9 +1393,6 @@ void z_init(mpi_ffl_handle *h) {
     upload(h, &h->tz_phi, phi);
     upload(h, &h->tz_tap_ptr, ptr);
     upload(h, &h->tz_taps, taps);
-    dev_alloc(h, &h->w_fine_z, (size_t)d.M * N * d.Nez);
-    dev_alloc(h, &h->w_projT, (size_t)d.M * N * d.Nz);
-    dev_alloc(h, &h->w_zcoef, (size_t)d.M * d.Nz * (2 * d.hw + 1) * S);
     h->z_ready = 1;
 }
 
@@ -1413,14 +1411,20 @@ Dims z_dims(const Dims &d) {
     return dz;
 }
 
+void ensure_projT(mpi_ffl_handle *h) {
+    if (!h->w_projT) dev_alloc(h, &h->w_projT, (size_t)h->d.M * h->d.N * h->d.Nz);
+}
+
 void zstage_h(mpi_ffl_handle *h, const float *proj, float *cz, cudaStream_t st) {
     const Dims &d = h->d;
+    ensure_projT(h);
     TIMED(MPI_FFL_K_ZDRIVE, launch_transpose_2d(proj, h->w_projT, d.M, d.Nz, d.N, st));
     TIMED(MPI_FFL_K_PSF_FWD, launch_psf_fwd(h->w_projT, h->t_htab, cz, z_dims(d), st));
 }
 
 void zstage_ht(mpi_ffl_handle *h, const float *cz, float *proj, cudaStream_t st) {
     const Dims &d = h->d;
+    ensure_projT(h);
     TIMED(MPI_FFL_K_PSF_ADJ, launch_psf_adj(cz, h->t_htab, h->w_projT, z_dims(d), st));
     TIMED(MPI_FFL_K_ZDRIVE, launch_transpose_2d(h->w_projT, proj, d.M, d.N, d.Nz, st));
 }
@@ -1434,10 +1438,35 @@ void zstage_evt(mpi_ffl_handle *h, const float *sig, float *cz, cudaStream_t st)
     TIMED(MPI_FFL_K_ZDRIVE, launch_resample_z_adj(sig, z_tables(h), h->t_gain, h->w_tz, cz, h->d, h->zigzag, st));
 }
 
+// Whether the folded z-drive kernels serve this shape; their tables are built on first use.
+bool use_zfold(mpi_ffl_handle *h) {
+    if (!zfold_fits(h->d)) return false;
+    const int rc = zfold_ready(h);
+    if (rc != MPI_FFL_OK) {
+        set_err(h, "building the z-drive tables failed");
+        throw Fail{rc};
+    }
+    return true;
+}
+
+void ensure_z_workspace(mpi_ffl_handle *h) {
+    const Dims &d = h->d;
+    if (!h->w_fine_z) dev_alloc(h, &h->w_fine_z, (size_t)d.M * d.N * d.Nez);
+    if (!h->w_zcoef) dev_alloc(h, &h->w_zcoef, (size_t)d.M * d.Nz * (2 * d.hw + 1) * d.S);
+}
+
 void forward_z_impl(mpi_ffl_handle *h, const float *x, float *b, cudaStream_t st) {
     const Dims &d = h->d;
     z_init(h);
+    const bool folded = use_zfold(h);
     stage_p(h, x, h->w_proj, st);
+    if (folded) {
+        TIMED(MPI_FFL_K_ZDRIVE, zfold_forward(h, h->w_proj, b, st));
+        h->launches += 2;  // a convolution and the band DFT's products in the same timed stage
+        check_launch(h, "z-drive forward");
+        return;
+    }
+    ensure_z_workspace(h);
     zstage_h(h, h->w_proj, h->w_fine_z, st);
     // E_z V_z B fused with S D_Gamma F: the time signal is not stored
     TIMED(MPI_FFL_K_ZDRIVE, launch_zdft_fwd(h->w_fine_z, z_tables(h), h->t_gain, h->t_tw1, h->t_tw2_ro, h->t_dgam, b,
@@ -1448,6 +1477,14 @@ void forward_z_impl(mpi_ffl_handle *h, const float *x, float *b, cudaStream_t st
 void adjoint_z_impl(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st) {
     const Dims &d = h->d;
     z_init(h);
+    if (use_zfold(h)) {
+        TIMED(MPI_FFL_K_ZDRIVE, zfold_adjoint(h, b, h->w_proj, st));
+        h->launches += 2;
+        stage_pt(h, h->w_proj, x, st);
+        check_launch(h, "z-drive adjoint");
+        return;
+    }
+    ensure_z_workspace(h);
     TIMED(MPI_FFL_K_ZDRIVE, launch_zdft_adj(b, h->t_tw1, h->t_tw2_qr, h->t_dgam, z_tables(h), h->t_gain,
                                             h->w_zcoef, h->w_fine_z, d, h->zigzag, st));
     zstage_ht(h, h->w_fine_z, h->w_proj, st);

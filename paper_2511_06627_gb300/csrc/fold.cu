@@ -314,7 +314,7 @@ void fold_forward(mpi_ffl_handle *h, int slot, const float *proj, const float *g
     for (int par = 0; par < d.n_par; ++par) {
         const int *rows = s->rows + (par ? s->nrows[0] : 0);
         g[par] = SgemmArgs{proj, d.N,      rows, s->nrows[par], d.N,  s->f[slot] + (size_t)par * d.N * s->ldf,
-                           s->ldf, data,   2 * d.nb, rows,      2 * d.nb, gain, d.Nz};
+                           s->ldf, data,   2 * d.nb, rows,      2 * d.nb, gain, d.Nz, nullptr, nullptr};
     }
     launch_sgemm(g, d.n_par, st);
 }
@@ -327,7 +327,7 @@ void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float
     for (int par = 0; par < d.n_par; ++par) {
         const int *rows = s->rows + (par ? s->nrows[0] : 0);
         g[par] = SgemmArgs{data, R,    rows, s->nrows[par], R,   s->a[0] + (size_t)par * R * s->lda,
-                           s->lda, proj, d.N, rows,          d.N, gain, d.Nz};
+                           s->lda, proj, d.N, rows,          d.N, gain, d.Nz, nullptr, nullptr};
     }
     launch_sgemm(g, d.n_par, st);
 }

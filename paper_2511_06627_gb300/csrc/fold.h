@@ -29,8 +29,9 @@ void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float
 int fold_psf_changed(mpi_ffl_handle *h);        // refolds the operands that were built
 void fold_release(mpi_ffl_handle *h);
 
-// C[crow[i]][n] = scale[arow[i] / rdiv] sum_k A[arow[i]][k] B[k][n] in FP32 (arow, crow and
-// scale may be NULL: row i, row i and 1). B is K x ldb, ldb a multiple of 4, on 16 bytes.
+// C[crow[i]][ccol[n]] = scale[arow[i] / rdiv] sum_k A[arow[i]][acol[k]] B[k][n] in FP32
+// (arow, crow, acol and ccol may be NULL: row i, column k or n; scale NULL: 1). B is K x
+// ldb, ldb a multiple of 4, on 16 bytes.
 struct SgemmArgs {
     const float *A;
     int64_t lda;
@@ -44,8 +45,17 @@ struct SgemmArgs {
     int N;
     const float *scale;
     int rdiv;
+    const int *acol, *ccol;
 };
-// n problems (1 or 2) of one kind in one launch
+constexpr int kSgemmMax = 9;  // problems of one launch
 void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st);
+
+// The z-drive scan with the raster and the PSF along z folded to tables (k_zfold.cu).
+bool zfold_fits(const Dims &d);                      // the rule by sizes
+int zfold_ready(mpi_ffl_handle *h);                  // tables and workspace, on first use
+void zfold_forward(mpi_ffl_handle *h, const float *proj, float *data, cudaStream_t st);
+void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream_t st);
+int zfold_psf_changed(mpi_ffl_handle *h);
+void zfold_release(mpi_ffl_handle *h);
 
 }  // namespace mpiffl

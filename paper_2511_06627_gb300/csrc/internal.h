@@ -207,6 +207,8 @@ struct mpi_ffl_handle {
     int *tz_optr = nullptr;
     int2 *tz_otap = nullptr;
     int tz_no = 0;
+    void *zfold_state = nullptr;  // folded tables and workspace (k_zfold.cu)
+    // workspace of the sample-by-sample kernels and of the z stages, on their first use
     float *w_fine_z = nullptr;  // M N N_ez
     float *w_zcoef = nullptr;   // M N_z W S (synthesis coefficients of the z adjoint)
     float *w_projT = nullptr;   // M N N_z (projections by column)

@@ -1,0 +1,400 @@
+// The z-drive scan (k_zdrive.cu has its model) with the slow raster and the PSF folded to
+// tables. A sample reads the z-convolved projection at (u = c_j, z = l + A sin(phase r)),
+// j = p S + r: the drive phase r sets the z offset and the period p the column. The sum
+// over the periods of a phase, with the band DFT's period twiddles, is then a fixed
+// combination of the detector's columns, and H_z commutes with it:
+//     G[m][z'][par][c][r] = sum_u K_par[c][r][u] p[m][z'][u]
+//         K_par[c][r][u] = sum_p hat(c_{pS+r} - u) tw_c(p), tw = cos(2 pi d p / P) (c = 0 or
+//         2d - 1), sin(2 pi d p / P) (c = 2d)
+//     T[m][l][c][r] = sum_z' hz[l - z'][r] G[m][z'][par(l)][c][r],
+//         hz[k][r] = v_r h(k + A sin(2 pi r / S + phi0)) as interpolated on the fine z grid
+//     data[m][l][k, +-d] = g_m D L^-1/2 sum_r (T[2d-1][r] +- i T[2d][r]) e^{2 pi i (kP +- d) r / L}
+// The first and last steps are FP32 matrix products (sgemm.cu, the last one per d), the
+// middle one a convolution along z per phase; neither the time signal, nor the fine z grid,
+// nor a transposed projection is formed. The tables are rounded once from FP64. The
+// adjoint runs the transposed steps in the opposite order.
+#include <cmath>
+#include <vector>
+
+#include "collapsed.h"
+#include "f32x2.cuh"
+#include "fold.h"
+#include "tc_ptx.cuh"
+
+namespace mpiffl {
+
+namespace {
+
+struct ZFold {
+    float *kf = nullptr;   // K, B operand of the forward [N][ldk], columns (par, c, r)
+    float *ka = nullptr;   // K, B operand of the adjoint [n_par W S][ldu]
+    float *hz = nullptr;   // [2 N_z - 1][S]
+    float *df = nullptr;   // DFT operands of the forward, per d [S or 2 S][2 or 4 K]
+    float *da = nullptr;   // and of the adjoint (their transposes)
+    int *cols = nullptr;   // per d: data column of operand column (k, sign, re / im)
+    float *g = nullptr;    // [M][N_z][n_par][W][S]
+    float *t = nullptr;    // [M][N_z][W][S]
+    int ldk = 0, ldu = 0;
+    bool ready = false;
+};
+
+ZFold *zs(const mpi_ffl_handle *h) { return reinterpret_cast<ZFold *>(h->zfold_state); }
+
+template <class T>
+bool zalloc(T **p, size_t n) {
+    if (*p) return true;
+    if (dev_malloc((void **)p, n * sizeof(T)) != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+        return false;
+    }
+    return true;
+}
+
+// One thread per (par, c, r) walks the periods in the order of increasing column, keeps the
+// sums of the two columns the sample lies between and writes a column once it is complete.
+// The slow position c = (N - 1) j / (L - 1) (from the other end on reversed lines) is exact.
+__global__ void __launch_bounds__(128) k_zfold_k(const double2 *__restrict__ unit_p, float *__restrict__ kf,
+                                                 float *__restrict__ ka, Dims d, int ldk, int ldu) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= d.n_par * d.W * d.S) return;
+    const int r = n % d.S, c = n / d.S % d.W, par = n / (d.S * d.W);
+    const int dd = (c + 1) / 2;
+    const bool sine = c > 0 && c % 2 == 0;
+    const long long N1 = d.N - 1, Lm1 = d.L - 1;
+    double acc0 = 0.0, acc1 = 0.0;
+    int u = 0;
+    auto flush = [&]() {
+        if (u < d.N) {
+            kf[(size_t)u * ldk + n] = (float)acc0;
+            ka[(size_t)n * ldu + u] = (float)acc0;
+        }
+        acc0 = acc1;
+        acc1 = 0.0;
+        ++u;
+    };
+    for (int q = 0; q < d.P; ++q) {
+        const int p = par ? d.P - 1 - q : q;
+        const long long j = (long long)p * d.S + r;
+        const long long num = N1 * (par ? Lm1 - j : j);
+        const int u0 = (int)(num / Lm1);
+        const double a = (double)(num - (long long)u0 * Lm1) / (double)Lm1;
+        while (u < u0) flush();
+        const double2 w = unit_p[(int)((long long)dd * p % d.P)];
+        const double tw = sine ? w.y : w.x;
+        acc0 = fma(1.0 - a, tw, acc0);
+        acc1 = fma(a, tw, acc1);
+    }
+    while (u < d.N) flush();
+}
+
+// hz[k][r]: taps h at offset k voxels of the fine cells n0_r and n0_r + 1, interpolated, times v_r
+__global__ void __launch_bounds__(128) k_zfold_h(const double *__restrict__ taps, const double2 *__restrict__ drive,
+                                                 float *__restrict__ hz, int Nz, int S, int Q, int D) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;  // offset k - (Nz - 1)
+    if (r >= S) return;
+    const double t = drive[r].x;  // Q A sin + D
+    const int n0 = (int)floor(t);
+    const double f = t - n0;
+    const double *h = taps + (size_t)Q * k + n0;  // taps[i] = h((i - D) / Q - (Nz - 1))
+    hz[(size_t)k * S + r] = (float)(drive[r].y * (f > 0.0 ? (1.0 - f) * h[0] + f * h[1] : h[0]));
+}
+
+// Place of the operands of offset d in their arrays: the forward's [rows][ldf] and the
+// adjoint's [cols][lda], leading dimensions rounded up to 4.
+struct DftOperand {
+    int rows, cols, ldf, lda;
+    size_t off_f, off_a, off_c;
+    __host__ __device__ DftOperand(const Dims &d, int dd) {
+        const int r0 = d.S, r1 = 2 * d.S, c0 = 2 * d.K, c1 = 4 * d.K;
+        rows = dd ? r1 : r0;
+        cols = dd ? c1 : c0;
+        ldf = (cols + 3) / 4 * 4;
+        lda = (rows + 3) / 4 * 4;
+        off_f = dd ? (size_t)r0 * ((c0 + 3) / 4 * 4) + (size_t)(dd - 1) * r1 * ldf : 0;
+        off_a = dd ? (size_t)c0 * ((r0 + 3) / 4 * 4) + (size_t)(dd - 1) * c1 * lda : 0;
+        off_c = dd ? c0 + (size_t)(dd - 1) * c1 : 0;
+    }
+};
+
+// Operand of harmonic offset d: rows (part, r), part 0 the cosine sums and 1 the sine sums
+// (d = 0 has part 0 only), columns (k, sign, re / im)
+__global__ void __launch_bounds__(128) k_zfold_dft(const float2 *__restrict__ dgam, float *__restrict__ df,
+                                                   float *__restrict__ da, int *__restrict__ cols, Dims d) {
+    const int dd = blockIdx.y;
+    const DftOperand q(d, dd);
+    const int rows = q.rows, ncol = q.cols;
+    const double isl = 1.0 / sqrt((double)d.L);
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < rows * ncol; t += gridDim.x * blockDim.x) {
+        const int row = t / ncol, col = t - row * ncol;
+        const int part = row / d.S, r = row - part * d.S;
+        const int k = dd ? col / 4 : col / 2, neg = dd ? (col >> 1) & 1 : 0, im = col & 1;
+        const int o = k * d.W + d.hw + (neg ? -dd : dd);
+        const long long w = (long long)(d.kmin + k) * d.P + (neg ? -dd : dd);
+        double s, c;
+        sincospi(2.0 * (double)(w * r % d.L) / (double)d.L, &s, &c);
+        const float2 g = dgam[o];
+        const double zr = isl * ((double)g.x * c - (double)g.y * s), zi = isl * ((double)g.x * s + (double)g.y * c);
+        // part 1 carries +-i z
+        const double sg = neg ? -1.0 : 1.0;
+        const double v = part == 0 ? (im ? zi : zr) : (im ? sg * zr : -sg * zi);
+        df[q.off_f + (size_t)row * q.ldf + col] = (float)v;
+        da[q.off_a + (size_t)col * q.lda + row] = (float)v;
+        if (row == 0) cols[q.off_c + col] = 2 * o + im;
+    }
+}
+
+// Convolution along z, one thread per drive phase r. Outputs o_i = q + n_par (R g + i) of
+// one class q modulo n_par: lines of trajectory par = q (forward, from every slice) or
+// slices (adjoint, from the lines of trajectory par). From one input to the next of its
+// class the taps of the R outputs move by one output, so each input costs one new tap and
+// W values for R W FMAs (pairs of outputs in one fma.rn.f32x2). The next input's values are
+// loaded ahead. Bound by the FP32 pipes and by the reads of the inputs from L2, which R
+// outputs share.
+template <int W, int R, bool ADJ>
+__global__ void __launch_bounds__(128) k_zconv(const float *__restrict__ in, const float *__restrict__ hz,
+                                               float *__restrict__ out, int Nz, int S, int np) {
+    const int ng = ((Nz + np - 1) / np + R - 1) / R;
+    int b = blockIdx.x;
+    const int grp = b % ng;
+    b /= ng;
+    int q = b % np;
+    b /= np;
+    int par = q;
+    if (ADJ) {
+        par = b % np;
+        b /= np;
+    }
+    const int m = b;
+    const int r = blockIdx.y * blockDim.x + threadIdx.x, re = min(r, S - 1);
+    const int o0 = q + np * R * grp;
+    if (o0 >= Nz) return;
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    const size_t WS = (size_t)W * S;
+    const size_t istride = ADJ ? WS : np * WS;
+    const float *src = in + (size_t)m * Nz * istride + (ADJ ? 0 : par * WS) + re;
+    const float *tap = hz + (size_t)(Nz - 1) * S + re;  // offset 0
+    f32x2 acc[R / 2][W];
+#pragma unroll
+    for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+        for (int c = 0; c < W; ++c) acc[i][c] = 0;
+    for (int cls = ADJ ? par : 0; cls < (ADJ ? par + 1 : np); ++cls) {
+        float w[R], v[W];
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const int k = ADJ ? cls - (o0 + np * i) : o0 + np * i - cls;
+            w[i] = __ldg(tap + (long long)min(max(k, 1 - Nz), Nz - 1) * S);
+        }
+        if (cls < Nz) {
+#pragma unroll
+            for (int c = 0; c < W; ++c) v[c] = __ldg(src + cls * istride + (size_t)c * S);
+        }
+        for (int j = cls; j < Nz; j += np) {
+            const int jn = j + np;
+            float vn[W], wn = 0.f;
+#pragma unroll
+            for (int c = 0; c < W; ++c) vn[c] = 0.f;
+            if (jn < Nz) {
+                wn = __ldg(tap + (long long)(ADJ ? jn - o0 : o0 - jn) * S);
+#pragma unroll
+                for (int c = 0; c < W; ++c) vn[c] = __ldg(src + jn * istride + (size_t)c * S);
+            }
+            f32x2 wp[R / 2];
+#pragma unroll
+            for (int i = 0; i < R / 2; ++i) wp[i] = pack2(w[2 * i], w[2 * i + 1]);
+#pragma unroll
+            for (int c = 0; c < W; ++c) {
+                const f32x2 vv = dup2(v[c]);
+#pragma unroll
+                for (int i = 0; i < R / 2; ++i) acc[i][c] = fma2(wp[i], vv, acc[i][c]);
+            }
+#pragma unroll
+            for (int i = R - 1; i > 0; --i) w[i] = w[i - 1];
+            w[0] = wn;
+#pragma unroll
+            for (int c = 0; c < W; ++c) v[c] = vn[c];
+        }
+    }
+    if (r >= S) return;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int o = o0 + np * i;
+        if (o >= Nz) break;
+        float *dst = out + ((size_t)m * Nz + o) * (ADJ ? np * WS : WS) + (ADJ ? par * WS : 0) + r;
+#pragma unroll
+        for (int c = 0; c < W; ++c) {
+            const float2 a = unpack2(acc[i / 2][c]);
+            dst[(size_t)c * S] = i & 1 ? a.y : a.x;
+        }
+    }
+}
+
+template <int W, bool ADJ>
+void zconv_w(const float *in, const float *hz, float *out, const Dims &d, cudaStream_t st) {
+    const int np = d.n_par, nl = (d.Nz + np - 1) / np;
+    const int threads = std::min(128, (d.S + 31) / 32 * 32), ny = (d.S + threads - 1) / threads;
+    auto go = [&](auto kernel, int R) {
+        const int blocks = d.M * (ADJ ? np : 1) * np * ((nl + R - 1) / R);
+        launch_dependent(kernel, dim3(blocks, ny), dim3(threads), 0, st, in, hz, out, d.Nz, d.S, np);
+    };
+    // sixteen outputs a thread halve the reads from L2; eight where sixteen leave SMs idle
+    const long long b16 = (long long)d.M * (ADJ ? np : 1) * np * ((nl + 15) / 16) * ny;
+    if (W <= 9 && b16 >= 2 * 152) go(k_zconv<W, W <= 9 ? 16 : 8, ADJ>, 16);
+    else go(k_zconv<W, 8, ADJ>, 8);
+}
+
+template <bool ADJ>
+void zconv(const float *in, const float *hz, float *out, const Dims &d, cudaStream_t st) {
+    switch (d.hw) {
+        case 0: zconv_w<1, ADJ>(in, hz, out, d, st); break;
+        case 1: zconv_w<3, ADJ>(in, hz, out, d, st); break;
+        case 2: zconv_w<5, ADJ>(in, hz, out, d, st); break;
+        case 3: zconv_w<7, ADJ>(in, hz, out, d, st); break;
+        case 4: zconv_w<9, ADJ>(in, hz, out, d, st); break;
+        case 5: zconv_w<11, ADJ>(in, hz, out, d, st); break;
+        case 6: zconv_w<13, ADJ>(in, hz, out, d, st); break;
+        case 7: zconv_w<15, ADJ>(in, hz, out, d, st); break;
+        default: zconv_w<17, ADJ>(in, hz, out, d, st); break;
+    }
+}
+
+size_t g_len(const Dims &d) { return (size_t)d.M * d.Nz * d.n_par * d.W * d.S; }
+size_t dft_f_len(const Dims &d) { return DftOperand(d, d.hw + 1).off_f; }
+size_t dft_a_len(const Dims &d) { return DftOperand(d, d.hw + 1).off_a; }
+
+bool fold_h(mpi_ffl_handle *h) {
+    const Dims &d = h->d;
+    const double a = h->fwhm / (2.0 * langevin_half_point_host());
+    const double kPi = 3.14159265358979323846;
+    std::vector<double> taps((size_t)d.Q * (2 * d.Nz - 2) + 2 * d.D + 2);
+    for (size_t i = 0; i < taps.size(); ++i)
+        taps[i] = 3.0 * langevin_d1_host((((double)i - d.D) / d.Q - (d.Nz - 1)) / a);
+    std::vector<double2> drive(d.S);
+    for (int r = 0; r < d.S; ++r) {
+        const double ph = 2.0 * kPi * r / d.S + h->phase;
+        drive[r] = make_double2(d.Q * h->amp * std::sin(ph) + d.D, h->amp * (2.0 * kPi / d.S) * std::cos(ph));
+    }
+    double *dt = nullptr;
+    double2 *dd = nullptr;
+    bool ok = zalloc(&dt, taps.size()) && zalloc(&dd, drive.size());
+    if (ok) {
+        cudaMemcpy(dt, taps.data(), taps.size() * sizeof(double), cudaMemcpyHostToDevice);
+        cudaMemcpy(dd, drive.data(), drive.size() * sizeof(double2), cudaMemcpyHostToDevice);
+        k_zfold_h<<<dim3((d.S + 127) / 128, 2 * d.Nz - 1), 128>>>(dt, dd, zs(h)->hz, d.Nz, d.S, d.Q, d.D);
+        ok = cudaStreamSynchronize(nullptr) == cudaSuccess;
+    }
+    if (dt) dev_free(dt);
+    if (dd) dev_free(dd);
+    return ok;
+}
+
+}  // namespace
+
+// Per (line, phase) the folded steps cost (n_par N + N_z) W FMAs at matrix-product speed,
+// the sample-by-sample kernels P (W + 4) at about a fifth of it (1.45 ms against 0.25 ms for
+// the pair at 256^2 x 128, 36 angles, P = 512). The intermediate G is kept in memory.
+bool zfold_fits(const Dims &d) {
+    const double folded = (double)(d.n_par * d.N + d.Nz) * d.W, sampled = 4.0 * d.P * (d.W + 4);
+    return folded <= sampled && g_len(d) * sizeof(float) <= (size_t)1 << 30 &&
+           (size_t)d.N * d.n_par * d.W * d.S * sizeof(float) <= (size_t)1 << 28;
+}
+
+int zfold_ready(mpi_ffl_handle *h) {
+    if (!h->zfold_state) h->zfold_state = new ZFold();
+    ZFold *s = zs(h);
+    if (s->ready) return MPI_FFL_OK;
+    const Dims &d = h->d;
+    const int nk = d.n_par * d.W * d.S;
+    s->ldk = (nk + 3) / 4 * 4;
+    s->ldu = (d.N + 3) / 4 * 4;
+    double2 *unit_p = nullptr;
+    bool ok = zalloc(&s->kf, (size_t)d.N * s->ldk) && zalloc(&s->ka, (size_t)nk * s->ldu) &&
+              zalloc(&s->hz, (size_t)(2 * d.Nz - 1) * d.S) && zalloc(&s->df, dft_f_len(d)) &&
+              zalloc(&s->da, dft_a_len(d)) && zalloc(&s->cols, (size_t)2 * d.nb) && zalloc(&s->g, g_len(d)) &&
+              zalloc(&s->t, (size_t)d.M * d.Nz * d.W * d.S) && zalloc(&unit_p, d.P);
+    if (ok) {
+        const double kPi = 3.14159265358979323846;
+        std::vector<double2> up(d.P);
+        for (int p = 0; p < d.P; ++p) up[p] = make_double2(std::cos(2.0 * kPi * p / d.P), std::sin(2.0 * kPi * p / d.P));
+        cudaMemcpy(unit_p, up.data(), up.size() * sizeof(double2), cudaMemcpyHostToDevice);
+        cudaMemset(s->kf, 0, (size_t)d.N * s->ldk * sizeof(float));  // the columns past the last
+        cudaMemset(s->ka, 0, (size_t)nk * s->ldu * sizeof(float));
+        cudaMemset(s->df, 0, dft_f_len(d) * sizeof(float));
+        cudaMemset(s->da, 0, dft_a_len(d) * sizeof(float));
+        k_zfold_k<<<(nk + 127) / 128, 128>>>(unit_p, s->kf, s->ka, d, s->ldk, s->ldu);
+        k_zfold_dft<<<dim3(64, d.hw + 1), 128>>>(h->t_dgam, s->df, s->da, s->cols, d);
+        ok = fold_h(h);
+    }
+    if (unit_p) dev_free(unit_p);
+    if (!ok) {  // nothing of a failed build is kept
+        zfold_release(h);
+        return MPI_FFL_ERR_OOM;
+    }
+    s->ready = true;
+    return MPI_FFL_OK;
+}
+
+int zfold_psf_changed(mpi_ffl_handle *h) {
+    const ZFold *s = zs(h);
+    return !s || !s->ready || fold_h(h) ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
+}
+
+namespace {
+
+// the band DFT's products, one per |delta|: T -> data or its transpose data -> T
+void dft_products(const mpi_ffl_handle *h, bool adjoint, const float *in, float *out, cudaStream_t st) {
+    const Dims &d = h->d;
+    const ZFold *s = zs(h);
+    const int WS = d.W * d.S, rows = d.M * d.Nz;
+    SgemmArgs g[kMaxHw + 1];
+    for (int dd = 0; dd <= d.hw; ++dd) {
+        const DftOperand q(d, dd);
+        const int *cols = s->cols + q.off_c;
+        const int c0 = dd ? (2 * dd - 1) * d.S : 0;  // first column of (2d - 1, r) in T
+        if (adjoint)
+            g[dd] = SgemmArgs{in, 2 * d.nb, nullptr, rows, q.cols, s->da + q.off_a, q.lda, out + c0, WS, nullptr,
+                              q.rows, h->t_gain, d.Nz, cols, nullptr};
+        else
+            g[dd] = SgemmArgs{in + c0, WS, nullptr, rows, q.rows, s->df + q.off_f, q.ldf, out, 2 * d.nb, nullptr,
+                              q.cols, h->t_gain, d.Nz, nullptr, cols};
+    }
+    launch_sgemm(g, d.hw + 1, st);
+}
+
+}  // namespace
+
+void zfold_forward(mpi_ffl_handle *h, const float *proj, float *data, cudaStream_t st) {
+    const Dims &d = h->d;
+    const ZFold *s = zs(h);
+    const int nk = d.n_par * d.W * d.S;
+    const SgemmArgs k{proj, d.N, nullptr, d.M * d.Nz, d.N, s->kf, s->ldk, s->g, nk, nullptr, nk, nullptr, 1, nullptr,
+                      nullptr};
+    launch_sgemm(&k, 1, st);
+    zconv<false>(s->g, s->hz, s->t, d, st);
+    dft_products(h, false, s->t, data, st);
+}
+
+void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream_t st) {
+    const Dims &d = h->d;
+    const ZFold *s = zs(h);
+    const int nk = d.n_par * d.W * d.S;
+    dft_products(h, true, data, s->t, st);
+    zconv<true>(s->t, s->hz, s->g, d, st);
+    const SgemmArgs k{s->g, nk, nullptr, d.M * d.Nz, nk, s->ka, s->ldu, proj, d.N, nullptr, d.N, nullptr, 1, nullptr,
+                      nullptr};
+    launch_sgemm(&k, 1, st);
+}
+
+void zfold_release(mpi_ffl_handle *h) {
+    ZFold *s = zs(h);
+    if (!s) return;
+    for (void *p : {(void *)s->kf, (void *)s->ka, (void *)s->hz, (void *)s->df, (void *)s->da, (void *)s->cols,
+                    (void *)s->g, (void *)s->t})
+        if (p) dev_free(p);
+    delete s;
+    h->zfold_state = nullptr;
+}
+
+}  // namespace mpiffl

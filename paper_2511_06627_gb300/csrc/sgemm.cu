@@ -7,6 +7,7 @@
 // FMAs, and so are the roundings).
 #include <algorithm>
 
+#include "f32x2.cuh"
 #include "fold.h"
 #include "tc_ptx.cuh"
 
@@ -16,24 +17,6 @@ namespace {
 
 constexpr int kSgK = 16;  // K per stage, two stages
 
-using f32x2 = unsigned long long;
-
-__device__ __forceinline__ f32x2 dup2(float a) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-
 // 16 bytes global -> shared, the last 16 - n of them zero
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, int n) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(n)
@@ -41,20 +24,30 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, int n) {
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+struct SgemmBatch {
+    SgemmArgs g[kSgemmMax];
+    int first[kSgemmMax + 1];  // first block of each problem
+};
+
+// K of one run of sums: longer products add their runs' sums, so that rounding errors grow
+// with the run and the number of runs, not with K
+constexpr int kSgRun = 256;
+
 // One BM x BN tile per block. A warp covers 8 row groups x 4 column groups: its A loads
 // take 8 distinct 16-byte units side by side (a thread's rows come in runs of 4, BM / (TM / 4)
 // rows apart), its B loads 4.
 template <int BM, int BN, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_sgemm(SgemmArgs g0, SgemmArgs g1, int n0) {
+__global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_sgemm(const __grid_constant__ SgemmBatch batch) {
     constexpr int T = (BM / TM) * (BN / TN);
     constexpr int LA = BM + 4;
     constexpr int NA = (BM * kSgK / 4 + T - 1) / T, NB = (BN * kSgK / 4 + T - 1) / T;
     static_assert(BM / TM == 8 && TM % 4 == 0 && TN % 4 == 0 && T % 32 == 0, "warp layout");
     __shared__ __align__(16) float sA[2][kSgK][LA];
     __shared__ __align__(16) float sB[2][kSgK][BN];
-    const bool second = (int)blockIdx.x >= n0;
-    const SgemmArgs g = second ? g1 : g0;
-    const int b = (int)blockIdx.x - (second ? n0 : 0);
+    int pi = 0;
+    while ((int)blockIdx.x >= batch.first[pi + 1]) ++pi;  // uniform
+    const SgemmArgs &g = batch.g[pi];
+    const int b = (int)blockIdx.x - batch.first[pi];
     const int ntn = (g.N + BN - 1) / BN;
     const int m0 = b / ntn * BM, c0 = b % ntn * BN;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -68,7 +61,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_sgemm(SgemmArgs g0, S
         const bool in = i < BM * kSgK / 4 && r < g.M;
         ap[u] = in ? g.A + (size_t)(g.arow ? __ldg(g.arow + r) : r) * g.lda : nullptr;
     }
-    const bool vec = g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
+    const bool vec = !g.acol && g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
     float4 ra[NA];
     auto load_a = [&](int k0) {
 #pragma unroll
@@ -79,10 +72,10 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_sgemm(SgemmArgs g0, S
                 if (vec && k + 4 <= g.K) {
                     ra[u] = __ldg(reinterpret_cast<const float4 *>(ap[u] + k));
                 } else {
-                    if (k < g.K) ra[u].x = __ldg(ap[u] + k);
-                    if (k + 1 < g.K) ra[u].y = __ldg(ap[u] + k + 1);
-                    if (k + 2 < g.K) ra[u].z = __ldg(ap[u] + k + 2);
-                    if (k + 3 < g.K) ra[u].w = __ldg(ap[u] + k + 3);
+                    auto at = [&](int kk) {
+                        return kk < g.K ? __ldg(ap[u] + (g.acol ? __ldg(g.acol + kk) : kk)) : 0.f;
+                    };
+                    ra[u] = make_float4(at(k), at(k + 1), at(k + 2), at(k + 3));
                 }
             }
         }
@@ -110,11 +103,11 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_sgemm(SgemmArgs g0, S
         }
     };
 
-    f32x2 acc[TM][TN / 2];
+    f32x2 acc[TM][TN / 2], sum[TM][TN / 2];
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-        for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0;
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = sum[i][j] = 0;
     copy_b(0, 0);
     ptx::grid_dep_wait();  // A comes from the previous kernel
     ptx::grid_dep_launch();
@@ -154,9 +147,18 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_sgemm(SgemmArgs g0, S
             store_a(s ^ 1);
             cp_async_wait();
         }
+        if ((t + 1) % (kSgRun / kSgK) == 0 || t + 1 == nk) {
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN / 2; ++j) {
+                    sum[i][j] = add2(sum[i][j], acc[i][j]);
+                    acc[i][j] = 0;
+                }
+        }
         __syncthreads();
     }
-    const bool vecc = g.ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
+    const bool vecc = !g.ccol && g.ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int r = m0 + (i / 4) * (BM / (TM / 4)) + 4 * tr + (i & 3);
@@ -166,15 +168,15 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_sgemm(SgemmArgs g0, S
 #pragma unroll
         for (int j = 0; j < TN / 4; ++j) {
             const int c = c0 + j * (BN / (TN / 4)) + 4 * tc;
-            const float2 lo = unpack2(acc[i][2 * j]), hi = unpack2(acc[i][2 * j + 1]);
+            const float2 lo = unpack2(sum[i][2 * j]), hi = unpack2(sum[i][2 * j + 1]);
             const float4 v = make_float4(sc * lo.x, sc * lo.y, sc * hi.x, sc * hi.y);
             if (vecc && c + 4 <= g.N) {
                 *reinterpret_cast<float4 *>(dst + c) = v;
             } else {
-                if (c < g.N) dst[c] = v.x;
-                if (c + 1 < g.N) dst[c + 1] = v.y;
-                if (c + 2 < g.N) dst[c + 2] = v.z;
-                if (c + 3 < g.N) dst[c + 3] = v.w;
+                const float e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (c + q < g.N) dst[g.ccol ? __ldg(g.ccol + c + q) : c + q] = e[q];
             }
         }
     }
@@ -182,11 +184,15 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_sgemm(SgemmArgs g0, S
 
 template <int BM, int BN, int TM, int TN>
 void run(const SgemmArgs *g, int n, cudaStream_t st) {
-    auto tiles = [](const SgemmArgs &a) { return (a.M + BM - 1) / BM * ((a.N + BN - 1) / BN); };
-    const int n0 = tiles(g[0]), n1 = n > 1 ? tiles(g[1]) : 0;
-    if (n0 + n1 == 0) return;
-    launch_dependent(k_sgemm<BM, BN, TM, TN>, dim3(n0 + n1), dim3((BM / TM) * (BN / TN)), 0, st, g[0],
-                     g[n > 1 ? 1 : 0], n0);
+    SgemmBatch b{};
+    for (int i = 0; i < kSgemmMax; ++i) {
+        const int tiles = i < n ? (g[i].M + BM - 1) / BM * ((g[i].N + BN - 1) / BN) : 0;
+        if (i < n) b.g[i] = g[i];
+        b.first[i + 1] = b.first[i] + tiles;
+    }
+    const int total = b.first[kSgemmMax];
+    if (total > 0)
+        launch_dependent(k_sgemm<BM, BN, TM, TN>, dim3(total), dim3((BM / TM) * (BN / TN)), 0, st, b);
 }
 
 }  // namespace

@@ -84,3 +84,37 @@ def test_staged_path_against_the_oracle(name):
         bare = np.vdot(gb[m], ref["data"] / gains[m[0]]).real
         assert abs(float(gg[m[0]]) - bare) < OP_TOL * np.linalg.norm(gb) * np.linalg.norm(ref["data"])
     op.close()
+
+
+# the z-drive scan: folded tables with odd phases, harmonics and slices, one trajectory and
+# two, both convolution widths, more phases than a block has threads; and a raster with few
+# periods a column, which keeps the sample-by-sample kernels
+ZDRIVE = {
+    "odd": dict(nx=21, nz=9, n_angles=3, S=15, P=30, k_max=5, half_width=1),
+    "one trajectory": dict(nx=18, nz=11, n_angles=2, zigzag=0, S=24, P=20, k_max=4, half_width=2),
+    "sixteen lines": dict(nx=24, nz=67, n_angles=60, S=16, P=40, k_max=3, half_width=1),
+    "many phases": dict(nx=16, nz=5, n_angles=2, S=140, P=20, k_max=7, half_width=0),
+    "sampled": dict(nx=40, nz=8, n_angles=3, S=32, P=6, k_max=5, half_width=1),
+}
+
+
+@pytest.mark.parametrize("name", list(ZDRIVE))
+def test_zdrive_against_the_oracle(name):
+    from oracle import zdrive
+
+    st, op = _make(**ZDRIVE[name])
+    rng = np.random.default_rng(7)
+    gains = (1 + 0.1 * rng.standard_normal(st.n_angles)).astype(np.float32)
+    op.set_gain(gains)
+    st.gains = gains.astype(np.float64)
+    m = np.array([st.n_angles - 1])
+    x = rng.standard_normal((st.nz, st.nx, st.nx)).astype(np.float32)
+    y = np.zeros(st.data_shape, dtype=np.complex64)
+    y[m] = rng.standard_normal(y[m].shape) + 1j * rng.standard_normal(y[m].shape)
+    for fwhm in (2.5, 3.25):
+        op.set_fwhm(fwhm)
+        st.fwhm = fwhm
+        ref = zdrive.forward_stages_z(x, st, angles=m)["data"]
+        assert rel_l2(_n(op.forward_zdrive(_t(x)))[m], to_interleaved(ref)) < OP_TOL
+        assert rel_l2(_n(op.adjoint_zdrive(_t(to_interleaved(y)))), zdrive.adjoint_stages_z(y[m], st, angles=m)["vol"]) < OP_TOL
+    op.close()
