@@ -49,6 +49,7 @@ struct SgemmArgs {
 };
 constexpr int kSgemmMax = 9;  // problems of one launch
 void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st);
+int sgemm_tiles(const SgemmArgs &g);  // its blocks with the largest tiles
 
 // The z-drive scan with the raster and the PSF along z folded to tables (k_zfold.cu).
 bool zfold_fits(const Dims &d);                      // the rule by sizes

@@ -13,6 +13,7 @@
 // middle one a convolution along z per phase; neither the time signal, nor the fine z grid,
 // nor a transposed projection is formed. The tables are rounded once from FP64. The
 // adjoint runs the transposed steps in the opposite order.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -34,6 +35,7 @@ struct ZFold {
     int *cols = nullptr;   // per d: data column of operand column (k, sign, re / im)
     float *g = nullptr;    // [M][N_z][n_par][W][S]
     float *t = nullptr;    // [M][N_z][W][S]
+    float *part = nullptr; // [parts of K][M][N_z][N], sums of the adjoint's last product
     int ldk = 0, ldu = 0;
     bool ready = false;
 };
@@ -231,38 +233,211 @@ __global__ void __launch_bounds__(128) k_zconv(const float *__restrict__ in, con
     }
 }
 
-template <int W, bool ADJ>
-void zconv_w(const float *in, const float *hz, float *out, const Dims &d, cudaStream_t st) {
-    const int np = d.n_par, nl = (d.Nz + np - 1) / np;
-    const int threads = std::min(128, (d.S + 31) / 32 * 32), ny = (d.S + threads - 1) / threads;
-    auto go = [&](auto kernel, int R) {
-        const int blocks = d.M * (ADJ ? np : 1) * np * ((nl + R - 1) / R);
-        launch_dependent(kernel, dim3(blocks, ny), dim3(threads), 0, st, in, hz, out, d.Nz, d.S, np);
+// The same sums with the inputs streamed through shared memory (S a multiple of 4, up to
+// 128): one thread copies kZcIn inputs' W S values at a time into a ring of kZcStages
+// stages, and NG groups of S threads take R outputs each from it, so an input is read from
+// L2 once for NG R outputs. The new taps are loaded a stage ahead. The sums of a thread go
+// through fma.rn.f32x2 in pairs of values c; the taps are kept as pairs of equal halves.
+// 55 us each way at 256^2 x 128 and 36 angles (the plain form above: 153 us with 8 outputs a
+// thread, 75 us with 16); FMA-bound would be 18 us, the rest is the shared loads and moves of
+// a thread with only R W FMAs an input.
+constexpr int kZcIn = 4, kZcStages = 4, kZcAhead = kZcStages - 2;
+
+template <int W, int R, int NG, bool ADJ>
+__global__ void __launch_bounds__(128 * NG) k_zconv_ring(const float *__restrict__ in,
+                                                         const float *__restrict__ hz, float *__restrict__ out,
+                                                         int Nz, int S, int np, int *err) {
+    extern __shared__ __align__(128) float zring[];  // kZcStages x kZcIn x W S
+    __shared__ uint64_t full[kZcStages], empty[kZcStages];
+    const int Sp = (S + 31) & ~31;
+    const int ng = ((Nz + np - 1) / np + R * NG - 1) / (R * NG);
+    int b = blockIdx.x;
+    const int grp = b % ng;
+    b /= ng;
+    const int q = b % np;
+    b /= np;
+    int par = q;
+    if (ADJ) {
+        par = b % np;
+        b /= np;
+    }
+    const int m = b;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) {
+        for (int k = 0; k < kZcStages; ++k) {
+            ptx::mbar_init(&full[k], 1);
+            ptx::mbar_init(&empty[k], NG * Sp / 32);
+        }
+        ptx::fence_mbar_init();
+    }
+    __syncthreads();
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    const size_t WS = (size_t)W * S;
+    const size_t istride = ADJ ? WS : np * WS;
+    const float *src = in + (size_t)m * Nz * istride + (ADJ ? 0 : par * WS);
+    // inputs in order: the classes modulo np one after another (adjoint: the class par);
+    // a stage holds inputs of one class
+    const int ncls = ADJ ? 1 : min(np, Nz), cls0 = ADJ ? par : 0;
+    const int cnt0 = (Nz - cls0 + np - 1) / np, st0 = (cnt0 + kZcIn - 1) / kZcIn;
+    const int cnt1 = ncls > 1 ? (Nz - 1 + np - 1) / np : 0, nst = st0 + (cnt1 + kZcIn - 1) / kZcIn;
+    auto issue = [&](int s) {
+        const int k = s % kZcStages;
+        const int c = s < st0 ? cls0 : 1, u = kZcIn * (s < st0 ? s : s - st0);
+        const int n = min(kZcIn, (s < st0 ? cnt0 : cnt1) - u);
+        ptx::mbar_arrive_expect_tx(&full[k], (uint32_t)(n * WS) * 4u);
+        for (int e = 0; e < n; ++e)
+            ptx::bulk_g2s(zring + (size_t)(k * kZcIn + e) * WS, src + (size_t)(c + np * (u + e)) * istride,
+                          (uint32_t)WS * 4u, &full[k]);
     };
-    // sixteen outputs a thread halve the reads from L2; eight where sixteen leave SMs idle
-    const long long b16 = (long long)d.M * (ADJ ? np : 1) * np * ((nl + 15) / 16) * ny;
-    if (W <= 9 && b16 >= 2 * 152) go(k_zconv<W, W <= 9 ? 16 : 8, ADJ>, 16);
-    else go(k_zconv<W, 8, ADJ>, 8);
+    if (tid == 0)
+        for (int s = 0; s < min(nst, kZcAhead); ++s) issue(s);
+    const int r = tid % Sp, re = min(r, S - 1);
+    const int o0 = q + np * R * (grp * NG + tid / Sp);
+    const bool work = o0 < Nz;  // a group past the last output only waits and arrives
+    const float *tap = hz + (size_t)(Nz - 1) * S + re;  // offset 0
+    auto tap_at = [&](int k) { return __ldg(tap + (long long)min(max(k, 1 - Nz), Nz - 1) * S); };
+    constexpr int WP = W / 2;  // pairs of values; the last value goes alone
+    f32x2 acc[R][WP > 0 ? WP : 1];
+    float acl[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        acl[i] = 0.f;
+#pragma unroll
+        for (int c = 0; c < WP; ++c) acc[i][c] = 0;
+    }
+    bool good = true;
+    int s = 0;
+    for (int ci = 0; ci < ncls; ++ci) {
+        const int c = ci ? 1 : cls0, cnt = ci ? cnt1 : cnt0;
+        f32x2 w[R];  // taps of the outputs at the current input
+        float nt[kZcIn];
+#pragma unroll
+        for (int i = 0; i < R; ++i) w[i] = dup2(tap_at(ADJ ? c - (o0 + np * i) : o0 + np * i - c));
+        // the tap that enters after input u is that of output 0 at input u + 1
+        auto next_tap = [&](int u) { return tap_at(ADJ ? c + np * (u + 1) - o0 : o0 - c - np * (u + 1)); };
+#pragma unroll
+        for (int e = 0; e < kZcIn; ++e) nt[e] = next_tap(e);
+        for (int u = 0; u < cnt; u += kZcIn, ++s) {
+            const int k = s % kZcStages;
+            float nn[kZcIn];
+#pragma unroll
+            for (int e = 0; e < kZcIn; ++e) nn[e] = next_tap(u + kZcIn + e);
+            if (tid == 0 && s + kZcAhead < nst) {
+                const int sn = s + kZcAhead, kn = sn % kZcStages;
+                if (sn >= kZcStages && !ptx::mbar_wait_bounded(&empty[kn], ((sn / kZcStages) - 1) & 1, 1u << 24)) {
+                    atomicExch(err, 1);  // nothing more is issued: the waits below run out
+                } else {
+                    ptx::fence_proxy_async_smem();  // the stage's generic reads, then its refill
+                    issue(sn);
+                }
+            }
+            __syncwarp();
+            if (!__all_sync(0xffffffffu, ptx::mbar_wait_bounded(&full[k], (s / kZcStages) & 1, 1u << 24))) {
+                good = false;
+                break;
+            }
+            if (work) {  // uniform over the warp
+                const float *v0 = zring + (size_t)k * kZcIn * WS + re;
+#pragma unroll
+                for (int e = 0; e < kZcIn; ++e) {
+                    if (u + e >= cnt) break;  // uniform
+                    const float *v = v0 + e * WS;
+#pragma unroll
+                    for (int p = 0; p < WP; ++p) {
+                        const f32x2 vv = pack2(v[2 * p * S], v[(2 * p + 1) * S]);
+#pragma unroll
+                        for (int i = 0; i < R; ++i) acc[i][p] = fma2(w[i], vv, acc[i][p]);
+                    }
+                    const float vl = v[(W - 1) * S];
+#pragma unroll
+                    for (int i = 0; i < R; ++i) acl[i] = fmaf(unpack2(w[i]).x, vl, acl[i]);
+#pragma unroll
+                    for (int i = R - 1; i > 0; --i) w[i] = w[i - 1];
+                    w[0] = dup2(nt[e]);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < kZcIn; ++e) nt[e] = nn[e];
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&empty[k]);
+        }
+        if (!good) break;
+    }
+    if (!good) {
+        if (lane == 0) atomicExch(err, 1);
+        return;
+    }
+    if (r >= S) return;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int o = o0 + np * i;
+        if (o >= Nz) break;
+        float *dst = out + ((size_t)m * Nz + o) * (ADJ ? np * WS : WS) + (ADJ ? par * WS : 0) + r;
+#pragma unroll
+        for (int p = 0; p < WP; ++p) {
+            const float2 a = unpack2(acc[i][p]);
+            dst[(size_t)(2 * p) * S] = a.x;
+            dst[(size_t)(2 * p + 1) * S] = a.y;
+        }
+        dst[(size_t)(W - 1) * S] = acl[i];
+    }
+}
+
+template <int W, bool ADJ>
+void zconv_w(const float *in, const float *hz, float *out, const Dims &d, int *err, cudaStream_t st) {
+    constexpr int R = 8;
+    const int np = d.n_par, nl = (d.Nz + np - 1) / np;
+    const int outer = d.M * (ADJ ? np : 1) * np;
+    const size_t smem = sizeof(float) * kZcStages * kZcIn * W * d.S;
+    if (d.S % 4 == 0 && d.S <= 128) {
+        // as many groups a block (4, or 2 where the sums of wide bands need the registers) as
+        // leave a block for every SM
+        auto go = [&](auto kernel, int NG) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            launch_dependent(kernel, dim3(outer * ((nl + R * NG - 1) / (R * NG))), dim3((d.S + 31) / 32 * 32 * NG),
+                             smem, st, in, hz, out, d.Nz, d.S, np, err);
+        };
+        auto blocks = [&](int NG) { return outer * ((nl + R * NG - 1) / (R * NG)); };
+        if (W <= 9 && blocks(4) >= 128) go(k_zconv_ring<W, R, W <= 9 ? 4 : 2, ADJ>, 4);
+        else if (blocks(2) >= 128) go(k_zconv_ring<W, R, 2, ADJ>, 2);
+        else go(k_zconv_ring<W, R, 1, ADJ>, 1);
+        return;
+    }
+    const int threads = std::min(128, (d.S + 31) / 32 * 32), ny = (d.S + threads - 1) / threads;
+    launch_dependent(k_zconv<W, R, ADJ>, dim3(outer * ((nl + R - 1) / R), ny), dim3(threads), 0, st, in, hz, out, d.Nz,
+                     d.S, np);
 }
 
 template <bool ADJ>
-void zconv(const float *in, const float *hz, float *out, const Dims &d, cudaStream_t st) {
+void zconv(const float *in, const float *hz, float *out, const Dims &d, int *err, cudaStream_t st) {
     switch (d.hw) {
-        case 0: zconv_w<1, ADJ>(in, hz, out, d, st); break;
-        case 1: zconv_w<3, ADJ>(in, hz, out, d, st); break;
-        case 2: zconv_w<5, ADJ>(in, hz, out, d, st); break;
-        case 3: zconv_w<7, ADJ>(in, hz, out, d, st); break;
-        case 4: zconv_w<9, ADJ>(in, hz, out, d, st); break;
-        case 5: zconv_w<11, ADJ>(in, hz, out, d, st); break;
-        case 6: zconv_w<13, ADJ>(in, hz, out, d, st); break;
-        case 7: zconv_w<15, ADJ>(in, hz, out, d, st); break;
-        default: zconv_w<17, ADJ>(in, hz, out, d, st); break;
+        case 0: zconv_w<1, ADJ>(in, hz, out, d, err, st); break;
+        case 1: zconv_w<3, ADJ>(in, hz, out, d, err, st); break;
+        case 2: zconv_w<5, ADJ>(in, hz, out, d, err, st); break;
+        case 3: zconv_w<7, ADJ>(in, hz, out, d, err, st); break;
+        case 4: zconv_w<9, ADJ>(in, hz, out, d, err, st); break;
+        case 5: zconv_w<11, ADJ>(in, hz, out, d, err, st); break;
+        case 6: zconv_w<13, ADJ>(in, hz, out, d, err, st); break;
+        case 7: zconv_w<15, ADJ>(in, hz, out, d, err, st); break;
+        default: zconv_w<17, ADJ>(in, hz, out, d, err, st); break;
     }
 }
 
 size_t g_len(const Dims &d) { return (size_t)d.M * d.Nz * d.n_par * d.W * d.S; }
 size_t dft_f_len(const Dims &d) { return DftOperand(d, d.hw + 1).off_f; }
 size_t dft_a_len(const Dims &d) { return DftOperand(d, d.hw + 1).off_a; }
+
+// K of one part of the adjoint's last product: whole runs of 256, at most kSgemmMax parts,
+// about four blocks an SM
+int z_kper(const Dims &d) {
+    const int nk = d.n_par * d.W * d.S;
+    SgemmArgs a{};
+    a.M = d.M * d.Nz;
+    a.N = d.N;
+    const int want = std::max(1, std::min(kSgemmMax, 600 / std::max(1, sgemm_tiles(a)) + 1));
+    return std::max(256, ((nk + want - 1) / want + 255) / 256 * 256);
+}
 
 bool fold_h(mpi_ffl_handle *h) {
     const Dims &d = h->d;
@@ -293,8 +468,8 @@ bool fold_h(mpi_ffl_handle *h) {
 }  // namespace
 
 // Per (line, phase) the folded steps cost (n_par N + N_z) W FMAs at matrix-product speed,
-// the sample-by-sample kernels P (W + 4) at about a fifth of it (1.45 ms against 0.25 ms for
-// the pair at 256^2 x 128, 36 angles, P = 512). The intermediate G is kept in memory.
+// the sample-by-sample kernels P (W + 4) at about a fifth of it (1.45 ms against 0.42 ms for
+// the line stages of a pair at 256^2 x 128, 36 angles, P = 512). The intermediate G is kept in memory.
 bool zfold_fits(const Dims &d) {
     const double folded = (double)(d.n_par * d.N + d.Nz) * d.W, sampled = 4.0 * d.P * (d.W + 4);
     return folded <= sampled && g_len(d) * sizeof(float) <= (size_t)1 << 30 &&
@@ -313,7 +488,8 @@ int zfold_ready(mpi_ffl_handle *h) {
     bool ok = zalloc(&s->kf, (size_t)d.N * s->ldk) && zalloc(&s->ka, (size_t)nk * s->ldu) &&
               zalloc(&s->hz, (size_t)(2 * d.Nz - 1) * d.S) && zalloc(&s->df, dft_f_len(d)) &&
               zalloc(&s->da, dft_a_len(d)) && zalloc(&s->cols, (size_t)2 * d.nb) && zalloc(&s->g, g_len(d)) &&
-              zalloc(&s->t, (size_t)d.M * d.Nz * d.W * d.S) && zalloc(&unit_p, d.P);
+              zalloc(&s->t, (size_t)d.M * d.Nz * d.W * d.S) && zalloc(&unit_p, d.P) &&
+              zalloc(&s->part, (size_t)((nk + z_kper(d) - 1) / z_kper(d)) * d.M * d.Nz * d.N);
     if (ok) {
         const double kPi = 3.14159265358979323846;
         std::vector<double2> up(d.P);
@@ -372,7 +548,7 @@ void zfold_forward(mpi_ffl_handle *h, const float *proj, float *data, cudaStream
     const SgemmArgs k{proj, d.N, nullptr, d.M * d.Nz, d.N, s->kf, s->ldk, s->g, nk, nullptr, nk, nullptr, 1, nullptr,
                       nullptr};
     launch_sgemm(&k, 1, st);
-    zconv<false>(s->g, s->hz, s->t, d, st);
+    zconv<false>(s->g, s->hz, s->t, d, h->w_err, st);
     dft_products(h, false, s->t, data, st);
 }
 
@@ -381,17 +557,25 @@ void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream
     const ZFold *s = zs(h);
     const int nk = d.n_par * d.W * d.S;
     dft_products(h, true, data, s->t, st);
-    zconv<true>(s->t, s->hz, s->g, d, st);
-    const SgemmArgs k{s->g, nk, nullptr, d.M * d.Nz, nk, s->ka, s->ldu, proj, d.N, nullptr, d.N, nullptr, 1, nullptr,
-                      nullptr};
-    launch_sgemm(&k, 1, st);
+    zconv<true>(s->t, s->hz, s->g, d, h->w_err, st);
+    // K is long (n_par W S): split over as many problems as fill the GPU, each into its own
+    // sums, which are added in a fixed order
+    SgemmArgs g[kSgemmMax];
+    const int kper = z_kper(d), np = (nk + kper - 1) / kper;
+    const int64_t rows = (int64_t)d.M * d.Nz;
+    for (int i = 0; i < np; ++i)
+        g[i] = SgemmArgs{s->g + (size_t)i * kper, nk, nullptr, (int)rows, std::min(kper, nk - i * kper),
+                         s->ka + (size_t)i * kper * s->ldu, s->ldu, np > 1 ? s->part + i * rows * d.N : proj, d.N,
+                         nullptr, d.N, nullptr, 1, nullptr, nullptr};
+    launch_sgemm(g, np, st);
+    if (np > 1) launch_coil_pad(s->part, nullptr, proj, rows, d.Nz, d.N, d.N, st, np, rows * d.N);
 }
 
 void zfold_release(mpi_ffl_handle *h) {
     ZFold *s = zs(h);
     if (!s) return;
     for (void *p : {(void *)s->kf, (void *)s->ka, (void *)s->hz, (void *)s->df, (void *)s->da, (void *)s->cols,
-                    (void *)s->g, (void *)s->t})
+                    (void *)s->g, (void *)s->t, (void *)s->part})
         if (p) dev_free(p);
     delete s;
     h->zfold_state = nullptr;
