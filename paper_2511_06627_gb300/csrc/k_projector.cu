@@ -334,7 +334,7 @@ void launch_project(const float *vol, const float *volT, const AngleParam *ang, 
     k_project<<<grid, threads, smem, st>>>(vol, volT, ang, agroups, proj, N, Nz, rays);
 }
 
-// Interleaved variant (same shapes as the pipelined one). The volume is copied once with
+// Interleaved variant (detectors of any size up to 496 bins). The volume is copied once with
 // each line's kZc slices innermost, volI[z block][y][x][kZc]. A march step is one tensor
 // copy of the step's line: a row of volI for row-marched angles, a column (32-byte
 // pieces N rows apart) for column-marched ones. The copy writes shared memory with the
@@ -390,8 +390,8 @@ size_t il_len(int N, int Nz) { return (size_t)((Nz + kZc - 1) / kZc) * kZc * N *
 
 // volI[zb][y][x][e] = vol[kZc zb + e][y][x] (zero past Nz). A block of 8 x 32 threads
 // moves a 32 x 32 tile of one slice block:
-// thread (tx, ty) loads 4 consecutive x of row ty of every slice (eight 16-byte loads;
-// N % 4 == 0) and forms each position's two halves in registers. The tile goes through
+// thread (tx, ty) loads 4 consecutive x of row ty of every slice (VEC: eight 16-byte loads,
+// N % 4 == 0 and the volume on 16 bytes) and forms each position's two halves in registers. The tile goes through
 // shared memory as 16-byte halves: half h of tile row r, column c sits at 16-byte slot
 // 64 r + 8 (c >> 2) + ((2 (c & 3) + h) ^ sw), sw = (c >> 2) ^ 2 (r & 3). The rows are
 // then written from the tile, 32 consecutive 16-byte units of one output row per warp
@@ -402,6 +402,7 @@ __device__ __forceinline__ int il_tile_slot(int r, int c, int h) {
     return 64 * r + 8 * (c >> 2) + ((2 * (c & 3) + h) ^ (((c >> 2) ^ (2 * (r & 3))) & 7));
 }
 
+template <bool VEC>
 __global__ void __launch_bounds__(256) k_interleave(const float *__restrict__ vol, float *__restrict__ volI, int N,
                                                     int Nz) {
     __shared__ float4 tile[32 * 64];  // 32 rows x 32 columns x 2 halves
@@ -415,7 +416,17 @@ __global__ void __launch_bounds__(256) k_interleave(const float *__restrict__ vo
     for (int e = 0; e < kZc; ++e) {
         const int z = zb * kZc + e;
         v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (z < Nz && y < N && xs < N) v[e] = __ldg(reinterpret_cast<const float4 *>(vol + ((size_t)z * N + y) * N + xs));
+        if (z < Nz && y < N && xs < N) {
+            const float *src = vol + ((size_t)z * N + y) * N + xs;
+            if (VEC) {
+                v[e] = __ldg(reinterpret_cast<const float4 *>(src));
+            } else {
+                v[e].x = __ldg(src);
+                if (xs + 1 < N) v[e].y = __ldg(src + 1);
+                if (xs + 2 < N) v[e].z = __ldg(src + 2);
+                if (xs + 3 < N) v[e].w = __ldg(src + 3);
+            }
+        }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -446,7 +457,8 @@ __global__ void __launch_bounds__(256) k_interleave(const float *__restrict__ vo
 
 void launch_interleave(const float *vol, float *volI, int N, int Nz, cudaStream_t st) {
     dim3 grid((N + 31) / 32, (N + 31) / 32, (Nz + kZc - 1) / kZc), block(8, 32);
-    launch_dependent(k_interleave, grid, block, 0, st, vol, volI, N, Nz);
+    const bool vec = N % 4 == 0 && (reinterpret_cast<uintptr_t>(vol) & 15) == 0;
+    launch_dependent(vec ? k_interleave<true> : k_interleave<false>, grid, block, 0, st, vol, volI, N, Nz);
 }
 
 // Tensor maps of volI as a 4-D array (kZc floats, x, y, z block): boxes of one row
@@ -698,7 +710,10 @@ void launch_il(dim3 grid, int threads, cudaStream_t st, const IlMaps &maps, cons
                      agroups, proj, N, Nz, rays, err, inject, pack);
 }
 
-bool project_il_ok(int N) { return N % 4 == 0 && pipe_ld(N) > 0 && pipe_threads_ok(N); }
+// Any detector of up to 496 bins: the copy's own strides (32 N bytes) suit the tensor maps,
+// and the boxes' zero fill past N takes the place of a ragged line's last positions. (101
+// bins, 21 angles and 37 slices: 113 us through the plain projector, 26 us this way.)
+bool project_il_ok(int N) { return pipe_ld(N) > 0 && pipe_threads_ok(N); }
 
 void launch_project_il(const IlMaps &maps, const AngleParam *ang, const int *agroups,
                        int n_agroups, float *proj, int N, int Nz, cudaStream_t st, int *err, uint32_t inject,

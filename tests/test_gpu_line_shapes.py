@@ -118,3 +118,18 @@ def test_zdrive_against_the_oracle(name):
         assert rel_l2(_n(op.forward_zdrive(_t(x)))[m], to_interleaved(ref)) < OP_TOL
         assert rel_l2(_n(op.adjoint_zdrive(_t(to_interleaved(y)))), zdrive.adjoint_stages_z(y[m], st, angles=m)["vol"]) < OP_TOL
     op.close()
+
+
+@pytest.mark.parametrize("nx,nz,off", [(21, 9, 0), (102, 8, 0), (259, 3, 0), (64, 9, 1), (33, 5, 3)])
+def test_interleaved_projector_on_ragged_detectors(nx, nz, off):
+    """Detectors that are not a multiple of four bins, on both sides of one tensor box, and
+    volumes that do not start on 16 bytes, against the oracle's projection."""
+    from oracle import projection
+
+    st, op = _make(nx=nx, nz=nz, n_angles=7, S=16, P=40)
+    x = np.random.default_rng(8).standard_normal((nz, nx, nx)).astype(np.float32)
+    buf = torch.zeros(x.size + 4, device="cuda")
+    vol = buf[off:off + x.size].view(x.shape)
+    vol.copy_(torch.from_numpy(x))
+    assert rel_l2(_n(op.project(vol)), projection.project(x, st.angles)) < OP_TOL
+    op.close()
