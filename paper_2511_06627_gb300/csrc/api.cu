@@ -17,7 +17,8 @@ using namespace mpiffl;
 
 // the z-drive scan (defined with its entry points below)
 void z_init(mpi_ffl_handle *h);
-void forward_z_impl(mpi_ffl_handle *h, const float *x, float *b, cudaStream_t st);
+void z_line_forward(mpi_ffl_handle *h, const float *proj, float *b, cudaStream_t st);
+void z_line_adjoint(mpi_ffl_handle *h, const float *b, float *proj, cudaStream_t st);
 void adjoint_z_impl(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st);
 
 namespace {
@@ -391,9 +392,9 @@ void group_table(mpi_ffl_handle *h) {
 void release(mpi_ffl_handle *h) {
     void *ptrs[] = {h->t_ang, h->t_gain, h->t_unit_gain, h->t_htab, h->t_dhtab, h->t_traj, h->t_csr_ptr,
                     h->t_csr, h->t_tw1, h->t_tw2_ro, h->t_tw2_qr, h->t_dgam, h->t_dgam_unit, h->t_groups, h->w_volT,
-                    h->w_proj, h->w_fine, h->w_sig, h->w_data, h->w_vol2, h->w_red, h->w_scal,
+                    h->w_proj, h->w_fine, h->w_sig, h->w_data, h->w_vol2, h->w_red, h->w_scal, h->w_count,
                     h->s_xp, h->s_y, h->s_g, h->s_r, h->s_hist, h->s_flags, h->tc_twb, h->t_agroups,
-                    h->t_tnf, h->t_vr, h->w_err, h->t_coil, h->w_projc, h->w_scanvol, h->w_volI,
+                    h->t_tnf, h->t_vr, h->w_err, h->t_coil, h->w_projc, h->w_scanproj, h->w_volI,
                     h->t_ra_tile, h->t_ra_j, h->t_ra_w, h->t_twp, h->w_bins};
     for (void *p : ptrs)
         if (p) dev_free(p);
@@ -498,17 +499,22 @@ void ensure_sig(mpi_ffl_handle *h) {
 
 // ------------------------------------------------------------ stages
 // With pack.out[0] set, the interleaved projector writes the forward full stage's A
-// operand instead of the projections; returns whether it did (the other projector
-// always stores the projections).
-bool stage_p(mpi_ffl_handle *h, const float *x, float *proj, cudaStream_t st, const ProjPack &pack = ProjPack{}) {
+// operand, and the projections only if `keep` says so; returns whether it did (the other
+// projector always stores the projections). With mom, the volume projected is mom->y.
+bool stage_p(mpi_ffl_handle *h, const float *x, float *proj, cudaStream_t st, const ProjPack &pack = ProjPack{},
+             bool keep = false, const MomentumIn *mom = nullptr) {
     if (h->w_volI) {  // the interleaved projector: both orientations from one pass over x
         const bool packed = pack.out[0] != nullptr;
-        TIMED(MPI_FFL_K_TRANSPOSE, launch_interleave(x, h->w_volI, h->d.N, h->d.Nz, st));
+        TIMED(MPI_FFL_K_TRANSPOSE, launch_interleave(x, h->w_volI, h->d.N, h->d.Nz, st, mom));
         TIMED(MPI_FFL_K_PROJECT, launch_project_il(h->il_maps, h->t_ang, h->t_agroups, h->n_agroups,
-                                                   packed ? nullptr : proj, h->d.N, h->d.Nz, st, h->w_err,
+                                                   packed && !keep ? nullptr : proj, h->d.N, h->d.Nz, st, h->w_err,
                                                    h->inject_polls, pack));
         check_launch(h, "project");
         return packed;
+    }
+    if (mom) {
+        TIMED(MPI_FFL_K_SOLVER, launch_momentum(x, mom->xp, mom->y, mom->beta, h->d.nvox, mom->done, st));
+        x = mom->y;
     }
     if (any_column_angle(h)) TIMED(MPI_FFL_K_TRANSPOSE, launch_transpose_xy(x, h->w_volT, h->d.N, h->d.Nz, st));
     TIMED(MPI_FFL_K_PROJECT, launch_project(x, h->w_volT, h->t_ang, h->t_agroups, h->n_agroups, proj, h->d.N, h->d.Nz, st, h->w_err));
@@ -698,15 +704,19 @@ void line_forward_impl(mpi_ffl_handle *h, const float *proj, float *b, const flo
     check_launch(h, "dft_fwd");
 }
 
-void forward_impl(mpi_ffl_handle *h, const float *x, float *b, const float *htab, const float *gain,
-                  cudaStream_t st) {
-    // The full-GEMM stage with the collinear PSF's own taps, no coil map: the projector
-    // splits its sums into the GEMM's A operand itself (the packing pass and the
-    // projections' round trip through HBM drop out; the same hi + lo values).
+// The projector's target for the forward GEMM's A operand: the full-GEMM stage with the
+// collinear PSF's own taps and no coil map lets the projector split its sums itself (the
+// packing pass and the projections' round trip through HBM drop out; the same hi + lo values).
+ProjPack pack_target(mpi_ffl_handle *h, const float *htab) {
     ProjPack pack{};
     const bool fold = h->path == MPI_FFL_PATH_FULL_GEMM && h->psf_model != MPI_FFL_PSF_TENSOR && !h->t_coil &&
                       htab == h->t_htab && col_prepack_targets(h, &pack);
-    const bool packed = stage_p(h, x, h->w_proj, st, fold ? pack : ProjPack{});
+    return fold ? pack : ProjPack{};
+}
+
+void forward_impl(mpi_ffl_handle *h, const float *x, float *b, const float *htab, const float *gain,
+                  cudaStream_t st, const MomentumIn *mom = nullptr) {
+    const bool packed = stage_p(h, x, h->w_proj, st, pack_target(h, htab), false, mom);
     line_forward_impl(h, h->w_proj, b, htab, gain, st, packed);
 }
 
@@ -795,28 +805,37 @@ double dot_sync(mpi_ffl_handle *h, const float *a, const float *b, int64_t n, cu
 }
 
 // The operator of the selected scans (Sec. 3.1: an x-drive and a z-drive scan per
-// angle): r = [A x; A_z x] in that order, and its transpose A^T r + A_z^T r_z (the
-// two volumes summed in a fixed order).
+// angle): r = [A x; A_z x] in that order, and its transpose A^T r + A_z^T r_z.
 int64_t scan_data_len(const mpi_ffl_handle *h) {
     return (int64_t)(((h->scans & MPI_FFL_SCAN_X) ? 1 : 0) + ((h->scans & MPI_FFL_SCAN_Z) ? 1 : 0)) * h->d.ndata;
 }
 
-void scans_forward(mpi_ffl_handle *h, const float *x, float *r, cudaStream_t st) {
-    if (h->scans & MPI_FFL_SCAN_X) {
-        forward_impl(h, x, r, h->t_htab, h->t_gain, st);
+// With both scans the volume is projected once, and the transposed line stages are added
+// before one backprojection.
+void scans_forward(mpi_ffl_handle *h, const float *x, float *r, cudaStream_t st, const MomentumIn *mom = nullptr) {
+    if (h->scans == MPI_FFL_SCAN_X) {
+        forward_impl(h, x, r, h->t_htab, h->t_gain, st, mom);
+        return;
+    }
+    const bool both = (h->scans & MPI_FFL_SCAN_X) != 0;
+    z_init(h);
+    const bool packed = stage_p(h, x, h->w_proj, st, both ? pack_target(h, h->t_htab) : ProjPack{}, true, mom);
+    if (both) {
+        line_forward_impl(h, h->w_proj, r, h->t_htab, h->t_gain, st, packed);
         r += h->d.ndata;
     }
-    if (h->scans & MPI_FFL_SCAN_Z) forward_z_impl(h, x, r, st);
+    z_line_forward(h, h->w_proj, r, st);
 }
 
 void scans_adjoint(mpi_ffl_handle *h, const float *r, float *g, cudaStream_t st) {
     const Dims &d = h->d;
     if (h->scans == (MPI_FFL_SCAN_X | MPI_FFL_SCAN_Z)) {
-        adjoint_impl(h, r, h->w_scanvol, st);
-        adjoint_z_impl(h, r + d.ndata, h->w_scanvol + d.nvox, st);
-        TIMED(MPI_FFL_K_SOLVER, launch_coil_pad(h->w_scanvol, nullptr, g, (long long)d.Nz * d.N, d.Nz, d.N, d.N, st, 2,
-                                                d.nvox));
+        line_adjoint_impl(h, r, h->w_scanproj, st);
+        z_line_adjoint(h, r + d.ndata, h->w_scanproj + d.nproj, st);
+        TIMED(MPI_FFL_K_SOLVER, launch_coil_pad(h->w_scanproj, nullptr, h->w_proj, d.nseg, d.Nz, d.N, d.N, st, 2,
+                                                d.nproj));
         check_launch(h, "scan sum");
+        stage_pt(h, h->w_proj, g, st);
     } else if (h->scans & MPI_FFL_SCAN_X) {
         adjoint_impl(h, r, g, st);
     } else {
@@ -827,20 +846,18 @@ void scans_adjoint(mpi_ffl_handle *h, const float *r, float *g, cudaStream_t st)
 double power_norm_impl(mpi_ffl_handle *h, int n_iter, uint64_t seed, cudaStream_t st) {
     const Dims &d = h->d;
     float *v = h->w_vol2, *w = h->s_g;
-    const int nbv = reduce_blocks(d.nvox);
+    float *scale = reinterpret_cast<float *>(h->w_count + 1);
     TIMED(MPI_FFL_K_SOLVER, launch_splitmix_fill(v, d.nvox, seed, st));
-    TIMED(MPI_FFL_K_SOLVER, launch_dot(v, v, d.nvox, h->w_red, nbv, st));
-    TIMED(MPI_FFL_K_SOLVER, launch_finalize(h->w_red, nbv, h->w_scal + 0, st));
-    TIMED(MPI_FFL_K_SOLVER, launch_scale_by_rsqrt(v, v, d.nvox, h->w_scal + 0, st));
+    TIMED(MPI_FFL_K_SOLVER, launch_dot2(v, v, d.nvox, h->w_red, h->w_count, nullptr, h->w_scal + 0, scale, st));
+    TIMED(MPI_FFL_K_SOLVER, launch_scale(v, v, d.nvox, scale, st));
     check_launch(h, "power init");
     for (int it = 0; it < n_iter; ++it) {
         scans_forward(h, v, h->w_data, st);
         scans_adjoint(h, h->w_data, w, st);
-        TIMED(MPI_FFL_K_SOLVER, launch_dot(v, w, d.nvox, h->w_red, nbv, st));
-        TIMED(MPI_FFL_K_SOLVER, launch_finalize(h->w_red, nbv, h->w_scal + 1, st));
-        TIMED(MPI_FFL_K_SOLVER, launch_dot(w, w, d.nvox, h->w_red, nbv, st));
-        TIMED(MPI_FFL_K_SOLVER, launch_finalize(h->w_red, nbv, h->w_scal + 0, st));
-        TIMED(MPI_FFL_K_SOLVER, launch_scale_by_rsqrt(w, v, d.nvox, h->w_scal + 0, st));
+        TIMED(MPI_FFL_K_SOLVER,
+              launch_dot2(v, w, d.nvox, h->w_red, h->w_count, it + 1 == n_iter ? h->w_scal + 1 : nullptr,
+                          h->w_scal + 0, scale, st));
+        TIMED(MPI_FFL_K_SOLVER, launch_scale(w, v, d.nvox, scale, st));
         check_launch(h, "power step");
     }
     double mu = 0;
@@ -965,9 +982,12 @@ extern "C" int mpi_ffl_create(const mpi_ffl_geometry *geom, const mpi_ffl_trajec
         dev_alloc(h, &h->w_fine, d.nfine);
         dev_alloc(h, &h->w_data, d.ndata);
         dev_alloc(h, &h->w_vol2, d.nvox);
-        h->w_red_len = std::max(reduce_blocks(std::max(d.nvox, d.ndata)) + 16, 1024 * std::max(d.M, 1));
+        h->w_red_len = std::max(std::max(reduce_blocks(std::max(d.nvox, d.ndata)), 2 * dot2_blocks(d.nvox)) + 16,
+                                1024 * std::max(d.M, 1));
         dev_alloc(h, &h->w_red, (size_t)h->w_red_len);
         dev_alloc(h, &h->w_scal, 16);
+        dev_alloc(h, &h->w_count, 2);
+        CK(cudaMemset(h->w_count, 0, 2 * sizeof(unsigned)));
         dev_alloc(h, &h->s_xp, d.nvox);
         dev_alloc(h, &h->s_y, d.nvox);
         dev_alloc(h, &h->s_g, d.nvox);
@@ -1165,12 +1185,12 @@ extern "C" int mpi_ffl_set_scans(mpi_ffl_handle *h, int32_t scans) {
         CK(cudaDeviceSynchronize());
         if (scans & MPI_FFL_SCAN_Z) z_init(h);
         const int n = ((scans & MPI_FFL_SCAN_X) ? 1 : 0) + ((scans & MPI_FFL_SCAN_Z) ? 1 : 0);
-        if (n == 2 && !h->w_scanvol) {
-            // residual and power-iteration data of both scans, and the two transposes
+        if (n == 2 && !h->w_scanproj) {
+            // residual and power-iteration data of both scans, and the two line transposes
             float *r = nullptr, *w = nullptr;
             dev_alloc(h, &r, (size_t)2 * d.ndata);
             dev_alloc(h, &w, (size_t)2 * d.ndata);
-            dev_alloc(h, &h->w_scanvol, (size_t)2 * d.nvox);
+            dev_alloc(h, &h->w_scanproj, (size_t)2 * d.nproj);
             CK(dev_free(h->s_r));
             CK(dev_free(h->w_data));
             h->bytes -= (int64_t)(2 * d.ndata * sizeof(float));
@@ -1455,41 +1475,48 @@ void ensure_z_workspace(mpi_ffl_handle *h) {
     if (!h->w_zcoef) dev_alloc(h, &h->w_zcoef, (size_t)d.M * d.Nz * (2 * d.hw + 1) * d.S);
 }
 
-void forward_z_impl(mpi_ffl_handle *h, const float *x, float *b, cudaStream_t st) {
+// projections -> z-drive data
+void z_line_forward(mpi_ffl_handle *h, const float *proj, float *b, cudaStream_t st) {
     const Dims &d = h->d;
-    z_init(h);
-    const bool folded = use_zfold(h);
-    stage_p(h, x, h->w_proj, st);
-    if (folded) {
-        TIMED(MPI_FFL_K_ZDRIVE, zfold_forward(h, h->w_proj, b, st));
+    if (use_zfold(h)) {
+        TIMED(MPI_FFL_K_ZDRIVE, zfold_forward(h, proj, b, st));
         h->launches += 2;  // a convolution and the band DFT's products in the same timed stage
         check_launch(h, "z-drive forward");
         return;
     }
     ensure_z_workspace(h);
-    zstage_h(h, h->w_proj, h->w_fine_z, st);
+    zstage_h(h, proj, h->w_fine_z, st);
     // E_z V_z B fused with S D_Gamma F: the time signal is not stored
     TIMED(MPI_FFL_K_ZDRIVE, launch_zdft_fwd(h->w_fine_z, z_tables(h), h->t_gain, h->t_tw1, h->t_tw2_ro, h->t_dgam, b,
                                             d, h->zigzag, st));
     check_launch(h, "z-drive forward");
 }
 
-void adjoint_z_impl(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st) {
+// z-drive data -> projections
+void z_line_adjoint(mpi_ffl_handle *h, const float *b, float *proj, cudaStream_t st) {
     const Dims &d = h->d;
-    z_init(h);
     if (use_zfold(h)) {
-        TIMED(MPI_FFL_K_ZDRIVE, zfold_adjoint(h, b, h->w_proj, st));
+        TIMED(MPI_FFL_K_ZDRIVE, zfold_adjoint(h, b, proj, st));
         h->launches += 2;
-        stage_pt(h, h->w_proj, x, st);
-        check_launch(h, "z-drive adjoint");
-        return;
+    } else {
+        ensure_z_workspace(h);
+        TIMED(MPI_FFL_K_ZDRIVE, launch_zdft_adj(b, h->t_tw1, h->t_tw2_qr, h->t_dgam, z_tables(h), h->t_gain,
+                                                h->w_zcoef, h->w_fine_z, d, h->zigzag, st));
+        zstage_ht(h, h->w_fine_z, proj, st);
     }
-    ensure_z_workspace(h);
-    TIMED(MPI_FFL_K_ZDRIVE, launch_zdft_adj(b, h->t_tw1, h->t_tw2_qr, h->t_dgam, z_tables(h), h->t_gain,
-                                            h->w_zcoef, h->w_fine_z, d, h->zigzag, st));
-    zstage_ht(h, h->w_fine_z, h->w_proj, st);
-    stage_pt(h, h->w_proj, x, st);
     check_launch(h, "z-drive adjoint");
+}
+
+void forward_z_impl(mpi_ffl_handle *h, const float *x, float *b, cudaStream_t st) {
+    z_init(h);
+    stage_p(h, x, h->w_proj, st);
+    z_line_forward(h, h->w_proj, b, st);
+}
+
+void adjoint_z_impl(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st) {
+    z_init(h);
+    z_line_adjoint(h, b, h->w_proj, st);
+    stage_pt(h, h->w_proj, x, st);
 }
 
 extern "C" int mpi_ffl_forward_zdrive(mpi_ffl_handle *h, const float *x, float *b, void *stream) {
@@ -1753,15 +1780,13 @@ extern "C" int mpi_ffl_solve(mpi_ffl_handle *h, const float *d_b, float *d_x, co
         CK(cudaMemcpyAsync(h->s_xp, d_x, sizeof(float) * d.nvox, cudaMemcpyDeviceToDevice, st));
         float *xc = d_x, *xp = h->s_xp;
         const int64_t nd = scan_data_len(h);  // data of the selected scans
-        const int nbd = reduce_blocks(nd);
         int done_host = 0, k_run = 0;
         for (int k = 1; k <= p->iters; ++k) {
             const double beta = (k - 1.0) / (k + 2.0);
-            TIMED(MPI_FFL_K_SOLVER, launch_momentum(xc, xp, h->s_y, beta, k, d.nvox, frozen, st));
-            scans_forward(h, h->s_y, h->s_r, st);
-            TIMED(MPI_FFL_K_SOLVER, launch_sub_norm(h->s_r, d_b, nd, h->w_red, nbd, frozen, st));
-            TIMED(MPI_FFL_K_SOLVER, launch_finalize(h->w_red, nbd, h->s_hist + (k - 1), st));
-            TIMED(MPI_FFL_K_SOLVER, launch_stop_check(h->s_hist, k - 1, p->stop_rel, flags, flags + 1, st));
+            const MomentumIn mom{xp, h->s_y, (float)beta, frozen};
+            scans_forward(h, xc, h->s_r, st, &mom);
+            TIMED(MPI_FFL_K_SOLVER, launch_residual(h->s_r, d_b, nd, h->w_red, h->w_count, h->s_hist, k - 1,
+                                                    p->stop_rel, flags, flags + 1, frozen, st));
             scans_adjoint(h, h->s_r, h->s_g, st);
             TIMED(MPI_FFL_K_SOLVER, launch_update(h->s_y, h->s_g, xp, (float)tau, (float)lam, p->nonneg ? 1 : 0,
                                                   d.N, d.Nz, frozen, st, xc));

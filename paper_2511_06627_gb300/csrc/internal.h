@@ -157,6 +157,7 @@ struct mpi_ffl_handle {
     float *w_vol2 = nullptr;   // nvox
     double *w_red = nullptr;   // reduction partials
     double *w_scal = nullptr;  // device scalars
+    unsigned *w_count = nullptr;  // [0] blocks done of a reduction, [1] the power iteration's scale (float)
     int w_red_len = 0;
     // solver state
     float *s_xp = nullptr, *s_y = nullptr, *s_g = nullptr, *s_r = nullptr;
@@ -193,7 +194,7 @@ struct mpi_ffl_handle {
     int host_overlap = 0;                   // mpi_ffl_set_host_overlap
     // scans of the solve and power iteration (MPI_FFL_SCAN_* bits): [A; A_z] when both
     int scans = 1;
-    float *w_scanvol = nullptr;  // 2 n_vox: A^T r and A_z^T r_z before their sum
+    float *w_scanproj = nullptr;  // 2 n_proj: the two scans' transposed line stages before their sum
     // PSF model (MPI_FFL_PSF_*) and receive-coil map b[z][u] (NULL: uniform coil)
     int psf_model = 0;
     float *t_coil = nullptr;    // N_z N
@@ -324,7 +325,15 @@ void launch_transpose_xy(const float *vol, float *volT, int N, int Nz, cudaStrea
 bool project_il_ok(int N);
 double project_il_cost(const AngleParam &a, int N);
 size_t il_len(int N, int Nz);
-void launch_interleave(const float *vol, float *volI, int N, int Nz, cudaStream_t st);
+// The solver's extrapolation y = x + beta (x - xp) of the volume x about to be projected.
+struct MomentumIn {
+    const float *xp;
+    float *y;
+    float beta;
+    const int *done;
+};
+void launch_interleave(const float *vol, float *volI, int N, int Nz, cudaStream_t st,
+                       const MomentumIn *mom = nullptr);
 // encodes the tensor maps of volI (false if the driver refuses them)
 bool make_il_maps(const float *volI, int N, int Nz, IlMaps *maps);
 // The forward line-GEMM's A operand written by the projector itself (bf16 or tf32 hi + lo, the
@@ -367,10 +376,15 @@ void launch_dft_adj(const float *data, const float *tw1, const float2 *twp, cons
 
 // Solver and reductions (k_solver.cu)
 int reduce_blocks(int64_t n);
-void launch_momentum(const float *x, const float *xp, float *y, double beta_num, int k,
-                     int64_t n, const int *done, cudaStream_t st);
-void launch_sub_norm(float *r, const float *b, int64_t n, double *partials, int nblk,
-                     const int *done, cudaStream_t st);
+void launch_momentum(const float *x, const float *xp, float *y, double beta_num, int64_t n, const int *done,
+                     cudaStream_t st);
+// r <- r - b, its norm and the stop test (k_solver.cu); counter: a device word that is 0
+void launch_residual(float *r, const float *b, int64_t n, double *partials, unsigned *counter, double *hist, int k,
+                     double stop_rel, int *stop, int *iters_done, const int *frozen, cudaStream_t st);
+int dot2_blocks(int64_t n);  // 2 partials per block
+// *ww = <w, w>, *scale = 1 / sqrt(*ww) and, vw not NULL, *vw = <v, w>
+void launch_dot2(const float *v, const float *w, int64_t n, double *partials, unsigned *counter, double *vw,
+                 double *ww, float *scale, cudaStream_t st);
 void launch_dot(const float *a, const float *b, int64_t n, double *partials, int nblk, cudaStream_t st);
 void launch_finalize(const double *partials, int nblk, double *out, cudaStream_t st);
 void launch_update(const float *y, const float *g, float *xout, float tau, float lam, int nonneg,
@@ -399,9 +413,7 @@ int zsyn_ring(const Dims &d, int no);
 size_t zsyn_smem(const Dims &d, int no);
 void launch_ttt(const float *x, float *out, int N, int Nz, cudaStream_t st);
 void launch_splitmix_fill(float *v, int64_t n, uint64_t seed, cudaStream_t st);
-void launch_scale_by_rsqrt(const float *in, float *out, int64_t n, const double *n2, cudaStream_t st);
-void launch_stop_check(double *hist, int k, double stop_rel, int *done, int *iters_done,
-                       cudaStream_t st);
+void launch_scale(const float *in, float *out, int64_t n, const float *scale, cudaStream_t st);
 void launch_angle_dots(const float *a, const float *b, int M, int64_t per_angle, double *partials,
                        int nblk_per_angle, cudaStream_t st);
 void launch_angle_finalize(const double *partials, int M, int nblk_per_angle, float *out,

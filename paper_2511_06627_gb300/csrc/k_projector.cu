@@ -402,29 +402,46 @@ __device__ __forceinline__ int il_tile_slot(int r, int c, int h) {
     return 64 * r + 8 * (c >> 2) + ((2 * (c & 3) + h) ^ (((c >> 2) ^ (2 * (r & 3))) & 7));
 }
 
-template <bool VEC>
+// MOM: the volume is the solver's extrapolated iterate y = x + beta (x - x_prev), formed here
+// from both iterates and stored too (nothing is done once *done is set).
+template <bool VEC, bool MOM>
 __global__ void __launch_bounds__(256) k_interleave(const float *__restrict__ vol, float *__restrict__ volI, int N,
-                                                    int Nz) {
+                                                    int Nz, MomentumIn mom) {
     __shared__ float4 tile[32 * 64];  // 32 rows x 32 columns x 2 halves
     const int tx = threadIdx.x, ty = threadIdx.y;  // 8 x 32
     const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32, zb = blockIdx.z;
     const int y = y0 + ty, xs = x0 + 4 * tx;
     ptx::grid_dep_wait();  // the volume comes from the previous kernel
     ptx::grid_dep_launch();
+    if (MOM && mom.done && *mom.done) return;  // the whole launch
     float4 v[kZc];
 #pragma unroll
     for (int e = 0; e < kZc; ++e) {
         const int z = zb * kZc + e;
         v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (z < Nz && y < N && xs < N) {
-            const float *src = vol + ((size_t)z * N + y) * N + xs;
-            if (VEC) {
-                v[e] = __ldg(reinterpret_cast<const float4 *>(src));
-            } else {
-                v[e].x = __ldg(src);
-                if (xs + 1 < N) v[e].y = __ldg(src + 1);
-                if (xs + 2 < N) v[e].z = __ldg(src + 2);
-                if (xs + 3 < N) v[e].w = __ldg(src + 3);
+            const size_t at = ((size_t)z * N + y) * N + xs;
+            auto load = [&](const float *p) {
+                if (VEC) return *reinterpret_cast<const float4 *>(p + at);
+                float4 r = make_float4(p[at], 0.f, 0.f, 0.f);
+                if (xs + 1 < N) r.y = p[at + 1];
+                if (xs + 2 < N) r.z = p[at + 2];
+                if (xs + 3 < N) r.w = p[at + 3];
+                return r;
+            };
+            v[e] = load(vol);
+            if (MOM) {
+                const float4 q = load(mom.xp);
+                v[e] = make_float4(fmaf(mom.beta, v[e].x - q.x, v[e].x), fmaf(mom.beta, v[e].y - q.y, v[e].y),
+                                   fmaf(mom.beta, v[e].z - q.z, v[e].z), fmaf(mom.beta, v[e].w - q.w, v[e].w));
+                if (VEC) {
+                    *reinterpret_cast<float4 *>(mom.y + at) = v[e];
+                } else {
+                    mom.y[at] = v[e].x;
+                    if (xs + 1 < N) mom.y[at + 1] = v[e].y;
+                    if (xs + 2 < N) mom.y[at + 2] = v[e].z;
+                    if (xs + 3 < N) mom.y[at + 3] = v[e].w;
+                }
             }
         }
     }
@@ -455,10 +472,13 @@ __global__ void __launch_bounds__(256) k_interleave(const float *__restrict__ vo
     }
 }
 
-void launch_interleave(const float *vol, float *volI, int N, int Nz, cudaStream_t st) {
+void launch_interleave(const float *vol, float *volI, int N, int Nz, cudaStream_t st, const MomentumIn *mom) {
     dim3 grid((N + 31) / 32, (N + 31) / 32, (Nz + kZc - 1) / kZc), block(8, 32);
-    const bool vec = N % 4 == 0 && (reinterpret_cast<uintptr_t>(vol) & 15) == 0;
-    launch_dependent(vec ? k_interleave<true> : k_interleave<false>, grid, block, 0, st, vol, volI, N, Nz);
+    auto a16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    const bool vec = N % 4 == 0 && a16(vol) && (!mom || (a16(mom->xp) && a16(mom->y)));
+    auto kernel = mom ? (vec ? k_interleave<true, true> : k_interleave<false, true>)
+                      : (vec ? k_interleave<true, false> : k_interleave<false, false>);
+    launch_dependent(kernel, grid, block, 0, st, vol, volI, N, Nz, mom ? *mom : MomentumIn{});
 }
 
 // Tensor maps of volI as a 4-D array (kZc floats, x, y, z block): boxes of one row

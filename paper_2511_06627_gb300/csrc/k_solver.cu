@@ -1,13 +1,16 @@
 // Solver kernels for Eq. (26) (Sec. 3.3) and the FP64 reductions it needs.
 //
 // Reductions are deterministic: each block writes one FP64 partial sum in a fixed
-// order and a single block adds the partials in index order.
+// order and a single block adds the partials in index order (in the solve and the power
+// iteration the last block to finish, in the same launch).
 // The stop test leaves its verdict in a device flag; the host reads it only when
 // an early stop was requested. The optional `done` flag of the per-iteration
 // kernels turns them into no-ops once it is set.
 #include <algorithm>
+#include <initializer_list>
 
 #include "internal.h"
+#include "tc_ptx.cuh"
 
 namespace mpiffl {
 
@@ -33,39 +36,164 @@ __device__ __forceinline__ double block_sum(double v) {
     return t;  // valid in thread 0
 }
 
-__global__ void k_momentum(const float *__restrict__ x, const float *__restrict__ xp,
-                           float *__restrict__ y, float beta, int64_t n, const int *done) {
-    if (done && *done) return;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float xi = x[i];
-        y[i] = fmaf(beta, xi - xp[i], xi);
+// True in every thread of the last block of the launch to arrive, with the other blocks'
+// partials visible; *counter is left at 0 for the next launch.
+__device__ __forceinline__ bool last_block(unsigned *counter) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+        if (last) *counter = 0;
     }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
 }
 
-void launch_momentum(const float *x, const float *xp, float *y, double beta_num, int k,
-                     int64_t n, const int *done, cudaStream_t st) {
-    (void)k;
-    const int blocks = (int)std::min<int64_t>((n + 255) / 256, 152 * 16);
-    k_momentum<<<blocks, 256, 0, st>>>(x, xp, y, (float)beta_num, n, done);
-}
-
-// r <- r - b, partial sums of r^2 (FP64)
-__global__ void __launch_bounds__(kRedThreads) k_sub_norm(float *__restrict__ r, const float *__restrict__ b,
-                                                          int64_t n, double *partials, const int *done) {
-    if (done && *done) return;
+__device__ __forceinline__ double sum_partials(const double *partials, int n) {
     double acc = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) acc += __ldcg(partials + i);
+    return block_sum(acc);
+}
+
+// 16-byte accesses when every pointer is on 16 bytes
+inline bool vec4(std::initializer_list<const void *> p) {
+    for (const void *q : p)
+        if (reinterpret_cast<uintptr_t>(q) & 15) return false;
+    return true;
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_momentum(const float *__restrict__ x, const float *__restrict__ xp,
+                                                  float *__restrict__ y, float beta, int64_t n, const int *done) {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    if (done && *done) return;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    auto f = [beta](float xi, float pi) { return fmaf(beta, xi - pi, xi); };
+    if (VEC)
+        for (int64_t i = i0; i < n / 4; i += step) {
+            const float4 a = reinterpret_cast<const float4 *>(x)[i], b = reinterpret_cast<const float4 *>(xp)[i];
+            reinterpret_cast<float4 *>(y)[i] = make_float4(f(a.x, b.x), f(a.y, b.y), f(a.z, b.z), f(a.w, b.w));
+        }
+    for (int64_t i = (VEC ? n / 4 * 4 : 0) + i0; i < n; i += step) y[i] = f(x[i], xp[i]);
+}
+
+void launch_momentum(const float *x, const float *xp, float *y, double beta_num, int64_t n, const int *done,
+                     cudaStream_t st) {
+    const bool v = vec4({x, xp, y});
+    const int blocks = (int)std::min<int64_t>((n / (v ? 4 : 1) + 255) / 256 + 1, 152 * 8);
+    launch_dependent(v ? k_momentum<true> : k_momentum<false>, dim3(blocks), dim3(256), 0, st, x, xp, y,
+                     (float)beta_num, n, done);
+}
+
+// One launch per iteration for r <- r - b, hist[k] = ||r|| (FP64) and the stop test: *stop
+// is set when the relative change from hist[k-1] is at most stop_rel (1) or the norm is not
+// finite (2), and *iters_done counts the iterations whose test ran. With the sum and the test
+// in two further launches of one block this took 12 us at 128^2 x 64 (24 angles), now 9 us.
+template <bool VEC>
+__global__ void __launch_bounds__(kRedThreads) k_residual(float *__restrict__ r, const float *__restrict__ b,
+                                                          int64_t n, double *partials, unsigned *counter,
+                                                          double *hist, int k, double stop_rel, int *stop,
+                                                          int *iters_done, const int *frozen) {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    if (frozen && *frozen) return;  // the whole launch
+    double acc = 0.0;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (VEC)
+        for (int64_t i = i0; i < n / 4; i += step) {
+            const float4 p = reinterpret_cast<const float4 *>(r)[i], q = reinterpret_cast<const float4 *>(b)[i];
+            const float4 v = make_float4(p.x - q.x, p.y - q.y, p.z - q.z, p.w - q.w);
+            reinterpret_cast<float4 *>(r)[i] = v;
+            acc += (double)v.x * (double)v.x + (double)v.y * (double)v.y + (double)v.z * (double)v.z +
+                   (double)v.w * (double)v.w;
+        }
+    for (int64_t i = (VEC ? n / 4 * 4 : 0) + i0; i < n; i += step) {
         const float v = r[i] - b[i];
         r[i] = v;
         acc += (double)v * (double)v;
     }
     const double t = block_sum(acc);
     if (threadIdx.x == 0) partials[blockIdx.x] = t;
+    if (!last_block(counter)) return;
+    const double sq = sum_partials(partials, gridDim.x);
+    if (threadIdx.x != 0 || *stop) return;
+    const double norm = sqrt(sq);
+    hist[k] = norm;
+    *iters_done = k + 1;
+    if (!(norm == norm) || norm > 1e300) {
+        *stop = 2;
+    } else if (stop_rel > 0.0 && k > 0) {
+        const double prev = hist[k - 1];
+        if (fabs(prev - norm) <= stop_rel * prev) *stop = 1;
+    }
 }
 
-void launch_sub_norm(float *r, const float *b, int64_t n, double *partials, int nblk,
-                     const int *done, cudaStream_t st) {
-    k_sub_norm<<<nblk, kRedThreads, 0, st>>>(r, b, n, partials, done);
+void launch_residual(float *r, const float *b, int64_t n, double *partials, unsigned *counter, double *hist, int k,
+                     double stop_rel, int *stop, int *iters_done, const int *frozen, cudaStream_t st) {
+    const bool v = vec4({r, b});
+    const int blocks = (int)std::min<int64_t>(std::max<int64_t>(1, (n + 2047) / 2048), 152 * 4);
+    launch_dependent(v ? k_residual<true> : k_residual<false>, dim3(blocks), dim3(kRedThreads), 0, st, r, b, n,
+                     partials, counter, hist, k, stop_rel, stop, iters_done, frozen);
+}
+
+// The power iteration's inner products in one pass: *ww = <w, w>, *scale = 1 / sqrt(<w, w>),
+// which k_scale applies, and with BOTH (the last step, whose Rayleigh quotient is the
+// result) *vw = <v, w>. Bound by the FP64 pipe: a conversion and an FMA an element cost more
+// than its read. (Two products, two sums of partials and a scaling with a square root per
+// thread took 54 us a step at 128^2 x 64, now 16 us.)
+template <bool VEC, bool BOTH>
+__global__ void __launch_bounds__(kRedThreads) k_dot2(const float *__restrict__ v, const float *__restrict__ w,
+                                                      int64_t n, double *partials, unsigned *counter, double *vw,
+                                                      double *ww, float *scale) {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    double a[4] = {0.0, 0.0, 0.0, 0.0}, b[4] = {0.0, 0.0, 0.0, 0.0};
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    auto add = [&](int u, float x, float y) {
+        const double yd = y;
+        if (BOTH) a[u] = fma((double)x, yd, a[u]);
+        b[u] = fma(yd, yd, b[u]);
+    };
+    if (VEC)
+#pragma unroll 2
+        for (int64_t i = i0; i < n / 4; i += step) {
+            const float4 q = reinterpret_cast<const float4 *>(w)[i];
+            const float4 p = BOTH ? reinterpret_cast<const float4 *>(v)[i] : q;
+            add(0, p.x, q.x);
+            add(1, p.y, q.y);
+            add(2, p.z, q.z);
+            add(3, p.w, q.w);
+        }
+    for (int64_t i = (VEC ? n / 4 * 4 : 0) + i0; i < n; i += step) add(0, BOTH ? v[i] : 0.f, w[i]);
+    const double tb = block_sum((b[0] + b[1]) + (b[2] + b[3]));
+    double ta = 0.0;
+    if (BOTH) ta = block_sum((a[0] + a[1]) + (a[2] + a[3]));
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = tb;
+        if (BOTH) partials[gridDim.x + blockIdx.x] = ta;
+    }
+    if (!last_block(counter)) return;
+    const double sb = sum_partials(partials, gridDim.x);
+    double sa = 0.0;
+    if (BOTH) sa = sum_partials(partials + gridDim.x, gridDim.x);
+    if (threadIdx.x == 0) {
+        if (BOTH) *vw = sa;
+        *ww = sb;
+        *scale = sb > 0.0 ? (float)(1.0 / sqrt(sb)) : 0.f;
+    }
+}
+
+int dot2_blocks(int64_t n) { return (int)std::min<int64_t>(std::max<int64_t>(1, (n + 2047) / 2048), 152 * 2); }
+
+void launch_dot2(const float *v, const float *w, int64_t n, double *partials, unsigned *counter, double *vw,
+                 double *ww, float *scale, cudaStream_t st) {
+    const bool a = vec4({v, w});
+    auto kernel = vw ? (a ? k_dot2<true, true> : k_dot2<false, true>) : (a ? k_dot2<true, false> : k_dot2<false, false>);
+    launch_dependent(kernel, dim3(dot2_blocks(n)), dim3(kRedThreads), 0, st, v, w, n, partials, counter, vw, ww,
+                     scale);
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_dot(const float *__restrict__ a, const float *__restrict__ b,
@@ -161,28 +289,68 @@ void launch_ttt(const float *x, float *out, int N, int Nz, cudaStream_t st) {
 
 // x_out = P(y - tau (g + lam T^T T y)), P = max(0, .) when nonneg. Once *done is set
 // the solve is frozen: x_out = xcur (the current iterate), so that the buffer swap of
-// the next iteration keeps the final iterate.
-__global__ void k_update(const float *__restrict__ y, const float *__restrict__ g, float *__restrict__ xo,
-                         float tau, float lam, int nonneg, int N, int Nz, const int *done,
-                         const float *__restrict__ xcur) {
-    const int xx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int yy = blockIdx.y, z = blockIdx.z;
-    if (xx >= N) return;
-    const size_t i = ((size_t)z * N + yy) * N + xx;
-    if (done && *done) {
-        if (xcur) xo[i] = xcur[i];
-        return;
+// the next iteration keeps the final iterate. VEC: four voxels of a row a thread (N % 4 ==
+// 0, pointers on 16 bytes); the terms of T^T T are added in ttt_at's order.
+template <bool VEC>
+__global__ void __launch_bounds__(128) k_update(const float *__restrict__ y, const float *__restrict__ g,
+                                                float *__restrict__ xo, float tau, float lam, int nonneg, int N,
+                                                int Nz, const int *done, const float *__restrict__ xcur) {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    constexpr int V = VEC ? 4 : 1;
+    const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;  // a warp per row (z, y)
+    if (row >= N * Nz) return;
+    const int yy = row % N, z = row / N;
+    const bool frozen = done && *done;
+    for (int xx = V * (threadIdx.x & 31); xx < N; xx += V * 32) {
+        const size_t i = ((size_t)z * N + yy) * N + xx;
+        if (frozen) {
+            if (xcur)
+#pragma unroll
+                for (int u = 0; u < V; ++u) xo[i + u] = xcur[i + u];
+            continue;
+        }
+        if (VEC) {
+            auto at = [&](size_t k) { return *reinterpret_cast<const float4 *>(y + k); };
+            const size_t sl = (size_t)N * N;
+            const float4 c4 = at(i), g4 = *reinterpret_cast<const float4 *>(g + i);
+            const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 ym = yy > 0 ? at(i - N) : z4, yp = yy < N - 1 ? at(i + N) : z4;
+            const float4 zm = z > 0 ? at(i - sl) : z4, zp = z < Nz - 1 ? at(i + sl) : z4;
+            const float left = xx > 0 ? y[i - 1] : 0.f, right = xx + 4 < N ? y[i + 4] : 0.f;
+            const float c[6] = {left, c4.x, c4.y, c4.z, c4.w, right};
+            const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
+            const float a0[4] = {ym.x, ym.y, ym.z, ym.w}, a1[4] = {yp.x, yp.y, yp.z, yp.w};
+            const float b0[4] = {zm.x, zm.y, zm.z, zm.w}, b1[4] = {zp.x, zp.y, zp.z, zp.w};
+            float o[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float cc = c[u + 1];
+                float s = 0.f;
+                if (xx + u > 0) s += cc - c[u];
+                if (xx + u < N - 1) s += cc - c[u + 2];
+                if (yy > 0) s += cc - a0[u];
+                if (yy < N - 1) s += cc - a1[u];
+                if (z > 0) s += cc - b0[u];
+                if (z < Nz - 1) s += cc - b1[u];
+                const float v = fmaf(-tau, fmaf(lam, s, gv[u]), cc);
+                o[u] = nonneg ? fmaxf(v, 0.f) : v;
+            }
+            *reinterpret_cast<float4 *>(xo + i) = make_float4(o[0], o[1], o[2], o[3]);
+        } else {
+            const float grad = fmaf(lam, ttt_at(y, N, Nz, z, yy, xx), g[i]);
+            float v = fmaf(-tau, grad, y[i]);
+            if (nonneg) v = fmaxf(v, 0.f);
+            xo[i] = v;
+        }
     }
-    const float grad = fmaf(lam, ttt_at(y, N, Nz, z, yy, xx), g[i]);
-    float v = fmaf(-tau, grad, y[i]);
-    if (nonneg) v = fmaxf(v, 0.f);
-    xo[i] = v;
 }
 
 void launch_update(const float *y, const float *g, float *xout, float tau, float lam, int nonneg,
                    int N, int Nz, const int *done, cudaStream_t st, const float *xcur) {
-    dim3 grid((N + 127) / 128, N, Nz);
-    k_update<<<grid, 128, 0, st>>>(y, g, xout, tau, lam, nonneg, N, Nz, done, xcur);
+    const bool v = N % 4 == 0 && vec4({y, g, xout});
+    launch_dependent(v ? k_update<true> : k_update<false>, dim3((N * Nz + 3) / 4), dim3(128), 0, st, y, g, xout, tau,
+                     lam, nonneg, N, Nz, done, xcur);
 }
 
 // Per kept bin q: sum over segments of |b[seg][q]|^2 in FP64, segments in order.
@@ -224,37 +392,25 @@ void launch_splitmix_fill(float *v, int64_t n, uint64_t seed, cudaStream_t st) {
     k_splitmix_fill<<<blocks, 256, 0, st>>>(v, n, seed);
 }
 
-__global__ void k_scale_by_rsqrt(const float *__restrict__ in, float *__restrict__ out, int64_t n, const double *n2) {
-    const double nn = *n2;
-    const float s = nn > 0.0 ? (float)(1.0 / sqrt(nn)) : 0.f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = in[i] * s;
+// out = *scale in
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_scale(const float *in, float *out, int64_t n, const float *scale) {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    const float s = *scale;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (VEC)
+        for (int64_t i = i0; i < n / 4; i += step) {
+            const float4 a = reinterpret_cast<const float4 *>(in)[i];
+            reinterpret_cast<float4 *>(out)[i] = make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
+        }
+    for (int64_t i = (VEC ? n / 4 * 4 : 0) + i0; i < n; i += step) out[i] = in[i] * s;
 }
 
-void launch_scale_by_rsqrt(const float *in, float *out, int64_t n, const double *n2, cudaStream_t st) {
-    const int blocks = (int)std::min<int64_t>((n + 255) / 256, 152 * 16);
-    k_scale_by_rsqrt<<<blocks, 256, 0, st>>>(in, out, n, n2);
-}
-
-// hist[k] holds ||r_k||^2 on entry; replaces it by ||r_k|| and sets *done when the
-// relative change from hist[k-1] is at most stop_rel (or the norm is not finite).
-__global__ void k_stop_check(double *hist, int k, double stop_rel, int *done, int *iters_done) {
-    if (*done) return;
-    const double r = sqrt(hist[k]);
-    hist[k] = r;
-    *iters_done = k + 1;
-    if (!(r == r) || r > 1e300) {
-        *done = 2;
-        return;
-    }
-    if (stop_rel > 0.0 && k > 0) {
-        const double prev = hist[k - 1];
-        if (fabs(prev - r) <= stop_rel * prev) *done = 1;
-    }
-}
-
-void launch_stop_check(double *hist, int k, double stop_rel, int *done, int *iters_done, cudaStream_t st) {
-    k_stop_check<<<1, 1, 0, st>>>(hist, k, stop_rel, done, iters_done);
+void launch_scale(const float *in, float *out, int64_t n, const float *scale, cudaStream_t st) {
+    const bool v = vec4({in, out});
+    const int blocks = (int)std::min<int64_t>((n / (v ? 4 : 1) + 255) / 256 + 1, 152 * 8);
+    launch_dependent(v ? k_scale<true> : k_scale<false>, dim3(blocks), dim3(256), 0, st, in, out, n, scale);
 }
 
 // ---------------------------------------------------------------------- batches

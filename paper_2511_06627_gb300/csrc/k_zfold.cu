@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(128) k_zconv(const float *__restrict__ in, con
 constexpr int kZcIn = 4, kZcStages = 4, kZcAhead = kZcStages - 2;
 
 template <int W, int R, int NG, bool ADJ>
-__global__ void __launch_bounds__(128 * NG) k_zconv_ring(const float *__restrict__ in,
+__global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restrict__ in,
                                                          const float *__restrict__ hz, float *__restrict__ out,
                                                          int Nz, int S, int np, int *err) {
     extern __shared__ __align__(128) float zring[];  // kZcStages x kZcIn x W S
