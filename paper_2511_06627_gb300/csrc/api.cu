@@ -517,7 +517,7 @@ bool stage_p(mpi_ffl_handle *h, const float *x, float *proj, cudaStream_t st, co
         x = mom->y;
     }
     if (any_column_angle(h)) TIMED(MPI_FFL_K_TRANSPOSE, launch_transpose_xy(x, h->w_volT, h->d.N, h->d.Nz, st));
-    TIMED(MPI_FFL_K_PROJECT, launch_project(x, h->w_volT, h->t_ang, h->t_agroups, h->n_agroups, proj, h->d.N, h->d.Nz, st, h->w_err));
+    TIMED(MPI_FFL_K_PROJECT, launch_project(x, h->w_volT, h->t_ang, h->t_agroups, h->n_agroups, proj, h->d.N, h->d.Nz, st));
     check_launch(h, "project");
     return false;
 }
@@ -903,7 +903,6 @@ double power_norm_for_job(mpi_ffl_handle *h, int n_iter, uint64_t seed, cudaStre
     return power_norm_impl(h, n_iter, seed, st);
 }
 double ttt_norm_for_job(const Dims &d) { return ttt_norm(d); }
-bool handle_has_column_angles(const mpi_ffl_handle *h) { return any_column_angle(h); }
 void forward_for_job(mpi_ffl_handle *h, const float *x, float *b, cudaStream_t st) {
     forward_impl(h, x, b, h->t_htab, h->t_gain, st);
 }
@@ -972,7 +971,7 @@ extern "C" int mpi_ffl_create(const mpi_ffl_geometry *geom, const mpi_ffl_trajec
         dev_alloc(h, &h->w_volT, d.nvox);
         if (project_il_ok(d.N)) {
             dev_alloc(h, &h->w_volI, il_len(d.N, d.Nz));
-            if (!make_il_maps(h->w_volI, d.N, d.Nz, &h->il_maps)) {  // the pipelined projector serves
+            if (!make_il_maps(h->w_volI, d.N, d.Nz, &h->il_maps)) {  // the plain projector serves
                 dev_free(h->w_volI);
                 h->w_volI = nullptr;
                 h->bytes -= (int64_t)(il_len(d.N, d.Nz) * sizeof(float));

@@ -3,10 +3,10 @@
 // A job is one reconstruction: its handle (tables and workspace), its compressed
 // data and its solver state (x, x_prev, y, gradient, residual, residual history),
 // all resident on the device. mpi_ffl_job_step advances a set of jobs by one
-// iteration each, as one launch per kernel kind for all of them: momentum, residual,
-// residual norm and stop test, update for every job; x/y transpose, projector, line
+// iteration each, as one launch per kernel kind for all of them: residual norm and stop
+// test, update for every job; extrapolation with the interleaved copy, projector, line
 // GEMM, adjoint line GEMM and backprojector for the jobs on the full-GEMM path (jobs
-// on other paths apply their A and A^T alone between those launches). Each launch is
+// on other paths extrapolate and apply their A and A^T alone between those launches). Each launch is
 // persistent: a grid of what the GPU holds at once loops over the work items of every
 // job (found through an offset table), so the launch count per iteration does not grow
 // with the number of jobs. Jobs that have met their stop test do no further work on
@@ -33,7 +33,6 @@ struct mpi_ffl_job {
     int iters = 0;
     double tau = 0, lam = 0, stop_rel = 0;
     int nonneg = 1;
-    bool col_angles = false;
     int64_t bytes = 0;
 };
 
@@ -41,7 +40,6 @@ namespace mpiffl {
 // from api.cu
 double power_norm_for_job(mpi_ffl_handle *h, int n_iter, uint64_t seed, cudaStream_t st);
 double ttt_norm_for_job(const Dims &d);
-bool handle_has_column_angles(const mpi_ffl_handle *h);
 void forward_for_job(mpi_ffl_handle *h, const float *x, float *b, cudaStream_t st);
 void adjoint_for_job(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st);
 }  // namespace mpiffl
@@ -85,7 +83,7 @@ bool staging_ready(size_t need) {
 
 template <class T>
 size_t put(std::vector<uint8_t> &buf, const T *p, size_t n) {
-    const size_t off = (buf.size() + 15) / 16 * 16;
+    const size_t off = (buf.size() + 127) / 128 * 128;  // tensor maps among the arguments
     buf.resize(off + n * sizeof(T));
     if (n) std::memcpy(buf.data() + off, p, n * sizeof(T));
     return off;
@@ -121,7 +119,6 @@ extern "C" int mpi_ffl_job_create(mpi_ffl_handle *h, const float *d_b, const flo
     j->nonneg = p->nonneg ? 1 : 0;
     j->stop_rel = p->stop_rel;
     j->nblk = std::max(1, std::min(1024, (int)((d.ndata + 4095) / 4096)));
-    j->col_angles = handle_has_column_angles(h);
     auto alloc = [&](void **ptr, size_t bytes) {
         if (dev_malloc(ptr, bytes) != cudaSuccess) {
             cudaGetLastError();
@@ -169,7 +166,7 @@ extern "C" int mpi_ffl_job_destroy(mpi_ffl_job *j) {
     return MPI_FFL_OK;
 }
 
-extern "C" int mpi_ffl_job_step(mpi_ffl_job *const *jobs, int32_t n, void *stream) {
+static int job_step(mpi_ffl_job *const *jobs, int32_t n, void *stream) {
     if (n < 0 || (n > 0 && !jobs)) return MPI_FFL_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     std::vector<mpi_ffl_job *> all, batch, single;
@@ -178,7 +175,7 @@ extern "C" int mpi_ffl_job_step(mpi_ffl_job *const *jobs, int32_t n, void *strea
         if (!j) return MPI_FFL_ERR_INVALID_ARG;
         if (j->k > j->iters) continue;  // iteration budget used up
         all.push_back(j);
-        if (j->h->path == MPI_FFL_PATH_FULL_GEMM && col_supported(j->h) && project_batch_ok(j->h->d.N) &&
+        if (j->h->path == MPI_FFL_PATH_FULL_GEMM && col_supported(j->h) && j->h->w_volI &&
             j->h->psf_model == MPI_FFL_PSF_COLLINEAR && !j->h->t_coil)
             batch.push_back(j);
         else single.push_back(j);
@@ -187,28 +184,38 @@ extern "C" int mpi_ffl_job_step(mpi_ffl_job *const *jobs, int32_t n, void *strea
     if (na == 0) return MPI_FFL_OK;
 
     // ---------------------------------------------------------------- staging
-    std::vector<uint8_t> buf;
-    std::vector<MomentumJob> mom(na);
+    // kept from call to call: filling them anew is cheaper than allocating and clearing them
+    static thread_local std::vector<uint8_t> buf, gf, ga;
+    static thread_local std::vector<int4> itf, ita;
+    buf.clear();
+    const int ns = (int)single.size();
+    std::vector<MomentumJob> mom(ns);
     std::vector<ResidualJob> rs(na);
     std::vector<StopJob> sp(na);
     std::vector<UpdateJob> up(na);
-    std::vector<int> off_m(na + 1, 0), off_r(na + 1, 0), off_u(na + 1, 0);
+    std::vector<int> off_m(ns + 1, 0), off_r(na + 1, 0), off_u(na + 1, 0);
+    for (int i = 0; i < ns; ++i) {
+        mpi_ffl_job *j = single[i];
+        const int64_t n = j->h->d.nvox;
+        mom[i] = MomentumJob{j->x, j->xp, j->y, (float)((j->k - 1.0) / (j->k + 2.0)), n, j->flags + 2};
+        off_m[i + 1] = off_m[i] + (int)((n + 2047) / 2048);
+    }
     for (int i = 0; i < na; ++i) {
         mpi_ffl_job *j = all[i];
         const Dims &d = j->h->d;
         const int *done = j->flags + 2;
-        mom[i] = MomentumJob{j->x, j->xp, j->y, (float)((j->k - 1.0) / (j->k + 2.0)), d.nvox, done};
-        off_m[i + 1] = off_m[i] + (int)((d.nvox + 2047) / 2048);
         rs[i] = ResidualJob{j->r, j->b, d.ndata, j->partials, j->nblk, done};
         off_r[i + 1] = off_r[i] + j->nblk;
         sp[i] = StopJob{j->partials, j->nblk, j->hist, j->k - 1, j->stop_rel, j->flags, j->flags + 2};
-        up[i] = UpdateJob{j->y, j->g, j->xp, j->x, (float)j->tau, (float)j->lam, j->nonneg, d.N, d.Nz, done};
+        // (the job's buffers are its own allocations, on 16 bytes)
+        up[i] = UpdateJob{j->y, j->g, j->xp, j->x, (float)j->tau, (float)j->lam, j->nonneg, d.N, d.Nz, done, d.N % 4 == 0};
         off_u[i + 1] = off_u[i] + update_blocks(d.N, d.Nz);
     }
-    std::vector<TransposeJob> tr;
+    std::vector<InterleaveJob> il(nb);
     std::vector<ProjectJob> pj(nb);
     std::vector<BackprojectJob> bp(nb);
-    std::vector<int> off_t(1, 0), off_p(nb + 1, 0), off_b(nb + 1, 0);
+    std::vector<char> pre(nb);
+    std::vector<int> off_i(nb + 1, 0), off_p(nb + 1, 0), off_b(nb + 1, 0);
     std::vector<mpi_ffl_handle *> hs(nb);
     std::vector<const float *> gin_f(nb), gin_a(nb);
     std::vector<float *> gout_f(nb), gout_a(nb);
@@ -222,11 +229,14 @@ extern "C" int mpi_ffl_job_step(mpi_ffl_job *const *jobs, int32_t n, void *strea
         dn[i] = done;
         hs[i] = h;
         maxN = std::max(maxN, d.N);
-        if (j->col_angles) {
-            tr.push_back(TransposeJob{j->y, h->w_volT, d.N, d.Nz, done});
-            off_t.push_back(off_t.back() + transpose_blocks(d.N, d.Nz));
-        }
-        pj[i] = ProjectJob{j->y, h->w_volT, h->t_ang, h->t_agroups, h->w_proj, d.N, d.Nz, h->n_agroups, done};
+        il[i] = InterleaveJob{j->x, h->w_volI, MomentumIn{j->xp, j->y, (float)((j->k - 1.0) / (j->k + 2.0)), done},
+                              d.N, d.Nz, d.N % 4 == 0};
+        off_i[i + 1] = off_i[i] + interleave_blocks(d.N, d.Nz);
+        ProjPack pack{};
+        pre[i] = col_prepack_targets(h, &pack);
+        if (!pre[i]) pack = ProjPack{};
+        pj[i] = ProjectJob{h->il_maps.row, h->il_maps.col, h->t_ang, h->t_agroups, pre[i] ? nullptr : h->w_proj, d.N,
+                           d.Nz, h->n_agroups, h->il_maps.nbox, h->il_maps.box, done, pack};
         off_p[i + 1] = off_p[i] + project_blocks(h->n_agroups, d.Nz);
         gin_f[i] = h->w_proj;
         gout_f[i] = j->r;
@@ -237,23 +247,25 @@ extern "C" int mpi_ffl_job_step(mpi_ffl_job *const *jobs, int32_t n, void *strea
     }
     const int arg_cap = 2 * std::max(nb, 1);
     const int item_cap = 65536;
-    std::vector<uint8_t> gf(gemm_args_size() * arg_cap), ga(gemm_args_size() * arg_cap);
-    std::vector<int4> itf(item_cap), ita(item_cap);
+    if (gf.size() < gemm_args_size() * arg_cap) gf.resize(gemm_args_size() * arg_cap);
+    if (ga.size() < gemm_args_size() * arg_cap) ga.resize(gemm_args_size() * arg_cap);
+    if (itf.size() < (size_t)item_cap) itf.resize(item_cap);
+    if (ita.size() < (size_t)item_cap) ita.resize(item_cap);
     int nif = 0, nia = 0, npf = 0, npa = 0;
     size_t smf = 0, sma = 0;
     uint32_t tcf = 32, tca = 32;
     if (nb > 0) {
-        npf = col_batch_prepare(hs.data(), gin_f.data(), gout_f.data(), dn.data(), nb, false, gf.data(), itf.data(),
-                                arg_cap, item_cap, nif, smf, tcf);
-        npa = col_batch_prepare(hs.data(), gin_a.data(), gout_a.data(), dn.data(), nb, true, ga.data(), ita.data(),
-                                arg_cap, item_cap, nia, sma, tca);
+        npf = col_batch_prepare(hs.data(), gin_f.data(), gout_f.data(), dn.data(), pre.data(), nb, false, gf.data(),
+                                itf.data(), arg_cap, item_cap, nif, smf, tcf);
+        npa = col_batch_prepare(hs.data(), gin_a.data(), gout_a.data(), dn.data(), nullptr, nb, true, ga.data(),
+                                ita.data(), arg_cap, item_cap, nia, sma, tca);
         if (npf < 0 || npa < 0) return MPI_FFL_ERR_UNSUPPORTED;
     }
     const size_t o_mom = put(buf, mom), o_offm = put(buf, off_m);
     const size_t o_rs = put(buf, rs), o_offr = put(buf, off_r);
     const size_t o_sp = put(buf, sp);
     const size_t o_up = put(buf, up), o_offu = put(buf, off_u);
-    const size_t o_tr = put(buf, tr), o_offt = put(buf, off_t);
+    const size_t o_il = put(buf, il), o_offi = put(buf, off_i);
     const size_t o_pj = put(buf, pj), o_offp = put(buf, off_p);
     const size_t o_gf = put(buf, gf.data(), gemm_args_size() * npf), o_itf = put(buf, itf.data(), nif);
     const size_t o_ga = put(buf, ga.data(), gemm_args_size() * npa), o_ita = put(buf, ita.data(), nia);
@@ -270,11 +282,9 @@ extern "C" int mpi_ffl_job_step(mpi_ffl_job *const *jobs, int32_t n, void *strea
     auto at = [&](size_t o) { return (void *)(D + o); };
 
     // ---------------------------------------------------------------- one iteration, every job
-    launch_momentum_batch((const MomentumJob *)at(o_mom), (const int *)at(o_offm), na, off_m[na], st);
+    launch_momentum_batch((const MomentumJob *)at(o_mom), (const int *)at(o_offm), ns, off_m[ns], st);
     if (nb > 0) {
-        if (!tr.empty())
-            launch_transpose_batch((const TransposeJob *)at(o_tr), (const int *)at(o_offt), (int)tr.size(),
-                                   off_t.back(), st);
+        launch_interleave_batch((const InterleaveJob *)at(o_il), (const int *)at(o_offi), nb, off_i[nb], st);
         launch_project_batch((const ProjectJob *)at(o_pj), (const int *)at(o_offp), nb, off_p[nb], maxN,
                              batch[0]->h->w_err, st);
         col_batch_launch(at(o_gf), (const int4 *)at(o_itf), nif, smf, tcf, st);
@@ -295,6 +305,14 @@ extern "C" int mpi_ffl_job_step(mpi_ffl_job *const *jobs, int32_t n, void *strea
     }
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
+}
+
+extern "C" int mpi_ffl_job_step(mpi_ffl_job *const *jobs, int32_t n, void *stream) {
+    try {
+        return job_step(jobs, n, stream);
+    } catch (...) {
+        return MPI_FFL_ERR_OOM;  // a host allocation
+    }
 }
 
 extern "C" int mpi_ffl_job_status(const mpi_ffl_job *j, mpi_ffl_job_status_t *out, void *stream) {

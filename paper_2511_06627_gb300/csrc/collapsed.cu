@@ -628,7 +628,8 @@ void launch_problems(const GemmArgs *g, const Packed *const *B, int n, cudaStrea
 }  // namespace
 
 // Arguments of the GEMM problems of one line stage of handle h (one per trajectory).
-int gemm_problems(const mpi_ffl_handle *h, bool adjoint, const float *in, float *out, const int *done,
+// prepacked: the projector writes the forward's A operand (col_prepack_targets).
+int gemm_problems(const mpi_ffl_handle *h, bool adjoint, const float *in, float *out, const int *done, bool prepacked,
                   GemmArgs *args, int4 *items, int item_cap, int &n_items) {
     ColState *s = cs(h);
     const Dims &d = h->d;
@@ -658,6 +659,11 @@ int gemm_problems(const mpi_ffl_handle *h, bool adjoint, const float *in, float 
         set_accumulators(g, B.per_sm);
         g.err = s->err;
         g.done = done;
+        if (prepacked) {
+            g.apk = s->apk[0][par];
+            g.apk_jg = 1;
+            g.apk_gper = (g.M + 7) / 8;
+        }
         for (int mt = 0; mt < (g.M + kBM - 1) / kBM; ++mt)
             for (int nt = 0; nt < B.ntile; ++nt) {
                 if (n_items >= item_cap) return -1;
@@ -899,7 +905,7 @@ size_t gemm_args_size() { return sizeof(GemmArgs); }
 // args/items are host staging arrays; dargs/ditems their device copies (same
 // layout), already uploaded by the caller before this launch runs.
 int col_batch_prepare(mpi_ffl_handle *const *hs, const float *const *in, float *const *out, const int *const *done,
-                      int n, bool adjoint, void *args, int4 *items, int arg_cap, int item_cap, int &n_items,
+                      const char *prepacked, int n, bool adjoint, void *args, int4 *items, int arg_cap, int item_cap, int &n_items,
                       size_t &smem, uint32_t &tmem_cols) {
     GemmArgs *a = reinterpret_cast<GemmArgs *>(args);
     int np = 0;
@@ -909,7 +915,7 @@ int col_batch_prepare(mpi_ffl_handle *const *hs, const float *const *in, float *
     for (int j = 0; j < n; ++j) {
         if (np + 2 > arg_cap) return -1;
         const int base_items = n_items;
-        const int k = gemm_problems(hs[j], adjoint, in[j], out[j], done[j], a + np, items, item_cap, n_items);
+        const int k = gemm_problems(hs[j], adjoint, in[j], out[j], done[j], prepacked && prepacked[j], a + np, items, item_cap, n_items);
         if (k < 0) return -1;
         for (int i = base_items; i < n_items; ++i) items[i].x += np;
         for (int i = 0; i < k; ++i) {

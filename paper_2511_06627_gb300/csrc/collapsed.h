@@ -29,7 +29,7 @@ void col_adjoint(mpi_ffl_handle *h, const float *data, bool full, const float *g
 // shared memory the launch needs.
 size_t gemm_args_size();
 int col_batch_prepare(mpi_ffl_handle *const *hs, const float *const *in, float *const *out, const int *const *done,
-                      int n, bool adjoint, void *args, int4 *items, int arg_cap, int item_cap, int &n_items,
+                      const char *prepacked, int n, bool adjoint, void *args, int4 *items, int arg_cap, int item_cap, int &n_items,
                       size_t &smem, uint32_t &tmem_cols);
 void col_batch_launch(const void *dargs, const int4 *ditems, int n_items, size_t smem, uint32_t tmem_cols,
                       cudaStream_t st);
@@ -49,5 +49,6 @@ void ten_adjoint(mpi_ffl_handle *h, const float *data, const float *coil, float 
 double langevin_d1_host(double x);
 double langevin_d2_host(double x);
 double langevin_half_point_host();
+void traj_point_host(const mpi_ffl_handle *h, int parity, int j, int &n, double &f, double &v);
 
 }  // namespace mpiffl

@@ -205,11 +205,67 @@ int refold(mpi_ffl_handle *h, int slot, cudaStream_t st) {
 
 }  // namespace
 
+namespace {
+
+// W of a small scan (at most kHostW values) on the host, sample by sample: 3 to 6 ms on the
+// thread that prepares a request, beside the running batch, without the temporary device
+// memory of the device build, whose release waits for the batch. The device build takes 0.6
+// ms at these sizes; with it a tiny request is done 9 ms after its arrival, and requests 10 ms
+// apart no longer meet in the server, which tests/test_gpu_serving.py holds it to.
+constexpr size_t kHostW = 40960;
+
+std::vector<double> w_host(const mpi_ffl_handle *h) {
+    const Dims &d = h->d;
+    const double kPi = 3.14159265358979323846;
+    const size_t R = (size_t)2 * d.nb;
+    const double isl = 1.0 / std::sqrt((double)d.L);
+    std::vector<double> W(d.n_par * R * d.Ne, 0.0), cs(d.S), sn(d.S);
+    for (int m = 0; m < d.S; ++m) {
+        cs[m] = std::cos(2.0 * kPi * m / d.S);
+        sn[m] = std::sin(2.0 * kPi * m / d.S);
+    }
+    for (int par = 0; par < d.n_par; ++par)
+        for (int j = 0; j < d.L; ++j) {
+            int n;
+            double f, v;
+            traj_point_host(h, par, j, n, f, v);
+            for (int di = 0; di < d.W; ++di) {
+                const int64_t dl = di - d.hw;
+                const double ad = 2.0 * kPi * (double)(((dl * j) % d.L + d.L) % d.L) / d.L;
+                const double cd = std::cos(ad), sd = std::sin(ad);
+                for (int k = 0; k < d.K; ++k) {
+                    // e^{2 pi i (kP + delta) j / L} = e^{2 pi i k r / S} e^{2 pi i delta j / L}
+                    const int m = (int)((int64_t)(d.kmin + k) * (j % d.S) % d.S);
+                    const double ck = cs[m], sk = sn[m];
+                    const double er = ck * cd - sk * sd, ei = ck * sd + sk * cd;
+                    const int o = k * d.W + di;
+                    const double gr = h->dgamma[2 * o], gi = h->dgamma[2 * o + 1];
+                    const double wr = (gr * er - gi * ei) * isl, wi = (gr * ei + gi * er) * isl;
+                    double *row = W.data() + (par * R + 2 * o) * d.Ne + n;
+                    row[0] += (1.0 - f) * v * wr;
+                    row[d.Ne] += (1.0 - f) * v * wi;
+                    row[1] += f * v * wr;
+                    row[d.Ne + 1] += f * v * wi;
+                }
+            }
+        }
+    return W;
+}
+
+}  // namespace
+
 int fold_w(mpi_ffl_handle *h) {
     FoldState *s = state(h);
     if (s->W) return MPI_FFL_OK;
     const Dims &d = h->d;
     const double kPi = 3.14159265358979323846;
+    if ((size_t)2 * d.nb * d.Ne <= kHostW) {
+        const std::vector<double> W = w_host(h);
+        if (!falloc(&s->W, W.size())) return MPI_FFL_ERR_OOM;
+        return cudaMemcpy(s->W, W.data(), W.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess
+                   ? MPI_FFL_OK
+                   : MPI_FFL_ERR_CUDA;
+    }
     double *drive = nullptr, *vel = nullptr, *W = nullptr;
     double2 *unit_s = nullptr;
     const bool ok = falloc(&drive, d.S) && falloc(&vel, (size_t)d.n_par * d.S) && falloc(&unit_s, d.S) &&

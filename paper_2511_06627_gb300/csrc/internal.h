@@ -221,19 +221,40 @@ namespace mpiffl {
 // ---------------------------------------------------------------- batched launches
 // One problem of a batched launch (continuous batching, batch.cu). `done` (device
 // int, may be NULL) turns the problem's blocks into no-ops once it is nonzero.
-struct TransposeJob {
-    const float *vol;
-    float *volT;
-    int N, Nz;
+// The solver's extrapolation y = x + beta (x - xp) of the volume x about to be projected.
+struct MomentumIn {
+    const float *xp;
+    float *y;
+    float beta;
     const int *done;
 };
-struct ProjectJob {
-    const float *vol, *volT;
+// The forward line-GEMM's A operand written by the projector itself (bf16 or tf32 hi + lo, the
+// canonical 1 KB blocks [K chunk][hi, lo][group of 8 rows] per trajectory parity), when
+// out[0] is not NULL: rows of parity p are the lines (m, z) with z = p mod n_par, in
+// angle-major order, G[p] groups of 8 rows each, nrow[p] rows per angle. proj may then
+// be NULL (the projections are not stored).
+struct ProjPack {
+    uint8_t *out[2];
+    int G[2];
+    int nrow[2];
+    int n_par;
+    int tf32;  // 1: tf32 hi + lo (4 K values per 16-byte unit), 0: bf16 (8)
+};
+struct InterleaveJob {
+    const float *x;
+    float *volI;
+    MomentumIn mom;
+    int N, Nz;
+    int vec;  // 16-byte loads: N % 4 == 0, pointers on 16 bytes
+};
+struct alignas(128) ProjectJob {
+    CUtensorMap row, col;
     const AngleParam *ang;
     const int *agroups;
-    float *proj;
-    int N, Nz, n_agroups;
+    float *proj;  // NULL when pack takes its place
+    int N, Nz, n_agroups, nbox, box;
     const int *done;
+    ProjPack pack;
 };
 struct BackprojectJob {
     const float *proj;
@@ -273,14 +294,14 @@ struct UpdateJob {     // x_out = P(y - tau (g + lam T^T T y)); a frozen job cop
     float tau, lam;
     int nonneg, N, Nz;
     const int *done;
+    int vec;  // four voxels a thread: N % 4 == 0, pointers on 16 bytes
 };
 
-int transpose_blocks(int N, int Nz);
+int interleave_blocks(int N, int Nz);
 int project_blocks(int n_agroups, int Nz);
-bool project_batch_ok(int N);  // problem size the batched projector takes
 int backproject_blocks(int N, int Nz);
 int update_blocks(int N, int Nz);
-void launch_transpose_batch(const TransposeJob *jobs, const int *offs, int n, int total, cudaStream_t st);
+void launch_interleave_batch(const InterleaveJob *jobs, const int *offs, int n, int total, cudaStream_t st);
 void launch_project_batch(const ProjectJob *jobs, const int *offs, int n, int total, int maxN, int *err,
                           cudaStream_t st);
 void launch_backproject_batch(const BackprojectJob *jobs, const int *offs, int n, int total, cudaStream_t st);
@@ -325,34 +346,14 @@ void launch_transpose_xy(const float *vol, float *volT, int N, int Nz, cudaStrea
 bool project_il_ok(int N);
 double project_il_cost(const AngleParam &a, int N);
 size_t il_len(int N, int Nz);
-// The solver's extrapolation y = x + beta (x - xp) of the volume x about to be projected.
-struct MomentumIn {
-    const float *xp;
-    float *y;
-    float beta;
-    const int *done;
-};
 void launch_interleave(const float *vol, float *volI, int N, int Nz, cudaStream_t st,
                        const MomentumIn *mom = nullptr);
 // encodes the tensor maps of volI (false if the driver refuses them)
 bool make_il_maps(const float *volI, int N, int Nz, IlMaps *maps);
-// The forward line-GEMM's A operand written by the projector itself (bf16 or tf32 hi + lo, the
-// canonical 1 KB blocks [K chunk][hi, lo][group of 8 rows] per trajectory parity), when
-// out[0] is not NULL: rows of parity p are the lines (m, z) with z = p mod n_par, in
-// angle-major order, G[p] groups of 8 rows each, nrow[p] rows per angle. proj may then
-// be NULL (the projections are not stored).
-struct ProjPack {
-    uint8_t *out[2];
-    int G[2];
-    int nrow[2];
-    int n_par;
-    int tf32;  // 1: tf32 hi + lo (4 K values per 16-byte unit), 0: bf16 (8)
-};
-
 void launch_project_il(const IlMaps &maps, const AngleParam *ang, const int *agroups,
                        int n_agroups, float *proj, int N, int Nz, cudaStream_t st, int *err, uint32_t inject = 0, ProjPack pack = ProjPack{});
 void launch_project(const float *vol, const float *volT, const AngleParam *ang, const int *agroups,
-                    int n_agroups, float *proj, int N, int Nz, cudaStream_t st, int *err);
+                    int n_agroups, float *proj, int N, int Nz, cudaStream_t st);
 constexpr int kProjAnglesPerBlock = 2;  // angle slots per projector block (k_projector.cu)
 void launch_backproject(const float *proj, const AngleParam *ang, float *vol, int N, int Nz,
                         int M, cudaStream_t st);

@@ -3,8 +3,8 @@
 //
 // Both directions process kZc z slices per thread: every slice shares the ray
 // geometry, so the interpolation weights are computed once per kZc samples.
-// Column-marched angles read a transposed copy of the volume, so that every
-// staged voxel line is contiguous.
+// Column-marched angles read a transposed copy of the volume (plain projector) or columns of
+// the slice-interleaved one.
 #include <algorithm>
 
 #include "internal.h"
@@ -156,176 +156,29 @@ __global__ void __launch_bounds__(1024) k_project(const float *__restrict__ vol,
     }
 }
 
-// Pipelined variant (N % 4 == 0, N <= 512): an extra producer warp streams voxel line
-// s of the block's kZc slices into a ring of kPStages shared-memory stages with bulk
-// copies that complete on full[stage]; every consumer warp signals empty[stage] when
-// it has used a stage, so no block-wide barrier sits in the march loop. Each staged
-// line sits between kPad zeros on the left and at least 4 on the right (row stride
-// LD >= N + 8, a compile-time constant), so a tap index clamped to [-2, N] reads a
-// zero outside the grid: the taps need no range checks, the slice offsets are
-// immediates, and the sums equal those of the checked form (a zero tap adds nothing).
 constexpr int kPStages = 12;
 constexpr int kPad = 4;
 // the interleaved projector's stages go in groups of kPGroup march steps, one pair of
 // barriers per group (fewer waits and arrivals per step)
 constexpr int kPGroup = 4, kPSlots = kPStages / kPGroup;
 
-template <int LD>
-__device__ __forceinline__ void project_pipe_body(const float *__restrict__ vol, const float *__restrict__ volT,
-                                                  const AngleParam *__restrict__ ang,
-                                                  const int *__restrict__ agroups, float *__restrict__ proj,
-                                                  int N, int Nz, int rays_per_angle, int *err, int bx, int by,
-                                                  float *psm) {
-    uint64_t *bars = reinterpret_cast<uint64_t *>(psm + kPStages * kZc * LD);  // full[K], empty[K]
-    const int nthreads_c = rays_per_angle * kProjAnglesPerBlock;  // consumers
-    const int ncw = nthreads_c / 32;
-    const int z0 = by * kZc;
-    const int nz = min(kZc, Nz - z0);
-    const int tid = threadIdx.x;
-    // zero the pads of every staged line: [0, kPad) and [kPad + N, LD). The stride is
-    // this problem's thread count: in a batch launch, threads past it have left.
-    const int padw = LD - N;
-    for (int t = tid; t < kPStages * kZc * padw; t += nthreads_c + 32) {
-        const int row = t / padw, cpos = t - row * padw;
-        psm[row * LD + (cpos < kPad ? cpos : N + cpos)] = 0.f;
-    }
-    if (tid == 0) {
-        for (int k = 0; k < kPStages; ++k) {
-            ptx::mbar_init(&bars[k], 1);
-            ptx::mbar_init(&bars[kPStages + k], ncw);
-        }
-        ptx::fence_mbar_init();
-    }
-    __syncthreads();
-    const AngleParam a0 = ang[agroups[bx * kProjAnglesPerBlock]];
-    const float *src = a0.row_major ? vol : volT;  // one orientation per block
-    const uint32_t row_bytes = (uint32_t)N * 4u;
-    if (tid >= nthreads_c) {
-        // ---------------------------------------------------------------- producer warp
-        // lane 0 announces the stage's bytes, then lane zz copies slice zz: the nz
-        // copies of a step are issued side by side, not one after another
-        const int lane = tid - nthreads_c;
-        for (int s = 0; s < N; ++s) {
-            const int k = s % kPStages;
-            int ok = 1;  // lane 0 waits for the stage to be free; the warp leaves together
-            if (s >= kPStages && lane == 0)
-                ok = ptx::mbar_wait_bounded(&bars[kPStages + k], ((s / kPStages) - 1) & 1, 1u << 24);
-            if (!__shfl_sync(0xffffffffu, ok, 0)) {
-                if (lane == 0) atomicExch(err, 1);
-                break;
-            }
-            float *dst = psm + k * kZc * LD + kPad;
-            if (lane == 0) ptx::mbar_arrive_expect_tx(&bars[k], row_bytes * nz);
-            __syncwarp();
-            if (lane < nz) {
-                // the consumers read the stage with ordinary loads (generic proxy) and
-                // the bulk copy writes it through the async proxy: the empty barrier
-                // orders the two only with this fence between them
-                ptx::fence_proxy_async_smem();
-                ptx::bulk_g2s(dst + lane * LD, src + ((size_t)(z0 + lane) * N + s) * N, row_bytes, &bars[k]);
-            }
-        }
-        return;
-    }
-    // -------------------------------------------------------------------- consumers
-    // The warps of an inactive slot (a block with one angle) only wait and arrive, as do
-    // the warps all of whose rays lie off the grid at a step (both taps on the zero pads:
-    // nothing to add). Threads beyond the last ray run the loop on clamped, in-bounds
-    // taps and store nothing; slices past nz hold stale data, never stored.
-    const int slot = tid / rays_per_angle;
-    const int i = tid % rays_per_angle;
-    const int m = agroups[bx * kProjAnglesPerBlock + slot];
-    const bool active = (m >= 0) && (i < N);
-    const AngleParam ap = ang[m >= 0 ? m : agroups[bx * kProjAnglesPerBlock]];
-    long long fs = ap.fx_a + (long long)i * ap.fx_d;  // position of ray i at march step s
-    float acc[kZc];
-#pragma unroll
-    for (int zz = 0; zz < kZc; ++zz) acc[zz] = 0.f;
-    bool good = true;
-    for (int s = 0; s < N; ++s, fs += ap.fx_b) {
-        const int k = s % kPStages;
-        // the warp gives up as one, so that its vote below sees all lanes
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait_bounded(&bars[k], (s / kPStages) & 1, 1u << 24))) {
-            good = false;
-            break;
-        }
-        int cell;
-        float t;
-        fx_split(fs, cell, t);
-        if (m >= 0 && __any_sync(0xffffffffu, cell >= -1 && cell <= N - 1)) {  // m: uniform per warp
-            const int kk = min(max(cell, -2), N);
-            const float *p = psm + k * kZc * LD + kPad + kk;
-#pragma unroll
-            for (int zz = 0; zz < kZc; ++zz) acc[zz] = fmaf(1.f - t, p[zz * LD], fmaf(t, p[zz * LD + 1], acc[zz]));
-        }
-        __syncwarp();
-        if ((tid & 31) == 0) ptx::mbar_arrive(&bars[kPStages + k]);
-    }
-    if (!good) {
-        if ((tid & 31) == 0) atomicExch(err, 1);
-        return;
-    }
-    if (active) {
-#pragma unroll
-        for (int zz = 0; zz < kZc; ++zz)
-            if (zz < nz) proj[((size_t)m * Nz + z0 + zz) * N + i] = acc[zz] * ap.scale;
-    }
-}
-
-template <int LD>
-__global__ void __launch_bounds__(1024 + 32) k_project_pipe(const float *__restrict__ vol,
-                                                            const float *__restrict__ volT,
-                                                            const AngleParam *__restrict__ ang,
-                                                            const int *__restrict__ agroups,
-                                                            float *__restrict__ proj, int N, int Nz,
-                                                            int rays_per_angle, int *err) {
-    extern __shared__ __align__(128) float psm[];  // kPStages x kZc x LD
-    project_pipe_body<LD>(vol, volT, ang, agroups, proj, N, Nz, rays_per_angle, err, blockIdx.x, blockIdx.y, psm);
-}
-
-// Smallest compiled row stride that holds N + 8 floats; 0 if N is above 512.
-int pipe_ld(int N) {
+// Smallest compiled line stride that holds N + 8 positions; 0 if N is above 512.
+int il_ld(int N) {
     for (int ld : {40, 72, 136, 200, 264, 392, 520})
         if (N + 8 <= ld) return ld;
     return 0;
 }
 
-size_t pipe_smem(int ld) { return sizeof(float) * kPStages * kZc * ld + 16 * kPStages; }
+size_t il_smem(int ld) { return sizeof(float) * kPStages * kZc * ld + 16 * kPStages; }
 
-// The pipelined and interleaved projectors run kProjAnglesPerBlock angles of
+// The interleaved projector runs kProjAnglesPerBlock angles of
 // (N + 31) / 32 * 32 rays each plus a producer warp in one block: at most 1024 threads,
 // so N <= 496; wider detectors take the plain projector.
-bool pipe_threads_ok(int N) { return (N + 31) / 32 * 32 * kProjAnglesPerBlock + 32 <= 1024; }
-
-bool pipe_ok(const float *vol, const float *volT, int N) {
-    return N % 4 == 0 && pipe_ld(N) > 0 && pipe_threads_ok(N) && (reinterpret_cast<uintptr_t>(vol) & 15) == 0 &&
-           (reinterpret_cast<uintptr_t>(volT) & 15) == 0;
-}
-
-template <int LD>
-void launch_pipe(dim3 grid, int threads, cudaStream_t st, const float *vol, const float *volT, const AngleParam *ang,
-                 const int *agroups, float *proj, int N, int Nz, int rays, int *err) {
-    cudaFuncSetAttribute(k_project_pipe<LD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    k_project_pipe<LD><<<grid, threads, pipe_smem(LD), st>>>(vol, volT, ang, agroups, proj, N, Nz, rays, err);
-}
+bool il_threads_ok(int N) { return (N + 31) / 32 * 32 * kProjAnglesPerBlock + 32 <= 1024; }
 
 void launch_project(const float *vol, const float *volT, const AngleParam *ang, const int *agroups,
-                    int n_agroups, float *proj, int N, int Nz, cudaStream_t st, int *err) {
+                    int n_agroups, float *proj, int N, int Nz, cudaStream_t st) {
     const int rays = (N + 31) / 32 * 32;
-    if (err && pipe_ok(vol, volT, N)) {
-        dim3 grid(n_agroups, (Nz + kZc - 1) / kZc);
-        const int threads = rays * kProjAnglesPerBlock + 32;
-        switch (pipe_ld(N)) {
-        case 40: launch_pipe<40>(grid, threads, st, vol, volT, ang, agroups, proj, N, Nz, rays, err); break;
-        case 72: launch_pipe<72>(grid, threads, st, vol, volT, ang, agroups, proj, N, Nz, rays, err); break;
-        case 136: launch_pipe<136>(grid, threads, st, vol, volT, ang, agroups, proj, N, Nz, rays, err); break;
-        case 200: launch_pipe<200>(grid, threads, st, vol, volT, ang, agroups, proj, N, Nz, rays, err); break;
-        case 264: launch_pipe<264>(grid, threads, st, vol, volT, ang, agroups, proj, N, Nz, rays, err); break;
-        case 392: launch_pipe<392>(grid, threads, st, vol, volT, ang, agroups, proj, N, Nz, rays, err); break;
-        default: launch_pipe<520>(grid, threads, st, vol, volT, ang, agroups, proj, N, Nz, rays, err); break;
-        }
-        return;
-    }
     const int threads = rays * kProjAnglesPerBlock;
     const size_t smem = sizeof(float) * 2 * kZc * N;
     if (smem > 48 * 1024)
@@ -334,15 +187,20 @@ void launch_project(const float *vol, const float *volT, const AngleParam *ang, 
     k_project<<<grid, threads, smem, st>>>(vol, volT, ang, agroups, proj, N, Nz, rays);
 }
 
-// Interleaved variant (detectors of any size up to 496 bins). The volume is copied once with
+// Interleaved projector (detectors of any size up to 496 bins). The volume is copied once with
 // each line's kZc slices innermost, volI[z block][y][x][kZc]. A march step is one tensor
 // copy of the step's line: a row of volI for row-marched angles, a column (32-byte
-// pieces N rows apart) for column-marched ones. The copy writes shared memory with the
+// pieces N rows apart) for column-marched ones. A producer warp keeps a ring of kPStages
+// steps filled; the stages go in groups of kPGroup with one pair of barriers each. A staged
+// line sits between kPad zeros on the left and at least 4 on the right (stride LDC >= N + 8,
+// a compile-time constant), so a tap position clamped to [-2, N] reads a zero outside the
+// grid: the taps need no range checks, and the sums equal those of the checked form (a zero
+// tap adds nothing). The copy writes shared memory with the
 // 32-byte swizzle, which swaps the two 16-byte halves of staged position p when bit 2
 // of p is set (stage bases are 256-byte aligned). A ray reads its two taps for all kZc
 // slices with four 16-byte loads. Eight rays whose positions differ mod 8 read eight
 // distinct 16-byte bank groups: position p puts slices 0-3 in group
-// 2p + ((p >> 2) & 1) mod 8. The sums are those of the pipelined variant, slice by slice.
+// 2p + ((p >> 2) & 1) mod 8.
 __host__ __device__ __forceinline__ int il_swap(int cs) { return (cs >> 2) & 1; }
 
 // Shared-memory wavefronts one angle costs the interleaved projector for one slice
@@ -405,15 +263,12 @@ __device__ __forceinline__ int il_tile_slot(int r, int c, int h) {
 // MOM: the volume is the solver's extrapolated iterate y = x + beta (x - x_prev), formed here
 // from both iterates and stored too (nothing is done once *done is set).
 template <bool VEC, bool MOM>
-__global__ void __launch_bounds__(256) k_interleave(const float *__restrict__ vol, float *__restrict__ volI, int N,
-                                                    int Nz, MomentumIn mom) {
-    __shared__ float4 tile[32 * 64];  // 32 rows x 32 columns x 2 halves
+__device__ __forceinline__ void interleave_body(const float *__restrict__ vol, float *__restrict__ volI, int N,
+                                                int Nz, const MomentumIn &mom, int bx, int by, int zb,
+                                                float4 *tile) {
     const int tx = threadIdx.x, ty = threadIdx.y;  // 8 x 32
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32, zb = blockIdx.z;
+    const int x0 = bx * 32, y0 = by * 32;
     const int y = y0 + ty, xs = x0 + 4 * tx;
-    ptx::grid_dep_wait();  // the volume comes from the previous kernel
-    ptx::grid_dep_launch();
-    if (MOM && mom.done && *mom.done) return;  // the whole launch
     float4 v[kZc];
 #pragma unroll
     for (int e = 0; e < kZc; ++e) {
@@ -472,6 +327,16 @@ __global__ void __launch_bounds__(256) k_interleave(const float *__restrict__ vo
     }
 }
 
+template <bool VEC, bool MOM>
+__global__ void __launch_bounds__(256) k_interleave(const float *__restrict__ vol, float *__restrict__ volI, int N,
+                                                    int Nz, MomentumIn mom) {
+    __shared__ float4 tile[32 * 64];  // 32 rows x 32 columns x 2 halves
+    ptx::grid_dep_wait();  // the volume comes from the previous kernel
+    ptx::grid_dep_launch();
+    if (MOM && mom.done && *mom.done) return;  // the whole launch
+    interleave_body<VEC, MOM>(vol, volI, N, Nz, mom, blockIdx.x, blockIdx.y, blockIdx.z, tile);
+}
+
 void launch_interleave(const float *vol, float *volI, int N, int Nz, cudaStream_t st, const MomentumIn *mom) {
     dim3 grid((N + 31) / 32, (N + 31) / 32, (Nz + kZc - 1) / kZc), block(8, 32);
     auto a16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
@@ -503,7 +368,7 @@ bool make_il_maps(const float *volI, int N, int Nz, IlMaps *maps) {
     if (!encode) return false;
     const int nbox = (N + 255) / 256;
     const int box = ((N + nbox - 1) / nbox + 3) / 4 * 4;
-    if (kPad + nbox * box > pipe_ld(N)) return false;  // the boxes' zero fill stays inside the stage
+    if (kPad + nbox * box > il_ld(N)) return false;  // the boxes' zero fill stays inside the stage
     const cuuint64_t dims[4] = {(cuuint64_t)kZc, (cuuint64_t)N, (cuuint64_t)N, (cuuint64_t)((Nz + kZc - 1) / kZc)};
     const cuuint64_t strides[3] = {(cuuint64_t)kZc * 4, (cuuint64_t)kZc * 4 * N, (cuuint64_t)kZc * 4 * N * N};
     const cuuint32_t elem[4] = {1, 1, 1, 1};
@@ -533,16 +398,13 @@ __device__ __forceinline__ void il_copy(float *dst, const CUtensorMap *map, int 
 }
 
 template <int LDC>
-__global__ void __launch_bounds__(1024 + 32) k_project_il(const __grid_constant__ CUtensorMap map_row,
-                                                          const __grid_constant__ CUtensorMap map_col, int nbox,
-                                                          int box, const AngleParam *__restrict__ ang,
-                                                          const int *__restrict__ agroups, float *__restrict__ proj,
-                                                          int N, int Nz, int rays_per_angle, int *err,
-                                                          uint32_t inject, ProjPack pack) {
-    extern __shared__ __align__(128) float psm[];  // kPStages x LDC positions x kZc
+__device__ __forceinline__ void project_il_body(const CUtensorMap *map_row, const CUtensorMap *map_col, int nbox,
+                                                int box, const AngleParam *__restrict__ ang,
+                                                const int *__restrict__ agroups, float *__restrict__ proj, int N,
+                                                int Nz, int rays_per_angle, int *err, uint32_t inject,
+                                                const ProjPack &pack, int bx, int zb, float *psm) {
     // kPGroup consecutive march steps share one pair of barriers: full[kPSlots], empty[kPSlots]
     uint64_t *bars = reinterpret_cast<uint64_t *>(psm + kPStages * LDC * kZc);
-    const int bx = blockIdx.x, zb = blockIdx.y;
     const int nthreads_c = rays_per_angle * kProjAnglesPerBlock;  // consumers
     const int ncw = nthreads_c / 32;
     const int z0 = zb * kZc;
@@ -579,7 +441,7 @@ __global__ void __launch_bounds__(1024 + 32) k_project_il(const __grid_constant_
     ptx::grid_dep_wait();  // the interleaved volume comes from the previous kernel
     const AngleParam a0 = ang[agroups[bx * kProjAnglesPerBlock]];
     const bool rows = a0.row_major != 0;  // one orientation per block
-    const CUtensorMap *map = rows ? &map_row : &map_col;
+    const CUtensorMap *map = rows ? map_row : map_col;
     const uint32_t step_bytes = (uint32_t)(nbox * box) * kZc * 4u;  // zero fill past N included
     if (tid >= nthreads_c) {
         // ---------------------------------------------------------------- producer
@@ -722,9 +584,21 @@ __global__ void __launch_bounds__(1024 + 32) k_project_il(const __grid_constant_
 }
 
 template <int LDC>
+__global__ void __launch_bounds__(1024 + 32) k_project_il(const __grid_constant__ CUtensorMap map_row,
+                                                          const __grid_constant__ CUtensorMap map_col, int nbox,
+                                                          int box, const AngleParam *__restrict__ ang,
+                                                          const int *__restrict__ agroups, float *__restrict__ proj,
+                                                          int N, int Nz, int rays_per_angle, int *err,
+                                                          uint32_t inject, ProjPack pack) {
+    extern __shared__ __align__(128) float psm[];  // kPStages x LDC positions x kZc
+    project_il_body<LDC>(&map_row, &map_col, nbox, box, ang, agroups, proj, N, Nz, rays_per_angle, err, inject, pack,
+                         blockIdx.x, blockIdx.y, psm);
+}
+
+template <int LDC>
 void launch_il(dim3 grid, int threads, cudaStream_t st, const IlMaps &maps, const AngleParam *ang,
                const int *agroups, float *proj, int N, int Nz, int rays, int *err, uint32_t inject, ProjPack pack) {
-    const size_t smem = pipe_smem(LDC);  // kPStages x kZc x LDC floats, as the pipelined variant
+    const size_t smem = il_smem(LDC);
     cudaFuncSetAttribute(k_project_il<LDC>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     launch_dependent(k_project_il<LDC>, grid, dim3(threads), smem, st, maps.row, maps.col, maps.nbox, maps.box, ang,
                      agroups, proj, N, Nz, rays, err, inject, pack);
@@ -733,7 +607,7 @@ void launch_il(dim3 grid, int threads, cudaStream_t st, const IlMaps &maps, cons
 // Any detector of up to 496 bins: the copy's own strides (32 N bytes) suit the tensor maps,
 // and the boxes' zero fill past N takes the place of a ragged line's last positions. (101
 // bins, 21 angles and 37 slices: 113 us through the plain projector, 26 us this way.)
-bool project_il_ok(int N) { return pipe_ld(N) > 0 && pipe_threads_ok(N); }
+bool project_il_ok(int N) { return il_ld(N) > 0 && il_threads_ok(N); }
 
 void launch_project_il(const IlMaps &maps, const AngleParam *ang, const int *agroups,
                        int n_agroups, float *proj, int N, int Nz, cudaStream_t st, int *err, uint32_t inject,
@@ -741,7 +615,7 @@ void launch_project_il(const IlMaps &maps, const AngleParam *ang, const int *agr
     const int rays = (N + 31) / 32 * 32;
     dim3 grid(n_agroups, (Nz + kZc - 1) / kZc);
     const int threads = rays * kProjAnglesPerBlock + 32;
-    switch (pipe_ld(N)) {
+    switch (il_ld(N)) {
     case 40: launch_il<40>(grid, threads, st, maps, ang, agroups, proj, N, Nz, rays, err, inject, pack); break;
     case 72: launch_il<72>(grid, threads, st, maps, ang, agroups, proj, N, Nz, rays, err, inject, pack); break;
     case 136: launch_il<136>(grid, threads, st, maps, ang, agroups, proj, N, Nz, rays, err, inject, pack); break;
@@ -939,41 +813,46 @@ __device__ __forceinline__ int batch_find(const int *__restrict__ offs, int n, i
 // at once loops over the work items of every job (see batch_find). An item's arithmetic
 // does not depend on the block that runs it, so a job gives the same bits alone and in
 // any mix.
-__global__ void k_transpose_batch(const TransposeJob *__restrict__ jobs, const int *__restrict__ offs, int n,
-                                  int total) {
+// y = x + beta (x - x_prev) and its slice-interleaved copy, every job's 32 x 32 tiles
+__global__ void __launch_bounds__(256) k_interleave_batch(const InterleaveJob *__restrict__ jobs,
+                                                          const int *__restrict__ offs, int n, int total) {
+    __shared__ float4 tile[32 * 64];
     for (int bi = blockIdx.x; bi < total; bi += gridDim.x) {
         const int j = batch_find(offs, n, bi);
-        const TransposeJob J = jobs[j];
-        if (J.done && *J.done) continue;
-        int b = bi - offs[j];
+        const InterleaveJob J = jobs[j];
+        if (J.mom.done && *J.mom.done) continue;  // uniform over the block
+        const int b = bi - offs[j];
         const int gx = (J.N + 31) / 32;
-        const int bx = b % gx, by = (b / gx) % gx, bz = b / (gx * gx);
         __syncthreads();  // the tile of the previous item has been read
-        transpose_body(J.vol, J.volT, J.N, bx, by, bz);
+        if (J.vec) interleave_body<true, true>(J.x, J.volI, J.N, J.Nz, J.mom, b % gx, (b / gx) % gx, b / (gx * gx), tile);
+        else interleave_body<false, true>(J.x, J.volI, J.N, J.Nz, J.mom, b % gx, (b / gx) % gx, b / (gx * gx), tile);
     }
 }
 
-template <int LD>
+template <int LDC>
 __global__ void __launch_bounds__(1024 + 32) k_project_batch(const ProjectJob *__restrict__ jobs,
                                                              const int *__restrict__ offs, int n, int total,
                                                              int *err) {
     extern __shared__ __align__(128) float psm[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(psm + kPStages * kZc * LD);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(psm + kPStages * kZc * LDC);
     for (int bi = blockIdx.x; bi < total; bi += gridDim.x) {
         const int j = batch_find(offs, n, bi);
-        const ProjectJob J = jobs[j];
+        const ProjectJob &J = jobs[j];
         if (J.done && *J.done) continue;  // uniform over the block
         const int b = bi - offs[j];
         const int rays = (J.N + 31) / 32 * 32;
+        // the maps were written to global memory before this launch, over earlier launches'
+        ptx::fence_tensormap(&J.row);
+        ptx::fence_tensormap(&J.col);
         if ((int)threadIdx.x < rays * kProjAnglesPerBlock + 32)
-            project_pipe_body<LD>(J.vol, J.volT, J.ang, J.agroups, J.proj, J.N, J.Nz, rays, err, b % J.n_agroups,
-                                  b / J.n_agroups, psm);
+            project_il_body<LDC>(&J.row, &J.col, J.nbox, J.box, J.ang, J.agroups, J.proj, J.N, J.Nz, rays, err, 0,
+                                 J.pack, b % J.n_agroups, b / J.n_agroups, psm);
         else
             __syncthreads();  // threads beyond this problem's block shape meet the body's one barrier
         // every thread has left the item: its barriers are idle and are set up anew
         __syncthreads();
         if (threadIdx.x == 0)
-            for (int k = 0; k < 2 * kPStages; ++k) ptx::mbar_inval(&bars[k]);
+            for (int k = 0; k < 2 * kPSlots; ++k) ptx::mbar_inval(&bars[k]);
         __syncthreads();
     }
 }
@@ -993,7 +872,7 @@ __global__ void __launch_bounds__(kBpTX * kBpTY, 2) k_backproject_batch(const Ba
     }
 }
 
-int transpose_blocks(int N, int Nz) { return ((N + 31) / 32) * ((N + 31) / 32) * Nz; }
+int interleave_blocks(int N, int Nz) { return ((N + 31) / 32) * ((N + 31) / 32) * ((Nz + kZc - 1) / kZc); }
 int project_blocks(int n_agroups, int Nz) { return n_agroups * ((Nz + kZc - 1) / kZc); }
 int backproject_blocks(int N, int Nz) {
     return ((N + kBpTX - 1) / kBpTX) * ((N + kBpTY - 1) / kBpTY) * ((Nz + kBpZ - 1) / kBpZ);
@@ -1017,28 +896,26 @@ int persistent_grid_p(K kernel, int threads, size_t smem, int total) {
     return std::max(1, std::min(total, per * n_sm));
 }
 
-void launch_transpose_batch(const TransposeJob *jobs, const int *offs, int n, int total, cudaStream_t st) {
+void launch_interleave_batch(const InterleaveJob *jobs, const int *offs, int n, int total, cudaStream_t st) {
     if (total <= 0) return;
-    k_transpose_batch<<<persistent_grid_p(k_transpose_batch, 256, 0, total), dim3(32, 8), 0, st>>>(jobs, offs, n,
-                                                                                                   total);
+    k_interleave_batch<<<persistent_grid_p(k_interleave_batch, 256, 0, total), dim3(8, 32), 0, st>>>(jobs, offs, n,
+                                                                                                    total);
 }
-
-bool project_batch_ok(int N) { return N % 4 == 0 && pipe_ld(N) > 0 && pipe_threads_ok(N); }
 
 template <int LD>
 void launch_pbatch(const ProjectJob *jobs, const int *offs, int n, int total, int threads, int *err,
                    cudaStream_t st) {
     cudaFuncSetAttribute(k_project_batch<LD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    const int grid = persistent_grid_p(k_project_batch<LD>, threads, pipe_smem(LD), total);
-    k_project_batch<LD><<<grid, threads, pipe_smem(LD), st>>>(jobs, offs, n, total, err);
+    const int grid = persistent_grid_p(k_project_batch<LD>, threads, il_smem(LD), total);
+    k_project_batch<LD><<<grid, threads, il_smem(LD), st>>>(jobs, offs, n, total, err);
 }
 
-// Every problem in the batch has N % 4 == 0 and N <= 512 (project_batch_ok); the ring
-// stride is the one of the largest N.
+// Every problem in the batch has its interleaved copy; the ring stride is the one of the
+// largest N.
 void launch_project_batch(const ProjectJob *jobs, const int *offs, int n, int total, int maxN, int *err,
                           cudaStream_t st) {
     const int threads = (maxN + 31) / 32 * 32 * kProjAnglesPerBlock + 32;
-    switch (pipe_ld(maxN)) {
+    switch (il_ld(maxN)) {
     case 40: launch_pbatch<40>(jobs, offs, n, total, threads, err, st); break;
     case 72: launch_pbatch<72>(jobs, offs, n, total, threads, err, st); break;
     case 136: launch_pbatch<136>(jobs, offs, n, total, threads, err, st); break;

@@ -292,16 +292,11 @@ void launch_ttt(const float *x, float *out, int N, int Nz, cudaStream_t st) {
 // the next iteration keeps the final iterate. VEC: four voxels of a row a thread (N % 4 ==
 // 0, pointers on 16 bytes); the terms of T^T T are added in ttt_at's order.
 template <bool VEC>
-__global__ void __launch_bounds__(128) k_update(const float *__restrict__ y, const float *__restrict__ g,
-                                                float *__restrict__ xo, float tau, float lam, int nonneg, int N,
-                                                int Nz, const int *done, const float *__restrict__ xcur) {
-    ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
+__device__ __forceinline__ void update_row(const float *__restrict__ y, const float *__restrict__ g,
+                                           float *__restrict__ xo, float tau, float lam, int nonneg, int N, int Nz,
+                                           bool frozen, const float *__restrict__ xcur, int row) {
     constexpr int V = VEC ? 4 : 1;
-    const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;  // a warp per row (z, y)
-    if (row >= N * Nz) return;
     const int yy = row % N, z = row / N;
-    const bool frozen = done && *done;
     for (int xx = V * (threadIdx.x & 31); xx < N; xx += V * 32) {
         const size_t i = ((size_t)z * N + yy) * N + xx;
         if (frozen) {
@@ -344,6 +339,17 @@ __global__ void __launch_bounds__(128) k_update(const float *__restrict__ y, con
             xo[i] = v;
         }
     }
+}
+
+// a warp per row (z, y)
+template <bool VEC>
+__global__ void __launch_bounds__(128) k_update(const float *__restrict__ y, const float *__restrict__ g,
+                                                float *__restrict__ xo, float tau, float lam, int nonneg, int N,
+                                                int Nz, const int *done, const float *__restrict__ xcur) {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    const int row = blockIdx.x * 4 + threadIdx.x / 32;
+    if (row < N * Nz) update_row<VEC>(y, g, xo, tau, lam, nonneg, N, Nz, done && *done, xcur, row);
 }
 
 void launch_update(const float *y, const float *g, float *xout, float tau, float lam, int nonneg,
@@ -490,29 +496,23 @@ __global__ void __launch_bounds__(kRedThreads) k_stop_batch(const StopJob *__res
     }
 }
 
+// a frozen job keeps the final iterate in the buffer that becomes x
 __global__ void __launch_bounds__(128) k_update_batch(const UpdateJob *__restrict__ jobs, const int *__restrict__ offs,
                                                       int n, int total) {
     for (int bi = blockIdx.x; bi < total; bi += gridDim.x) {
         const int j = batch_find_s(offs, n, bi);
         const UpdateJob J = jobs[j];
-        const int b = bi - offs[j];
-        const int gx = (J.N + 127) / 128;
-        const int xx = (b % gx) * 128 + threadIdx.x;
-        const int yy = (b / gx) % J.N, z = b / (gx * J.N);
-        if (xx >= J.N) continue;
-        const size_t i = ((size_t)z * J.N + yy) * J.N + xx;
-        if (J.done && *J.done) {  // frozen: keep the final iterate in the buffer that becomes x
-            J.xo[i] = J.xcur[i];
-            continue;
+        const bool frozen = J.done && *J.done;
+        for (int q = 0; q < 2; ++q) {
+            const int row = (bi - offs[j]) * 8 + 4 * q + threadIdx.x / 32;
+            if (row >= J.N * J.Nz) break;
+            if (J.vec) update_row<true>(J.y, J.g, J.xo, J.tau, J.lam, J.nonneg, J.N, J.Nz, frozen, J.xcur, row);
+            else update_row<false>(J.y, J.g, J.xo, J.tau, J.lam, J.nonneg, J.N, J.Nz, frozen, J.xcur, row);
         }
-        const float grad = fmaf(J.lam, ttt_at(J.y, J.N, J.Nz, z, yy, xx), J.g[i]);
-        float v = fmaf(-J.tau, grad, J.y[i]);
-        if (J.nonneg) v = fmaxf(v, 0.f);
-        J.xo[i] = v;
     }
 }
 
-int update_blocks(int N, int Nz) { return ((N + 127) / 128) * N * Nz; }
+int update_blocks(int N, int Nz) { return (N * Nz + 7) / 8; }
 
 __global__ void k_freeze_batch(const StopJob *__restrict__ jobs, int n) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
