@@ -3,8 +3,8 @@
 // of one angle: proj[seg][N] -> fine[seg][N_e] -> sig[seg][L] -> data[seg][nb].
 //
 // H   : full-support polyphase convolution on the fine grid. Output e has phase
-//       (e - D) mod Q; a thread owns kPsfTF outputs of one phase and slides a
-//       register window over the tap table, so each tap load feeds kPsfTF FMAs.
+//       (e - D) mod Q; a thread owns kPsfTF outputs of one phase of two lines and slides a
+//       register window over the tap table, so each tap load feeds 2 kPsfTF FMAs.
 // EVB : velocity-weighted linear interpolation at the FFL positions; the
 //       trajectory table is read once per group of kGroup lines that share it.
 //       The transpose gathers through a per-trajectory CSR (fine cell <- samples).
@@ -12,6 +12,7 @@
 //       b[k, d] = L^-1/2 sum_r e^{2 pi i (kP+d) r / L} sum_p s[pS+r] e^{2 pi i d p / P},
 //       exactly equal to Eq. (27) on the kept bins. The inner sum over periods
 //       costs 2w+1 FMAs per sample (the signal is real); the outer one is small.
+#include "f32x2.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
 
@@ -19,23 +20,32 @@ namespace mpiffl {
 
 // ----------------------------------------------------------------------------- H
 
+// Both directions take lines two at a time: a thread's sums of the two lines are the halves of
+// an fma.rn.f32x2 with the same taps, so the issue slots that loads and tap duplication need
+// stay free beside the FMAs (one line at a time, an FMA was followed by a shared load or a
+// move in every fifth slot and a thread of 9 sums issued 11 instructions for 9 FMAs).
+
 // Nine outputs per thread: at Q = 8 the 30 register blocks of the 8 phases of a
 // 256-bin line fill one round of 256 threads, and lanes of different blocks read taps
 // 9 Q words apart, in distinct banks (with eight, 34 blocks took two rounds and four
 // lanes shared each bank).
 constexpr int kPsfTF = 9;
-// sixteen outputs per lane in the transpose: 16 FMAs per pair of shared loads
+// sixteen outputs per lane in the transpose: 16 FMA pairs per pair of shared loads
 constexpr int kPsfTA = 16;
 static_assert(kPsfTF <= kPsfT && kPsfTA <= kPsfT, "the tap table is padded for the windows");
 
+// FP32-bound: 2.5 GFMA at 256^2 x 128 and 36 angles in 121 us (144 us one line at a
+// time), of 67 us at the FMA rate.
 __global__ void __launch_bounds__(256) k_psf_fwd(const float *__restrict__ proj,
                                                  const float *__restrict__ htab,
                                                  float *__restrict__ fine, Dims d) {
-    extern __shared__ float sm[];
-    float *sp = sm;            // N
-    float *sh = sm + d.N;      // htab_len
-    const int seg = blockIdx.x;
-    for (int i = threadIdx.x; i < d.N; i += blockDim.x) sp[i] = proj[(size_t)seg * d.N + i];
+    extern __shared__ __align__(16) float sm[];
+    f32x2 *sp = reinterpret_cast<f32x2 *>(sm);  // N pairs (line, next line)
+    float *sh = sm + 2 * d.N;                   // htab_len
+    const int seg = 2 * blockIdx.x;
+    const bool two = seg + 1 < d.nseg;
+    const float *p0 = proj + (size_t)seg * d.N;
+    for (int i = threadIdx.x; i < d.N; i += blockDim.x) sp[i] = pack2(p0[i], two ? p0[d.N + i] : 0.f);
     for (int i = threadIdx.x; i < d.htab_len; i += blockDim.x) sh[i] = htab[i];
     __syncthreads();
     const int Q = d.Q;
@@ -45,109 +55,123 @@ __global__ void __launch_bounds__(256) k_psf_fwd(const float *__restrict__ proj,
         const int q = task % Q;
         const int ab = task / Q;
         const int base = q - d.D + d.htab_off + Q * ab * kPsfTF;
-        float w[kPsfTF], acc[kPsfTF];
+        f32x2 w[kPsfTF], acc[kPsfTF];
 #pragma unroll
         for (int t = 0; t < kPsfTF; ++t) {
-            w[t] = sh[base + Q * t];
-            acc[t] = 0.f;
+            w[t] = dup2(sh[base + Q * t]);
+            acc[t] = 0;
         }
         // unrolled by the window length, so that the window's shift is a renaming of
         // registers rather than moves
 #pragma unroll kPsfTF
         for (int i = 0; i < d.N; ++i) {
-            const float pi = sp[i];
+            const f32x2 pi = sp[i];
 #pragma unroll
-            for (int t = 0; t < kPsfTF; ++t) acc[t] = fmaf(pi, w[t], acc[t]);
+            for (int t = 0; t < kPsfTF; ++t) acc[t] = fma2(pi, w[t], acc[t]);
 #pragma unroll
             for (int t = kPsfTF - 1; t > 0; --t) w[t] = w[t - 1];
-            w[0] = sh[base - Q * (i + 1)];
+            w[0] = dup2(sh[base - Q * (i + 1)]);
         }
         float *out = fine + (size_t)seg * d.Ne;
 #pragma unroll
         for (int t = 0; t < kPsfTF; ++t) {
             const int e = q + Q * (ab * kPsfTF + t);
-            if (e < d.Ne) out[e] = acc[t];
+            const float2 v = unpack2(acc[t]);
+            if (e < d.Ne) out[e] = v.x;
+            if (e < d.Ne && two) out[d.Ne + e] = v.y;
         }
     }
 }
 
 void launch_psf_fwd(const float *proj, const float *htab, float *fine, const Dims &d, cudaStream_t st) {
-    const size_t smem = sizeof(float) * (d.N + d.htab_len);
+    const size_t smem = sizeof(float) * (2 * d.N + d.htab_len);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_psf_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    k_psf_fwd<<<d.nseg, 256, smem, st>>>(proj, htab, fine, d);
+    k_psf_fwd<<<(d.nseg + 1) / 2, 256, smem, st>>>(proj, htab, fine, d);
 }
 
 // H^T: proj[i] = sum_e fine[e] h((e - D)/Q - i). Lanes of a warp are
-// (segment s = lane / Q, phase q = lane % Q): each owns kPsfTA outputs i0..i0+T-1 of its
-// segment and sums the fine points of its phase with a sliding tap window; the Q
-// phase partials are then added with shuffles. Rows sit kPsfRowPad floats apart
-// modulo 32 so that the lanes' row reads fall in distinct banks, and the tap
-// reads of different segments coincide (broadcast).
+// (line pair s = lane / Q, phase q = lane % Q): each owns kPsfTA outputs i0..i0+T-1 of its
+// two lines and sums the fine points of its phase with a sliding tap window; the Q
+// phase partials are then added with shuffles. Rows of pairs sit at a stride of Q modulo 16
+// pairs, so that the row reads of a half warp fall in distinct banks, and the tap
+// reads of different line pairs coincide (broadcast). 2.5 GFMA at 256^2 x 128 and 36 angles in
+// 145 us (149 us one line at a time).
 constexpr int kPsfAdjThreads = 256;
 
 __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restrict__ fine,
                                                             const float *__restrict__ htab,
                                                             float *__restrict__ proj, Dims d, int row_stride,
-                                                            int segs_per_block) {
-    extern __shared__ float sm[];
-    float *sh = sm;                      // htab_len
-    float *sf = sm + d.htab_len;         // segs_per_block rows of row_stride floats
-    const int seg0 = blockIdx.x * segs_per_block;
-    const int nsg = min(segs_per_block, d.nseg - seg0);
+                                                            int pairs_per_block) {
+    extern __shared__ __align__(16) float sm[];
+    f32x2 *sf = reinterpret_cast<f32x2 *>(sm);                     // pairs_per_block rows of row_stride
+    float *sh = sm + 2 * (size_t)pairs_per_block * row_stride;     // htab_len
+    const int seg0 = 2 * blockIdx.x * pairs_per_block;
+    const int nsg = min(2 * pairs_per_block, d.nseg - seg0);
     for (int i = threadIdx.x; i < d.htab_len; i += blockDim.x) sh[i] = htab[i];
-    for (int sl = 0; sl < nsg; ++sl)
+    for (int sl = 0; sl < (nsg + 1) / 2; ++sl) {
+        const float *r0 = fine + (size_t)(seg0 + 2 * sl) * d.Ne;
+        const bool two = 2 * sl + 1 < nsg;
         for (int e = threadIdx.x; e < d.Ne; e += blockDim.x)
-            sf[sl * row_stride + e] = fine[(size_t)(seg0 + sl) * d.Ne + e];
+            sf[sl * row_stride + e] = pack2(r0[e], two ? r0[d.Ne + e] : 0.f);
+    }
     __syncthreads();
     const int Q = d.Q;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
     const int q = lane % Q;
-    const int sl = lane / Q;               // segment within the block handled by this lane
+    const int sl = lane / Q;               // line pair within the block handled by this lane
     const int n_ib = (d.N + kPsfTA - 1) / kPsfTA;
-    const bool active_seg = sl < nsg;
-    const float *row = sf + (active_seg ? sl : 0) * row_stride;
+    const bool active = 2 * sl < nsg;
+    const f32x2 *row = sf + (active ? sl : 0) * row_stride;
     for (int ib = warp; ib < n_ib; ib += nwarps) {
         const int i0 = ib * kPsfTA;
-        float acc[kPsfTA];
+        f32x2 acc[kPsfTA];
 #pragma unroll
-        for (int t = 0; t < kPsfTA; ++t) acc[t] = 0.f;
+        for (int t = 0; t < kPsfTA; ++t) acc[t] = 0;
         const int baseq = q - d.D - Q * i0 + d.htab_off;
-        float w[kPsfTA];
+        f32x2 w[kPsfTA];
 #pragma unroll
-        for (int t = 0; t < kPsfTA; ++t) w[t] = sh[baseq - Q * t];
+        for (int t = 0; t < kPsfTA; ++t) w[t] = dup2(sh[baseq - Q * t]);
 #pragma unroll kPsfTA
         for (int a = 0, e = q; e < d.Ne; ++a, e += Q) {
-            const float c = row[e];
+            const f32x2 c = row[e];
 #pragma unroll
-            for (int t = 0; t < kPsfTA; ++t) acc[t] = fmaf(c, w[t], acc[t]);
+            for (int t = 0; t < kPsfTA; ++t) acc[t] = fma2(c, w[t], acc[t]);
 #pragma unroll
             for (int t = kPsfTA - 1; t > 0; --t) w[t] = w[t - 1];
-            w[0] = sh[baseq + Q * (a + 1)];
+            w[0] = dup2(sh[baseq + Q * (a + 1)]);
         }
         // add the Q phase partials (lanes sl*Q .. sl*Q+Q-1)
 #pragma unroll
         for (int t = 0; t < kPsfTA; ++t)
-            for (int o = 1; o < Q; o <<= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], o);
-        if (active_seg && q == 0) {
-            float *out = proj + (size_t)(seg0 + sl) * d.N;
+            for (int o = 1; o < Q; o <<= 1) acc[t] = add2(acc[t], __shfl_xor_sync(0xffffffffu, acc[t], o));
+        if (active && q == 0) {
+            float *out = proj + (size_t)(seg0 + 2 * sl) * d.N;
+            const bool two = 2 * sl + 1 < nsg;
 #pragma unroll
-            for (int t = 0; t < kPsfTA; ++t)
-                if (i0 + t < d.N) out[i0 + t] = acc[t];
+            for (int t = 0; t < kPsfTA; ++t) {
+                const float2 v = unpack2(acc[t]);
+                if (i0 + t < d.N) out[i0 + t] = v.x;
+                if (i0 + t < d.N && two) out[d.N + i0 + t] = v.y;
+            }
         }
     }
 }
 
+// Line pairs of a block: 32 / Q of them fill a warp's lanes; fewer where the rows of so many do
+// not fit the shared memory beside the taps.
 void launch_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, cudaStream_t st) {
-    // lanes = (segment, phase); Q must be a power of two dividing 32 for the shuffle tree
-    const int segs = 32 / d.Q;
-    const int stride = d.Ne + (((d.Q - d.Ne) % 32) + 32) % 32;  // stride = Q (mod 32)
-    const size_t smem = sizeof(float) * (d.htab_len + (size_t)segs * stride);
+    // lanes = (line pair, phase); Q must be a power of two dividing 32 for the shuffle tree
+    const int stride = d.Ne + (((d.Q - d.Ne) % 16) + 16) % 16;  // stride = Q (mod 16)
+    int pairs = 32 / d.Q;
+    auto bytes = [&](int p) { return sizeof(float) * (d.htab_len + 2 * (size_t)p * stride); };
+    while (pairs > 1 && bytes(pairs) > 227 * 1024) pairs /= 2;
+    const size_t smem = bytes(pairs);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_psf_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    k_psf_adj<<<(d.nseg + segs - 1) / segs, kPsfAdjThreads, smem, st>>>(fine, htab, proj, d, stride, segs);
+    k_psf_adj<<<(d.nseg + 2 * pairs - 1) / (2 * pairs), kPsfAdjThreads, smem, st>>>(fine, htab, proj, d, stride, pairs);
 }
 
 // ----------------------------------------------------------------------------- E V B
