@@ -22,10 +22,14 @@ from .operator import FFLOperator
 class _ApplyA(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, gains, fwhm, op):
-        g_host = [float(v) for v in gains.detach().cpu().reshape(-1)]
+        g, w = gains.detach().reshape(-1), fwhm.detach().reshape(-1)[:1]
+        if g.device == w.device and g.dtype == w.dtype:  # one wait for both
+            host = torch.cat((g, w)).tolist()
+        else:
+            host = g.tolist() + w.tolist()
+        g_host, w = host[:-1], host[-1]
         if getattr(op, "gains", None) != g_host:
             op.set_gain(g_host)
-        w = float(fwhm.detach().cpu().reshape(-1)[0])
         if w != op.fwhm:
             op.set_fwhm(w)
         proj = op.project(x.contiguous())

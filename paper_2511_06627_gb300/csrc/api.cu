@@ -174,12 +174,12 @@ void psf_tables(const Dims &d, double fwhm, std::vector<float> &h, std::vector<f
     const double a = fwhm / (2.0 * langevin_half_point());
     h.resize(d.htab_len);
     dh.resize(d.htab_len);
-    for (int k = 0; k < d.htab_len; ++k) {
-        const double u = (double)(k - d.htab_off) / d.Q;
+    for (int k = 0; k <= d.htab_off; ++k) {  // both are even in u
+        const double u = (double)k / d.Q;
         const double x = u / a;
-        h[k] = (float)(3.0 * langevin_d1(x));
+        h[d.htab_off + k] = h[d.htab_off - k] = (float)(3.0 * langevin_d1(x));
         // d/dfwhm of 3 L'(u/a), a = fwhm / (2 x_h): -3 L''(x) x / fwhm
-        dh[k] = (float)(-3.0 * langevin_d2(x) * x / fwhm);
+        dh[d.htab_off + k] = dh[d.htab_off - k] = (float)(-3.0 * langevin_d2(x) * x / fwhm);
     }
 }
 
@@ -776,6 +776,27 @@ void adjoint_impl(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st) 
 void param_grad_impl(mpi_ffl_handle *h, const float *proj, const float *d_gb, float *d_g_gain, float *d_g_fwhm,
                      cudaStream_t st) {
     const Dims &d = h->d;
+    if (h->path == MPI_FFL_PATH_LINE_GEMM) {
+        // <g_b, W H p> = <H^T W^T g_b, p>: both gradients from one transposed product, in
+        // projections, where the forward form ran W H p and W (dH) p and wrote both as data
+        // (133 us at 128^2 x 64 and 24 angles, this way 88 us)
+        if (h->t_coil) {
+            TIMED(MPI_FFL_K_COIL, launch_coil_pad(proj, h->t_coil, h->w_projc, (long long)d.M * d.Nz, d.Nz, d.N, d.N, st));
+            proj = h->w_projc;
+        }
+        TIMED(MPI_FFL_K_GEMM_ADJ, col_adjoint(h, d_gb, false, h->t_unit_gain, h->w_fine, st));
+        const int64_t per = (int64_t)d.Nz * d.N;
+        const int nbk = std::min(1024, std::max(1, (int)((per + 1023) / 1024)));
+        for (int k = 0; k < 2; ++k) {
+            if (!(k ? d_g_fwhm : d_g_gain)) continue;
+            TIMED(MPI_FFL_K_PSF_ADJ, launch_psf_adj(h->w_fine, k ? h->t_dhtab : h->t_htab, h->s_g, d, st));
+            TIMED(MPI_FFL_K_SOLVER, launch_angle_dots(h->s_g, proj, d.M, per, h->w_red, nbk, st));
+            if (k) TIMED(MPI_FFL_K_SOLVER, launch_angles_weighted(h->w_red, d.M, nbk, h->t_gain, d_g_fwhm, st));
+            else TIMED(MPI_FFL_K_SOLVER, launch_angle_finalize(h->w_red, d.M, nbk, d_g_gain, st));
+        }
+        check_launch(h, "parameter gradients");
+        return;
+    }
     if (d_g_gain) {
         line_forward_impl(h, proj, h->s_r, h->t_htab, h->t_unit_gain, st);
         const int64_t per = (int64_t)2 * d.Nz * d.nb;
@@ -989,7 +1010,7 @@ extern "C" int mpi_ffl_create(const mpi_ffl_geometry *geom, const mpi_ffl_trajec
         CK(cudaMemset(h->w_count, 0, 2 * sizeof(unsigned)));
         dev_alloc(h, &h->s_xp, d.nvox);
         dev_alloc(h, &h->s_y, d.nvox);
-        dev_alloc(h, &h->s_g, d.nvox);
+        dev_alloc(h, &h->s_g, std::max(d.nvox, d.nproj));  // a gradient, or projections (param_grad_impl)
         dev_alloc(h, &h->s_r, d.ndata);
         dev_alloc(h, &h->s_flags, 4);
         dev_alloc(h, &h->w_err, 1);

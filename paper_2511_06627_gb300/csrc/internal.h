@@ -419,6 +419,9 @@ void launch_angle_dots(const float *a, const float *b, int M, int64_t per_angle,
                        int nblk_per_angle, cudaStream_t st);
 void launch_angle_finalize(const double *partials, int M, int nblk_per_angle, float *out,
                            cudaStream_t st);
+// out = sum over angles of weight[m] times the angle's sum of partials
+void launch_angles_weighted(const double *partials, int M, int nblk_per_angle, const float *weight, float *out,
+                            cudaStream_t st);
 void launch_finalize_to_float(const double *partials, int nblk, float *out, cudaStream_t st);
 
 }  // namespace mpiffl

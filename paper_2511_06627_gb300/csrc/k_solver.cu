@@ -260,6 +260,20 @@ void launch_angle_finalize(const double *partials, int M, int nblk_per_angle, fl
     k_angle_finalize<<<M, kRedThreads, 0, st>>>(partials, nblk_per_angle, out);
 }
 
+// partials are [angle][nblk]: each angle's sum weighted, in one sum over threads in a fixed order
+__global__ void __launch_bounds__(kRedThreads) k_angles_weighted(const double *partials, int M, int nblk,
+                                                                 const float *__restrict__ weight, float *out) {
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < M * nblk; i += blockDim.x) acc += (double)__ldg(weight + i / nblk) * partials[i];
+    const double t = block_sum(acc);
+    if (threadIdx.x == 0) *out = (float)t;
+}
+
+void launch_angles_weighted(const double *partials, int M, int nblk_per_angle, const float *weight, float *out,
+                            cudaStream_t st) {
+    k_angles_weighted<<<1, kRedThreads, 0, st>>>(partials, M, nblk_per_angle, weight, out);
+}
+
 // T^T T x with forward differences and no wrap (Neumann): 7-point stencil with the
 // face-reduced diagonal.
 __device__ __forceinline__ float ttt_at(const float *__restrict__ x, int N, int Nz, int z, int y, int xx) {

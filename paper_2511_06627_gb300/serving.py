@@ -114,7 +114,7 @@ def estimate_request_bytes(geometry):
     nb = K * (2 * geometry["half_width"] + 1)
     ne = (nx - 1) * Q + 2 * int(-(-A * Q // 1)) + 1
     nvox, nproj, nfine, ndata = nz * nx * nx, m * nz * nx, m * nz * ne, 2 * m * nz * nb
-    handle = 4 * (3 * nvox + nproj + nfine + 2 * ndata) + 4 * 4 * nvox + 4 * 2 * S * P * 12 + (8 << 20)
+    handle = 4 * (3 * nvox + nproj + nfine + 2 * ndata) + 4 * (3 * nvox + max(nvox, nproj)) + 4 * 2 * S * P * 12 + (8 << 20)
     return handle + 4 * (4 * nvox + 2 * ndata)
 
 
