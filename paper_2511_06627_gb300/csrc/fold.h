@@ -31,7 +31,9 @@ void fold_release(mpi_ffl_handle *h);
 
 // C[crow[i]][ccol[n]] = scale[arow[i] / rdiv] sum_k A[arow[i]][acol[k]] B[k][n] in FP32
 // (arow, crow, acol and ccol may be NULL: row i, column k or n; scale NULL: 1). B is K x
-// ldb, ldb a multiple of 4, on 16 bytes.
+// ldb, ldb a multiple of 4, on 16 bytes; its rows hold bcols values that may be read (a
+// multiple of 4; 0: ldb). nbatch: that many such products, their operands sA, sB (a
+// multiple of 4) and sC values apart.
 struct SgemmArgs {
     const float *A;
     int64_t lda;
@@ -46,6 +48,8 @@ struct SgemmArgs {
     const float *scale;
     int rdiv;
     const int *acol, *ccol;
+    int nbatch = 1, bcols = 0;
+    int64_t sA = 0, sB = 0, sC = 0;
 };
 constexpr int kSgemmMax = 9;  // problems of one launch
 void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st);

@@ -41,7 +41,7 @@ struct SgemmBatch {
 
 // K of one run of sums: longer products add their runs' sums, so that rounding errors grow
 // with the run and the number of runs, not with K
-constexpr int kSgRun = 256;
+constexpr int kSgRun = 320;
 
 // One BM x BN tile per block. A warp covers 8 row groups x 4 column groups of TM x TN sums
 // each (a thread's rows are 8 apart, its columns come in runs of 4, BN / (TN / 4) apart). A
@@ -69,49 +69,56 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
     int pi = 0;
     while ((int)blockIdx.x >= batch.first[pi + 1]) ++pi;  // uniform
     const SgemmArgs &g = batch.g[pi];
-    const int b = (int)blockIdx.x - batch.first[pi];
-    const int ntn = (g.N + BN - 1) / BN;
+    const int ntn = (g.N + BN - 1) / BN, nt = (g.M + BM - 1) / BM * ntn;
+    const int bi = ((int)blockIdx.x - batch.first[pi]) / nt, b = (int)blockIdx.x - batch.first[pi] - bi * nt;
     const int m0 = b / ntn * BM, c0 = b % ntn * BN;
+    const float *gA = g.A + bi * g.sA, *gB = g.B + bi * g.sB;
+    const int bcols = g.bcols ? g.bcols : g.ldb;
     const int tid = threadIdx.x, lane = tid & 31, kg = tid / TG;
     const int tr = lane >> 2, tc = (tid % TG >> 5) * 4 + (lane & 3);
 
-    // this thread's part of a stage of A: K quad i mod 4 of row i / 4, i = tid + u T
+    // This thread's part of a stage of A: K quad tid mod 4 of the rows tid / 4 + u T / 4. Past
+    // the last row the tile's rows again, whose sums are not stored (not one row for all of
+    // them: copies of one address to many places take turns, 64 rows in tiles of 56 took three
+    // times as long).
+    static_assert(T % (kSgK / 4) == 0 && T % (BN / 4) == 0, "a thread keeps its K quad and its columns");
+    const int ka = 4 * (tid % (kSgK / 4));
     const float *ap[NA];
 #pragma unroll
     for (int u = 0; u < NA; ++u) {
-        const int i = tid + u * T, r = m0 + i / (kSgK / 4);
-        const bool in = i < BM * kSgK / 4 && r < g.M;
-        ap[u] = in ? g.A + (size_t)(g.arow ? __ldg(g.arow + r) : r) * g.lda : nullptr;
+        const int r = m0 + (tid + u * T) / (kSgK / 4) % min(BM, g.M - m0);
+        ap[u] = gA + (size_t)(g.arow ? __ldg(g.arow + r) : r) * g.lda;
     }
-    const bool vec = !g.acol && g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(g.A) & 15) == 0;
+    const bool vec = !g.acol && g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(gA) & 15) == 0;
     auto copy_a = [&](int t) {
-        float *st = smf + (t % kSgStages) * kStage;
+        float *st = smf + (t % kSgStages) * kStage + (tid / (kSgK / 4)) * kSgRow + ka;
+        const int k = t * kSgK + ka, n = min(4, max(0, g.K - k)), ks = min(k, (g.K - 1) & ~3);
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
-            const int i = tid + u * T;
-            if (i >= BM * kSgK / 4) break;
-            const int k = t * kSgK + 4 * (i % (kSgK / 4));
-            float *dst = st + (i / (kSgK / 4)) * kSgRow + 4 * (i % (kSgK / 4));
+            if ((BM * kSgK / 4) % T && tid + u * T >= BM * kSgK / 4) break;
+            float *dst = st + u * (T / (kSgK / 4)) * kSgRow;
             if (vec) {
-                const int n = ap[u] ? min(4, max(0, g.K - k)) : 0;
-                cp_async16(dst, n ? ap[u] + k : g.A, 4 * n);
+                cp_async16(dst, ap[u] + ks, 4 * n);
             } else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const bool in = ap[u] && k + e < g.K;
-                    cp_async4(dst + e, in ? ap[u] + (g.acol ? __ldg(g.acol + k + e) : k + e) : g.A, in ? 4 : 0);
+                    const bool in = k + e < g.K;
+                    cp_async4(dst + e, in ? ap[u] + (g.acol ? __ldg(g.acol + k + e) : k + e) : gA, in ? 4 : 0);
                 }
             }
         }
     };
+    // of B: columns cb of the rows tid / (BN / 4) + u T / (BN / 4)
+    const int cb = c0 + 4 * (tid % (BN / 4)), kb0 = tid / (BN / 4);
+    const float *bp = gB + min(cb, bcols - 4);
+    const int kvalid = cb < bcols ? g.K : 0;
     auto copy_b = [&](int t) {
-        float *st = smf + (t % kSgStages) * kStage + BM * kSgRow;
+        float *st = smf + (t % kSgStages) * kStage + BM * kSgRow + 4 * tid;
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
-            const int i = tid + u * T, kk = i / (BN / 4), c = 4 * (i % (BN / 4));
-            if (i >= BN * kSgK / 4) break;
-            const bool in = t * kSgK + kk < g.K && c0 + c < g.ldb;
-            cp_async16(st + kk * BN + c, in ? g.B + (size_t)(t * kSgK + kk) * g.ldb + c0 + c : g.B, in ? 16 : 0);
+            if ((BN * kSgK / 4) % T && tid + u * T >= BN * kSgK / 4) break;
+            const int kk = t * kSgK + kb0 + u * (T / (BN / 4));
+            cp_async16(st + 4 * u * T, bp + (int64_t)min(kk, g.K - 1) * g.ldb, kk < kvalid ? 16 : 0);
         }
     };
 
@@ -199,13 +206,14 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
                     acc[i][j] = add2(acc[i][j], pack2(o.x, o.y));
                 }
     }
-    const bool vecc = !g.ccol && g.ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
+    float *gC = g.C + bi * g.sC;
+    const bool vecc = !g.ccol && g.ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(gC) & 15) == 0;
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int r = m0 + tr + 8 * i;
         if (r >= g.M) continue;
         const float sc = g.scale ? __ldg(g.scale + (g.arow ? __ldg(g.arow + r) : r) / g.rdiv) : 1.f;
-        float *dst = g.C + (size_t)(g.crow ? __ldg(g.crow + r) : r) * g.ldc;
+        float *dst = gC + (size_t)(g.crow ? __ldg(g.crow + r) : r) * g.ldc;
 #pragma unroll
         for (int j = 0; j < TN / 4; ++j) {
             const int c = c0 + j * (BN / (TN / 4)) + 4 * tc;
@@ -222,6 +230,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
     }
 }
 
+int batches(const SgemmArgs *g, int i, int n) { return i < n ? std::max(0, g[i].nbatch) : 0; }
+
 template <int BM, int BN, int TM, int TN, int KG>
 void run(const SgemmArgs *g, int n, cudaStream_t st) {
     constexpr int T = (BM / TM) * (BN / TN) * KG;
@@ -231,7 +241,7 @@ void run(const SgemmArgs *g, int n, cudaStream_t st) {
         const int tiles = i < n ? (g[i].M + BM - 1) / BM * ((g[i].N + BN - 1) / BN) : 0;
         if (i < n) b.g[i] = g[i];
         if (i < n && g[i].K > kSgRun * KG) runs = true;
-        b.first[i + 1] = b.first[i] + tiles;
+        b.first[i + 1] = b.first[i] + tiles * batches(g, i, n);
     }
     const int total = b.first[kSgemmMax];
     if (total == 0) return;
@@ -246,13 +256,35 @@ void run(const SgemmArgs *g, int n, cudaStream_t st) {
 int sgemm_tiles(const SgemmArgs &g) { return (g.M + 63) / 64 * ((g.N + 127) / 128); }
 
 // 8 x 8 sums a thread (the fewest shared loads an FMA) where such tiles come to four blocks
-// an SM: 4608 x 2304 x 256 in 120 us, 60% of the FP32 FMA rate (4 x 8 sums in 32 x 64 tiles
-// and two groups along K: 143 us). Smaller products take the smaller tiles: 4608 x 288 x 256
-// in 25 us (34 us with the large tiles), 1536 x 168 x 128 in 6.3 us (13.3 us).
+// an SM: 4608 x 2304 x 256 in 106 us, 68% of the FP32 FMA rate (4 x 8 sums in 32 x 64 tiles
+// and two groups along K: 129 us). Smaller products take the smaller tiles: 4608 x 288 x 256
+// in 22 us (29 us with the large tiles), 1536 x 168 x 128 in 5.5 us (11 us).
+//
+// Batches of products with few rows each (one per frequency or angle) take tiles of 64 columns
+// whose height fits the rows: the least padding, a tile's loads of B counted as 24 rows. 127
+// of 72 x 576 x 256 take 66 us in one tile of 72 rows each (20 TFMA/s), 74 us in two of 40, 90
+// in three of 32 and 110 in two of 64. Where that leaves an SM without its three blocks, the
+// smallest tiles: 72 of 64 x 288 x 256 in 23 us (25 us in tiles of 64 rows).
 void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st) {
-    int big = 0;
-    for (int i = 0; i < n; ++i) big += sgemm_tiles(g[i]);
-    if (big >= 600) run<64, 128, 8, 8, 1>(g, n, st);
+    int big = 0, rows = 0;
+    for (int i = 0; i < n; ++i) {
+        big += sgemm_tiles(g[i]);
+        if (g[i].nbatch != 1) rows = std::max(rows, g[i].M);
+    }
+    int height = 0;
+    if (rows > 0) {
+        for (int h : {32, 40, 56, 64, 72})
+            if (!height || (rows + h - 1) / h * (h + 24) < (rows + height - 1) / height * (height + 24)) height = h;
+        int64_t tiles = 0;
+        for (int i = 0; i < n; ++i)
+            tiles += (int64_t)g[i].nbatch * ((g[i].M + height - 1) / height) * ((g[i].N + 63) / 64);
+        if (tiles < 3 * 152) height = 32;
+    }
+    if (height == 40) run<40, 64, 5, 8, 2>(g, n, st);
+    else if (height == 56) run<56, 64, 7, 8, 2>(g, n, st);
+    else if (height == 64) run<64, 64, 8, 8, 2>(g, n, st);
+    else if (height == 72) run<72, 64, 9, 8, 2>(g, n, st);
+    else if (height == 0 && big >= 600) run<64, 128, 8, 8, 1>(g, n, st);
     else run<32, 64, 4, 8, 2>(g, n, st);
 }
 
