@@ -883,7 +883,7 @@ def run_ours(args, cfg, rank, world, local_rank):
                                 "x_drive_path": path, "z_drive_path": "FP32, E_z V_z B fused with S D F",
                                 "step": "[A; A_z] x then A^T b + A_z^T b_z"}
         # tensor PSF (Appendix B, Eq. (31)): every line reads every slice of its projection;
-        # A and A^T run as per-line (per-slice) split-K GEMMs on the bf16 hi+lo operands
+        # the DFT along z turns the sum over slices into one FP32 product per frequency
         op.set_psf_model("tensor")
         for _ in range(2):
             op.forward(x, out=b)
@@ -898,26 +898,16 @@ def run_ours(args, cfg, rank, world, local_rank):
         t_ms, t_n = tprof["tensor"]
         nz_ = dims["nvox"] // (dims["N"] * dims["N"])
         R_ = dims["ndata"] // (dims["M"] * nz_)
-        flops = 2.0 * dims["M"] * nz_ * (nz_ * dims["N"]) * R_  # one direction, FP32 contraction
+        # one direction: along z (2 N_z x N_z), 2 N_z products by n_par 2n_b x N matrices, back
+        n_par_ = 2 if cfg["zigzag"] else 1
+        flops = 2.0 * dims["M"] * 2 * nz_ * (nz_ * (dims["N"] + R_) + n_par_ * R_ * dims["N"])
         sec = t_ms / max(t_n, 1) / 1e3
-        peak, peak_src = bf16_peak_tflops()
-        # issued MMA work: J = 128 // M8 lines of one trajectory share a problem (rows M8 J,
-        # M8 = M rounded up to 8, in 128-row tiles) and its window spans N_z + step (J - 1)
-        # slices
-        step_ = 2 if cfg["zigzag"] else 1
-        M8_ = (dims["M"] + 7) // 8 * 8
-        J_ = max(1, min(128 // M8_, (nz_ + step_ - 1) // step_))
-        issue_factor = (128 * ((M8_ * J_ + 127) // 128) / (dims["M"] * J_)) * (nz_ + step_ * (J_ - 1)) / nz_
         result["tensor_psf"] = {
             "pairs_per_s": 1e3 / ten_ms, "ms_per_pair": ten_ms,
             "stage_ms_per_launch": round(t_ms / max(t_n, 1), 4),
-            "tensor_tflops": round(3 * flops / sec / 1e12, 2),
-            "tensor_frac": round(3 * flops / sec / 1e12 / peak, 4),
-            "issued_frac": round(3 * flops * issue_factor / sec / 1e12 / peak, 4),
-            "peak": f"{peak} TFLOP/s bf16 ({peak_src})",
-            "note": "stage = coil weighting + padding, per-line (per-slice) GEMMs over all slices (3 bf16 "
-                    "products of 2 M N_z (N_z N) 2n_b flops), sum of the K splits; issued counts the 128-row "
-                    "MMA tiles that hold J lines x M8 angles and the window's step (J - 1) extra slices"}
+            "fp32_tflops": round(flops / sec / 1e12, 2),
+            "fp32_frac": round(flops / sec / 1e12 / FP32_PEAK_TFLOPS, 4),
+            "note": "stage = three FP32 products: DFT along z, one product per frequency, inverse DFT"}
         op.set_psf_model("collinear")
         # detection limit (Sec. 4.2, Fig. 5) of a synthetic sensitivity series at the
         # phantom scale: reconstruction with Eq. (26), box statistics on the GPU, line fit

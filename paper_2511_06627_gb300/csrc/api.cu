@@ -419,6 +419,7 @@ void release(mpi_ffl_handle *h) {
     col_release(h);
     fold_release(h);
     zfold_release(h);
+    ten_release(h);
 }
 
 // ------------------------------------------------------------ host buffers
@@ -1133,22 +1134,9 @@ static int set_path_impl(mpi_ffl_handle *h, int32_t path) {
     return MPI_FFL_OK;
 }
 
-// the tensor-PSF tables hold split operands of the handle's precision
-static int refresh_tensor(mpi_ffl_handle *h, int rc) {
-    if (rc != MPI_FFL_OK || h->psf_model != MPI_FFL_PSF_TENSOR) return rc;
-    return guarded(h, [&]() {
-        CK(cudaDeviceSynchronize());
-        const int r = ten_refresh(h, false);
-        if (r != MPI_FFL_OK) h->err = "rebuilding the tensor-PSF operands failed";
-        return r;
-    });
-}
+extern "C" int mpi_ffl_set_precision(mpi_ffl_handle *h, int32_t precision) { return set_precision_impl(h, precision); }
 
-extern "C" int mpi_ffl_set_precision(mpi_ffl_handle *h, int32_t precision) {
-    return refresh_tensor(h, set_precision_impl(h, precision));
-}
-
-extern "C" int mpi_ffl_set_path(mpi_ffl_handle *h, int32_t path) { return refresh_tensor(h, set_path_impl(h, path)); }
+extern "C" int mpi_ffl_set_path(mpi_ffl_handle *h, int32_t path) { return set_path_impl(h, path); }
 
 extern "C" int mpi_ffl_set_psf_model(mpi_ffl_handle *h, int32_t model) {
     return guarded(h, [&]() {

@@ -60,13 +60,11 @@ struct GemmArgs {
     int tf32;            // 1: tf32 hi + lo operands (32 K elements per stage), 0: bf16 (64)
     int nacc;            // accumulators in TMEM: K chunk kc adds into accumulator kc % nacc
     int acc_stride;      // TMEM columns between accumulators (a multiple of 32, >= BN)
-    int b_tstride;       // K chunks per N tile in B's storage (0: nkc); B may be a K window of a table
     // A pre-split in its canonical layout (NULL: the producer warps split g.A). 1 KB blocks
-    // (group of 8 rows, K chunk) ordered [chunk][hi, lo][group]; tile row group
-    // j * apk_gper + g (g < apk_gper, j < apk_jg) takes the blocks of group g at chunk
-    // apk_cbase + j * apk_cstep + kc, so each j is one contiguous copy per half.
+    // (group of 8 rows, K chunk) ordered [chunk][hi, lo][group], apk_gper groups: a tile's
+    // groups of one chunk are one contiguous copy per half.
     const uint8_t *apk;
-    int apk_jg, apk_gper, apk_cbase, apk_cstep;
+    int apk_gper;
     // failure-detection test hook: > 0 makes every block wait this many polls on the
     // final-MMA barrier before any copy or MMA is issued (so nothing ever arrives
     // there), record a timeout and free its TMEM (mpi_ffl_test_inject_timeout)
@@ -339,10 +337,10 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int mt, int nt, uin
     } else {
         // ------------------------------------------------------------ B loader
         if (lane == 0) {
-            const uint8_t *bt = g.B + (size_t)nt * (g.b_tstride ? g.b_tstride : g.nkc) * 2 * bytesB;
+            const uint8_t *bt = g.B + (size_t)nt * g.nkc * 2 * bytesB;
             // pre-split A: the row groups of this m tile that hold rows
             const int rg0 = mt * (kBM / 8);
-            const int nrg = g.apk ? max(0, min(kBM / 8, g.apk_jg * g.apk_gper - rg0)) : 0;
+            const int nrg = g.apk ? max(0, min(kBM / 8, g.apk_gper - rg0)) : 0;
             for (int kc = 0; kc < g.nkc; ++kc) {
                 const int s = kc % g.stages;
                 if (kc >= g.stages && !ptx::mbar_wait_bounded(&bars[g.stages + s], ((kc / g.stages) - 1) & 1, kWait)) {
@@ -353,15 +351,10 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs &g, int mt, int nt, uin
                 uint8_t *sb = sa + 2 * bytesA;
                 ptx::mbar_arrive_expect_tx(&bars[s], 2 * bytesB + 2048u * (uint32_t)nrg);
                 ptx::bulk_g2s(sb, bt + (size_t)kc * 2 * bytesB, 2 * bytesB, &bars[s]);
-                for (int r = 0; r < nrg;) {  // one copy per half for each run of one j
-                    const int rg = rg0 + r, j = rg / g.apk_gper, gg = rg - j * g.apk_gper;
-                    const int len = min(g.apk_gper - gg, nrg - r);
-                    const size_t c2 = 2 * (size_t)(g.apk_cbase + j * g.apk_cstep + kc);
-                    const uint8_t *hi = g.apk + (c2 * g.apk_gper + gg) * 1024u;
-                    const uint8_t *lo = g.apk + ((c2 + 1) * g.apk_gper + gg) * 1024u;
-                    ptx::bulk_g2s(sa + r * 1024u, hi, 1024u * len, &bars[s]);
-                    ptx::bulk_g2s(sa + bytesA + r * 1024u, lo, 1024u * len, &bars[s]);
-                    r += len;
+                if (nrg > 0) {
+                    const uint8_t *hi = g.apk + (2 * (size_t)kc * g.apk_gper + rg0) * 1024u;
+                    ptx::bulk_g2s(sa, hi, 1024u * nrg, &bars[s]);
+                    ptx::bulk_g2s(sa + bytesA, hi + (size_t)g.apk_gper * 1024u, 1024u * nrg, &bars[s]);
                 }
             }
         }
@@ -503,7 +496,6 @@ struct ColState {
     // per operand format (0 bf16, 1 tf32) and trajectory: forward / adjoint operands of
     // W (line) and W H (full)
     Packed evf_f[2][2], evf_a[2][2], full_f[2][2], full_a[2][2];
-    struct TensorState *ten = nullptr;  // slice-coupled operator of the tensor PSF
     int *rows[2] = {nullptr, nullptr};  // line indices of each trajectory
     int nrows[2] = {0, 0};
     int *err = nullptr;
@@ -525,7 +517,7 @@ struct PackLines {
 };
 
 // A rows of the full line stage, split once per call into the canonical layout the
-// producer warps would write, as k_pack_rows does for the tensor PSF: row r of
+// producer warps would write: row r of
 // trajectory blockIdx.y is line arow[r] of in (stride lda, Ka valid values, zero past
 // Ka and past the last row). One thread per 16-byte row of a block (8 bf16 or 4 tf32
 // values), split exactly as the producers split.
@@ -661,7 +653,6 @@ int gemm_problems(const mpi_ffl_handle *h, bool adjoint, const float *in, float 
         g.done = done;
         if (prepacked) {
             g.apk = s->apk[0][par];
-            g.apk_jg = 1;
             g.apk_gper = (g.M + 7) / 8;
         }
         for (int mt = 0; mt < (g.M + kBM - 1) / kBM; ++mt)
@@ -782,12 +773,9 @@ void col_init(mpi_ffl_handle *h) {
     s->ok = true;
 }
 
-void ten_release(ColState *s);
-
 void col_release(mpi_ffl_handle *h) {
     ColState *s = cs(h);
     if (!s) return;
-    ten_release(s);
     for (int p = 0; p < 2; ++p) {
         for (int f = 0; f < 2; ++f)
             for (Packed *pk : {&s->evf_f[f][p], &s->evf_a[f][p], &s->full_f[f][p], &s->full_a[f][p]})
@@ -836,10 +824,7 @@ static void pack_full(mpi_ffl_handle *h, int dir, const float *in, GemmArgs *g, 
     for (int par = 0; par < s->n_par; ++par) {
         pl[par] = PackLines{g[par].arow, g[par].M, s->apk[dir][par]};
         g[par].apk = s->apk[dir][par];
-        g[par].apk_jg = 1;
         g[par].apk_gper = (g[par].M + 7) / 8;
-        g[par].apk_cbase = 0;
-        g[par].apk_cstep = 0;
     }
     if (prepacked) return;
     const int G = (std::max(g[0].M, s->n_par > 1 ? g[1].M : 0) + 7) / 8;
@@ -951,419 +936,6 @@ void col_batch_launch(const void *dargs, const int4 *ditems, int n_items, size_t
 
 void col_batch_init() {
     cudaFuncSetAttribute(k_gemm_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-}
-
-// ============================================================ tensor PSF (slices coupled)
-// With the in-plane tensor PSF (Appendix B, Eq. (31): an x drive read by a collinear
-// coil takes h_uu(u, z) = 3 [L'(xi) u^2/rho^2 + (L(xi)/xi) z^2/rho^2], xi = rho / a) the
-// PSF-convolved projection of line l mixes every slice z': c_l = sum_z' H_{l-z'} b.p_z',
-// with H_d[e][i] = h_uu(u_lo + e/Q - i, d). Folded with the line operator W_par of the
-// line's trajectory, line l's data are
-//     data[m][l] = g_m sum_z' W_{par(l), l-z'} (b . p)[m][z'],    W_{par,d} = W_par H_d,
-// one 2 n_b x N matrix per trajectory and slice offset (H_d is even in d). Stacked by
-// offset, T_par[t] = W_{par, Nz-1-t} (t = 0 .. 2 Nz - 2), line l is one GEMM whose K
-// runs over all slices (z', i) and whose B is the window t = Nz-1-l .. 2Nz-2-l of
-// T_par; its rows are the angles. The transpose is one GEMM per slice z' whose K runs
-// over all lines (l, o): B is the window t = Nz-1-z' .. 2Nz-2-z' of Tadj_s[t] =
-// W_{par(l), t-(Nz-1)}^T, where line l = z' + t - (Nz-1) has parity (s + t - Nz + 1) & 1
-// for slices of parity s.
-//
-// The rows of one such GEMM are the M angles only, so J = 128 / M lines of one
-// trajectory share a problem: line l + step j (step = 2 with zig-zag, else 1) reads the
-// window of line l shifted by step j slices, which is the same window applied to the
-// projection shifted by step j slices. Row (j, m) of the problem whose last line is
-// l_J reads the coil-weighted projection, padded with step (J - 1) zero slices in
-// front, from slice step (j + J - J_g) on; the window starts at t = Nz - 1 - l_J and
-// spans Nz + step (J - 1) slices. The tables carry step (J - 1) zero slices at both
-// ends so that a partial group keeps the same extent (its missing rows write
-// nothing). The transpose groups slices the same way.
-namespace {
-
-constexpr int kTenSplitK = 4096; // K per problem at most (64 bf16 chunks: 32 per accumulator)
-
-// N tile: the fewest tiles of at most 256 columns (one MMA), rounded up to 16. Fewer
-// tiles fetch the A rows fewer times; one block per SM holds up to 512 TMEM columns, two
-// accumulators of 256 or three of 160.
-int ten_bn(int Nv) {
-    const int tiles = (Nv + 255) / 256;
-    return std::min(256, ((Nv + tiles - 1) / tiles + 15) / 16 * 16);
-}
-
-struct TensorState {
-    int fmt = -1;              // operand format of the packed tables (0 bf16, 1 tf32)
-    Packed fwd[2], adj[2];     // T per trajectory (forward), Tadj per slice parity (adjoint)
-    int Np = 0, Op = 0;        // K per slice (forward) and per line (adjoint), multiples of 64
-    int step = 1, J = 1;       // line step of one trajectory; lines per problem
-    int Zp = 0, P0 = 0;        // padded slices per angle (a multiple of step), leading zeros
-    int Tpre = 0;              // zero offsets in front of and behind each table (step (J - 1))
-    double *Wd = nullptr;      // [n_par][Nz][2 n_b][N], offsets d >= 0
-    int M8 = 0;                // angles rounded up to a multiple of 8 (rows of a shift j)
-    uint8_t *apk_f = nullptr;  // split A of the forward: coil-weighted projections, padded
-    uint8_t *apk_a = nullptr;  // split A of the adjoint: data rows, padded
-    int cm[2] = {0, 0};        // K chunks per angle row of apk_f / apk_a (current format)
-    int nsplit[2] = {1, 1};    // K splits of the forward and adjoint problems
-    int ksplit[2] = {0, 0};    // K per split (a multiple of 64)
-    float *c_fwd = nullptr;    // [nsplit][M][Nz][2 n_b] partial sums
-    float *c_adj = nullptr;    // [nsplit][M][Nz][N] partial sums
-    int *idx = nullptr;        // per problem group: M8 J A rows, then M8 J C rows
-    GemmArgs *dargs = nullptr; // forward problems, then adjoint problems
-    int n_prob_f = 0;
-    int4 *ditems = nullptr;    // forward items, then adjoint items
-    int n_items_f = 0, n_items_a = 0;
-    size_t smem[2] = {0, 0};   // dynamic shared memory of the forward and adjoint launches
-    uint32_t cols[2] = {32, 32};  // TMEM columns a block of the forward and adjoint launches holds
-};
-
-// Forward table value T_par[n = o][k = (t + Tpre) Np + i] and adjoint table value
-// Tadj_s[n = i][k = (t + Tpre) Op + o], read from W_{par,|d|} (zero past |d| = Nz - 1).
-struct TenFwdSrc {
-    const double *Wd;
-    int par, Nz, R, N, Np, Tpre;
-    __device__ double operator()(int n, long long k) const {
-        const int ts = (int)(k / Np), i = (int)(k - (long long)ts * Np);
-        const int d = abs(Nz - 1 - (ts - Tpre));
-        if (i >= N || d > Nz - 1) return 0.0;
-        return Wd[(((size_t)par * Nz + d) * R + n) * N + i];
-    }
-};
-struct TenAdjSrc {
-    const double *Wd;
-    int s, n_par, Nz, R, N, Op, Tpre;
-    __device__ double operator()(int n, long long k) const {
-        const int ts = (int)(k / Op), o = (int)(k - (long long)ts * Op);
-        const int dd = ts - Tpre - (Nz - 1);
-        if (o >= R || abs(dd) > Nz - 1) return 0.0;
-        const int par = n_par == 1 ? 0 : ((dd + s) & 1);
-        return Wd[(((size_t)par * Nz + abs(dd)) * R + o) * N + n];
-    }
-};
-
-// A operand of the tensor-PSF GEMMs, split once per call: row m (angle) of the padded
-// block holds K = Zp * per values, value (zp, c) = b[z][c] in[(m Nz + z) ncols + c] for
-// z = zp - P0 in [0, Nz) and c < ncols, else 0 (b NULL: 1). 1 KB blocks per (group of 8
-// angles, K chunk, half), ordered [chunk][hi, lo][group], each in the canonical layout
-// the producer warps write: core-matrix column kg at kg * 128, row r7 at r7 * 16. One
-// thread per 16-byte row of a block (8 bf16 or 4 tf32 values), split as the producers
-// split.
-__global__ void __launch_bounds__(256) k_pack_rows(const float *__restrict__ in, const float *__restrict__ coil,
-                                                   int M, int Nz, int ncols, int per, int P0, int Zp, int cm,
-                                                   int tf32, uint8_t *__restrict__ out) {
-    const int kpc = tf32 ? kBK / 2 : kBK, epk = tf32 ? 4 : 8;
-    const long long total = (long long)((M + 7) / 8) * cm * 64;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const int kg = (int)(t & 7), r7 = (int)((t >> 3) & 7);
-        const long long gc = t >> 6;  // block: (angle group, chunk)
-        const int c = (int)(gc % cm), gq = (int)(gc / cm);
-        const int m = 8 * gq + r7;
-        float v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            v[e] = 0.f;
-            if (e < epk && m < M) {
-                const long long k = (long long)c * kpc + kg * epk + e;
-                const int zp = (int)(k / per), col = (int)(k - (long long)zp * per);
-                const int z = zp - P0;
-                if (z >= 0 && z < Nz && col < ncols) {
-                    v[e] = __ldg(in + ((size_t)m * Nz + z) * ncols + col);
-                    if (coil) v[e] *= __ldg(coil + (size_t)z * ncols + col);
-                }
-            }
-        }
-        uint4 hi, lo;
-        if (tf32) {
-            const float f[4] = {v[0], v[1], v[2], v[3]};
-            split4_tf32(f, hi, lo);
-        } else {
-            split8(v, hi, lo);
-        }
-        const int G = (M + 7) / 8;
-        const uint32_t off = (uint32_t)kg * 128u + (uint32_t)r7 * 16u;
-        *reinterpret_cast<uint4 *>(out + ((2 * (size_t)c) * G + gq) * 1024u + off) = hi;
-        *reinterpret_cast<uint4 *>(out + ((2 * (size_t)c + 1) * G + gq) * 1024u + off) = lo;
-    }
-}
-
-// h_uu at in-plane offset (u, z) voxels; a = FWHM / (2 x_h)
-double h_uu_host(double u, double z, double a) {
-    const double rho2 = u * u + z * z;
-    if (rho2 == 0.0) return 1.0;
-    const double xi = std::sqrt(rho2) / a;
-    double lx;  // L(xi) / xi
-    if (xi < 0.05) {
-        const double x2 = xi * xi;
-        lx = 1.0 / 3.0 - x2 / 45.0 + 2.0 * x2 * x2 / 945.0 - x2 * x2 * x2 / 4725.0;
-    } else {
-        lx = (1.0 / std::tanh(xi) - 1.0 / xi) / xi;
-    }
-    return 3.0 * (langevin_d1_host(xi) * u * u / rho2 + lx * z * z / rho2);
-}
-
-template <class T>
-bool talloc(T **p, size_t n) {
-    if (dev_malloc((void **)p, std::max<size_t>(1, n) * sizeof(T)) != cudaSuccess) {
-        *p = nullptr;
-        cudaGetLastError();
-        return false;
-    }
-    return true;
-}
-
-// W_{par,d} for d = 0 .. Nz-1 from W_par and the tensor PSF (FP64, on the device).
-bool ten_build_wd(const mpi_ffl_handle *h, ColState *s, TensorState *t) {
-    const Dims &d = h->d;
-    const int R = 2 * d.nb;
-    const int kmin = fold_kmin(d), Lk = fold_taps(d);
-    const double a = h->fwhm / (2.0 * langevin_half_point_host());
-    std::vector<double> g((size_t)d.Nz * Lk);
-    for (int dz = 0; dz < d.Nz; ++dz)
-        for (int k = 0; k < Lk; ++k) g[(size_t)dz * Lk + k] = h_uu_host((double)(k + kmin) / d.Q, dz, a);
-    double *dg = nullptr;
-    bool ok = fold_w_dev(h) && talloc(&dg, g.size());
-    if (ok && !t->Wd) ok = talloc(&t->Wd, (size_t)s->n_par * d.Nz * R * d.N);
-    if (ok) {
-        cudaMemcpy(dg, g.data(), g.size() * sizeof(double), cudaMemcpyHostToDevice);
-        launch_fold_taps(fold_w_dev(h), dg, t->Wd, d, s->n_par, d.Nz, nullptr);
-        ok = cudaDeviceSynchronize() == cudaSuccess;
-    }
-    if (dg) dev_free(dg);
-    cudaGetLastError();
-    return ok;
-}
-
-// Line (slice) groups of one trajectory (slice parity): first line and count.
-std::vector<int2> ten_groups(const Dims &d, int step, int J) {
-    std::vector<int2> g;
-    for (int p = 0; p < step; ++p)
-        for (int l = p; l < d.Nz; l += step * J) g.push_back(make_int2(l, std::min(J, (d.Nz - 1 - l) / step + 1)));
-    return g;
-}
-
-// Packed tables, problems and items for operand format fmt.
-bool ten_prepare(const mpi_ffl_handle *h, ColState *s, TensorState *t, int fmt) {
-    const Dims &d = h->d;
-    const int R = 2 * d.nb;
-    const int kpc = fmt ? kBK / 2 : kBK;
-    const long long tslices = 2LL * d.Nz - 1 + 2LL * t->Tpre;  // zero offsets at both ends
-    for (int par = 0; par < s->n_par; ++par)
-        if (!pack_dev(t->fwd[par], TenFwdSrc{t->Wd, par, d.Nz, R, d.N, t->Np, t->Tpre}, R, tslices * t->Np,
-                      ten_bn(R), fmt))
-            return false;
-    for (int sp = 0; sp < s->n_par; ++sp)
-        if (!pack_dev(t->adj[sp], TenAdjSrc{t->Wd, sp, s->n_par, d.Nz, R, d.N, t->Op, t->Tpre}, d.N,
-                      tslices * t->Op, ten_bn(d.N), fmt))
-            return false;
-    if (cudaDeviceSynchronize() != cudaSuccess) return false;
-    const std::vector<int2> groups = ten_groups(d, t->step, t->J);
-    const int rows = t->M8 * t->J;  // tile rows (j, m), m padded to M8
-    t->cm[0] = t->Zp * t->Np / kpc;
-    t->cm[1] = t->Zp * t->Op / kpc;
-    std::vector<int> idx(groups.size() * 2 * 2 * rows);
-    std::vector<GemmArgs> args;
-    std::vector<int4> items[2];
-    const int mtiles = (rows + kBM - 1) / kBM;
-    const int span = d.Nz + t->step * (t->J - 1);  // window slices (lines)
-    // one block per SM (it measured faster than two for these long-K problems), so the
-    // pipeline takes as many stages as fit: A and B both arrive by bulk copies
-    auto deep = [](int BN, int &stages) {
-        const size_t stage = 2u * kBM * kBK * 2 + 2u * BN * kBK * 2;
-        stages = (int)std::max<size_t>(2, std::min<size_t>(4, (220u * 1024u - 256u) / stage));
-        return stages * stage + 256;
-    };
-    int st_dir[2] = {0, 0};
-    t->smem[0] = t->smem[1] = std::max(deep(t->fwd[0].BN, st_dir[0]), deep(t->adj[0].BN, st_dir[1]));
-    for (int dir = 0; dir < 2; ++dir) {
-        const int per = dir ? t->Op : t->Np;  // K per line (adjoint) or per slice (forward)
-        const int BN = dir ? t->adj[0].BN : t->fwd[0].BN;
-        const size_t blk = (size_t)BN * kBK * 2;
-        const int stages = st_dir[dir];
-        const int base = (int)args.size();
-        for (size_t gi = 0; gi < groups.size(); ++gi) {
-            const int l0 = groups[gi].x, Jg = groups[gi].y;
-            const int llast = l0 + t->step * (Jg - 1);
-            int *ar = idx.data() + ((size_t)dir * groups.size() + gi) * 2 * rows;
-            int *cr = ar + rows;
-            for (int j = 0; j < t->J; ++j)
-                for (int m = 0; m < t->M8; ++m) {
-                    // row (j, m): angle m's padded block from slice step (j + J - Jg); the
-                    // A row list only gives the gain (A comes pre-split)
-                    ar[j * t->M8 + m] = m < d.M ? m : 0;
-                    cr[j * t->M8 + m] = (j < Jg && m < d.M) ? m * d.Nz + l0 + t->step * j : -1;
-                }
-            const int *dar = t->idx + (ar - idx.data());
-            const int *dcr = t->idx + (cr - idx.data());
-            // the window starts at t = Nz - 1 - llast (table slice + Tpre)
-            const long long kwin = (long long)(d.Nz - 1 - llast + t->Tpre) * per;
-            const Packed &B = dir ? t->adj[s->n_par == 1 ? 0 : (l0 & 1)] : t->fwd[s->n_par == 1 ? 0 : (l0 & 1)];
-            for (int ks = 0; ks < t->nsplit[dir]; ++ks) {
-                const int k0 = ks * t->ksplit[dir];
-                const int kn = std::min(t->ksplit[dir], span * per - k0);
-                GemmArgs g{};
-                g.A = nullptr;
-                g.lda = 0;
-                g.Ka = kn;
-                g.arow = dar;
-                g.M = rows;
-                g.apk = dir ? t->apk_a : t->apk_f;
-                g.apk_jg = Jg;
-                g.apk_gper = t->M8 / 8;
-                g.apk_cbase = (t->step * (t->J - Jg) * per + k0) / kpc;
-                g.apk_cstep = t->step * per / kpc;
-                g.B = B.dev + (size_t)((kwin + k0) / kpc) * 2 * blk;
-                g.BN = BN;
-                g.nkc = kn / kpc;
-                g.b_tstride = B.nkc;
-                g.C = (dir ? t->c_adj : t->c_fwd) + (size_t)ks * d.M * d.Nz * (dir ? d.N : R);
-                g.ldc = dir ? d.N : R;
-                g.crow = dcr;
-                g.Nc = dir ? d.N : R;
-                g.rscale = h->t_gain;
-                g.rdiv = 1;  // A row list = angle
-                g.prec = h->precision;
-                g.tf32 = fmt;
-                g.stages = stages;
-                // one block per SM: up to 512 TMEM columns, at most 4 accumulators
-                g.acc_stride = (g.BN + 31) / 32 * 32;
-                g.nacc = std::max(1, std::min({4, 512 / g.acc_stride, g.nkc}));
-                {
-                    const int cols = g.nacc * g.acc_stride;
-                    g.tmem_cols = cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
-                }
-                g.err = s->err;
-                g.done = nullptr;
-                t->cols[dir] = std::max(t->cols[dir], g.tmem_cols);
-                const int pi = (int)args.size() - base;
-                args.push_back(g);
-                for (int mt = 0; mt < mtiles; ++mt)
-                    for (int nt = 0; nt < B.ntile; ++nt) items[dir].push_back(make_int4(pi, mt, nt, 0));
-            }
-        }
-        if (dir == 0) t->n_prob_f = (int)args.size();
-    }
-    if (cudaMemcpy(t->idx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return false;
-    // the adjoint items index their problems from the adjoint part of the arguments
-    t->n_items_f = (int)items[0].size();
-    t->n_items_a = (int)items[1].size();
-    items[0].insert(items[0].end(), items[1].begin(), items[1].end());
-    if (t->dargs) dev_free(t->dargs);
-    if (t->ditems) dev_free(t->ditems);
-    t->dargs = nullptr;
-    t->ditems = nullptr;
-    if (!talloc(&t->dargs, args.size()) || !talloc(&t->ditems, items[0].size())) return false;
-    cudaMemcpy(t->dargs, args.data(), args.size() * sizeof(GemmArgs), cudaMemcpyHostToDevice);
-    cudaMemcpy(t->ditems, items[0].data(), items[0].size() * sizeof(int4), cudaMemcpyHostToDevice);
-    t->fmt = fmt;
-    return cudaGetLastError() == cudaSuccess;
-}
-
-}  // namespace
-
-void ten_release(ColState *s) {
-    TensorState *t = s->ten;
-    if (!t) return;
-    for (int p = 0; p < 2; ++p)
-        for (Packed *pk : {&t->fwd[p], &t->adj[p]})
-            if (pk->dev) dev_free(pk->dev);
-    for (void *p : {(void *)t->Wd, (void *)t->apk_f, (void *)t->apk_a, (void *)t->c_fwd, (void *)t->c_adj,
-                    (void *)t->idx, (void *)t->dargs, (void *)t->ditems})
-        if (p) dev_free(p);
-    delete t;
-    s->ten = nullptr;
-}
-
-int ten_init(mpi_ffl_handle *h) {
-    ColState *s = cs(h);
-    if (!s || !s->ok || !fold_w_dev(h)) return MPI_FFL_ERR_UNSUPPORTED;
-    const Dims &d = h->d;
-    const int R = 2 * d.nb;
-    ten_release(s);
-    TensorState *t = new TensorState();
-    s->ten = t;
-    t->Np = (d.N + kBK - 1) / kBK * kBK;
-    t->Op = (R + kBK - 1) / kBK * kBK;
-    t->step = s->n_par;
-    t->M8 = (d.M + 7) / 8 * 8;
-    t->J = std::max(1, std::min(kBM / t->M8, (d.Nz + t->step - 1) / t->step));
-    t->P0 = t->step * (t->J - 1);
-    t->Tpre = t->step * (t->J - 1);
-    t->Zp = (d.Nz + 2 * t->P0 + t->step - 1) / t->step * t->step;
-    // the accumulation in TMEM is not round-to-nearest, so its error grows with the MMAs
-    // chained into one accumulator: K is split into parts of at most kTenSplitK, summed
-    // in FP32 afterwards (in a fixed order)
-    const int span = d.Nz + t->step * (t->J - 1);
-    for (int dir = 0; dir < 2; ++dir) {
-        const int K = span * (dir ? t->Op : t->Np);
-        t->nsplit[dir] = (K + kTenSplitK - 1) / kTenSplitK;
-        t->ksplit[dir] = ((K + t->nsplit[dir] - 1) / t->nsplit[dir] + kBK - 1) / kBK * kBK;
-        t->nsplit[dir] = (K + t->ksplit[dir] - 1) / t->ksplit[dir];
-    }
-    const size_t ng = ten_groups(d, t->step, t->J).size();
-    // split A: 2 KB per (8 angles, K chunk); a tf32 chunk holds 32 values, a bf16 one 64
-    const size_t blocks_f = (size_t)(t->M8 / 8) * (t->Zp * t->Np / (kBK / 2));
-    const size_t blocks_a = (size_t)(t->M8 / 8) * (t->Zp * t->Op / (kBK / 2));
-    bool ok = talloc(&t->apk_f, blocks_f * 2048) && talloc(&t->apk_a, blocks_a * 2048) &&
-              talloc(&t->c_fwd, (size_t)t->nsplit[0] * d.M * d.Nz * R) &&
-              talloc(&t->c_adj, (size_t)t->nsplit[1] * d.M * d.Nz * d.N) &&
-              talloc(&t->idx, ng * 2 * 2 * (size_t)t->M8 * t->J);
-    ok = ok && ten_build_wd(h, s, t) && ten_prepare(h, s, t, h->precision == MPI_FFL_PREC_TF32 ? 1 : 0);
-    if (!ok) {
-        ten_release(s);
-        cudaGetLastError();
-        return MPI_FFL_ERR_OOM;
-    }
-    cudaFuncSetAttribute(k_gemm_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    return MPI_FFL_OK;
-}
-
-bool ten_ready(const mpi_ffl_handle *h) {
-    const ColState *s = cs(h);
-    return s && s->ten;
-}
-
-int ten_refresh(mpi_ffl_handle *h, bool psf_changed) {
-    ColState *s = cs(h);
-    if (!s || !s->ten) return MPI_FFL_OK;
-    TensorState *t = s->ten;
-    const int fmt = h->precision == MPI_FFL_PREC_TF32 ? 1 : 0;
-    if (psf_changed) {
-        if (!ten_build_wd(h, s, t)) return MPI_FFL_ERR_CUDA;
-        t->fmt = -1;
-    }
-    if (t->fmt != fmt && !ten_prepare(h, s, t, fmt)) return MPI_FFL_ERR_OOM;
-    return MPI_FFL_OK;
-}
-
-void ten_pack(TensorState *t, const float *in, const float *coil, int M, int Nz, int ncols, int per, int dir,
-              cudaStream_t st) {
-    const long long total = (long long)(t->M8 / 8) * t->cm[dir] * 64;
-    const int blocks = (int)std::min<long long>((total + 255) / 256, 152LL * 16);
-    k_pack_rows<<<std::max(1, blocks), 256, 0, st>>>(in, coil, M, Nz, ncols, per, t->P0, t->Zp, t->cm[dir], t->fmt,
-                                                    dir ? t->apk_a : t->apk_f);
-}
-
-// proj -> data: coil-weighted, padded A rows split once; the GEMM problems; sum of the K splits
-void ten_forward(mpi_ffl_handle *h, const float *proj, const float *coil, float *data, cudaStream_t st) {
-    ColState *s = cs(h);
-    TensorState *t = s->ten;
-    const Dims &d = h->d;
-    const long long rows = (long long)d.M * d.Nz;
-    ten_pack(t, proj, coil, d.M, d.Nz, d.N, t->Np, 0, st);
-    // one block per item (each holds up to 512 TMEM columns, one block per SM)
-    k_gemm_batch<<<t->n_items_f, kGemmThreads, t->smem[0] + 16, st>>>(t->dargs, t->ditems, t->n_items_f, t->cols[0],
-                                                                      (uint32_t)t->smem[0]);
-    launch_coil_pad(t->c_fwd, nullptr, data, rows, d.Nz, 2 * d.nb, 2 * d.nb, st, t->nsplit[0], rows * 2 * d.nb);
-}
-
-// data -> proj: padded data rows; the GEMM problems; sum of the K splits, coil weighting
-void ten_adjoint(mpi_ffl_handle *h, const float *data, const float *coil, float *proj, cudaStream_t st) {
-    ColState *s = cs(h);
-    TensorState *t = s->ten;
-    const Dims &d = h->d;
-    const long long rows = (long long)d.M * d.Nz;
-    ten_pack(t, data, nullptr, d.M, d.Nz, 2 * d.nb, t->Op, 1, st);
-    k_gemm_batch<<<t->n_items_a, kGemmThreads, t->smem[1] + 16, st>>>(t->dargs + t->n_prob_f, t->ditems + t->n_items_f,
-                                                                      t->n_items_a, t->cols[1], (uint32_t)t->smem[1]);
-    launch_coil_pad(t->c_adj, coil, proj, rows, d.Nz, d.N, d.N, st, t->nsplit[1], rows * d.N);
 }
 
 }  // namespace mpiffl

@@ -35,13 +35,11 @@ void col_batch_launch(const void *dargs, const int4 *ditems, int n_items, size_t
                       cudaStream_t st);
 void col_batch_init();
 
-// Slice-coupled operator of the tensor PSF (Appendix B, Eq. (31)): per-offset folded
-// line operators W_par H_d stacked by offset, one GEMM per line (forward) or per slice
-// (adjoint). ten_init builds the tables (FP64 fold, then split operands for the
-// handle's precision); ten_refresh rebuilds them after a PSF or precision change.
+// Slice-coupled operator of the tensor PSF (Appendix B, Eq. (31); k_tensor.cu): ten_init
+// builds its tables for the handle's PSF width, ten_ready says whether they are there.
 int ten_init(mpi_ffl_handle *h);
 bool ten_ready(const mpi_ffl_handle *h);
-int ten_refresh(mpi_ffl_handle *h, bool psf_changed);
+void ten_release(mpi_ffl_handle *h);
 void ten_forward(mpi_ffl_handle *h, const float *proj, const float *coil, float *data, cudaStream_t st);
 void ten_adjoint(mpi_ffl_handle *h, const float *data, const float *coil, float *proj, cudaStream_t st);
 

@@ -364,7 +364,7 @@ class FFLOperator:
     def set_psf_model(self, model):
         """PSF model of the x-drive operator: 'collinear' (1D L' along the drive axis, per
         line) or 'tensor' (the in-plane tensor PSF of Appendix B, Eq. (31): every line reads
-        every slice). Selecting 'tensor' builds its per-offset operator on the device."""
+        every slice). Selecting 'tensor' builds its per-frequency operator on the device."""
         if isinstance(model, str):
             model = _lib.PSF_MODELS[model]
         check(self._lib.mpi_ffl_set_psf_model(self._h, int(model)), self._h)

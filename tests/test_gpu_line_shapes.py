@@ -133,3 +133,63 @@ def test_interleaved_projector_on_ragged_detectors(nx, nz, off):
     vol.copy_(torch.from_numpy(x))
     assert rel_l2(_n(op.project(vol)), projection.project(x, st.angles)) < OP_TOL
     op.close()
+
+
+# the tensor PSF by frequencies along z: each tile height of the batched products (rows twice
+# the angles), odd and even slice counts, both trajectories and one, odd rows of bins
+TENSOR = {
+    "two slices": dict(nx=21, nz=2, n_angles=3, S=16, P=40, k_max=3, half_width=1),
+    "odd slices, 20 rows": dict(nx=18, nz=129, n_angles=10, S=20, P=40, k_max=8, half_width=3),
+    "40 rows": dict(nx=16, nz=128, n_angles=20, S=20, P=40, k_max=8, half_width=3),
+    "56 rows, one trajectory": dict(nx=17, nz=130, n_angles=28, zigzag=0, S=40, P=40, k_max=18, half_width=3),
+    "64 rows": dict(nx=16, nz=121, n_angles=31, S=20, P=40, k_max=8, half_width=3),
+    "72 rows": dict(nx=33, nz=128, n_angles=36, S=20, P=40, k_max=8, half_width=3),
+}
+
+
+@pytest.mark.parametrize("name", list(TENSOR))
+def test_tensor_psf_by_frequencies(name):
+    from oracle import tensor_psf
+
+    st, op = _make(**TENSOR[name])
+    op.set_path("full_gemm")
+    op.set_psf_model("tensor")
+    rng = np.random.default_rng(9)
+    gains = np.linspace(0.9, 1.1, st.n_angles)
+    op.set_gain(gains.astype(np.float32))
+    coil = rng.uniform(0.5, 1.5, (st.nz, st.nx)).astype(np.float32)
+    x = rng.standard_normal((st.nz, st.nx, st.nx)).astype(np.float32)
+    m = np.array([st.n_angles - 1])
+    y = np.zeros(st.data_shape, dtype=np.complex64)
+    y[m] = rng.standard_normal(y[m].shape) + 1j * rng.standard_normal(y[m].shape)
+    for c in (None, coil):
+        op.set_coil_map(c)
+        ref = tensor_psf.forward_stages(x, st, c, angles=m)["data"][0] * gains[m[0]]
+        assert rel_l2(_n(op.forward(_t(x)))[m[0]], to_interleaved(ref)) < OP_TOL
+        buf = torch.zeros(2 * y.size + 4, device="cuda")  # data that do not start on 16 bytes
+        yt = buf[1:1 + 2 * y.size].view(op.data_shape)
+        yt.copy_(_t(to_interleaved(y)))
+        ref = tensor_psf.adjoint_stages(y[m], st, c, angles=m)["vol"] * gains[m[0]]
+        assert rel_l2(_n(op.adjoint(yt)), ref) < OP_TOL
+    op.close()
+
+
+def test_tensor_tables_follow_a_width_set_under_the_other_model():
+    """The tables of the width in force, also when it was set while the collinear PSF was
+    selected or the path changed meanwhile."""
+    from oracle import tensor_psf
+
+    kw = dict(nx=20, nz=6, n_angles=3, S=16, P=40, k_max=3, half_width=1)
+    _, op = _make(**kw)
+    op.set_path("line_gemm")
+    op.set_psf_model("tensor")
+    op.set_psf_model("collinear")
+    op.set_fwhm(3.5)
+    op.set_psf_model("tensor")
+    st, _ = _make(**dict(kw, fwhm=3.5))
+    x = np.random.default_rng(10).standard_normal((st.nz, st.nx, st.nx)).astype(np.float32)
+    ref = to_interleaved(tensor_psf.forward(x, st))
+    assert rel_l2(_n(op.forward(_t(x))), ref) < OP_TOL
+    op.set_path("full_gemm")
+    assert rel_l2(_n(op.forward(_t(x))), ref) < OP_TOL
+    op.close()
