@@ -33,23 +33,27 @@ void fold_release(mpi_ffl_handle *h);
 // (arow, crow, acol and ccol may be NULL: row i, column k or n; scale NULL: 1). B is K x
 // ldb, ldb a multiple of 4, on 16 bytes; its rows hold bcols values that may be read (a
 // multiple of 4; 0: ldb). nbatch: that many such products, their operands sA, sB (a
-// multiple of 4) and sC values apart.
+// multiple of 4) and sC values apart. half > 0: two products E and O of half values of k
+// each, O's in columns ahalf (a multiple of 4) and rows bhalf further on; E + O goes to
+// column n, E - O to column c1 + n, or c1 - n when mirror is set (no acol and ccol, one batch).
 struct SgemmArgs {
-    const float *A;
-    int64_t lda;
-    const int *arow;
-    int M, K;
-    const float *B;
-    int ldb;
-    float *C;
-    int64_t ldc;
-    const int *crow;
-    int N;
-    const float *scale;
-    int rdiv;
-    const int *acol, *ccol;
+    const float *A = nullptr;
+    int64_t lda = 0;
+    const int *arow = nullptr;
+    int M = 0, K = 0;
+    const float *B = nullptr;
+    int ldb = 0;
+    float *C = nullptr;
+    int64_t ldc = 0;
+    const int *crow = nullptr;
+    int N = 0;
+    const float *scale = nullptr;
+    int rdiv = 1;
+    const int *acol = nullptr, *ccol = nullptr;
     int nbatch = 1, bcols = 0;
     int64_t sA = 0, sB = 0, sC = 0;
+    int half = 0, ahalf = 0, bhalf = 0, c1 = 0;
+    bool mirror = false;
 };
 constexpr int kSgemmMax = 9;  // problems of one launch
 void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st);

@@ -13,6 +13,12 @@
 // middle one a convolution along z per phase; neither the time signal, nor the fine z grid,
 // nor a transposed projection is formed. The tables are rounded once from FP64. The
 // adjoint runs the transposed steps in the opposite order.
+//
+// A reversed line passes the columns from the other end: K_1[u] = K_0[N - 1 - u]. With zig-zag
+// the products by K therefore split into an even and an odd one of half the columns each,
+//     G_{0,1} = K_e p_e +- K_o p_o,  K_{e,o}[u] = (K_0[u] +- K_0[N - 1 - u]) / 2,
+//     p_{e,o}[u] = p[u] +- p[N - 1 - u], u < N / 2 (the middle column of an odd N in e),
+// which is half the FMAs; the adjoint's convolution writes G_0 + G_1 and G_0 - G_1.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -27,8 +33,9 @@ namespace mpiffl {
 namespace {
 
 struct ZFold {
-    float *kf = nullptr;   // K, B operand of the forward [N][ldk], columns (par, c, r)
-    float *ka = nullptr;   // K, B operand of the adjoint [n_par W S][ldu]
+    // K as the B operand of the forward, [N][ldk] with columns (par, c, r), and of the adjoint,
+    // [n_par W S][ldu]; halved: [e, o][Nh][W S] and [e, o][W S][ldu], Nh = (N + 1) / 2
+    float *kf = nullptr, *ka = nullptr;
     float *hz = nullptr;   // [2 N_z - 1][S]
     float *df = nullptr;   // DFT operands of the forward, per d [S or 2 S][2 or 4 K]
     float *da = nullptr;   // and of the adjoint (their transposes)
@@ -36,6 +43,7 @@ struct ZFold {
     float *g = nullptr;    // [M][N_z][n_par][W][S]
     float *t = nullptr;    // [M][N_z][W][S]
     float *part = nullptr; // [parts of K][M][N_z][N], sums of the adjoint's last product
+    float *eo = nullptr;   // [M][N_z][e, o][ldu] of the projections (halved)
     int ldk = 0, ldu = 0;
     bool ready = false;
 };
@@ -56,10 +64,10 @@ bool zalloc(T **p, size_t n) {
 // One thread per (par, c, r) walks the periods in the order of increasing column, keeps the
 // sums of the two columns the sample lies between and writes a column once it is complete.
 // The slow position c = (N - 1) j / (L - 1) (from the other end on reversed lines) is exact.
-__global__ void __launch_bounds__(128) k_zfold_k(const double2 *__restrict__ unit_p, float *__restrict__ kf,
-                                                 float *__restrict__ ka, Dims d, int ldk, int ldu) {
+__global__ void __launch_bounds__(128) k_zfold_k(const double2 *__restrict__ unit_p, double *__restrict__ K, Dims d,
+                                                 int nk) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= d.n_par * d.W * d.S) return;
+    if (n >= nk) return;
     const int r = n % d.S, c = n / d.S % d.W, par = n / (d.S * d.W);
     const int dd = (c + 1) / 2;
     const bool sine = c > 0 && c % 2 == 0;
@@ -67,10 +75,7 @@ __global__ void __launch_bounds__(128) k_zfold_k(const double2 *__restrict__ uni
     double acc0 = 0.0, acc1 = 0.0;
     int u = 0;
     auto flush = [&]() {
-        if (u < d.N) {
-            kf[(size_t)u * ldk + n] = (float)acc0;
-            ka[(size_t)n * ldu + u] = (float)acc0;
-        }
+        if (u < d.N) K[(size_t)u * nk + n] = acc0;
         acc0 = acc1;
         acc1 = 0.0;
         ++u;
@@ -88,6 +93,41 @@ __global__ void __launch_bounds__(128) k_zfold_k(const double2 *__restrict__ uni
         acc1 = fma(a, tw, acc1);
     }
     while (u < d.N) flush();
+}
+
+// FP32 operands of K [N][nk]
+__global__ void __launch_bounds__(256) k_zfold_operands(const double *__restrict__ K, float *__restrict__ kf,
+                                                        float *__restrict__ ka, int N, int nk, int ldk, int ldu,
+                                                        bool halved) {
+    const int rows = halved ? 2 * ((N + 1) / 2) : N;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < rows * nk; t += gridDim.x * blockDim.x) {
+        const int n = t % nk, row = t / nk;
+        if (!halved) {
+            const float v = (float)K[t];
+            kf[(size_t)row * ldk + n] = v;
+            ka[(size_t)n * ldu + row] = v;
+            continue;
+        }
+        const int Nh = rows / 2, o = row / Nh, u = row - o * Nh, um = N - 1 - u;
+        const double a = K[(size_t)u * nk + n], b = K[(size_t)um * nk + n];
+        const float v = (float)(u == um ? (o ? 0.0 : a) : 0.5 * (o ? a - b : a + b));
+        kf[(size_t)row * ldk + n] = v;
+        ka[((size_t)o * nk + n) * ldu + u] = v;
+    }
+}
+
+// eo[row][e, o][u] = p[u] +- p[N - 1 - u], u < Nh; bound by L2
+__global__ void __launch_bounds__(256) k_zfold_eo(const float *__restrict__ p, float *__restrict__ eo, int rows, int N,
+                                                  int ld) {
+    const int Nh = (N + 1) / 2, total = rows * Nh;
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        const int row = t / Nh, u = t - row * Nh, um = N - 1 - u;
+        const float a = p[(size_t)row * N + u], b = p[(size_t)row * N + um];
+        eo[(size_t)row * 2 * ld + u] = u == um ? a : a + b;
+        eo[(size_t)row * 2 * ld + ld + u] = u == um ? 0.f : a - b;
+    }
 }
 
 // hz[k][r]: taps h at offset k voxels of the fine cells n0_r and n0_r + 1, interpolated, times v_r
@@ -238,15 +278,15 @@ __global__ void __launch_bounds__(128) k_zconv(const float *__restrict__ in, con
 // stages, and NG groups of S threads take R outputs each from it, so an input is read from
 // L2 once for NG R outputs. The new taps are loaded a stage ahead. The sums of a thread go
 // through fma.rn.f32x2 in pairs of values c; the taps are kept as pairs of equal halves.
-// 55 us each way at 256^2 x 128 and 36 angles (the plain form above: 153 us with 8 outputs a
+// 55 us forward at 256^2 x 128 and 36 angles, 67 us back in halves (the plain form above: 153 us with 8 outputs a
 // thread, 75 us with 16); FMA-bound would be 18 us, the rest is the shared loads and moves of
 // a thread with only R W FMAs an input.
-constexpr int kZcIn = 4, kZcStages = 4, kZcAhead = kZcStages - 2;
+constexpr int kZcIn = 4, kZcStages = 4, kZcAhead = kZcStages - 2, kZcR = 8;
 
 template <int W, int R, int NG, bool ADJ>
 __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restrict__ in,
                                                          const float *__restrict__ hz, float *__restrict__ out,
-                                                         int Nz, int S, int np, int *err) {
+                                                         int Nz, int S, int np, bool halves, int *err) {
     extern __shared__ __align__(128) float zring[];  // kZcStages x kZcIn x W S
     __shared__ uint64_t full[kZcStages], empty[kZcStages];
     const int Sp = (S + 31) & ~31;
@@ -257,7 +297,7 @@ __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restr
     const int q = b % np;
     b /= np;
     int par = q;
-    if (ADJ) {
+    if (ADJ && !halves) {
         par = b % np;
         b /= np;
     }
@@ -276,9 +316,10 @@ __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restr
     const size_t WS = (size_t)W * S;
     const size_t istride = ADJ ? WS : np * WS;
     const float *src = in + (size_t)m * Nz * istride + (ADJ ? 0 : par * WS);
-    // inputs in order: the classes modulo np one after another (adjoint: the class par);
-    // a stage holds inputs of one class
-    const int ncls = ADJ ? 1 : min(np, Nz), cls0 = ADJ ? par : 0;
+    // inputs in order: the classes modulo np one after another (adjoint: the class par alone,
+    // or both for halves); a stage holds inputs of one class
+    const bool one = ADJ && !halves;
+    const int ncls = one ? 1 : min(np, Nz), cls0 = one ? par : 0;
     const int cnt0 = (Nz - cls0 + np - 1) / np, st0 = (cnt0 + kZcIn - 1) / kZcIn;
     const int cnt1 = ncls > 1 ? (Nz - 1 + np - 1) / np : 0, nst = st0 + (cnt1 + kZcIn - 1) / kZcIn;
     auto issue = [&](int s) {
@@ -306,10 +347,30 @@ __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restr
 #pragma unroll
         for (int c = 0; c < WP; ++c) acc[i][c] = 0;
     }
+    // a thread's W values of output i: f(value index, sum)
+    auto each = [&](int i, auto f) {
+#pragma unroll
+        for (int p = 0; p < WP; ++p) {
+            const float2 a = unpack2(acc[i][p]);
+            f(2 * p, a.x);
+            f(2 * p + 1, a.y);
+        }
+        f(W - 1, acl[i]);
+    };
+    auto at = [&](int i) { return out + ((size_t)m * Nz + o0 + np * i) * (ADJ ? np * WS : WS) + (one ? par * WS : 0) + r; };
     bool good = true;
     int s = 0;
     for (int ci = 0; ci < ncls; ++ci) {
         const int c = ci ? 1 : cls0, cnt = ci ? cnt1 : cnt0;
+        if (ADJ && ci == 1) {  // the sums of trajectory 0 wait in their place of the output
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                if (r < S && o0 + np * i < Nz) each(i, [&](int v, float x) { at(i)[(size_t)v * S] = x; });
+                acl[i] = 0.f;
+#pragma unroll
+                for (int p = 0; p < WP; ++p) acc[i][p] = 0;
+            }
+        }
         f32x2 w[R];  // taps of the outputs at the current input
         float nt[kZcIn];
 #pragma unroll
@@ -371,32 +432,48 @@ __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restr
     if (r >= S) return;
 #pragma unroll
     for (int i = 0; i < R; ++i) {
-        const int o = o0 + np * i;
-        if (o >= Nz) break;
-        float *dst = out + ((size_t)m * Nz + o) * (ADJ ? np * WS : WS) + (ADJ ? par * WS : 0) + r;
-#pragma unroll
-        for (int p = 0; p < WP; ++p) {
-            const float2 a = unpack2(acc[i][p]);
-            dst[(size_t)(2 * p) * S] = a.x;
-            dst[(size_t)(2 * p + 1) * S] = a.y;
-        }
-        dst[(size_t)(W - 1) * S] = acl[i];
+        if (o0 + np * i >= Nz) break;
+        float *dst = at(i);
+        each(i, [&](int v, float x) {
+            float *w = dst + (size_t)v * S;
+            if (ADJ && halves) {  // G_0 + G_1 and G_0 - G_1
+                const float g0 = ncls == 2 ? *w : x, g1 = ncls == 2 ? x : 0.f;
+                w[0] = g0 + g1;
+                w[WS] = g0 - g1;
+            } else {
+                *w = x;
+            }
+        });
     }
+}
+
+bool zconv_streams(const Dims &d) { return d.S % 4 == 0 && d.S <= 128; }
+
+// The even and odd halves of the products by K, where the convolution can write them and a
+// half's rows start on 16 bytes; rounding errors grow with the length of a sum, so that halves
+// stay within a run of the products (320). The adjoint's convolution then takes both
+// trajectories in one thread, so that its threads must fill the GPU (12 warps an SM): at 256^2
+// x 128 and 36 angles (73728 threads) a pair takes 522 us in halves and 575 us whole, at 156^2
+// x 83 and 35 angles (26880) 205 and 192 us.
+bool halved(const Dims &d) {
+    const int64_t threads = (int64_t)d.M * d.n_par * ((d.Nz / 2 + kZcR - 1) / kZcR) * ((d.S + 31) / 32 * 32);
+    return d.n_par == 2 && zconv_streams(d) && d.N <= 640 && threads >= 12 * 32 * 128;
 }
 
 template <int W, bool ADJ>
 void zconv_w(const float *in, const float *hz, float *out, const Dims &d, int *err, cudaStream_t st) {
-    constexpr int R = 8;
+    constexpr int R = kZcR;
     const int np = d.n_par, nl = (d.Nz + np - 1) / np;
-    const int outer = d.M * (ADJ ? np : 1) * np;
     const size_t smem = sizeof(float) * kZcStages * kZcIn * W * d.S;
-    if (d.S % 4 == 0 && d.S <= 128) {
+    if (zconv_streams(d)) {
+        const bool hv = halved(d);
+        const int outer = d.M * (ADJ && !hv ? np : 1) * np;
         // as many groups a block (4, or 2 where the sums of wide bands need the registers) as
         // leave a block for every SM
         auto go = [&](auto kernel, int NG) {
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             launch_dependent(kernel, dim3(outer * ((nl + R * NG - 1) / (R * NG))), dim3((d.S + 31) / 32 * 32 * NG),
-                             smem, st, in, hz, out, d.Nz, d.S, np, err);
+                             smem, st, in, hz, out, d.Nz, d.S, np, hv, err);
         };
         auto blocks = [&](int NG) { return outer * ((nl + R * NG - 1) / (R * NG)); };
         if (W <= 9 && blocks(4) >= 128) go(k_zconv_ring<W, R, W <= 9 ? 4 : 2, ADJ>, 4);
@@ -405,7 +482,7 @@ void zconv_w(const float *in, const float *hz, float *out, const Dims &d, int *e
         return;
     }
     const int threads = std::min(128, (d.S + 31) / 32 * 32), ny = (d.S + threads - 1) / threads;
-    launch_dependent(k_zconv<W, R, ADJ>, dim3(outer * ((nl + R - 1) / R), ny), dim3(threads), 0, st, in, hz, out, d.Nz,
+    launch_dependent(k_zconv<W, R, ADJ>, dim3(d.M * (ADJ ? np : 1) * np * ((nl + R - 1) / R), ny), dim3(threads), 0, st, in, hz, out, d.Nz,
                      d.S, np);
 }
 
@@ -428,15 +505,26 @@ size_t g_len(const Dims &d) { return (size_t)d.M * d.Nz * d.n_par * d.W * d.S; }
 size_t dft_f_len(const Dims &d) { return DftOperand(d, d.hw + 1).off_f; }
 size_t dft_a_len(const Dims &d) { return DftOperand(d, d.hw + 1).off_a; }
 
-// K of one part of the adjoint's last product: whole runs of 256, at most kSgemmMax parts,
-// about four blocks an SM
+// K of one part of the adjoint's last product, at most kSgemmMax parts: halved, of each half
+// and at most 320, parts that make one wave of the products' blocks (3 an SM); else whole runs
+// of 256 and about four blocks an SM
 int z_kper(const Dims &d) {
-    const int nk = d.n_par * d.W * d.S;
+    const int nk = (halved(d) ? 1 : d.n_par) * d.W * d.S;
     SgemmArgs a{};
     a.M = d.M * d.Nz;
-    a.N = d.N;
-    const int want = std::max(1, std::min(kSgemmMax, 600 / std::max(1, sgemm_tiles(a)) + 1));
+    a.N = halved(d) ? (d.N + 1) / 2 : d.N;
+    const int tiles = std::max(1, sgemm_tiles(a));
+    if (halved(d)) {
+        const int want = std::max(1, std::min(kSgemmMax, 3 * 152 / tiles));
+        return std::min(320, ((nk + want - 1) / want + 15) / 16 * 16);
+    }
+    const int want = std::max(1, std::min(kSgemmMax, 600 / tiles + 1));
     return std::max(256, ((nk + want - 1) / want + 255) / 256 * 256);
+}
+
+int z_parts(const Dims &d) {
+    const int nk = (halved(d) ? 1 : d.n_par) * d.W * d.S;
+    return (nk + z_kper(d) - 1) / z_kper(d);
 }
 
 bool fold_h(mpi_ffl_handle *h) {
@@ -481,29 +569,35 @@ int zfold_ready(mpi_ffl_handle *h) {
     ZFold *s = zs(h);
     if (s->ready) return MPI_FFL_OK;
     const Dims &d = h->d;
-    const int nk = d.n_par * d.W * d.S;
+    const bool hv = halved(d);
+    const int nk = (hv ? 1 : d.n_par) * d.W * d.S, Nh = (d.N + 1) / 2;
     s->ldk = (nk + 3) / 4 * 4;
-    s->ldu = (d.N + 3) / 4 * 4;
+    s->ldu = ((hv ? Nh : d.N) + 3) / 4 * 4;
+    const size_t kf_len = (size_t)(hv ? 2 * Nh : d.N) * s->ldk, ka_len = (size_t)(hv ? 2 : 1) * nk * s->ldu;
     double2 *unit_p = nullptr;
-    bool ok = zalloc(&s->kf, (size_t)d.N * s->ldk) && zalloc(&s->ka, (size_t)nk * s->ldu) &&
+    double *K = nullptr;
+    bool ok = zalloc(&s->kf, kf_len) && zalloc(&s->ka, ka_len) && zalloc(&K, (size_t)d.N * nk) &&
+              (!hv || zalloc(&s->eo, (size_t)d.M * d.Nz * 2 * s->ldu)) &&
               zalloc(&s->hz, (size_t)(2 * d.Nz - 1) * d.S) && zalloc(&s->df, dft_f_len(d)) &&
               zalloc(&s->da, dft_a_len(d)) && zalloc(&s->cols, (size_t)2 * d.nb) && zalloc(&s->g, g_len(d)) &&
               zalloc(&s->t, (size_t)d.M * d.Nz * d.W * d.S) && zalloc(&unit_p, d.P) &&
-              zalloc(&s->part, (size_t)((nk + z_kper(d) - 1) / z_kper(d)) * d.M * d.Nz * d.N);
+              zalloc(&s->part, (size_t)z_parts(d) * d.M * d.Nz * d.N);
     if (ok) {
         const double kPi = 3.14159265358979323846;
         std::vector<double2> up(d.P);
         for (int p = 0; p < d.P; ++p) up[p] = make_double2(std::cos(2.0 * kPi * p / d.P), std::sin(2.0 * kPi * p / d.P));
         cudaMemcpy(unit_p, up.data(), up.size() * sizeof(double2), cudaMemcpyHostToDevice);
-        cudaMemset(s->kf, 0, (size_t)d.N * s->ldk * sizeof(float));  // the columns past the last
-        cudaMemset(s->ka, 0, (size_t)nk * s->ldu * sizeof(float));
+        cudaMemset(s->kf, 0, kf_len * sizeof(float));  // the columns past the last
+        cudaMemset(s->ka, 0, ka_len * sizeof(float));
         cudaMemset(s->df, 0, dft_f_len(d) * sizeof(float));
         cudaMemset(s->da, 0, dft_a_len(d) * sizeof(float));
-        k_zfold_k<<<(nk + 127) / 128, 128>>>(unit_p, s->kf, s->ka, d, s->ldk, s->ldu);
+        k_zfold_k<<<(nk + 127) / 128, 128>>>(unit_p, K, d, nk);
+        k_zfold_operands<<<608, 256>>>(K, s->kf, s->ka, d.N, nk, s->ldk, s->ldu, hv);
         k_zfold_dft<<<dim3(64, d.hw + 1), 128>>>(h->t_dgam, s->df, s->da, s->cols, d);
         ok = fold_h(h);
     }
     if (unit_p) dev_free(unit_p);
+    if (K) dev_free(K);
     if (!ok) {  // nothing of a failed build is kept
         zfold_release(h);
         return MPI_FFL_ERR_OOM;
@@ -544,9 +638,31 @@ void dft_products(const mpi_ffl_handle *h, bool adjoint, const float *in, float 
 void zfold_forward(mpi_ffl_handle *h, const float *proj, float *data, cudaStream_t st) {
     const Dims &d = h->d;
     const ZFold *s = zs(h);
-    const int nk = d.n_par * d.W * d.S;
-    const SgemmArgs k{proj, d.N, nullptr, d.M * d.Nz, d.N, s->kf, s->ldk, s->g, nk, nullptr, nk, nullptr, 1, nullptr,
-                      nullptr};
+    const int rows = d.M * d.Nz, nk = d.W * d.S;
+    SgemmArgs k{};
+    k.M = rows;
+    k.B = s->kf;
+    k.ldb = s->ldk;
+    k.C = s->g;
+    k.ldc = d.n_par * nk;
+    k.rdiv = 1;
+    if (halved(d)) {
+        const int Nh = (d.N + 1) / 2;
+        launch_dependent(k_zfold_eo, dim3(std::min(608, (rows * Nh + 255) / 256)), dim3(256), 0, st, proj, s->eo, rows,
+                         d.N, s->ldu);
+        k.A = s->eo;
+        k.lda = 2 * s->ldu;
+        k.N = nk;
+        k.half = Nh;
+        k.ahalf = s->ldu;
+        k.bhalf = Nh;
+        k.c1 = nk;
+    } else {
+        k.A = proj;
+        k.lda = d.N;
+        k.K = d.N;
+        k.N = d.n_par * nk;
+    }
     launch_sgemm(&k, 1, st);
     zconv<false>(s->g, s->hz, s->t, d, h->w_err, st);
     dft_products(h, false, s->t, data, st);
@@ -555,18 +671,36 @@ void zfold_forward(mpi_ffl_handle *h, const float *proj, float *data, cudaStream
 void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream_t st) {
     const Dims &d = h->d;
     const ZFold *s = zs(h);
-    const int nk = d.n_par * d.W * d.S;
+    const bool hv = halved(d);
+    const int nk = (hv ? 1 : d.n_par) * d.W * d.S;
     dft_products(h, true, data, s->t, st);
     zconv<true>(s->t, s->hz, s->g, d, h->w_err, st);
     // K is long (n_par W S): split over as many problems as fill the GPU, each into its own
     // sums, which are added in a fixed order
     SgemmArgs g[kSgemmMax];
-    const int kper = z_kper(d), np = (nk + kper - 1) / kper;
+    const int kper = z_kper(d), np = z_parts(d);
     const int64_t rows = (int64_t)d.M * d.Nz;
-    for (int i = 0; i < np; ++i)
-        g[i] = SgemmArgs{s->g + (size_t)i * kper, nk, nullptr, (int)rows, std::min(kper, nk - i * kper),
-                         s->ka + (size_t)i * kper * s->ldu, s->ldu, np > 1 ? s->part + i * rows * d.N : proj, d.N,
-                         nullptr, d.N, nullptr, 1, nullptr, nullptr};
+    for (int i = 0; i < np; ++i) {
+        const int K = std::min(kper, nk - i * kper);
+        g[i].A = s->g + (size_t)i * kper;
+        g[i].lda = d.n_par * d.W * d.S;
+        g[i].M = (int)rows;
+        g[i].B = s->ka + (size_t)i * kper * s->ldu;
+        g[i].ldb = s->ldu;
+        g[i].C = np > 1 ? s->part + i * rows * d.N : proj;
+        g[i].ldc = d.N;
+        g[i].rdiv = 1;
+        if (hv) {
+            g[i].N = (d.N + 1) / 2;
+            g[i].half = K;
+            g[i].ahalf = g[i].bhalf = nk;
+            g[i].c1 = d.N - 1;
+            g[i].mirror = true;
+        } else {
+            g[i].N = d.N;
+            g[i].K = K;
+        }
+    }
     launch_sgemm(g, np, st);
     if (np > 1) launch_coil_pad(s->part, nullptr, proj, rows, d.Nz, d.N, d.N, st, np, rows * d.N);
 }
@@ -575,7 +709,7 @@ void zfold_release(mpi_ffl_handle *h) {
     ZFold *s = zs(h);
     if (!s) return;
     for (void *p : {(void *)s->kf, (void *)s->ka, (void *)s->hz, (void *)s->df, (void *)s->da, (void *)s->cols,
-                    (void *)s->g, (void *)s->t, (void *)s->part})
+                    (void *)s->g, (void *)s->t, (void *)s->part, (void *)s->eo})
         if (p) dev_free(p);
     delete s;
     h->zfold_state = nullptr;

@@ -3,7 +3,7 @@
 // Bound by the FP32 pipes and by shared-memory loads together: a thread keeps TM x TN sums
 // and reads TM + TN shared values per k, A four k at a time. The sums go two columns at a
 // time through fma.rn.f32x2, which leaves half the issue slots to the loads and to the
-// duplication of the A values. Both operands come through a ring of kSgStages stages filled
+// duplication of the A values. Both operands come through a ring of four stages filled
 // by cp.async, so that a stage's latency (about a microsecond) is spread over three.
 #include <algorithm>
 
@@ -15,7 +15,9 @@ namespace mpiffl {
 
 namespace {
 
-constexpr int kSgK = 16, kSgStages = 4;
+constexpr int kSgK = 16;
+// stages of the ring: three where sums wait in shared memory, so that three blocks fit an SM
+__host__ __device__ constexpr int sg_stages(int mode) { return mode ? 3 : 4; }
 constexpr int kSgRow = kSgK + 4;  // floats of a staged A row: 8 rows start in distinct bank groups
 
 // 16 bytes global -> shared, the last 16 - n of them zero
@@ -48,24 +50,25 @@ constexpr int kSgRun = 320;
 // 16-byte shared load takes two cycles where neighbouring lanes share the address (the A
 // loads here), four where they do not (B). KG: groups of threads that take their share of
 // each stage's K and add their sums at the end (more warps for products with few tiles).
-// RUNS: K above kSgRun, the runs' sums are added in shared memory.
+// MODE 1: K above kSgRun, the runs' sums are added in shared memory. MODE 2: two products of
+// half values of k each; the first one's sums wait there for the second's.
 __host__ __device__ constexpr int sgemm_stage_floats(int BM, int BN) { return BM * kSgRow + kSgK * BN; }
-__host__ __device__ constexpr int sgemm_ring_floats(int BM, int BN, int join) {
-    const int ring = kSgStages * sgemm_stage_floats(BM, BN);
+__host__ __device__ constexpr int sgemm_ring_floats(int BM, int BN, int join, int stages) {
+    const int ring = stages * sgemm_stage_floats(BM, BN);
     return ring > join ? ring : join;
 }
 
-template <int BM, int BN, int TM, int TN, int KG, bool RUNS>
+template <int BM, int BN, int TM, int TN, int KG, int MODE>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) * (BN / TN) * KG))
     k_sgemm(const __grid_constant__ SgemmBatch batch) {
     constexpr int TG = (BM / TM) * (BN / TN), T = TG * KG;
     constexpr int NA = (BM * kSgK / 4 + T - 1) / T, NB = (BN * kSgK / 4 + T - 1) / T;
     constexpr int KS = kSgK / KG;
-    constexpr int kStage = sgemm_stage_floats(BM, BN);
+    constexpr int kStage = sgemm_stage_floats(BM, BN), kSgStages = sg_stages(MODE);
     static_assert(BM / TM == 8 && TN % 4 == 0 && TG % 32 == 0 && KS % 4 == 0, "warp layout");
-    // the ring (the groups' sums take its place at the end), then RUNS: float2 [TM][TN / 2][T]
+    // the ring (the groups' sums take its place at the end), then MODE > 0: float2 [TM][TN / 2][T]
     extern __shared__ __align__(16) float smf[];
-    float2 *sum = reinterpret_cast<float2 *>(smf + sgemm_ring_floats(BM, BN, (KG - 1) * TG * TM * TN));
+    float2 *sum = reinterpret_cast<float2 *>(smf + sgemm_ring_floats(BM, BN, (KG - 1) * TG * TM * TN, kSgStages));
     int pi = 0;
     while ((int)blockIdx.x >= batch.first[pi + 1]) ++pi;  // uniform
     const SgemmArgs &g = batch.g[pi];
@@ -90,9 +93,12 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
         ap[u] = gA + (size_t)(g.arow ? __ldg(g.arow + r) : r) * g.lda;
     }
     const bool vec = !g.acol && g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(gA) & 15) == 0;
+    const int Kv = MODE == 2 ? g.half : g.K, th = (Kv + kSgK - 1) / kSgK;  // values and stages of a product
     auto copy_a = [&](int t) {
         float *st = smf + (t % kSgStages) * kStage + (tid / (kSgK / 4)) * kSgRow + ka;
-        const int k = t * kSgK + ka, n = min(4, max(0, g.K - k)), ks = min(k, (g.K - 1) & ~3);
+        const bool second = MODE == 2 && t >= th;
+        const int k = (second ? t - th : t) * kSgK + ka, n = min(4, max(0, Kv - k));
+        const int ks = min(k, (Kv - 1) & ~3) + (second ? g.ahalf : 0);
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
             if ((BM * kSgK / 4) % T && tid + u * T >= BM * kSgK / 4) break;
@@ -102,8 +108,9 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
             } else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const bool in = k + e < g.K;
-                    cp_async4(dst + e, in ? ap[u] + (g.acol ? __ldg(g.acol + k + e) : k + e) : gA, in ? 4 : 0);
+                    const bool in = k + e < Kv;
+                    cp_async4(dst + e, in ? ap[u] + (MODE == 2 ? ks + e : g.acol ? __ldg(g.acol + k + e) : k + e) : gA,
+                              in ? 4 : 0);
                 }
             }
         }
@@ -111,14 +118,16 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
     // of B: columns cb of the rows tid / (BN / 4) + u T / (BN / 4)
     const int cb = c0 + 4 * (tid % (BN / 4)), kb0 = tid / (BN / 4);
     const float *bp = gB + min(cb, bcols - 4);
-    const int kvalid = cb < bcols ? g.K : 0;
+    const int kvalid = cb < bcols ? Kv : 0;
     auto copy_b = [&](int t) {
         float *st = smf + (t % kSgStages) * kStage + BM * kSgRow + 4 * tid;
+        const bool second = MODE == 2 && t >= th;
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
             if ((BN * kSgK / 4) % T && tid + u * T >= BN * kSgK / 4) break;
-            const int kk = t * kSgK + kb0 + u * (T / (BN / 4));
-            cp_async16(st + 4 * u * T, bp + (int64_t)min(kk, g.K - 1) * g.ldb, kk < kvalid ? 16 : 0);
+            const int kk = (second ? t - th : t) * kSgK + kb0 + u * (T / (BN / 4));
+            cp_async16(st + 4 * u * T, bp + (int64_t)(min(kk, Kv - 1) + (second ? g.bhalf : 0)) * g.ldb,
+                       kk < kvalid ? 16 : 0);
         }
     };
 
@@ -128,7 +137,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
     for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0;
-    const int nk = (g.K + kSgK - 1) / kSgK;
+    const int nk = MODE == 2 ? 2 * th : th;
     ptx::grid_dep_wait();  // A comes from the previous kernel
     ptx::grid_dep_launch();
 #pragma unroll
@@ -172,7 +181,15 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
                 }
             }
         }
-        if (RUNS && ((t + 1) % (kSgRun * KG / kSgK) == 0 || t + 1 == nk)) {  // a thread's own words
+        if (MODE == 2 && t + 1 == th)  // a thread's own words
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN / 2; ++j) {
+                    sum[(i * (TN / 2) + j) * T + tid] = unpack2(acc[i][j]);
+                    acc[i][j] = 0;
+                }
+        if (MODE == 1 && ((t + 1) % (kSgRun * KG / kSgK) == 0 || t + 1 == nk)) {  // a thread's own words
             const bool first = t < kSgRun * KG / kSgK;
 #pragma unroll
             for (int i = 0; i < TM; ++i)
@@ -186,6 +203,16 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
                 }
         }
     }
+    if (MODE == 2)  // E - O in its place in shared memory, E + O in registers
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < TN / 2; ++j) {
+                float2 &w = sum[(i * (TN / 2) + j) * T + tid];
+                const float2 o = unpack2(acc[i][j]), e = w;
+                w = make_float2(e.x - o.x, e.y - o.y);
+                acc[i][j] = pack2(e.x + o.x, e.y + o.y);
+            }
     if (KG > 1) {  // group 0 adds the other groups' sums in their order
         __syncthreads();
         float2 *join = reinterpret_cast<float2 *>(smf);
@@ -226,6 +253,28 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
                 for (int q = 0; q < 4; ++q)
                     if (c + q < g.N) dst[g.ccol ? __ldg(g.ccol + c + q) : c + q] = e[q];
             }
+            if (MODE == 2) {
+                float d[4];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    float2 w = sum[(i * (TN / 2) + 2 * j + q) * T + tid];
+                    for (int k = 1; k < KG; ++k) {
+                        const float2 v = sum[(i * (TN / 2) + 2 * j + q) * T + k * TG + tid];
+                        w = make_float2(w.x + v.x, w.y + v.y);
+                    }
+                    d[2 * q] = sc * w.x;
+                    d[2 * q + 1] = sc * w.y;
+                }
+                const int c1 = g.mirror ? g.c1 - c - 3 : g.c1 + c;
+                if (vecc && c + 4 <= g.N && c1 % 4 == 0) {
+                    *reinterpret_cast<float4 *>(dst + c1) =
+                        g.mirror ? make_float4(d[3], d[2], d[1], d[0]) : make_float4(d[0], d[1], d[2], d[3]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (c + q < g.N) dst[g.mirror ? g.c1 - c - q : c1 + q] = d[q];
+                }
+            }
         }
     }
 }
@@ -236,17 +285,19 @@ template <int BM, int BN, int TM, int TN, int KG>
 void run(const SgemmArgs *g, int n, cudaStream_t st) {
     constexpr int T = (BM / TM) * (BN / TN) * KG;
     SgemmBatch b{};
-    bool runs = false;
+    bool runs = false;  // of the products of one launch: all halved or none
     for (int i = 0; i < kSgemmMax; ++i) {
         const int tiles = i < n ? (g[i].M + BM - 1) / BM * ((g[i].N + BN - 1) / BN) : 0;
         if (i < n) b.g[i] = g[i];
-        if (i < n && g[i].K > kSgRun * KG) runs = true;
+        if (i < n && (g[i].half > 0 || g[i].K > kSgRun * KG)) runs = true;
         b.first[i + 1] = b.first[i] + tiles * batches(g, i, n);
     }
     const int total = b.first[kSgemmMax];
     if (total == 0) return;
-    const size_t smem = sizeof(float) * (sgemm_ring_floats(BM, BN, (KG - 1) * T / KG * TM * TN) + (runs ? TM * TN * T : 0));
-    auto kernel = runs ? k_sgemm<BM, BN, TM, TN, KG, true> : k_sgemm<BM, BN, TM, TN, KG, false>;
+    const size_t smem = sizeof(float) * (sgemm_ring_floats(BM, BN, (KG - 1) * T / KG * TM * TN, sg_stages(runs)) + (runs ? TM * TN * T : 0));
+    auto kernel = runs ? k_sgemm<BM, BN, TM, TN, KG, 1> : k_sgemm<BM, BN, TM, TN, KG, 0>;
+    if constexpr (TM == 4 || KG == 1)
+        if (g[0].half > 0) kernel = k_sgemm<BM, BN, TM, TN, KG, 2>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     launch_dependent(kernel, dim3(total), dim3(T), smem, st, b);
 }
@@ -255,10 +306,12 @@ void run(const SgemmArgs *g, int n, cudaStream_t st) {
 
 int sgemm_tiles(const SgemmArgs &g) { return (g.M + 63) / 64 * ((g.N + 127) / 128); }
 
-// 8 x 8 sums a thread (the fewest shared loads an FMA) where such tiles come to four blocks
-// an SM: 4608 x 2304 x 256 in 106 us, 68% of the FP32 FMA rate (4 x 8 sums in 32 x 64 tiles
-// and two groups along K: 129 us). Smaller products take the smaller tiles: 4608 x 288 x 256
-// in 22 us (29 us with the large tiles), 1536 x 168 x 128 in 5.5 us (11 us).
+// 8 x 8 sums a thread (the fewest shared loads an FMA) where such tiles come to almost a wave
+// of three blocks an SM: 4608 x 2304 x 256 in 106 us, 68% of the FP32 FMA rate (4 x 8 sums in
+// 32 x 64 tiles and two groups along K: 129 us). Smaller products take the smaller tiles:
+// 4608 x 288 x 256 in 22 us (29 us with the large tiles), 1536 x 168 x 128 in 5.5 us (11 us).
+// Of the large tiles those of 56 rows where their waves are shorter: two halves of 4608 x 1152
+// x 128 in 59 us (two waves of 64 rows, the second a third full: 67 us).
 //
 // Batches of products with few rows each (one per frequency or angle) take tiles of 64 columns
 // whose height fits the rows: the least padding, a tile's loads of B counted as 24 rows. 127
@@ -266,9 +319,11 @@ int sgemm_tiles(const SgemmArgs &g) { return (g.M + 63) / 64 * ((g.N + 127) / 12
 // in three of 32 and 110 in two of 64. Where that leaves an SM without its three blocks, the
 // smallest tiles: 72 of 64 x 288 x 256 in 23 us (25 us in tiles of 64 rows).
 void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st) {
-    int big = 0, rows = 0;
+    constexpr int kWave = 3 * 152;
+    int n64 = 0, n56 = 0, rows = 0;
     for (int i = 0; i < n; ++i) {
-        big += sgemm_tiles(g[i]);
+        n64 += sgemm_tiles(g[i]);
+        n56 += (g[i].M + 55) / 56 * ((g[i].N + 127) / 128);
         if (g[i].nbatch != 1) rows = std::max(rows, g[i].M);
     }
     int height = 0;
@@ -278,13 +333,15 @@ void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st) {
         int64_t tiles = 0;
         for (int i = 0; i < n; ++i)
             tiles += (int64_t)g[i].nbatch * ((g[i].M + height - 1) / height) * ((g[i].N + 63) / 64);
-        if (tiles < 3 * 152) height = 32;
+        if (tiles < kWave) height = 32;
     }
     if (height == 40) run<40, 64, 5, 8, 2>(g, n, st);
     else if (height == 56) run<56, 64, 7, 8, 2>(g, n, st);
     else if (height == 64) run<64, 64, 8, 8, 2>(g, n, st);
     else if (height == 72) run<72, 64, 9, 8, 2>(g, n, st);
-    else if (height == 0 && big >= 600) run<64, 128, 8, 8, 1>(g, n, st);
+    else if (height == 0 && n64 >= 400 && (n56 + kWave - 1) / kWave * 56 < (n64 + kWave - 1) / kWave * 64)
+        run<56, 128, 7, 8, 1>(g, n, st);
+    else if (height == 0 && n64 >= 400) run<64, 128, 8, 8, 1>(g, n, st);
     else run<32, 64, 4, 8, 2>(g, n, st);
 }
 

@@ -95,6 +95,11 @@ ZDRIVE = {
     "sixteen lines": dict(nx=24, nz=67, n_angles=60, S=16, P=40, k_max=3, half_width=1),
     "many phases": dict(nx=16, nz=5, n_angles=2, S=140, P=20, k_max=7, half_width=0),
     "sampled": dict(nx=40, nz=8, n_angles=3, S=32, P=6, k_max=5, half_width=1),
+    # the products by K in halves of the columns (scans that fill the GPU): odd and not a
+    # multiple of four, odd slices, no harmonic offsets; and the large tiles of both products
+    "odd columns in halves": dict(nx=23, nz=95, n_angles=64, S=64, P=30, k_max=5, half_width=1),
+    "66 columns": dict(nx=66, nz=96, n_angles=64, S=60, P=70, k_max=6, half_width=0),
+    "large halves": dict(nx=19, nz=112, n_angles=60, S=128, P=20, k_max=5, half_width=3),
 }
 
 
