@@ -22,7 +22,7 @@ from .operator import FFLOperator
 class _ApplyA(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, gains, fwhm, op):
-        g, w = gains.detach().reshape(-1), fwhm.detach().reshape(-1)[:1]
+        g, w = gains.detach().reshape(-1), fwhm.detach().reshape(-1)[0].reshape(1)  # no width: IndexError
         if g.device == w.device and g.dtype == w.dtype:  # one wait for both
             host = torch.cat((g, w)).tolist()
         else:
