@@ -12,6 +12,8 @@
 //       b[k, d] = L^-1/2 sum_r e^{2 pi i (kP+d) r / L} sum_p s[pS+r] e^{2 pi i d p / P},
 //       exactly equal to Eq. (27) on the kept bins. The inner sum over periods
 //       costs 2w+1 FMAs per sample (the signal is real); the outer one is small.
+#include <algorithm>
+
 #include "f32x2.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
@@ -33,9 +35,23 @@ constexpr int kPsfTF = 9;
 // sixteen outputs per lane in the transpose: 16 FMA pairs per pair of shared loads
 constexpr int kPsfTA = 16;
 static_assert(kPsfTF <= kPsfT && kPsfTA <= kPsfT, "the tap table is padded for the windows");
+// Few lines (less than a warp of tasks a scheduler): the time is one thread's chain of packed
+// FMAs, so threads take fewer outputs, and a line's tasks are spread over blocks of one row
+// of the grid (blockIdx.y), four warps of them each. The sums and their order are the same.
+// Pairs of the line-GEMM path: 110 lines of 184 bins 142 -> 126 us (one line a thread: 133 us),
+// 297 lines of 48 bins 67 -> 64 us (66 us).
+constexpr int kPsfTFew = 5, kPsfTAFew = 8;
+constexpr int kPsfSMs = 152;
+
+// Blocks that share the tasks of one block's lines: gx blocks with `warps` warps of tasks each
+static int psf_split(int gx, int warps) {
+    return gx < kPsfSMs ? std::min((warps + 3) / 4, (2 * kPsfSMs + gx - 1) / gx) : 1;
+}
+static bool psf_few(int gx, int warps) { return (long long)gx * warps < 4 * kPsfSMs; }
 
 // FP32-bound: 2.5 GFMA at 256^2 x 128 and 36 angles in 121 us (144 us one line at a
 // time), of 67 us at the FMA rate.
+template <int T>
 __global__ void __launch_bounds__(256) k_psf_fwd(const float *__restrict__ proj,
                                                  const float *__restrict__ htab,
                                                  float *__restrict__ fine, Dims d) {
@@ -50,32 +66,34 @@ __global__ void __launch_bounds__(256) k_psf_fwd(const float *__restrict__ proj,
     __syncthreads();
     const int Q = d.Q;
     const int n_a = (d.Ne + Q - 1) / Q;               // fine points per phase (upper bound)
-    const int n_ab = (n_a + kPsfTF - 1) / kPsfTF;       // register blocks per phase
-    for (int task = threadIdx.x; task < Q * n_ab; task += blockDim.x) {
+    const int n_ab = (n_a + T - 1) / T;       // register blocks per phase
+    const int share = ((Q * n_ab + 31) / 32 + gridDim.y - 1) / gridDim.y * 32;  // tasks of this block
+    const int end = min(Q * n_ab, (int)(blockIdx.y + 1) * share);
+    for (int task = blockIdx.y * share + threadIdx.x; task < end; task += blockDim.x) {
         const int q = task % Q;
         const int ab = task / Q;
-        const int base = q - d.D + d.htab_off + Q * ab * kPsfTF;
-        f32x2 w[kPsfTF], acc[kPsfTF];
+        const int base = q - d.D + d.htab_off + Q * ab * T;
+        f32x2 w[T], acc[T];
 #pragma unroll
-        for (int t = 0; t < kPsfTF; ++t) {
+        for (int t = 0; t < T; ++t) {
             w[t] = dup2(sh[base + Q * t]);
             acc[t] = 0;
         }
         // unrolled by the window length, so that the window's shift is a renaming of
         // registers rather than moves
-#pragma unroll kPsfTF
+#pragma unroll T
         for (int i = 0; i < d.N; ++i) {
             const f32x2 pi = sp[i];
 #pragma unroll
-            for (int t = 0; t < kPsfTF; ++t) acc[t] = fma2(pi, w[t], acc[t]);
+            for (int t = 0; t < T; ++t) acc[t] = fma2(pi, w[t], acc[t]);
 #pragma unroll
-            for (int t = kPsfTF - 1; t > 0; --t) w[t] = w[t - 1];
+            for (int t = T - 1; t > 0; --t) w[t] = w[t - 1];
             w[0] = dup2(sh[base - Q * (i + 1)]);
         }
         float *out = fine + (size_t)seg * d.Ne;
 #pragma unroll
-        for (int t = 0; t < kPsfTF; ++t) {
-            const int e = q + Q * (ab * kPsfTF + t);
+        for (int t = 0; t < T; ++t) {
+            const int e = q + Q * (ab * T + t);
             const float2 v = unpack2(acc[t]);
             if (e < d.Ne) out[e] = v.x;
             if (e < d.Ne && two) out[d.Ne + e] = v.y;
@@ -83,11 +101,20 @@ __global__ void __launch_bounds__(256) k_psf_fwd(const float *__restrict__ proj,
     }
 }
 
-void launch_psf_fwd(const float *proj, const float *htab, float *fine, const Dims &d, cudaStream_t st) {
+template <int T>
+static void run_psf_fwd(const float *proj, const float *htab, float *fine, const Dims &d, int warps, cudaStream_t st) {
     const size_t smem = sizeof(float) * (2 * d.N + d.htab_len);
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_psf_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    k_psf_fwd<<<(d.nseg + 1) / 2, 256, smem, st>>>(proj, htab, fine, d);
+        cudaFuncSetAttribute(k_psf_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    const int gx = (d.nseg + 1) / 2;
+    k_psf_fwd<T><<<dim3(gx, psf_split(gx, warps)), 256, smem, st>>>(proj, htab, fine, d);
+}
+
+void launch_psf_fwd(const float *proj, const float *htab, float *fine, const Dims &d, cudaStream_t st) {
+    const int n_a = (d.Ne + d.Q - 1) / d.Q;
+    auto warps = [&](int t) { return (d.Q * ((n_a + t - 1) / t) + 31) / 32; };
+    if (psf_few((d.nseg + 1) / 2, warps(kPsfTF))) run_psf_fwd<kPsfTFew>(proj, htab, fine, d, warps(kPsfTFew), st);
+    else run_psf_fwd<kPsfTF>(proj, htab, fine, d, warps(kPsfTF), st);
 }
 
 // H^T: proj[i] = sum_e fine[e] h((e - D)/Q - i). Lanes of a warp are
@@ -99,6 +126,7 @@ void launch_psf_fwd(const float *proj, const float *htab, float *fine, const Dim
 // 145 us (149 us one line at a time).
 constexpr int kPsfAdjThreads = 256;
 
+template <int T>
 __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restrict__ fine,
                                                             const float *__restrict__ htab,
                                                             float *__restrict__ proj, Dims d, int row_stride,
@@ -122,36 +150,38 @@ __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restr
     const int nwarps = blockDim.x >> 5;
     const int q = lane % Q;
     const int sl = lane / Q;               // line pair within the block handled by this lane
-    const int n_ib = (d.N + kPsfTA - 1) / kPsfTA;
+    const int n_ib = (d.N + T - 1) / T;
     const bool active = 2 * sl < nsg;
     const f32x2 *row = sf + (active ? sl : 0) * row_stride;
-    for (int ib = warp; ib < n_ib; ib += nwarps) {
-        const int i0 = ib * kPsfTA;
-        f32x2 acc[kPsfTA];
+    const int share = (n_ib + gridDim.y - 1) / gridDim.y;  // warp tasks of this block
+    const int end = min(n_ib, (int)(blockIdx.y + 1) * share);
+    for (int ib = blockIdx.y * share + warp; ib < end; ib += nwarps) {
+        const int i0 = ib * T;
+        f32x2 acc[T];
 #pragma unroll
-        for (int t = 0; t < kPsfTA; ++t) acc[t] = 0;
+        for (int t = 0; t < T; ++t) acc[t] = 0;
         const int baseq = q - d.D - Q * i0 + d.htab_off;
-        f32x2 w[kPsfTA];
+        f32x2 w[T];
 #pragma unroll
-        for (int t = 0; t < kPsfTA; ++t) w[t] = dup2(sh[baseq - Q * t]);
-#pragma unroll kPsfTA
+        for (int t = 0; t < T; ++t) w[t] = dup2(sh[baseq - Q * t]);
+#pragma unroll T
         for (int a = 0, e = q; e < d.Ne; ++a, e += Q) {
             const f32x2 c = row[e];
 #pragma unroll
-            for (int t = 0; t < kPsfTA; ++t) acc[t] = fma2(c, w[t], acc[t]);
+            for (int t = 0; t < T; ++t) acc[t] = fma2(c, w[t], acc[t]);
 #pragma unroll
-            for (int t = kPsfTA - 1; t > 0; --t) w[t] = w[t - 1];
+            for (int t = T - 1; t > 0; --t) w[t] = w[t - 1];
             w[0] = dup2(sh[baseq + Q * (a + 1)]);
         }
         // add the Q phase partials (lanes sl*Q .. sl*Q+Q-1)
 #pragma unroll
-        for (int t = 0; t < kPsfTA; ++t)
+        for (int t = 0; t < T; ++t)
             for (int o = 1; o < Q; o <<= 1) acc[t] = add2(acc[t], __shfl_xor_sync(0xffffffffu, acc[t], o));
         if (active && q == 0) {
             float *out = proj + (size_t)(seg0 + 2 * sl) * d.N;
             const bool two = 2 * sl + 1 < nsg;
 #pragma unroll
-            for (int t = 0; t < kPsfTA; ++t) {
+            for (int t = 0; t < T; ++t) {
                 const float2 v = unpack2(acc[t]);
                 if (i0 + t < d.N) out[i0 + t] = v.x;
                 if (i0 + t < d.N && two) out[d.N + i0 + t] = v.y;
@@ -161,17 +191,27 @@ __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restr
 }
 
 // Line pairs of a block: 32 / Q of them fill a warp's lanes; fewer where the rows of so many do
-// not fit the shared memory beside the taps.
-void launch_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, cudaStream_t st) {
+// not fit the shared memory beside the taps, at most two where the lines are few.
+template <int T>
+static void run_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, int pairs, cudaStream_t st) {
     // lanes = (line pair, phase); Q must be a power of two dividing 32 for the shuffle tree
     const int stride = d.Ne + (((d.Q - d.Ne) % 16) + 16) % 16;  // stride = Q (mod 16)
-    int pairs = 32 / d.Q;
     auto bytes = [&](int p) { return sizeof(float) * (d.htab_len + 2 * (size_t)p * stride); };
     while (pairs > 1 && bytes(pairs) > 227 * 1024) pairs /= 2;
     const size_t smem = bytes(pairs);
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_psf_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    k_psf_adj<<<(d.nseg + 2 * pairs - 1) / (2 * pairs), kPsfAdjThreads, smem, st>>>(fine, htab, proj, d, stride, pairs);
+        cudaFuncSetAttribute(k_psf_adj<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    const int gx = (d.nseg + 2 * pairs - 1) / (2 * pairs);
+    k_psf_adj<T><<<dim3(gx, psf_split(gx, (d.N + T - 1) / T)), kPsfAdjThreads, smem, st>>>(fine, htab, proj, d, stride,
+                                                                                          pairs);
+}
+
+void launch_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, cudaStream_t st) {
+    const int pairs = 32 / d.Q;
+    if (psf_few((d.nseg + 2 * pairs - 1) / (2 * pairs), (d.N + kPsfTA - 1) / kPsfTA))
+        run_psf_adj<kPsfTAFew>(fine, htab, proj, d, std::min(pairs, 2), st);
+    else
+        run_psf_adj<kPsfTA>(fine, htab, proj, d, pairs, st);
 }
 
 // ----------------------------------------------------------------------------- E V B

@@ -198,3 +198,17 @@ def test_tensor_tables_follow_a_width_set_under_the_other_model():
     op.set_path("full_gemm")
     assert rel_l2(_n(op.forward(_t(x))), ref) < OP_TOL
     op.close()
+
+
+@pytest.mark.parametrize("nx,nz,M", [(20, 5, 1), (184, 10, 11), (64, 16, 21), (184, 16, 14), (300, 16, 20)])
+def test_psf_stage_of_few_lines(nx, nz, M):
+    """H and its transpose where a line's outputs are spread over several blocks, with the small
+    and the large register tiles, odd numbers of lines and of blocks of outputs."""
+    st, op = _make(nx=nx, nz=nz, n_angles=M, S=12, P=20, Q=8)
+    h = operator.psf.h((np.arange(st.n_fine)[:, None] - st.D) / st.Q - np.arange(nx)[None, :], st.fwhm)
+    rng = np.random.default_rng(11)
+    p = rng.standard_normal((M, nz, nx)).astype(np.float32)
+    assert rel_l2(_n(op.apply_stage(1, _t(p))), p @ h.T) < OP_TOL
+    f = rng.standard_normal((M, nz, st.n_fine)).astype(np.float32)
+    assert rel_l2(_n(op.apply_stage(1, _t(f), transpose=True)), f @ h) < OP_TOL
+    op.close()
