@@ -190,7 +190,9 @@ int mpi_ffl_get_path(const mpi_ffl_handle *h);
 /* Replace the per-angle gains (host array of n_angles) or the PSF width. Both take
  * effect for work enqueued after the call returns; the call synchronises the device
  * before touching tables that queued work may still read. A new PSF width also
- * rebuilds the collapsed line operator (W H), which takes a moment on the host. */
+ * rebuilds the operators that the PSF is folded into. After any error of set_psf_fwhm but
+ * MPI_FFL_ERR_INVALID_ARG the width is the new one everywhere, and the handle fell back to
+ * the staged path or the collinear PSF if the selected one could not be rebuilt. */
 int mpi_ffl_set_gain(mpi_ffl_handle *h, const float *gain);
 int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm_vox);
 

@@ -1230,23 +1230,25 @@ extern "C" int mpi_ffl_set_gain(mpi_ffl_handle *h, const float *gain) {
     });
 }
 
+// Every table of the width follows it or is marked stale before this returns, whatever fails
+// on the way, so that no two paths or scans of a handle ever hold two widths: apart from an
+// invalid argument, an error means that the width is the new one and that the handle fell back
+// to a path or PSF model whose tables could be built.
 extern "C" int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm) {
     return guarded(h, [&]() {
         if (!(fwhm > 0.0)) {
             h->err = "fwhm must be > 0";
             return MPI_FFL_ERR_INVALID_ARG;
         }
-        h->fwhm = fwhm;
         std::vector<float> ht, dht;
         psf_tables(h->d, fwhm, ht, dht);
         CK(cudaDeviceSynchronize());
+        h->fwhm = fwhm;
         CK(cudaMemcpy(h->t_htab, ht.data(), sizeof(float) * ht.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->t_dhtab, dht.data(), sizeof(float) * dht.size(), cudaMemcpyHostToDevice));
         tc_tables_changed(h);
-        if (fold_psf_changed(h) != MPI_FFL_OK || zfold_psf_changed(h) != MPI_FFL_OK) {
-            h->err = "the folded line operator could not be rebuilt";
-            return MPI_FFL_ERR_CUDA;
-        }
+        fold_psf_changed(h);
+        zfold_psf_changed(h);
         // W H holds the PSF: rebuild the collapsed operator if it was built and the
         // full-GEMM path is selected; otherwise W (which holds no PSF) stays and W H is
         // rebuilt when the full-GEMM path is next selected
@@ -1254,24 +1256,34 @@ extern "C" int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm) {
         if (h->col_state) {
             if (h->path == MPI_FFL_PATH_FULL_GEMM) {
                 col_release(h);
-                col_init(h);
+                try {
+                    col_init(h);
+                } catch (...) {  // a host allocation
+                    col_release(h);
+                }
             } else {
                 col_mark_psf_stale(h);
             }
         }
+        int rc = MPI_FFL_OK;
         if (had && !col_supported(h) && (h->path == MPI_FFL_PATH_LINE_GEMM || h->path == MPI_FFL_PATH_FULL_GEMM)) {
+            col_release(h);  // nothing of a failed build is kept: set_path tries again
             h->path = MPI_FFL_PATH_STAGED;
             h->precision = MPI_FFL_PREC_FP32;
             h->psf_model = MPI_FFL_PSF_COLLINEAR;
             h->err = "collapsed operator could not be rebuilt; fell back to the staged path";
-            return MPI_FFL_ERR_OOM;
+            rc = MPI_FFL_ERR_OOM;
         }
-        if (h->psf_model == MPI_FFL_PSF_TENSOR && ten_init(h) != MPI_FFL_OK) {
-            h->psf_model = MPI_FFL_PSF_COLLINEAR;
-            h->err = "tensor-PSF operator could not be rebuilt; fell back to the collinear PSF";
-            return MPI_FFL_ERR_OOM;
+        if (h->psf_model == MPI_FFL_PSF_TENSOR) {
+            h->psf_model = MPI_FFL_PSF_COLLINEAR;  // unless its tables are built (or a host allocation throws)
+            if (ten_init(h) == MPI_FFL_OK) {
+                h->psf_model = MPI_FFL_PSF_TENSOR;
+            } else {
+                h->err = "tensor-PSF operator could not be rebuilt; fell back to the collinear PSF";
+                rc = MPI_FFL_ERR_OOM;
+            }
         }
-        return MPI_FFL_OK;
+        return rc;
     });
 }
 

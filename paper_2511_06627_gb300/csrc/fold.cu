@@ -24,6 +24,7 @@ struct FoldState {
     // FP32 operands of slot 0 (h) and 1 (d h / d fwhm): B of the forward [n_par][N][ldf]
     // and of the adjoint [n_par][2 n_b][lda]
     float *f[2] = {nullptr, nullptr}, *a[2] = {nullptr, nullptr};
+    bool stale[2] = {false, false};  // of another width: refolded on the next use
     int ldf = 0, lda = 0;
     int *rows = nullptr;  // lines of trajectory 0, then of trajectory 1
     int nrows[2] = {0, 0};
@@ -200,7 +201,9 @@ int refold(mpi_ffl_handle *h, int slot, cudaStream_t st) {
     k_fold_operands<<<dim3(std::min(608, (work + 255) / 256), d.n_par), 256, 0, st>>>(wh, s->f[slot], s->a[slot], R,
                                                                                      d.N, s->ldf, s->lda);
     // another stream may use the operands next, and the host taps may be freed
-    return cudaStreamSynchronize(st) == cudaSuccess ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return MPI_FFL_ERR_CUDA;
+    s->stale[slot] = false;
+    return MPI_FFL_OK;
 }
 
 }  // namespace
@@ -337,7 +340,7 @@ bool fold_fits(const Dims &d) {
 int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
     const Dims &d = h->d;
     FoldState *s = state(h);
-    if (s->f[slot]) return MPI_FFL_OK;
+    if (s->f[slot] && !s->stale[slot]) return MPI_FFL_OK;
     const int R = 2 * d.nb;
     if (!s->rows) {
         std::vector<int> rows;
@@ -388,14 +391,15 @@ void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float
     launch_sgemm(g, d.n_par, st);
 }
 
-int fold_psf_changed(mpi_ffl_handle *h) {
+void fold_psf_changed(mpi_ffl_handle *h) {
     FoldState *s = fs(h);
-    for (int slot = 0; s && slot < 2; ++slot)
-        if (s->f[slot]) {
-            const int rc = refold(h, slot, nullptr);
-            if (rc != MPI_FFL_OK) return rc;
-        }
-    return MPI_FFL_OK;
+    if (!s) return;
+    for (int slot = 0; slot < 2; ++slot) s->stale[slot] = s->f[slot] != nullptr;  // until refold has succeeded
+    try {
+        for (int slot = 0; slot < 2; ++slot)
+            if (s->stale[slot]) refold(h, slot, nullptr);
+    } catch (...) {  // a host allocation
+    }
 }
 
 void fold_release(mpi_ffl_handle *h) {

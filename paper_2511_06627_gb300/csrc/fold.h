@@ -26,7 +26,9 @@ bool fold_fits(const Dims &d);                  // the rule by sizes
 int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st);  // operands built on first use
 void fold_forward(mpi_ffl_handle *h, int slot, const float *proj, const float *gain, float *data, cudaStream_t st);
 void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float *proj, cudaStream_t st);
-int fold_psf_changed(mpi_ffl_handle *h);        // refolds the operands that were built
+// After a new width: refolds the operands that were built. Those it could not refold are
+// left to their next use, which tries again and reports.
+void fold_psf_changed(mpi_ffl_handle *h);
 void fold_release(mpi_ffl_handle *h);
 
 // C[crow[i]][ccol[n]] = scale[arow[i] / rdiv] sum_k A[arow[i]][acol[k]] B[k][n] in FP32
@@ -64,7 +66,7 @@ bool zfold_fits(const Dims &d);                      // the rule by sizes
 int zfold_ready(mpi_ffl_handle *h);                  // tables and workspace, on first use
 void zfold_forward(mpi_ffl_handle *h, const float *proj, float *data, cudaStream_t st);
 void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream_t st);
-int zfold_psf_changed(mpi_ffl_handle *h);
+void zfold_psf_changed(mpi_ffl_handle *h);           // as fold_psf_changed
 void zfold_release(mpi_ffl_handle *h);
 
 }  // namespace mpiffl

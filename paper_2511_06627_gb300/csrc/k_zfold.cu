@@ -45,7 +45,11 @@ struct ZFold {
     float *part = nullptr; // [parts of K][M][N_z][N], sums of the adjoint's last product
     float *eo = nullptr;   // [M][N_z][e, o][ldu] of the projections (halved)
     int ldk = 0, ldu = 0;
+    // inputs of hz, kept so that a new width allocates nothing: FP64 taps, and the drive per phase
+    double *taps = nullptr;
+    double2 *drive = nullptr;
     bool ready = false;
+    bool stale = false;  // hz is of another width: rebuilt on the next use
 };
 
 ZFold *zs(const mpi_ffl_handle *h) { return reinterpret_cast<ZFold *>(h->zfold_state); }
@@ -539,18 +543,14 @@ bool fold_h(mpi_ffl_handle *h) {
         const double ph = 2.0 * kPi * r / d.S + h->phase;
         drive[r] = make_double2(d.Q * h->amp * std::sin(ph) + d.D, h->amp * (2.0 * kPi / d.S) * std::cos(ph));
     }
-    double *dt = nullptr;
-    double2 *dd = nullptr;
-    bool ok = zalloc(&dt, taps.size()) && zalloc(&dd, drive.size());
-    if (ok) {
-        cudaMemcpy(dt, taps.data(), taps.size() * sizeof(double), cudaMemcpyHostToDevice);
-        cudaMemcpy(dd, drive.data(), drive.size() * sizeof(double2), cudaMemcpyHostToDevice);
-        k_zfold_h<<<dim3((d.S + 127) / 128, 2 * d.Nz - 1), 128>>>(dt, dd, zs(h)->hz, d.Nz, d.S, d.Q, d.D);
-        ok = cudaStreamSynchronize(nullptr) == cudaSuccess;
-    }
-    if (dt) dev_free(dt);
-    if (dd) dev_free(dd);
-    return ok;
+    ZFold *s = zs(h);
+    if (!zalloc(&s->taps, taps.size()) || !zalloc(&s->drive, drive.size())) return false;
+    cudaMemcpy(s->taps, taps.data(), taps.size() * sizeof(double), cudaMemcpyHostToDevice);
+    cudaMemcpy(s->drive, drive.data(), drive.size() * sizeof(double2), cudaMemcpyHostToDevice);
+    k_zfold_h<<<dim3((d.S + 127) / 128, 2 * d.Nz - 1), 128>>>(s->taps, s->drive, s->hz, d.Nz, d.S, d.Q, d.D);
+    if (cudaStreamSynchronize(nullptr) != cudaSuccess) return false;
+    s->stale = false;
+    return true;
 }
 
 }  // namespace
@@ -567,7 +567,7 @@ bool zfold_fits(const Dims &d) {
 int zfold_ready(mpi_ffl_handle *h) {
     if (!h->zfold_state) h->zfold_state = new ZFold();
     ZFold *s = zs(h);
-    if (s->ready) return MPI_FFL_OK;
+    if (s->ready) return !s->stale || fold_h(h) ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
     const Dims &d = h->d;
     const bool hv = halved(d);
     const int nk = (hv ? 1 : d.n_par) * d.W * d.S, Nh = (d.N + 1) / 2;
@@ -606,9 +606,14 @@ int zfold_ready(mpi_ffl_handle *h) {
     return MPI_FFL_OK;
 }
 
-int zfold_psf_changed(mpi_ffl_handle *h) {
-    const ZFold *s = zs(h);
-    return !s || !s->ready || fold_h(h) ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
+void zfold_psf_changed(mpi_ffl_handle *h) {
+    ZFold *s = zs(h);
+    if (!s || !s->ready) return;
+    s->stale = true;  // until fold_h has succeeded
+    try {
+        fold_h(h);
+    } catch (...) {  // a host allocation
+    }
 }
 
 namespace {
@@ -709,7 +714,7 @@ void zfold_release(mpi_ffl_handle *h) {
     ZFold *s = zs(h);
     if (!s) return;
     for (void *p : {(void *)s->kf, (void *)s->ka, (void *)s->hz, (void *)s->df, (void *)s->da, (void *)s->cols,
-                    (void *)s->g, (void *)s->t, (void *)s->part, (void *)s->eo})
+                    (void *)s->g, (void *)s->t, (void *)s->part, (void *)s->eo, (void *)s->taps, (void *)s->drive})
         if (p) dev_free(p);
     delete s;
     h->zfold_state = nullptr;

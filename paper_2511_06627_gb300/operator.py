@@ -358,8 +358,10 @@ class FFLOperator:
         self.gains = [float(g) for g in gains]
 
     def set_fwhm(self, fwhm):
-        check(self._lib.mpi_ffl_set_psf_fwhm(self._h, float(fwhm)), self._h)
-        self.fwhm = float(fwhm)
+        rc = self._lib.mpi_ffl_set_psf_fwhm(self._h, float(fwhm))
+        if rc != _lib.ERR_INVALID_ARG:  # any other error: the width is set, the path or model fell back
+            self.fwhm = float(fwhm)
+        check(rc, self._h)
 
     def set_psf_model(self, model):
         """PSF model of the x-drive operator: 'collinear' (1D L' along the drive axis, per
