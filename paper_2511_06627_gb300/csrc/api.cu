@@ -166,6 +166,11 @@ void traj_point_host(const mpi_ffl_handle *h, int par, int j, int &n, double &f,
     if (n > d.Ne - 2) n = d.Ne - 2;
     f = tt - n;
 }
+double z_drive_offset_host(const mpi_ffl_handle *h, int r) {
+    const double ph = 2.0 * 3.14159265358979323846 * r / h->d.S + h->phase;
+    const double t = h->d.Q * h->amp * std::sin(ph) + h->d.D;
+    return std::min(std::max(t, 0.0), 2.0 * h->d.D);
+}
 }  // namespace mpiffl
 
 namespace {
@@ -1378,7 +1383,7 @@ void z_init(mpi_ffl_handle *h) {
     std::vector<float> f0(S), v(S);
     for (int r = 0; r < S; ++r) {
         const double ph = 2.0 * kPi * r / S + h->phase;
-        const double t = Q * h->amp * std::sin(ph) + d.D;
+        const double t = z_drive_offset_host(h, r);
         n0[r] = (int)std::floor(t);
         f0[r] = (float)(t - n0[r]);
         v[r] = (float)(h->amp * (2.0 * kPi / S) * std::cos(ph));

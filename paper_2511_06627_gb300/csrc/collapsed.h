@@ -48,5 +48,9 @@ double langevin_d1_host(double x);
 double langevin_d2_host(double x);
 double langevin_half_point_host();
 void traj_point_host(const mpi_ffl_handle *h, int parity, int j, int &n, double &f, double &v);
+// The drive's offset A sin(phase r) on the fine z grid, Q A sin + D, held to [0, 2 D]: D = ceil(Q A
+// - 1e-9) takes a Q A that rounding left just above a whole number, and the lowest offset is
+// then some 1e-15 below 0, whose cell -1 is before the first tap and the first fine cell.
+double z_drive_offset_host(const mpi_ffl_handle *h, int r);
 
 }  // namespace mpiffl

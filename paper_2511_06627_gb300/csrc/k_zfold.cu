@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(128) k_zfold_h(const double *__restrict__ taps
                                                  float *__restrict__ hz, int Nz, int S, int Q, int D) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;  // offset k - (Nz - 1)
     if (r >= S) return;
-    const double t = drive[r].x;  // Q A sin + D
+    const double t = drive[r].x;  // Q A sin + D, in [0, 2 D]
     const int n0 = (int)floor(t);
     const double f = t - n0;
     const double *h = taps + (size_t)Q * k + n0;  // taps[i] = h((i - D) / Q - (Nz - 1))
@@ -541,7 +541,7 @@ bool fold_h(mpi_ffl_handle *h) {
     std::vector<double2> drive(d.S);
     for (int r = 0; r < d.S; ++r) {
         const double ph = 2.0 * kPi * r / d.S + h->phase;
-        drive[r] = make_double2(d.Q * h->amp * std::sin(ph) + d.D, h->amp * (2.0 * kPi / d.S) * std::cos(ph));
+        drive[r] = make_double2(z_drive_offset_host(h, r), h->amp * (2.0 * kPi / d.S) * std::cos(ph));
     }
     ZFold *s = zs(h);
     if (!zalloc(&s->taps, taps.size()) || !zalloc(&s->drive, drive.size())) return false;

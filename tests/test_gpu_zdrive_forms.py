@@ -1,0 +1,52 @@
+"""Forms of the z-drive scan's tables and kernels beside the ordinary ones."""
+
+import numpy as np
+import pytest
+
+from _helpers import OP_TOL, ensure_library, rel_l2
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import Setup, zdrive  # noqa: E402
+from oracle.data import to_interleaved  # noqa: E402
+
+GEOM = dict(nx=21, nz=9, n_angles=3, S=16, P=30, A=4.0, phi0=0.0, zigzag=1, Q=8, fwhm=2.5, k_min=1, k_max=5,
+            half_width=1)
+FORMS = {"folded": GEOM, "sampled": dict(GEOM, nx=40, nz=8, S=32, P=6)}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    ensure_library()
+
+
+def _t(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+
+def _check(op, st):
+    """A_z and A_z^T of one angle against the oracle."""
+    rng = np.random.default_rng(31)
+    m = np.array([st.n_angles - 1])
+    x = rng.standard_normal((st.nz, st.nx, st.nx)).astype(np.float32)
+    y = np.zeros(st.data_shape, dtype=np.complex64)
+    y[m] = rng.standard_normal(y[m].shape) + 1j * rng.standard_normal(y[m].shape)
+    b = op.forward_zdrive(_t(x)).double().cpu().numpy()
+    xa = op.adjoint_zdrive(_t(to_interleaved(y))).double().cpu().numpy()
+    op.sync_check()
+    assert rel_l2(b[m], to_interleaved(zdrive.forward_stages_z(x, st, angles=m)["data"])) < OP_TOL
+    assert rel_l2(xa, zdrive.adjoint_stages_z(y[m], st, angles=m)["vol"]) < OP_TOL
+
+
+@pytest.mark.parametrize("form", list(FORMS))
+def test_a_drive_amplitude_just_above_whole_fine_cells(form):
+    """Q A = 24 + 4e-15 still has a margin of 24 cells; where the sine is -1 the offset must not
+    fall to the cell below the first one. (The oracle takes A = 3, which differs by 4e-16.)"""
+    from paper_2511_06627_gb300 import FFLOperator
+
+    amp = (0.1 + 0.2) * 10
+    assert 8 * amp > 24 and np.ceil(8 * amp - 1e-9) == 24
+    op = FFLOperator(**dict(FORMS[form], A=amp))
+    _check(op, Setup(**dict(FORMS[form], A=3.0)))
+    op.close()
