@@ -111,6 +111,10 @@ void upload(mpi_ffl_handle *h, T **p, const std::vector<T> &v) {
     CK(cudaMemcpy(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
 }
 
+// Waits for the uploads of this call. A copy from pageable memory may return before its data is
+// in device memory, on the legacy stream, which a caller's non-blocking stream does not wait for.
+void uploads_done(mpi_ffl_handle *h) { CK(cudaStreamSynchronize(nullptr)); }
+
 // ------------------------------------------------------------ Langevin PSF
 // L'(x) = 1/x^2 - 1/sinh(x)^2 (Appendix B, Eq. (31) collinear term), with the
 // Taylor series 1/3 - x^2/15 + 2x^4/189 - x^6/675 for |x| < 0.05.
@@ -632,6 +636,7 @@ void ensure_ra_tables(mpi_ffl_handle *h) {
         upload(h, &h->t_ra_tile, tiles);
         upload(h, &h->t_ra_j, tj);
         upload(h, &h->t_ra_w, tw);
+        uploads_done(h);
         h->ra_ntile = ntile;
         h->ra_cap = cap;
     }
@@ -1184,6 +1189,7 @@ extern "C" int mpi_ffl_set_coil_map(mpi_ffl_handle *h, const float *b_zu) {
         if (!h->t_coil) dev_alloc(h, &h->t_coil, (size_t)d.Nz * d.N);
         if (!h->w_projc) dev_alloc(h, &h->w_projc, (size_t)d.M * d.Nz * d.N);
         CK(cudaMemcpy(h->t_coil, b_zu, sizeof(float) * d.Nz * d.N, cudaMemcpyHostToDevice));
+        uploads_done(h);
         return MPI_FFL_OK;
     });
 }
@@ -1231,6 +1237,7 @@ extern "C" int mpi_ffl_set_gain(mpi_ffl_handle *h, const float *gain) {
         for (int m = 0; m < h->d.M; ++m) h->gains[m] = gain[m];
         CK(cudaDeviceSynchronize());
         CK(cudaMemcpy(h->t_gain, h->gains.data(), sizeof(float) * h->d.M, cudaMemcpyHostToDevice));
+        uploads_done(h);
         return MPI_FFL_OK;
     });
 }
@@ -1251,6 +1258,7 @@ extern "C" int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm) {
         h->fwhm = fwhm;
         CK(cudaMemcpy(h->t_htab, ht.data(), sizeof(float) * ht.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->t_dhtab, dht.data(), sizeof(float) * dht.size(), cudaMemcpyHostToDevice));
+        uploads_done(h);
         tc_tables_changed(h);
         fold_psf_changed(h);
         zfold_psf_changed(h);
@@ -1438,6 +1446,7 @@ void z_init(mpi_ffl_handle *h) {
     upload(h, &h->tz_phi, phi);
     upload(h, &h->tz_tap_ptr, ptr);
     upload(h, &h->tz_taps, taps);
+    uploads_done(h);
     h->z_ready = 1;
 }
 
@@ -1703,7 +1712,10 @@ extern "C" int mpi_ffl_band_energy(mpi_ffl_handle *h, const float *d_x, double *
         const Dims &d = h->d;
         cudaStream_t st = S(stream);
         ensure_sig(h);
-        if (!h->t_dgam_unit) upload(h, &h->t_dgam_unit, std::vector<float2>(d.nb, make_float2(1.f, 0.f)));
+        if (!h->t_dgam_unit) {
+            upload(h, &h->t_dgam_unit, std::vector<float2>(d.nb, make_float2(1.f, 0.f)));
+            uploads_done(h);
+        }
         // s = E V B H P x on the staged kernels (FP32), then its energy and its kept bins
         stage_p(h, d_x, h->w_proj, st);
         TIMED(MPI_FFL_K_PSF_FWD, launch_psf_fwd(h->w_proj, h->t_htab, h->w_fine, d, st));

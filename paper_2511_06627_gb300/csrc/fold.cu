@@ -32,6 +32,14 @@ struct FoldState {
 
 FoldState *fs(const mpi_ffl_handle *h) { return reinterpret_cast<FoldState *>(h->fold_state); }
 
+// Host data to device memory, there when this returns: a copy from pageable memory may return
+// before, on the legacy stream, which the caller's non-blocking stream does not wait for.
+template <class T>
+bool fupload(T *p, const std::vector<T> &v) {
+    return cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice) == cudaSuccess &&
+           cudaStreamSynchronize(nullptr) == cudaSuccess;
+}
+
 template <class T>
 bool falloc(T **p, size_t n) {
     if (*p) return true;
@@ -265,9 +273,10 @@ int fold_w(mpi_ffl_handle *h) {
     if ((size_t)2 * d.nb * d.Ne <= kHostW) {
         const std::vector<double> W = w_host(h);
         if (!falloc(&s->W, W.size())) return MPI_FFL_ERR_OOM;
-        return cudaMemcpy(s->W, W.data(), W.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess
-                   ? MPI_FFL_OK
-                   : MPI_FFL_ERR_CUDA;
+        if (fupload(s->W, W)) return MPI_FFL_OK;
+        dev_free(s->W);  // not filled: the next call builds it
+        s->W = nullptr;
+        return MPI_FFL_ERR_CUDA;
     }
     double *drive = nullptr, *vel = nullptr, *W = nullptr;
     double2 *unit_s = nullptr;
@@ -350,7 +359,11 @@ int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
             s->nrows[par] = (int)rows.size() - (par ? s->nrows[0] : 0);
         }
         if (!falloc(&s->rows, rows.size())) return MPI_FFL_ERR_OOM;
-        cudaMemcpy(s->rows, rows.data(), rows.size() * sizeof(int), cudaMemcpyHostToDevice);
+        if (!fupload(s->rows, rows)) {
+            dev_free(s->rows);
+            s->rows = nullptr;
+            return MPI_FFL_ERR_CUDA;
+        }
     }
     s->ldf = (R + 3) / 4 * 4;
     s->lda = (d.N + 3) / 4 * 4;
