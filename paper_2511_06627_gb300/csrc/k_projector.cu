@@ -489,6 +489,11 @@ __device__ __forceinline__ void project_il_body(const CUtensorMap *map_row, cons
         const int gi = s0 / kPGroup, u = gi % kPSlots;
         // the warp gives up as one, so that its later votes and shuffles see all lanes
         if (!__all_sync(0xffffffffu, ptx::mbar_wait_bounded(&bars[u], (gi / kPSlots) & 1, 1u << 24))) {
+            // the groups that may have been issued land before the block's shared memory is given
+            // up or, in a batch, set up for the next item
+            if ((tid & 31) == 0)
+                for (int q = gi; q < gi + kPSlots && q * kPGroup < N; ++q)
+                    ptx::mbar_wait_bounded(&bars[q % kPSlots], (q / kPSlots) & 1, 1u << 24);
             good = false;
             break;
         }

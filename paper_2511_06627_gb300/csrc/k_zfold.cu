@@ -335,8 +335,9 @@ __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restr
             ptx::bulk_g2s(zring + (size_t)(k * kZcIn + e) * WS, src + (size_t)(c + np * (u + e)) * istride,
                           (uint32_t)WS * 4u, &full[k]);
     };
+    int issued = 0;  // stages thread 0 has issued
     if (tid == 0)
-        for (int s = 0; s < min(nst, kZcAhead); ++s) issue(s);
+        for (; issued < min(nst, kZcAhead); ++issued) issue(issued);
     const int r = tid % Sp, re = min(r, S - 1);
     const int o0 = q + np * R * (grp * NG + tid / Sp);
     const bool work = o0 < Nz;  // a group past the last output only waits and arrives
@@ -395,6 +396,7 @@ __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restr
                 } else {
                     ptx::fence_proxy_async_smem();  // the stage's generic reads, then its refill
                     issue(sn);
+                    issued = sn + 1;
                 }
             }
             __syncwarp();
@@ -431,6 +433,11 @@ __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restr
     }
     if (!good) {
         if (lane == 0) atomicExch(err, 1);
+        // Copies still in flight land before the block's shared memory is given up. (The first
+        // warp reads every stage: where its waits all succeed it has seen every copy land.)
+        if (tid == 0)
+            for (int q = max(0, issued - kZcStages); q < issued; ++q)
+                ptx::mbar_wait_bounded(&full[q % kZcStages], (q / kZcStages) & 1, 1u << 24);
         return;
     }
     if (r >= S) return;
