@@ -458,7 +458,8 @@ __global__ void __launch_bounds__(128 * NG, 1) k_zconv_ring(const float *__restr
     }
 }
 
-bool zconv_streams(const Dims &d) { return d.S % 4 == 0 && d.S <= 128; }
+constexpr int kZcMaxS = 128;
+bool zconv_streams(const Dims &d) { return d.S % 4 == 0 && d.S <= kZcMaxS; }
 
 // The even and odd halves of the products by K, where the convolution can write them and a
 // half's rows start on 16 bytes; rounding errors grow with the length of a sum, so that halves
@@ -482,7 +483,9 @@ void zconv_w(const float *in, const float *hz, float *out, const Dims &d, int *e
         // as many groups a block (4, or 2 where the sums of wide bands need the registers) as
         // leave a block for every SM
         auto go = [&](auto kernel, int NG) {
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            // one limit for every S: another thread's handle may set it between this and the launch
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(float) * kZcStages * kZcIn * W * kZcMaxS);
             launch_dependent(kernel, dim3(outer * ((nl + R * NG - 1) / (R * NG))), dim3((d.S + 31) / 32 * 32 * NG),
                              smem, st, in, hz, out, d.Nz, d.S, np, hv, err);
         };

@@ -1,5 +1,7 @@
 """Forms of the z-drive scan's tables and kernels beside the ordinary ones."""
 
+import threading
+
 import numpy as np
 import pytest
 
@@ -50,3 +52,36 @@ def test_a_drive_amplitude_just_above_whole_fine_cells(form):
     op = FFLOperator(**dict(FORMS[form], A=amp))
     _check(op, Setup(**dict(FORMS[form], A=3.0)))
     op.close()
+
+
+def test_scans_of_different_phases_in_two_threads():
+    """Two handles whose convolutions are one kernel with different amounts of shared memory,
+    each in its own thread and stream."""
+    from paper_2511_06627_gb300 import FFLOperator
+
+    ops = [FFLOperator(**dict(GEOM, nx=40, nz=24, P=40, k_max=3, half_width=4, S=S)) for S in (128, 16)]
+    xs = [torch.rand(op.vol_shape, device="cuda") for op in ops]
+    refs = [op.forward_zdrive(x) for op, x in zip(ops, xs)]
+    torch.cuda.synchronize()
+    results = [None, None]
+
+    def work(k):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                out = ops[k].new_data()
+                for _ in range(1500):
+                    ops[k].forward_zdrive(xs[k], out=out)
+            stream.synchronize()
+            results[k] = out
+        except Exception as e:  # noqa: BLE001
+            results[k] = e
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for got, ref in zip(results, refs):
+        assert isinstance(got, torch.Tensor), got
+        assert torch.equal(got, ref)
