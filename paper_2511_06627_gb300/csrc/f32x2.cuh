@@ -28,4 +28,26 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
     return r;
 }
 
+// The same names on one value, for kernels that take one line or two.
+template <bool TWO>
+struct Lines;
+template <>
+struct Lines<true> {
+    using V = f32x2;
+    static __device__ __forceinline__ V pair(float a, float b) { return pack2(a, b); }
+    static __device__ __forceinline__ V dup(float a) { return dup2(a); }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return fma2(a, b, c); }
+    static __device__ __forceinline__ V add(V a, V b) { return add2(a, b); }
+    static __device__ __forceinline__ float2 parts(V v) { return unpack2(v); }
+};
+template <>
+struct Lines<false> {
+    using V = float;
+    static __device__ __forceinline__ V pair(float a, float) { return a; }
+    static __device__ __forceinline__ V dup(float a) { return a; }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return fmaf(a, b, c); }
+    static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+    static __device__ __forceinline__ float2 parts(V v) { return make_float2(v, 0.f); }
+};
+
 }  // namespace mpiffl

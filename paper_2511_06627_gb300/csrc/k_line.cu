@@ -42,6 +42,10 @@ static_assert(kPsfTF <= kPsfT && kPsfTA <= kPsfT, "the tap table is padded for t
 // 297 lines of 48 bins 67 -> 64 us (66 us).
 constexpr int kPsfTFew = 5, kPsfTAFew = 8;
 constexpr int kPsfSMs = 152;
+// A pair of lines and the taps fit a block's shared memory for every x-drive scan that
+// mpi_ffl_create takes. Along z they may not (columns of 440 slices and more at Q = 32: a pair and
+// the taps need 264 KB, a line and the taps 199 KB): such columns go one at a time.
+constexpr int kPsfSmem = 227 * 1024;
 
 // Blocks that share the tasks of one block's lines: gx blocks with `warps` warps of tasks each
 static int psf_split(int gx, int warps) {
@@ -51,17 +55,20 @@ static bool psf_few(int gx, int warps) { return (long long)gx * warps < 4 * kPsf
 
 // FP32-bound: 2.5 GFMA at 256^2 x 128 and 36 angles in 121 us (144 us one line at a
 // time), of 67 us at the FMA rate.
-template <int T>
+template <int T, bool TWO>
 __global__ void __launch_bounds__(256) k_psf_fwd(const float *__restrict__ proj,
                                                  const float *__restrict__ htab,
                                                  float *__restrict__ fine, Dims d) {
     extern __shared__ __align__(16) float sm[];
-    f32x2 *sp = reinterpret_cast<f32x2 *>(sm);  // N pairs (line, next line)
-    float *sh = sm + 2 * d.N;                   // htab_len
-    const int seg = 2 * blockIdx.x;
-    const bool two = seg + 1 < d.nseg;
+    using X = Lines<TWO>;
+    using V = typename X::V;
+    constexpr int B = TWO ? 2 : 1;
+    V *sp = reinterpret_cast<V *>(sm);  // N pairs (line, next line)
+    float *sh = sm + B * d.N;           // htab_len
+    const int seg = B * blockIdx.x;
+    const bool two = TWO && seg + 1 < d.nseg;
     const float *p0 = proj + (size_t)seg * d.N;
-    for (int i = threadIdx.x; i < d.N; i += blockDim.x) sp[i] = pack2(p0[i], two ? p0[d.N + i] : 0.f);
+    for (int i = threadIdx.x; i < d.N; i += blockDim.x) sp[i] = X::pair(p0[i], two ? p0[d.N + i] : 0.f);
     for (int i = threadIdx.x; i < d.htab_len; i += blockDim.x) sh[i] = htab[i];
     __syncthreads();
     const int Q = d.Q;
@@ -73,48 +80,52 @@ __global__ void __launch_bounds__(256) k_psf_fwd(const float *__restrict__ proj,
         const int q = task % Q;
         const int ab = task / Q;
         const int base = q - d.D + d.htab_off + Q * ab * T;
-        f32x2 w[T], acc[T];
+        V w[T], acc[T];
 #pragma unroll
         for (int t = 0; t < T; ++t) {
-            w[t] = dup2(sh[base + Q * t]);
+            w[t] = X::dup(sh[base + Q * t]);
             acc[t] = 0;
         }
         // unrolled by the window length, so that the window's shift is a renaming of
         // registers rather than moves
 #pragma unroll T
         for (int i = 0; i < d.N; ++i) {
-            const f32x2 pi = sp[i];
+            const V pi = sp[i];
 #pragma unroll
-            for (int t = 0; t < T; ++t) acc[t] = fma2(pi, w[t], acc[t]);
+            for (int t = 0; t < T; ++t) acc[t] = X::fma(pi, w[t], acc[t]);
 #pragma unroll
             for (int t = T - 1; t > 0; --t) w[t] = w[t - 1];
-            w[0] = dup2(sh[base - Q * (i + 1)]);
+            w[0] = X::dup(sh[base - Q * (i + 1)]);
         }
         float *out = fine + (size_t)seg * d.Ne;
 #pragma unroll
         for (int t = 0; t < T; ++t) {
             const int e = q + Q * (ab * T + t);
-            const float2 v = unpack2(acc[t]);
+            const float2 v = X::parts(acc[t]);
             if (e < d.Ne) out[e] = v.x;
             if (e < d.Ne && two) out[d.Ne + e] = v.y;
         }
     }
 }
 
-template <int T>
+template <int T, bool TWO>
 static void run_psf_fwd(const float *proj, const float *htab, float *fine, const Dims &d, int warps, cudaStream_t st) {
-    const size_t smem = sizeof(float) * (2 * d.N + d.htab_len);
+    constexpr int B = TWO ? 2 : 1;
+    const size_t smem = sizeof(float) * (B * d.N + d.htab_len);
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_psf_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    const int gx = (d.nseg + 1) / 2;
-    k_psf_fwd<T><<<dim3(gx, psf_split(gx, warps)), 256, smem, st>>>(proj, htab, fine, d);
+        cudaFuncSetAttribute(k_psf_fwd<T, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPsfSmem);
+    const int gx = (d.nseg + B - 1) / B;
+    k_psf_fwd<T, TWO><<<dim3(gx, psf_split(gx, warps)), 256, smem, st>>>(proj, htab, fine, d);
 }
 
 void launch_psf_fwd(const float *proj, const float *htab, float *fine, const Dims &d, cudaStream_t st) {
     const int n_a = (d.Ne + d.Q - 1) / d.Q;
     auto warps = [&](int t) { return (d.Q * ((n_a + t - 1) / t) + 31) / 32; };
-    if (psf_few((d.nseg + 1) / 2, warps(kPsfTF))) run_psf_fwd<kPsfTFew>(proj, htab, fine, d, warps(kPsfTFew), st);
-    else run_psf_fwd<kPsfTF>(proj, htab, fine, d, warps(kPsfTF), st);
+    if (sizeof(float) * (2 * (size_t)d.N + d.htab_len) > kPsfSmem)
+        run_psf_fwd<kPsfTFew, false>(proj, htab, fine, d, warps(kPsfTFew), st);
+    else if (psf_few((d.nseg + 1) / 2, warps(kPsfTF)))
+        run_psf_fwd<kPsfTFew, true>(proj, htab, fine, d, warps(kPsfTFew), st);
+    else run_psf_fwd<kPsfTF, true>(proj, htab, fine, d, warps(kPsfTF), st);
 }
 
 // H^T: proj[i] = sum_e fine[e] h((e - D)/Q - i). Lanes of a warp are
@@ -126,22 +137,25 @@ void launch_psf_fwd(const float *proj, const float *htab, float *fine, const Dim
 // 145 us (149 us one line at a time).
 constexpr int kPsfAdjThreads = 256;
 
-template <int T>
+template <int T, bool TWO>
 __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restrict__ fine,
                                                             const float *__restrict__ htab,
                                                             float *__restrict__ proj, Dims d, int row_stride,
                                                             int pairs_per_block) {
     extern __shared__ __align__(16) float sm[];
-    f32x2 *sf = reinterpret_cast<f32x2 *>(sm);                     // pairs_per_block rows of row_stride
-    float *sh = sm + 2 * (size_t)pairs_per_block * row_stride;     // htab_len
-    const int seg0 = 2 * blockIdx.x * pairs_per_block;
-    const int nsg = min(2 * pairs_per_block, d.nseg - seg0);
+    using X = Lines<TWO>;
+    using V = typename X::V;
+    constexpr int B = TWO ? 2 : 1;
+    V *sf = reinterpret_cast<V *>(sm);                             // pairs_per_block rows of row_stride
+    float *sh = sm + B * (size_t)pairs_per_block * row_stride;     // htab_len
+    const int seg0 = B * blockIdx.x * pairs_per_block;
+    const int nsg = min(B * pairs_per_block, d.nseg - seg0);
     for (int i = threadIdx.x; i < d.htab_len; i += blockDim.x) sh[i] = htab[i];
-    for (int sl = 0; sl < (nsg + 1) / 2; ++sl) {
-        const float *r0 = fine + (size_t)(seg0 + 2 * sl) * d.Ne;
-        const bool two = 2 * sl + 1 < nsg;
+    for (int sl = 0; sl < (nsg + B - 1) / B; ++sl) {
+        const float *r0 = fine + (size_t)(seg0 + B * sl) * d.Ne;
+        const bool two = TWO && 2 * sl + 1 < nsg;
         for (int e = threadIdx.x; e < d.Ne; e += blockDim.x)
-            sf[sl * row_stride + e] = pack2(r0[e], two ? r0[d.Ne + e] : 0.f);
+            sf[sl * row_stride + e] = X::pair(r0[e], two ? r0[d.Ne + e] : 0.f);
     }
     __syncthreads();
     const int Q = d.Q;
@@ -151,38 +165,38 @@ __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restr
     const int q = lane % Q;
     const int sl = lane / Q;               // line pair within the block handled by this lane
     const int n_ib = (d.N + T - 1) / T;
-    const bool active = 2 * sl < nsg;
-    const f32x2 *row = sf + (active ? sl : 0) * row_stride;
+    const bool active = B * sl < nsg;
+    const V *row = sf + (active ? sl : 0) * row_stride;
     const int share = (n_ib + gridDim.y - 1) / gridDim.y;  // warp tasks of this block
     const int end = min(n_ib, (int)(blockIdx.y + 1) * share);
     for (int ib = blockIdx.y * share + warp; ib < end; ib += nwarps) {
         const int i0 = ib * T;
-        f32x2 acc[T];
+        V acc[T];
 #pragma unroll
         for (int t = 0; t < T; ++t) acc[t] = 0;
         const int baseq = q - d.D - Q * i0 + d.htab_off;
-        f32x2 w[T];
+        V w[T];
 #pragma unroll
-        for (int t = 0; t < T; ++t) w[t] = dup2(sh[baseq - Q * t]);
+        for (int t = 0; t < T; ++t) w[t] = X::dup(sh[baseq - Q * t]);
 #pragma unroll T
         for (int a = 0, e = q; e < d.Ne; ++a, e += Q) {
-            const f32x2 c = row[e];
+            const V c = row[e];
 #pragma unroll
-            for (int t = 0; t < T; ++t) acc[t] = fma2(c, w[t], acc[t]);
+            for (int t = 0; t < T; ++t) acc[t] = X::fma(c, w[t], acc[t]);
 #pragma unroll
             for (int t = T - 1; t > 0; --t) w[t] = w[t - 1];
-            w[0] = dup2(sh[baseq + Q * (a + 1)]);
+            w[0] = X::dup(sh[baseq + Q * (a + 1)]);
         }
         // add the Q phase partials (lanes sl*Q .. sl*Q+Q-1)
 #pragma unroll
         for (int t = 0; t < T; ++t)
-            for (int o = 1; o < Q; o <<= 1) acc[t] = add2(acc[t], __shfl_xor_sync(0xffffffffu, acc[t], o));
+            for (int o = 1; o < Q; o <<= 1) acc[t] = X::add(acc[t], __shfl_xor_sync(0xffffffffu, acc[t], o));
         if (active && q == 0) {
-            float *out = proj + (size_t)(seg0 + 2 * sl) * d.N;
-            const bool two = 2 * sl + 1 < nsg;
+            float *out = proj + (size_t)(seg0 + B * sl) * d.N;
+            const bool two = TWO && 2 * sl + 1 < nsg;
 #pragma unroll
             for (int t = 0; t < T; ++t) {
-                const float2 v = unpack2(acc[t]);
+                const float2 v = X::parts(acc[t]);
                 if (i0 + t < d.N) out[i0 + t] = v.x;
                 if (i0 + t < d.N && two) out[d.N + i0 + t] = v.y;
             }
@@ -191,27 +205,30 @@ __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restr
 }
 
 // Line pairs of a block: 32 / Q of them fill a warp's lanes; fewer where the rows of so many do
-// not fit the shared memory beside the taps, at most two where the lines are few.
-template <int T>
+// not fit the shared memory beside the taps, at most two where the lines are few. Where not even
+// one pair fits, one line a block.
+template <int T, bool TWO>
 static void run_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, int pairs, cudaStream_t st) {
     // lanes = (line pair, phase); Q must be a power of two dividing 32 for the shuffle tree
     const int stride = d.Ne + (((d.Q - d.Ne) % 16) + 16) % 16;  // stride = Q (mod 16)
-    auto bytes = [&](int p) { return sizeof(float) * (d.htab_len + 2 * (size_t)p * stride); };
-    while (pairs > 1 && bytes(pairs) > 227 * 1024) pairs /= 2;
+    constexpr int B = TWO ? 2 : 1;
+    auto bytes = [&](int p) { return sizeof(float) * (d.htab_len + B * (size_t)p * stride); };
+    while (pairs > 1 && bytes(pairs) > kPsfSmem) pairs /= 2;
     const size_t smem = bytes(pairs);
+    if (TWO && smem > kPsfSmem) return run_psf_adj<kPsfTAFew, false>(fine, htab, proj, d, 1, st);
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_psf_adj<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    const int gx = (d.nseg + 2 * pairs - 1) / (2 * pairs);
-    k_psf_adj<T><<<dim3(gx, psf_split(gx, (d.N + T - 1) / T)), kPsfAdjThreads, smem, st>>>(fine, htab, proj, d, stride,
+        cudaFuncSetAttribute(k_psf_adj<T, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPsfSmem);
+    const int gx = (d.nseg + B * pairs - 1) / (B * pairs);
+    k_psf_adj<T, TWO><<<dim3(gx, psf_split(gx, (d.N + T - 1) / T)), kPsfAdjThreads, smem, st>>>(fine, htab, proj, d, stride,
                                                                                           pairs);
 }
 
 void launch_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, cudaStream_t st) {
     const int pairs = 32 / d.Q;
     if (psf_few((d.nseg + 2 * pairs - 1) / (2 * pairs), (d.N + kPsfTA - 1) / kPsfTA))
-        run_psf_adj<kPsfTAFew>(fine, htab, proj, d, std::min(pairs, 2), st);
+        run_psf_adj<kPsfTAFew, true>(fine, htab, proj, d, std::min(pairs, 2), st);
     else
-        run_psf_adj<kPsfTA>(fine, htab, proj, d, pairs, st);
+        run_psf_adj<kPsfTA, true>(fine, htab, proj, d, pairs, st);
 }
 
 // ----------------------------------------------------------------------------- E V B
