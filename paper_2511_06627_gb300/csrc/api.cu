@@ -1492,21 +1492,31 @@ void zstage_evt(mpi_ffl_handle *h, const float *sig, float *cz, cudaStream_t st)
     TIMED(MPI_FFL_K_ZDRIVE, launch_resample_z_adj(sig, z_tables(h), h->t_gain, h->w_tz, cz, h->d, h->zigzag, st));
 }
 
-// Whether the folded z-drive kernels serve this shape; their tables are built on first use.
+// Whether the folded z-drive kernels serve this handle; their tables are built on first use.
+// They take more memory than the sample-by-sample kernels: where it is not to be had, those
+// serve the handle from then on.
 bool use_zfold(mpi_ffl_handle *h) {
-    if (!zfold_fits(h->d)) return false;
+    if (h->zfold_off || !zfold_fits(h->d)) return false;
     const int rc = zfold_ready(h);
-    if (rc != MPI_FFL_OK) {
+    if (rc == MPI_FFL_OK) return true;
+    if (rc != MPI_FFL_ERR_OOM) {
         set_err(h, "building the z-drive tables failed");
         throw Fail{rc};
     }
-    return true;
+    h->zfold_off = true;
+    return false;
 }
 
 void ensure_z_workspace(mpi_ffl_handle *h) {
     const Dims &d = h->d;
-    if (!h->w_fine_z) dev_alloc(h, &h->w_fine_z, (size_t)d.M * d.N * d.Nez);
-    if (!h->w_zcoef) dev_alloc(h, &h->w_zcoef, (size_t)d.M * d.Nz * (2 * d.hw + 1) * d.S);
+    try {
+        if (!h->w_fine_z) dev_alloc(h, &h->w_fine_z, (size_t)d.M * d.N * d.Nez);
+        if (!h->w_zcoef) dev_alloc(h, &h->w_zcoef, (size_t)d.M * d.Nz * (2 * d.hw + 1) * d.S);
+        ensure_projT(h);
+    } catch (...) {  // no memory for either form: the next call tries both again
+        h->zfold_off = false;
+        throw;
+    }
 }
 
 // projections -> z-drive data

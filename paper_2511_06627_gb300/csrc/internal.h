@@ -209,6 +209,7 @@ struct mpi_ffl_handle {
     int2 *tz_otap = nullptr;
     int tz_no = 0;
     void *zfold_state = nullptr;  // folded tables and workspace (k_zfold.cu)
+    bool zfold_off = false;       // no memory for them: the sample-by-sample kernels
     void *ten_state = nullptr;    // tables and workspace of the tensor PSF (k_tensor.cu)
     // workspace of the sample-by-sample kernels and of the z stages, on their first use
     float *w_fine_z = nullptr;  // M N N_ez

@@ -541,11 +541,14 @@ int z_parts(const Dims &d) {
     return (nk + z_kper(d) - 1) / z_kper(d);
 }
 
+size_t tap_len(const Dims &d) { return (size_t)d.Q * (2 * d.Nz - 2) + 2 * d.D + 2; }
+
+// hz for the handle's width; its buffers are there
 bool fold_h(mpi_ffl_handle *h) {
     const Dims &d = h->d;
     const double a = h->fwhm / (2.0 * langevin_half_point_host());
     const double kPi = 3.14159265358979323846;
-    std::vector<double> taps((size_t)d.Q * (2 * d.Nz - 2) + 2 * d.D + 2);
+    std::vector<double> taps(tap_len(d));
     for (size_t i = 0; i < taps.size(); ++i)
         taps[i] = 3.0 * langevin_d1_host((((double)i - d.D) / d.Q - (d.Nz - 1)) / a);
     std::vector<double2> drive(d.S);
@@ -554,7 +557,6 @@ bool fold_h(mpi_ffl_handle *h) {
         drive[r] = make_double2(z_drive_offset_host(h, r), h->amp * (2.0 * kPi / d.S) * std::cos(ph));
     }
     ZFold *s = zs(h);
-    if (!zalloc(&s->taps, taps.size()) || !zalloc(&s->drive, drive.size())) return false;
     cudaMemcpy(s->taps, taps.data(), taps.size() * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(s->drive, drive.data(), drive.size() * sizeof(double2), cudaMemcpyHostToDevice);
     k_zfold_h<<<dim3((d.S + 127) / 128, 2 * d.Nz - 1), 128>>>(s->taps, s->drive, s->hz, d.Nz, d.S, d.Q, d.D);
@@ -567,11 +569,17 @@ bool fold_h(mpi_ffl_handle *h) {
 
 // Per (line, phase) the folded steps cost (n_par N + N_z) W FMAs at matrix-product speed,
 // the sample-by-sample kernels P (W + 4) at about a fifth of it (1.45 ms against 0.42 ms for
-// the line stages of a pair at 256^2 x 128, 36 angles, P = 512). The intermediate G is kept in memory.
+// the line stages of a pair at 256^2 x 128, 36 angles, P = 512). The intermediates are kept in
+// memory: G at most 1 GB, T at most as much, the partial sums of the adjoint's last product at
+// most twice that and a set of projections (z_kper), together at most 4 GB. Where they cannot be
+// allocated the sample-by-sample kernels serve the handle (use_zfold).
 bool zfold_fits(const Dims &d) {
     const double folded = (double)(d.n_par * d.N + d.Nz) * d.W, sampled = 4.0 * d.P * (d.W + 4);
-    return folded <= sampled && g_len(d) * sizeof(float) <= (size_t)1 << 30 &&
-           (size_t)d.N * d.n_par * d.W * d.S * sizeof(float) <= (size_t)1 << 28;
+    if (folded > sampled || g_len(d) * sizeof(float) > (size_t)1 << 30 ||
+        (size_t)d.N * d.n_par * d.W * d.S * sizeof(float) > (size_t)1 << 28)
+        return false;
+    const size_t rows = (size_t)d.M * d.Nz;
+    return (g_len(d) + rows * d.W * d.S + z_parts(d) * rows * d.N) * sizeof(float) <= (size_t)4 << 30;
 }
 
 int zfold_ready(mpi_ffl_handle *h) {
@@ -586,12 +594,14 @@ int zfold_ready(mpi_ffl_handle *h) {
     const size_t kf_len = (size_t)(hv ? 2 * Nh : d.N) * s->ldk, ka_len = (size_t)(hv ? 2 : 1) * nk * s->ldu;
     double2 *unit_p = nullptr;
     double *K = nullptr;
-    bool ok = zalloc(&s->kf, kf_len) && zalloc(&s->ka, ka_len) && zalloc(&K, (size_t)d.N * nk) &&
+    int rc = MPI_FFL_ERR_OOM;
+    const bool ok = zalloc(&s->kf, kf_len) && zalloc(&s->ka, ka_len) && zalloc(&K, (size_t)d.N * nk) &&
               (!hv || zalloc(&s->eo, (size_t)d.M * d.Nz * 2 * s->ldu)) &&
               zalloc(&s->hz, (size_t)(2 * d.Nz - 1) * d.S) && zalloc(&s->df, dft_f_len(d)) &&
               zalloc(&s->da, dft_a_len(d)) && zalloc(&s->cols, (size_t)2 * d.nb) && zalloc(&s->g, g_len(d)) &&
               zalloc(&s->t, (size_t)d.M * d.Nz * d.W * d.S) && zalloc(&unit_p, d.P) &&
-              zalloc(&s->part, (size_t)z_parts(d) * d.M * d.Nz * d.N);
+              zalloc(&s->part, (size_t)z_parts(d) * d.M * d.Nz * d.N) && zalloc(&s->taps, tap_len(d)) &&
+              zalloc(&s->drive, d.S);
     if (ok) {
         const double kPi = 3.14159265358979323846;
         std::vector<double2> up(d.P);
@@ -604,13 +614,13 @@ int zfold_ready(mpi_ffl_handle *h) {
         k_zfold_k<<<(nk + 127) / 128, 128>>>(unit_p, K, d, nk);
         k_zfold_operands<<<608, 256>>>(K, s->kf, s->ka, d.N, nk, s->ldk, s->ldu, hv);
         k_zfold_dft<<<dim3(64, d.hw + 1), 128>>>(h->t_dgam, s->df, s->da, s->cols, d);
-        ok = fold_h(h);
+        rc = fold_h(h) ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
     }
     if (unit_p) dev_free(unit_p);
     if (K) dev_free(K);
-    if (!ok) {  // nothing of a failed build is kept
+    if (rc != MPI_FFL_OK) {  // nothing of a failed build is kept
         zfold_release(h);
-        return MPI_FFL_ERR_OOM;
+        return rc;
     }
     s->ready = true;
     return MPI_FFL_OK;

@@ -1,5 +1,6 @@
 """Forms of the z-drive scan's tables and kernels beside the ordinary ones."""
 
+import ctypes as C
 import threading
 
 import numpy as np
@@ -52,6 +53,33 @@ def test_a_drive_amplitude_just_above_whole_fine_cells(form):
     op = FFLOperator(**dict(FORMS[form], A=amp))
     _check(op, Setup(**dict(FORMS[form], A=3.0)))
     op.close()
+
+
+def test_without_memory_for_the_tables_the_sampled_kernels_serve():
+    """An allocation of the folded form that fails leaves the scan to the sample-by-sample
+    kernels, in both directions and at another width."""
+    from paper_2511_06627_gb300 import FFLOperator, MpiFflError
+    from paper_2511_06627_gb300 import _lib as L
+
+    lib = L.load()
+    served = 0
+    for n in range(1, 40):
+        op = FFLOperator(**GEOM)
+        x = torch.zeros(op.vol_shape, device="cuda")
+        assert lib.mpi_ffl_test_fail_alloc(n) == L.OK
+        try:
+            op.forward_zdrive(x)
+            served += 1
+            failed = False
+        except MpiFflError as e:
+            assert e.code == L.ERR_OOM, e
+            failed = True
+        lib.mpi_ffl_test_fail_alloc(0)
+        for fwhm in () if failed else (2.5, 3.25):
+            op.set_fwhm(fwhm)
+            _check(op, Setup(**dict(GEOM, fwhm=fwhm)))
+        op.close()
+    assert served >= 25  # the others fell on tables that both forms need
 
 
 def test_scans_of_different_phases_in_two_threads():
