@@ -153,7 +153,6 @@ double langevin_half_point() {
 
 namespace mpiffl {
 double langevin_d1_host(double x) { return langevin_d1(x); }
-double langevin_d2_host(double x) { return langevin_d2(x); }
 double langevin_half_point_host() { return langevin_half_point(); }
 // FFL sample j of a line with the given trajectory (parity): fine cell n, fraction f, velocity v
 void traj_point_host(const mpi_ffl_handle *h, int par, int j, int &n, double &f, double &v) {
@@ -179,16 +178,22 @@ double z_drive_offset_host(const mpi_ffl_handle *h, int r) {
 
 namespace {
 
-void psf_tables(const Dims &d, double fwhm, std::vector<float> &h, std::vector<float> &dh) {
+// The PSF and its derivative by the width at k / Q, k = 0 .. htab_off, in FP64 (both are even),
+// and the FP32 tap tables made of them. The folded operators take theirs from the same values.
+void psf_tables(const Dims &d, double fwhm, PsfTaps &t, std::vector<float> &h, std::vector<float> &dh) {
     const double a = fwhm / (2.0 * langevin_half_point());
+    t.h.resize(d.htab_off + 1);
+    t.dh.resize(d.htab_off + 1);
     h.resize(d.htab_len);
     dh.resize(d.htab_len);
-    for (int k = 0; k <= d.htab_off; ++k) {  // both are even in u
+    for (int k = 0; k <= d.htab_off; ++k) {
         const double u = (double)k / d.Q;
         const double x = u / a;
-        h[d.htab_off + k] = h[d.htab_off - k] = (float)(3.0 * langevin_d1(x));
+        t.h[k] = 3.0 * langevin_d1(x);
         // d/dfwhm of 3 L'(u/a), a = fwhm / (2 x_h): -3 L''(x) x / fwhm
-        dh[d.htab_off + k] = dh[d.htab_off - k] = (float)(-3.0 * langevin_d2(x) * x / fwhm);
+        t.dh[k] = -3.0 * langevin_d2(x) * x / fwhm;
+        h[d.htab_off + k] = h[d.htab_off - k] = (float)t.h[k];
+        dh[d.htab_off + k] = dh[d.htab_off - k] = (float)t.dh[k];
     }
 }
 
@@ -994,7 +999,7 @@ extern "C" int mpi_ffl_create(const mpi_ffl_geometry *geom, const mpi_ffl_trajec
         upload(h, &h->t_gain, h->gains);
         upload(h, &h->t_unit_gain, std::vector<float>(d.M, 1.f));
         std::vector<float> ht, dht;
-        psf_tables(d, h->fwhm, ht, dht);
+        psf_tables(d, h->fwhm, h->taps, ht, dht);
         upload(h, &h->t_htab, ht);
         upload(h, &h->t_dhtab, dht);
         trajectory_tables(h);
@@ -1144,9 +1149,18 @@ static int set_path_impl(mpi_ffl_handle *h, int32_t path) {
     return MPI_FFL_OK;
 }
 
-extern "C" int mpi_ffl_set_precision(mpi_ffl_handle *h, int32_t precision) { return set_precision_impl(h, precision); }
+// The staged path's operands follow a width at once while that path is selected, or when it is
+// selected: its calls then find them built (a captured graph of theirs too).
+static int staged_selected(mpi_ffl_handle *h, int rc) {
+    if (rc == MPI_FFL_OK && h->path == MPI_FFL_PATH_STAGED) fold_refresh(h);
+    return rc;
+}
 
-extern "C" int mpi_ffl_set_path(mpi_ffl_handle *h, int32_t path) { return set_path_impl(h, path); }
+extern "C" int mpi_ffl_set_precision(mpi_ffl_handle *h, int32_t precision) {
+    return staged_selected(h, set_precision_impl(h, precision));
+}
+
+extern "C" int mpi_ffl_set_path(mpi_ffl_handle *h, int32_t path) { return staged_selected(h, set_path_impl(h, path)); }
 
 extern "C" int mpi_ffl_set_psf_model(mpi_ffl_handle *h, int32_t model) {
     return guarded(h, [&]() {
@@ -1253,14 +1267,17 @@ extern "C" int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm) {
             return MPI_FFL_ERR_INVALID_ARG;
         }
         std::vector<float> ht, dht;
-        psf_tables(h->d, fwhm, ht, dht);
+        PsfTaps taps;
+        psf_tables(h->d, fwhm, taps, ht, dht);
         CK(cudaDeviceSynchronize());
         h->fwhm = fwhm;
+        h->taps = std::move(taps);
         CK(cudaMemcpy(h->t_htab, ht.data(), sizeof(float) * ht.size(), cudaMemcpyHostToDevice));
         CK(cudaMemcpy(h->t_dhtab, dht.data(), sizeof(float) * dht.size(), cudaMemcpyHostToDevice));
         uploads_done(h);
         tc_tables_changed(h);
         fold_psf_changed(h);
+        if (h->path == MPI_FFL_PATH_STAGED) fold_refresh(h);
         zfold_psf_changed(h);
         // W H holds the PSF: rebuild the collapsed operator if it was built and the
         // full-GEMM path is selected; otherwise W (which holds no PSF) stays and W H is

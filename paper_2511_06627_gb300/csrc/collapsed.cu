@@ -689,7 +689,7 @@ void col_init(mpi_ffl_handle *h) {
     if ((size_t)d.N * 2 * d.nb * 8 > (size_t)1 << 31) return;
     s->n_par = d.n_par;
     const int R = 2 * d.nb;
-    const double *WH = fold_wh(h, 0, nullptr), *W = fold_w_dev(h);
+    const double *WH = fold_wh(h, nullptr), *W = fold_w_dev(h);
     if (!WH || !W) {
         s->oom = true;
         return;

@@ -45,7 +45,6 @@ void ten_adjoint(mpi_ffl_handle *h, const float *data, const float *coil, float 
 
 // host-side model pieces shared with the table builders (api.cu)
 double langevin_d1_host(double x);
-double langevin_d2_host(double x);
 double langevin_half_point_host();
 void traj_point_host(const mpi_ffl_handle *h, int parity, int j, int &n, double &f, double &v);
 // The drive's offset A sin(phase r) on the fine z grid, Q A sin + D, held to [0, 2 D]: D = ceil(Q A

@@ -19,11 +19,12 @@ namespace {
 
 struct FoldState {
     double *W = nullptr;     // [n_par][2 n_b][N_e]
-    double *taps = nullptr;  // one slot's PSF taps
-    double *WH = nullptr;    // [n_par][2 n_b][N]
-    // FP32 operands of slot 0 (h) and 1 (d h / d fwhm): B of the forward [n_par][N][ldf]
-    // and of the adjoint [n_par][2 n_b][lda]
-    float *f[2] = {nullptr, nullptr}, *a[2] = {nullptr, nullptr};
+    double *taps = nullptr;  // PSF taps of slot 0, then of slot 1
+    double taps_fwhm = -1.0; // their width; < 0: none
+    double *WH = nullptr;    // [n_par][slots folded together][2 n_b][N]
+    // FP32 operands: B of the forward [n_par][N][ldf] of slot 0 (h) and 1 (d h / d fwhm), and of
+    // the adjoint [n_par][2 n_b][lda] of slot 0
+    float *f[2] = {nullptr, nullptr}, *a = nullptr;
     bool stale[2] = {false, false};  // of another width: refolded on the next use
     int ldf = 0, lda = 0;
     int *rows = nullptr;  // lines of trajectory 0, then of trajectory 1
@@ -121,61 +122,61 @@ __global__ void __launch_bounds__(256) k_fold_w(FoldTraj T, double *__restrict__
     }
 }
 
-// out[par][z][o][i] = sum_e W[par][o][e] g[z][e - D - Q i - kmin]: a block takes 8 rows o,
-// 128 columns i, one z and trajectory; e runs in tiles of 256 staged in shared memory with
-// the taps they meet.
-constexpr int kWdRows = 8, kWdCols = 128, kWdTile = 256;
+// out[par][z][o][i] = sum_e W[par][o][e] g[z][e - D - Q i - kmin]: a warp takes one row o and 32
+// columns i, a block two rows of one z and trajectory; e runs in tiles of 256 staged in shared
+// memory with the taps they meet, which lie there by residue modulo Q, so that the lanes of a
+// warp (taps Q apart) read neighbouring words. Bound by the FP64 pipe, two FMAs a clock and SM:
+// small blocks spread even one small fold over the GPU. With eight rows and 128 columns a block a
+// fold at 32^2 x 16 ran on 12 SMs and took 160 us.
+constexpr int kWdRows = 2, kWdCols = 32, kWdTile = 256;
 
-__global__ void __launch_bounds__(kWdCols) k_fold_taps(const double *__restrict__ W, const double *__restrict__ g,
-                                                       double *__restrict__ out, int R, int Ne, int N, int Nz, int D,
-                                                       int Q, int kmin, int Lk) {
+__global__ void __launch_bounds__(32 * kWdRows) k_fold_taps(const double *__restrict__ W,
+                                                            const double *__restrict__ g, double *__restrict__ out,
+                                                            int R, int Ne, int N, int Nz, int D, int Q, int kmin,
+                                                            int Lk) {
     __shared__ double sw[kWdRows][kWdTile];
-    extern __shared__ double sg[];  // kWdTile + Q (kWdCols - 1) taps
+    __shared__ double sg[kWdTile + 32 * kWdCols];  // [Q][kWdTile / Q + kWdCols] taps, Q <= 32
     const int ncb = (N + kWdCols - 1) / kWdCols;
     const int o0 = (blockIdx.x / ncb) * kWdRows, i0 = (blockIdx.x % ncb) * kWdCols;
     const int d = blockIdx.y, par = blockIdx.z;
-    const int il = threadIdx.x, i = i0 + il;
+    const int lane = threadIdx.x & 31, r = threadIdx.x >> 5, i = i0 + lane;
     const double *Wp = W + (size_t)par * R * Ne;
     const double *gd = g + (size_t)d * Lk;
-    const int span = kWdTile + Q * (kWdCols - 1);
-    double acc[kWdRows];
-#pragma unroll
-    for (int r = 0; r < kWdRows; ++r) acc[r] = 0.0;
+    const int per = kWdTile / Q + kWdCols, span = kWdTile + Q * (kWdCols - 1);
+    double acc = 0.0;
     for (int e0 = 0; e0 < Ne; e0 += kWdTile) {
         __syncthreads();
         for (int t = threadIdx.x; t < kWdRows * kWdTile; t += blockDim.x) {
-            const int r = t / kWdTile, e = e0 + t % kWdTile;
-            sw[r][t % kWdTile] = (o0 + r < R && e < Ne) ? Wp[(size_t)(o0 + r) * Ne + e] : 0.0;
+            const int rr = t / kWdTile, e = e0 + t % kWdTile;
+            sw[rr][t % kWdTile] = (o0 + rr < R && e < Ne) ? Wp[(size_t)(o0 + rr) * Ne + e] : 0.0;
         }
         // k = e - D - Q i runs from kb (e = e0, i = i0 + kWdCols - 1) upwards
         const int kb = e0 - D - Q * (i0 + kWdCols - 1) - kmin;
         for (int t = threadIdx.x; t < span; t += blockDim.x) {
             const int k = kb + t;
-            sg[t] = (k >= 0 && k < Lk) ? gd[k] : 0.0;
+            sg[(t % Q) * per + t / Q] = (k >= 0 && k < Lk) ? gd[k] : 0.0;
         }
         __syncthreads();
-        const double *gl = sg + Q * (kWdCols - 1 - il);
-        for (int e = 0; e < kWdTile; ++e) {
-            const double gv = gl[e];
-#pragma unroll
-            for (int r = 0; r < kWdRows; ++r) acc[r] = fma(sw[r][e], gv, acc[r]);
-        }
+        const double *gl = sg + kWdCols - 1 - lane;
+        for (int b = 0; b < kWdTile / Q; ++b)
+            for (int q = 0; q < Q; ++q) acc = fma(sw[r][b * Q + q], gl[q * per + b], acc);
     }
-    if (i < N)
-        for (int r = 0; r < kWdRows; ++r)
-            if (o0 + r < R) out[(((size_t)par * Nz + d) * R + o0 + r) * N + i] = acc[r];
+    if (i < N && o0 + r < R) out[(((size_t)par * Nz + d) * R + o0 + r) * N + i] = acc;
 }
 
-// FP32 operands of the staged path from W H: f[par][i][o] (columns past 2 n_b zero) and
-// a[par][o][i] (columns past N zero)
-__global__ void __launch_bounds__(256) k_fold_operands(const double *__restrict__ WH, float *__restrict__ f,
-                                                       float *__restrict__ a, int R, int N, int ldf, int lda) {
+// FP32 operands of the staged path from W H [n_par][ns][2 n_b][N], z = blockIdx.z of ns:
+// f_z[par][i][o] (columns past 2 n_b zero) and, of slot 0, a[par][o][i] (columns past N zero)
+__global__ void __launch_bounds__(256) k_fold_operands(const double *__restrict__ WH, float *__restrict__ f0,
+                                                       float *__restrict__ f1, float *__restrict__ a, int R, int N,
+                                                       int ldf, int lda) {
     const int par = blockIdx.y;
-    const double *src = WH + (size_t)par * R * N;
+    const double *src = WH + ((size_t)par * gridDim.z + blockIdx.z) * R * N;
+    float *f = blockIdx.z ? f1 : f0;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < N * ldf; t += gridDim.x * blockDim.x) {
         const int i = t / ldf, o = t - i * ldf;
         f[(size_t)par * N * ldf + t] = o < R ? (float)src[(size_t)o * N + i] : 0.f;
     }
+    if (!a || blockIdx.z) return;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < R * lda; t += gridDim.x * blockDim.x) {
         const int o = t / lda, i = t - o * lda;
         a[(size_t)par * R * lda + t] = i < N ? (float)src[(size_t)o * N + i] : 0.f;
@@ -187,30 +188,48 @@ FoldState *state(mpi_ffl_handle *h) {
     return fs(h);
 }
 
-// FP64 taps of slot 0 (h) or 1 (d h / d fwhm) at offsets (kmin + k) / Q
-std::vector<double> psf_taps(const mpi_ffl_handle *h, int slot) {
+// Taps of both slots at offsets (kmin + k) / Q on the device, for the handle's width
+int taps_ready(mpi_ffl_handle *h) {
+    FoldState *s = fs(h);
+    if (s->taps_fwhm == h->fwhm) return MPI_FFL_OK;
     const Dims &d = h->d;
-    std::vector<double> g(fold_taps(d));
-    const double a = h->fwhm / (2.0 * langevin_half_point_host());
-    for (size_t k = 0; k < g.size(); ++k) {
-        const double x = (double)((int)k + fold_kmin(d)) / d.Q / a;
-        g[k] = slot ? -3.0 * langevin_d2_host(x) * x / h->fwhm : 3.0 * langevin_d1_host(x);
+    const int n = fold_taps(d);
+    if (!falloc(&s->taps, 2 * (size_t)n)) return MPI_FFL_ERR_OOM;
+    std::vector<double> g(2 * (size_t)n);
+    for (int k = 0; k < n; ++k) {
+        g[k] = h->taps.h[std::abs(k + fold_kmin(d))];
+        g[n + k] = h->taps.dh[std::abs(k + fold_kmin(d))];
     }
-    return g;
+    s->taps_fwhm = -1.0;
+    if (!fupload(s->taps, g)) return MPI_FFL_ERR_CUDA;
+    s->taps_fwhm = h->fwhm;
+    return MPI_FFL_OK;
 }
 
-int refold(mpi_ffl_handle *h, int slot, cudaStream_t st) {
+// W H of slots [first, first + n) into s->WH
+int fold_slots(mpi_ffl_handle *h, int first, int n, cudaStream_t st) {
     const Dims &d = h->d;
+    int rc = fold_w(h);
+    if (rc == MPI_FFL_OK) rc = taps_ready(h);
+    if (rc != MPI_FFL_OK) return rc;
     FoldState *s = fs(h);
-    const int R = 2 * d.nb;
-    const double *wh = fold_wh(h, slot, st);
-    if (!wh) return MPI_FFL_ERR_OOM;
-    const int work = std::max(d.N * s->ldf, R * s->lda);
-    k_fold_operands<<<dim3(std::min(608, (work + 255) / 256), d.n_par), 256, 0, st>>>(wh, s->f[slot], s->a[slot], R,
-                                                                                     d.N, s->ldf, s->lda);
-    // another stream may use the operands next, and the host taps may be freed
+    if (!falloc(&s->WH, (size_t)d.n_par * 2 * 2 * d.nb * d.N)) return MPI_FFL_ERR_OOM;
+    launch_fold_taps(s->W, s->taps + (size_t)first * fold_taps(d), s->WH, d, d.n_par, n, st);
+    return MPI_FFL_OK;
+}
+
+// the operands of slots [first, first + n), whose buffers are there
+int refold(mpi_ffl_handle *h, int first, int n, cudaStream_t st) {
+    const Dims &d = h->d;
+    const int rc = fold_slots(h, first, n, st);
+    if (rc != MPI_FFL_OK) return rc;
+    FoldState *s = fs(h);
+    const int R = 2 * d.nb, work = std::max(d.N * s->ldf, R * s->lda);
+    k_fold_operands<<<dim3(std::min(608, (work + 255) / 256), d.n_par, n), 256, 0, st>>>(
+        s->WH, s->f[first], s->f[1], first == 0 ? s->a : nullptr, R, d.N, s->ldf, s->lda);
+    // another stream may use the operands next
     if (cudaStreamSynchronize(st) != cudaSuccess) return MPI_FFL_ERR_CUDA;
-    s->stale[slot] = false;
+    for (int k = first; k < first + n; ++k) s->stale[k] = false;
     return MPI_FFL_OK;
 }
 
@@ -315,23 +334,12 @@ const double *fold_w_dev(const mpi_ffl_handle *h) { return fs(h) ? fs(h)->W : nu
 void launch_fold_taps(const double *W, const double *g, double *out, const Dims &d, int n_par, int nz,
                       cudaStream_t st) {
     const int R = 2 * d.nb, ncb = (d.N + kWdCols - 1) / kWdCols;
-    const size_t smem = sizeof(double) * (kWdTile + d.Q * (kWdCols - 1));
-    if (smem > 32 * 1024) cudaFuncSetAttribute(k_fold_taps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_fold_taps<<<dim3(((R + kWdRows - 1) / kWdRows) * ncb, nz, n_par), kWdCols, smem, st>>>(
+    k_fold_taps<<<dim3(((R + kWdRows - 1) / kWdRows) * ncb, nz, n_par), 32 * kWdRows, 0, st>>>(
         W, g, out, R, d.Ne, d.N, nz, d.D, d.Q, fold_kmin(d), fold_taps(d));
 }
 
-const double *fold_wh(mpi_ffl_handle *h, int slot, cudaStream_t st) {
-    const Dims &d = h->d;
-    if (fold_w(h) != MPI_FFL_OK) return nullptr;
-    FoldState *s = fs(h);
-    if (!falloc(&s->taps, fold_taps(d)) || !falloc(&s->WH, (size_t)d.n_par * 2 * d.nb * d.N)) return nullptr;
-    const std::vector<double> g = psf_taps(h, slot);
-    // pageable memory: the copy has left the host vector when the call returns
-    if (cudaMemcpyAsync(s->taps, g.data(), g.size() * sizeof(double), cudaMemcpyHostToDevice, st) != cudaSuccess)
-        return nullptr;
-    launch_fold_taps(s->W, s->taps, s->WH, d, d.n_par, 1, st);
-    return s->WH;
+const double *fold_wh(mpi_ffl_handle *h, cudaStream_t st) {
+    return fold_slots(h, 0, 1, st) == MPI_FFL_OK ? fs(h)->WH : nullptr;
 }
 
 // The folded stage costs 2 n_b N FMAs a line, the stage kernels N N_e (H), about
@@ -368,14 +376,17 @@ int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
     s->ldf = (R + 3) / 4 * 4;
     s->lda = (d.N + 3) / 4 * 4;
     int rc = MPI_FFL_ERR_OOM;
-    if (falloc(&s->f[slot], (size_t)d.n_par * d.N * s->ldf) && falloc(&s->a[slot], (size_t)d.n_par * R * s->lda))
-        rc = refold(h, slot, st);
-    if (rc != MPI_FFL_OK)  // nothing of a failed build is kept: the next call tries again
-        for (float **p : {&s->f[slot], &s->a[slot]})
-            if (*p) {
+    if (falloc(&s->f[slot], (size_t)d.n_par * d.N * s->ldf) &&
+        (slot || falloc(&s->a, (size_t)d.n_par * R * s->lda)))
+        rc = refold(h, slot, 1, st);
+    if (rc != MPI_FFL_OK) {  // no operands of a failed build are kept: the next call tries again
+        for (float **p : {&s->f[slot], slot ? nullptr : &s->a})
+            if (p && *p) {
                 dev_free(*p);
                 *p = nullptr;
             }
+        s->stale[slot] = false;
+    }
     return rc;
 }
 
@@ -398,19 +409,23 @@ void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float
     SgemmArgs g[2];
     for (int par = 0; par < d.n_par; ++par) {
         const int *rows = s->rows + (par ? s->nrows[0] : 0);
-        g[par] = SgemmArgs{data, R,    rows, s->nrows[par], R,   s->a[0] + (size_t)par * R * s->lda,
+        g[par] = SgemmArgs{data, R,    rows, s->nrows[par], R,   s->a + (size_t)par * R * s->lda,
                            s->lda, proj, d.N, rows,          d.N, gain, d.Nz, nullptr, nullptr};
     }
     launch_sgemm(g, d.n_par, st);
 }
 
 void fold_psf_changed(mpi_ffl_handle *h) {
-    FoldState *s = fs(h);
-    if (!s) return;
-    for (int slot = 0; slot < 2; ++slot) s->stale[slot] = s->f[slot] != nullptr;  // until refold has succeeded
+    if (FoldState *s = fs(h))
+        for (int slot = 0; slot < 2; ++slot) s->stale[slot] = s->f[slot] != nullptr;
+}
+
+void fold_refresh(mpi_ffl_handle *h) {
+    const FoldState *s = fs(h);
+    if (!s || !(s->stale[0] || s->stale[1])) return;
     try {
-        for (int slot = 0; slot < 2; ++slot)
-            if (s->stale[slot]) refold(h, slot, nullptr);
+        const int first = s->stale[0] ? 0 : 1;
+        refold(h, first, s->stale[0] && s->stale[1] ? 2 : 1, nullptr);
     } catch (...) {  // a host allocation
     }
 }
@@ -418,8 +433,8 @@ void fold_psf_changed(mpi_ffl_handle *h) {
 void fold_release(mpi_ffl_handle *h) {
     FoldState *s = fs(h);
     if (!s) return;
-    for (void *p : {(void *)s->W, (void *)s->taps, (void *)s->WH, (void *)s->f[0], (void *)s->f[1], (void *)s->a[0],
-                    (void *)s->a[1], (void *)s->rows})
+    for (void *p : {(void *)s->W, (void *)s->taps, (void *)s->WH, (void *)s->f[0], (void *)s->f[1], (void *)s->a,
+                    (void *)s->rows})
         if (p) dev_free(p);
     delete s;
     h->fold_state = nullptr;

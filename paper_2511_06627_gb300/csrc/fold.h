@@ -17,18 +17,19 @@ inline int fold_taps(const Dims &d) { return d.Ne + d.Q * (d.N - 1); }
 // out[par][z][o][i] = sum_e W[par][o][e] g[z][e - D - Q i - kmin], z < nz, on the stream
 void launch_fold_taps(const double *W, const double *g, double *out, const Dims &d, int n_par, int nz,
                       cudaStream_t st);
-// W H in FP64 ([n_par][2 n_b][N]) for the handle's PSF (slot 0) or d H / d fwhm (slot 1),
-// valid until the next call; NULL when an allocation failed
-const double *fold_wh(mpi_ffl_handle *h, int slot, cudaStream_t st);
+// W H in FP64 ([n_par][2 n_b][N]) for the handle's PSF, valid until the next call or refold;
+// NULL when an allocation failed
+const double *fold_wh(mpi_ffl_handle *h, cudaStream_t st);
 
 // Staged path: W H in FP32, applied to the projections (forward) or to the data (adjoint).
 bool fold_fits(const Dims &d);                  // the rule by sizes
 int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st);  // operands built on first use
 void fold_forward(mpi_ffl_handle *h, int slot, const float *proj, const float *gain, float *data, cudaStream_t st);
 void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float *proj, cudaStream_t st);
-// After a new width: refolds the operands that were built. Those it could not refold are
-// left to their next use, which tries again and reports.
-void fold_psf_changed(mpi_ffl_handle *h);
+void fold_psf_changed(mpi_ffl_handle *h);       // marks the operands that were built as stale
+// Refolds the stale operands. Those it could not refold are left to their next use, which
+// tries again and reports.
+void fold_refresh(mpi_ffl_handle *h);
 void fold_release(mpi_ffl_handle *h);
 
 // C[crow[i]][ccol[n]] = scale[arow[i] / rdiv] sum_k A[arow[i]][acol[k]] B[k][n] in FP32
@@ -66,7 +67,8 @@ bool zfold_fits(const Dims &d);                      // the rule by sizes
 int zfold_ready(mpi_ffl_handle *h);                  // tables and workspace, on first use
 void zfold_forward(mpi_ffl_handle *h, const float *proj, float *data, cudaStream_t st);
 void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream_t st);
-void zfold_psf_changed(mpi_ffl_handle *h);           // as fold_psf_changed
+// Rebuilds the table of the width, or leaves it to its next use, which tries again and reports.
+void zfold_psf_changed(mpi_ffl_handle *h);
 void zfold_release(mpi_ffl_handle *h);
 
 }  // namespace mpiffl

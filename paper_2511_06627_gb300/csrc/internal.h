@@ -98,6 +98,11 @@ constexpr int kMaxHw = 8;          // largest supported half-width
 
 }  // namespace mpiffl
 
+// The PSF h and d h / d fwhm at k / Q, k = 0 .. htab_off, in FP64 (both are even in k).
+struct PsfTaps {
+    std::vector<double> h, dh;
+};
+
 struct mpi_ffl_handle {
     mpiffl::Dims d{};
     int device = 0;
@@ -108,6 +113,7 @@ struct mpi_ffl_handle {
     std::vector<double> angles;
     std::vector<float> gains;
     double fwhm = 0, amp = 0, phase = 0;
+    PsfTaps taps;               // of fwhm
     int zigzag = 1;
     std::vector<float> dgamma;  // nb complex
 

@@ -546,11 +546,10 @@ size_t tap_len(const Dims &d) { return (size_t)d.Q * (2 * d.Nz - 2) + 2 * d.D + 
 // hz for the handle's width; its buffers are there
 bool fold_h(mpi_ffl_handle *h) {
     const Dims &d = h->d;
-    const double a = h->fwhm / (2.0 * langevin_half_point_host());
     const double kPi = 3.14159265358979323846;
     std::vector<double> taps(tap_len(d));
-    for (size_t i = 0; i < taps.size(); ++i)
-        taps[i] = 3.0 * langevin_d1_host((((double)i - d.D) / d.Q - (d.Nz - 1)) / a);
+    const int last = d.Q * (d.Nz - 1) + d.D;  // taps[last] is h(0); one past the other end has weight 0
+    for (int i = 0; i < (int)taps.size(); ++i) taps[i] = h->taps.h[std::abs(i - last)];
     std::vector<double2> drive(d.S);
     for (int r = 0; r < d.S; ++r) {
         const double ph = 2.0 * kPi * r / d.S + h->phase;
