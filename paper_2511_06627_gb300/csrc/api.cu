@@ -16,7 +16,7 @@
 using namespace mpiffl;
 
 // the z-drive scan (defined with its entry points below)
-void z_init(mpi_ffl_handle *h);
+void z_check(mpi_ffl_handle *h);
 void z_line_forward(mpi_ffl_handle *h, const float *proj, float *b, cudaStream_t st);
 void z_line_adjoint(mpi_ffl_handle *h, const float *b, float *proj, cudaStream_t st);
 void adjoint_z_impl(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st);
@@ -855,7 +855,7 @@ void scans_forward(mpi_ffl_handle *h, const float *x, float *r, cudaStream_t st,
         return;
     }
     const bool both = (h->scans & MPI_FFL_SCAN_X) != 0;
-    z_init(h);
+    z_check(h);
     const bool packed = stage_p(h, x, h->w_proj, st, both ? pack_target(h, h->t_htab) : ProjPack{}, true, mom);
     if (both) {
         line_forward_impl(h, h->w_proj, r, h->t_htab, h->t_gain, st, packed);
@@ -1216,7 +1216,7 @@ extern "C" int mpi_ffl_set_scans(mpi_ffl_handle *h, int32_t scans) {
         }
         const Dims &d = h->d;
         CK(cudaDeviceSynchronize());
-        if (scans & MPI_FFL_SCAN_Z) z_init(h);
+        if (scans & MPI_FFL_SCAN_Z) z_check(h);
         const int n = ((scans & MPI_FFL_SCAN_X) ? 1 : 0) + ((scans & MPI_FFL_SCAN_Z) ? 1 : 0);
         if (n == 2 && !h->w_scanproj) {
             // residual and power-iteration data of both scans, and the two line transposes
@@ -1378,18 +1378,32 @@ int float_bits(float f) {
     return i;
 }
 
-// Tables of the z-drive scan, in double precision on the host: the slow raster's
-// detector column and fraction per (parity, j), the drive's fine z offset, fraction
-// and velocity per phase r = j mod S, the periods reading each column, and the
-// transpose's taps grouped by residue of the fine index modulo Q.
-void z_init(mpi_ffl_handle *h) {
-    if (h->z_ready) return;
+// The scans that the z-drive takes; the same for both forms of its kernels.
+void z_check(mpi_ffl_handle *h) {
+    if (h->z_checked) return;
     const Dims &d = h->d;
-    const int L = d.L, S = d.S, N = d.N, P = d.P, Q = d.Q, npar = d.n_par;
-    if ((size_t)(d.Nz + 1) * S * 4 > 200 * 1024) {
+    if ((size_t)(d.Nz + 1) * d.S * 4 > 200 * 1024) {
         h->err = "the z-drive transpose keeps (N_z + 1) x S floats in shared memory (at most 200 KB)";
         throw Fail{MPI_FFL_ERR_UNSUPPORTED};
     }
+    int no = 0;  // offsets o = e - Q l that a line's samples touch
+    for (int r = 0; r < d.S; ++r) no = std::max(no, (int)std::floor(z_drive_offset_host(h, r)) + 2);
+    if (zsyn_smem(d, no) > 227 * 1024 || zdft_fwd_smem(d) > 227 * 1024) {
+        h->err = "the fused z-drive kernels keep twiddles and tiles in shared memory (at most 227 KB)";
+        throw Fail{MPI_FFL_ERR_UNSUPPORTED};
+    }
+    h->tz_no = no;
+    h->z_checked = true;
+}
+
+// Tables of the sample-by-sample kernels and stages, on their first use, in double precision on
+// the host: the slow raster's detector column and fraction per (parity, j), the drive's fine z
+// offset, fraction and velocity per phase r = j mod S, the periods reading each column, and the
+// transpose's taps grouped by residue of the fine index modulo Q.
+void z_sampled_tables(mpi_ffl_handle *h) {
+    if (h->z_ready) return;
+    const Dims &d = h->d;
+    const int L = d.L, S = d.S, N = d.N, P = d.P, Q = d.Q, npar = d.n_par;
     const double slope = (double)(N - 1) / (double)(L - 1);
     std::vector<int> u0((size_t)npar * L);
     std::vector<float2> ua((size_t)npar * L);
@@ -1436,8 +1450,7 @@ void z_init(mpi_ffl_handle *h) {
     }
     ptr[Q] = (int)taps.size();
     // the same taps by offset o = e - Q l within a line's cells (the fused transpose)
-    int no = 0;
-    for (int r = 0; r < S; ++r) no = std::max(no, n0[r] + 2);
+    const int no = h->tz_no;
     std::vector<int> optr(no + 1, 0);
     std::vector<int2> otap;
     for (int o = 0; o < no; ++o) {
@@ -1448,21 +1461,20 @@ void z_init(mpi_ffl_handle *h) {
         }
     }
     optr[no] = (int)otap.size();
-    h->tz_no = no;
-    if (zsyn_smem(d, no) > 227 * 1024 || zdft_fwd_smem(d) > 227 * 1024) {
-        h->err = "the fused z-drive kernels keep twiddles and tiles in shared memory (at most 227 KB)";
-        throw Fail{MPI_FFL_ERR_UNSUPPORTED};
-    }
-    upload(h, &h->tz_optr, optr);
-    upload(h, &h->tz_otap, otap);
-    upload(h, &h->tz_ua, ua);
-    upload(h, &h->tz_n0, n0);
-    upload(h, &h->tz_f0, f0);
-    upload(h, &h->tz_v, v);
-    upload(h, &h->tz_plo, plo);
-    upload(h, &h->tz_phi, phi);
-    upload(h, &h->tz_tap_ptr, ptr);
-    upload(h, &h->tz_taps, taps);
+    // (tables of an earlier call that ran out of memory are there already)
+    auto up = [&](auto **p, const auto &v) {
+        if (!*p) upload(h, p, v);
+    };
+    up(&h->tz_optr, optr);
+    up(&h->tz_otap, otap);
+    up(&h->tz_ua, ua);
+    up(&h->tz_n0, n0);
+    up(&h->tz_f0, f0);
+    up(&h->tz_v, v);
+    up(&h->tz_plo, plo);
+    up(&h->tz_phi, phi);
+    up(&h->tz_tap_ptr, ptr);
+    up(&h->tz_taps, taps);
     uploads_done(h);
     h->z_ready = 1;
 }
@@ -1524,9 +1536,11 @@ bool use_zfold(mpi_ffl_handle *h) {
     return false;
 }
 
-void ensure_z_workspace(mpi_ffl_handle *h) {
+// Tables and workspace of the sample-by-sample kernels.
+void ensure_z_sampled(mpi_ffl_handle *h) {
     const Dims &d = h->d;
     try {
+        z_sampled_tables(h);
         if (!h->w_fine_z) dev_alloc(h, &h->w_fine_z, (size_t)d.M * d.N * d.Nez);
         if (!h->w_zcoef) dev_alloc(h, &h->w_zcoef, (size_t)d.M * d.Nz * (2 * d.hw + 1) * d.S);
         ensure_projT(h);
@@ -1545,7 +1559,7 @@ void z_line_forward(mpi_ffl_handle *h, const float *proj, float *b, cudaStream_t
         check_launch(h, "z-drive forward");
         return;
     }
-    ensure_z_workspace(h);
+    ensure_z_sampled(h);
     zstage_h(h, proj, h->w_fine_z, st);
     // E_z V_z B fused with S D_Gamma F: the time signal is not stored
     TIMED(MPI_FFL_K_ZDRIVE, launch_zdft_fwd(h->w_fine_z, z_tables(h), h->t_gain, h->t_tw1, h->t_tw2_ro, h->t_dgam, b,
@@ -1560,7 +1574,7 @@ void z_line_adjoint(mpi_ffl_handle *h, const float *b, float *proj, cudaStream_t
         TIMED(MPI_FFL_K_ZDRIVE, zfold_adjoint(h, b, proj, st));
         h->launches += 2;
     } else {
-        ensure_z_workspace(h);
+        ensure_z_sampled(h);
         TIMED(MPI_FFL_K_ZDRIVE, launch_zdft_adj(b, h->t_tw1, h->t_tw2_qr, h->t_dgam, z_tables(h), h->t_gain,
                                                 h->w_zcoef, h->w_fine_z, d, h->zigzag, st));
         zstage_ht(h, h->w_fine_z, proj, st);
@@ -1569,13 +1583,13 @@ void z_line_adjoint(mpi_ffl_handle *h, const float *b, float *proj, cudaStream_t
 }
 
 void forward_z_impl(mpi_ffl_handle *h, const float *x, float *b, cudaStream_t st) {
-    z_init(h);
+    z_check(h);
     stage_p(h, x, h->w_proj, st);
     z_line_forward(h, h->w_proj, b, st);
 }
 
 void adjoint_z_impl(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st) {
-    z_init(h);
+    z_check(h);
     z_line_adjoint(h, b, h->w_proj, st);
     stage_pt(h, h->w_proj, x, st);
 }
@@ -1613,7 +1627,8 @@ extern "C" int mpi_ffl_apply_stage_zdrive(mpi_ffl_handle *h, int32_t stage, int3
             h->err = "bad z-drive stage or NULL buffer";
             return MPI_FFL_ERR_INVALID_ARG;
         }
-        z_init(h);
+        z_check(h);
+        if (stage == 2) z_sampled_tables(h);
         cudaStream_t st = S(stream);
         if (stage == 1) {
             if (transpose) zstage_ht(h, in, out, st);

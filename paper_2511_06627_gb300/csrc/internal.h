@@ -206,7 +206,8 @@ struct mpi_ffl_handle {
     float *t_coil = nullptr;    // N_z N
     float *w_projc = nullptr;   // M N_z N: coil-weighted projections (collinear model)
     // z-drive scan (k_zdrive.cu): tables and workspace, built on first use
-    int z_ready = 0;
+    int z_ready = 0;          // the tables below are there
+    bool z_checked = false;   // z_check accepted the scan
     int *tz_n0 = nullptr, *tz_plo = nullptr, *tz_phi = nullptr, *tz_tap_ptr = nullptr;
     float *tz_f0 = nullptr, *tz_v = nullptr;
     float2 *tz_ua = nullptr;

@@ -21,6 +21,7 @@
 // which is half the FMAs; the adjoint's convolution writes G_0 + G_1 and G_0 - G_1.
 #include <algorithm>
 #include <cmath>
+#include <utility>
 #include <vector>
 
 #include "collapsed.h"
@@ -45,37 +46,34 @@ struct ZFold {
     float *part = nullptr; // [parts of K][M][N_z][N], sums of the adjoint's last product
     float *eo = nullptr;   // [M][N_z][e, o][ldu] of the projections (halved)
     int ldk = 0, ldu = 0;
-    // inputs of hz, kept so that a new width allocates nothing: FP64 taps, and the drive per phase
+    // inputs of the tables in one array, kept so that a new width allocates nothing: FP64 taps, the
+    // drive per phase, e^{2 pi i p / P}
     double *taps = nullptr;
-    double2 *drive = nullptr;
+    void *mem = nullptr;   // one allocation that holds all of these
     bool ready = false;
     bool stale = false;  // hz is of another width: rebuilt on the next use
 };
 
 ZFold *zs(const mpi_ffl_handle *h) { return reinterpret_cast<ZFold *>(h->zfold_state); }
 
-template <class T>
-bool zalloc(T **p, size_t n) {
-    if (*p) return true;
-    if (dev_malloc((void **)p, n * sizeof(T)) != cudaSuccess) {
-        *p = nullptr;
-        cudaGetLastError();
-        return false;
-    }
-    return true;
-}
-
 // One thread per (par, c, r) walks the periods in the order of increasing column, keeps the
 // sums of the two columns the sample lies between and writes a column once it is complete.
-// The slow position c = (N - 1) j / (L - 1) (from the other end on reversed lines) is exact.
-__global__ void __launch_bounds__(128) k_zfold_k(const double2 *__restrict__ unit_p, double *__restrict__ K, Dims d,
-                                                 int nk) {
+// The slow position c = (N - 1) j / (L - 1) (from the other end on reversed lines) goes on by a
+// whole number and an exact remainder a period. Bound by the latency of a thread's chain and by
+// the FP64 pipe, so a block is one warp: they spread over the SMs.
+__global__ void __launch_bounds__(32) k_zfold_k(const double2 *__restrict__ unit_p, double *__restrict__ K, Dims d,
+                                                int nk) {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= nk) return;
     const int r = n % d.S, c = n / d.S % d.W, par = n / (d.S * d.W);
     const int dd = (c + 1) / 2;
     const bool sine = c > 0 && c % 2 == 0;
-    const long long N1 = d.N - 1, Lm1 = d.L - 1;
+    const long long step = (long long)(d.N - 1) * d.S, start = (long long)(d.N - 1) * (par ? d.S - 1 - r : r);
+    const int Lm1 = d.L - 1, ustep = (int)(step / Lm1), rstep = (int)(step % Lm1);
+    const int pstep = par ? d.P - dd % d.P : dd % d.P;  // of dd p modulo P
+    const double inv = 1.0 / (double)Lm1;
+    int u0 = (int)(start / Lm1), rem = (int)(start % Lm1);
+    int ip = par ? (int)((long long)dd * (d.P - 1) % d.P) : 0;
     double acc0 = 0.0, acc1 = 0.0;
     int u = 0;
     auto flush = [&]() {
@@ -84,17 +82,21 @@ __global__ void __launch_bounds__(128) k_zfold_k(const double2 *__restrict__ uni
         acc1 = 0.0;
         ++u;
     };
+#pragma unroll 4
     for (int q = 0; q < d.P; ++q) {
-        const int p = par ? d.P - 1 - q : q;
-        const long long j = (long long)p * d.S + r;
-        const long long num = N1 * (par ? Lm1 - j : j);
-        const int u0 = (int)(num / Lm1);
-        const double a = (double)(num - (long long)u0 * Lm1) / (double)Lm1;
+        const double2 w = unit_p[ip];
+        const double a = (double)rem * inv, tw = sine ? w.y : w.x;
         while (u < u0) flush();
-        const double2 w = unit_p[(int)((long long)dd * p % d.P)];
-        const double tw = sine ? w.y : w.x;
         acc0 = fma(1.0 - a, tw, acc0);
         acc1 = fma(a, tw, acc1);
+        u0 += ustep;
+        rem += rstep;
+        if (rem >= Lm1) {
+            rem -= Lm1;
+            ++u0;
+        }
+        ip += pstep;
+        if (ip >= d.P) ip -= d.P;
     }
     while (u < d.N) flush();
 }
@@ -541,24 +543,37 @@ int z_parts(const Dims &d) {
     return (nk + z_kper(d) - 1) / z_kper(d);
 }
 
-size_t tap_len(const Dims &d) { return (size_t)d.Q * (2 * d.Nz - 2) + 2 * d.D + 2; }
+size_t tap_len(const Dims &d) { return ((size_t)d.Q * (2 * d.Nz - 2) + 2 * d.D + 2 + 1) & ~(size_t)1; }
+size_t input_len(const Dims &d) { return tap_len(d) + 2 * ((size_t)d.S + d.P); }
+double2 *drive_of(const ZFold *s, const Dims &d) { return reinterpret_cast<double2 *>(s->taps + tap_len(d)); }
 
-// hz for the handle's width; its buffers are there
-bool fold_h(mpi_ffl_handle *h) {
+// hz for the handle's width; all: the other inputs of the tables are uploaded too
+bool fold_h(mpi_ffl_handle *h, bool all) {
     const Dims &d = h->d;
     const double kPi = 3.14159265358979323846;
-    std::vector<double> taps(tap_len(d));
-    const int last = d.Q * (d.Nz - 1) + d.D;  // taps[last] is h(0); one past the other end has weight 0
-    for (int i = 0; i < (int)taps.size(); ++i) taps[i] = h->taps.h[std::abs(i - last)];
-    std::vector<double2> drive(d.S);
-    for (int r = 0; r < d.S; ++r) {
-        const double ph = 2.0 * kPi * r / d.S + h->phase;
-        drive[r] = make_double2(z_drive_offset_host(h, r), h->amp * (2.0 * kPi / d.S) * std::cos(ph));
+    std::vector<double> in(all ? input_len(d) : tap_len(d), 0.0);
+    const int last = d.Q * (d.Nz - 1) + d.D;  // in[last] is h(0); the one past the other end has weight 0
+    for (int i = 0; i <= 2 * last + 1; ++i) in[i] = h->taps.h[std::abs(i - last)];
+    if (all) {
+        double *p = in.data() + tap_len(d);
+        for (int r = 0; r < d.S; ++r) {
+            const double ph = 2.0 * kPi * r / d.S + h->phase;
+            *p++ = z_drive_offset_host(h, r);
+            *p++ = h->amp * (2.0 * kPi / d.S) * std::cos(ph);
+        }
+        for (int q = 0; q < d.P; ++q) {
+            *p++ = std::cos(2.0 * kPi * q / d.P);
+            *p++ = std::sin(2.0 * kPi * q / d.P);
+        }
     }
     ZFold *s = zs(h);
-    cudaMemcpy(s->taps, taps.data(), taps.size() * sizeof(double), cudaMemcpyHostToDevice);
-    cudaMemcpy(s->drive, drive.data(), drive.size() * sizeof(double2), cudaMemcpyHostToDevice);
-    k_zfold_h<<<dim3((d.S + 127) / 128, 2 * d.Nz - 1), 128>>>(s->taps, s->drive, s->hz, d.Nz, d.S, d.Q, d.D);
+    if (cudaMemcpy(s->taps, in.data(), in.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) return false;
+    k_zfold_h<<<dim3((d.S + 127) / 128, 2 * d.Nz - 1), 128>>>(s->taps, drive_of(s, d), s->hz, d.Nz, d.S, d.Q, d.D);
+    return true;
+}
+
+// Waits for the tables: the caller's stream does not wait for the legacy stream they are made on
+bool tables_done(ZFold *s) {
     if (cudaStreamSynchronize(nullptr) != cudaSuccess) return false;
     s->stale = false;
     return true;
@@ -584,38 +599,55 @@ bool zfold_fits(const Dims &d) {
 int zfold_ready(mpi_ffl_handle *h) {
     if (!h->zfold_state) h->zfold_state = new ZFold();
     ZFold *s = zs(h);
-    if (s->ready) return !s->stale || fold_h(h) ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
+    if (s->ready) return !s->stale || (fold_h(h, false) && tables_done(s)) ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
     const Dims &d = h->d;
     const bool hv = halved(d);
     const int nk = (hv ? 1 : d.n_par) * d.W * d.S, Nh = (d.N + 1) / 2;
+    const size_t rows = (size_t)d.M * d.Nz;
     s->ldk = (nk + 3) / 4 * 4;
     s->ldu = ((hv ? Nh : d.N) + 3) / 4 * 4;
-    const size_t kf_len = (size_t)(hv ? 2 * Nh : d.N) * s->ldk, ka_len = (size_t)(hv ? 2 : 1) * nk * s->ldu;
-    double2 *unit_p = nullptr;
+    // One allocation: a dozen of them took a third of a small scan's first product. K in FP64 lies
+    // where G will be, if it fits.
+    size_t used = 0;
+    std::vector<std::pair<void **, size_t>> place;
+    auto hold = [&](auto **p, size_t n) {
+        place.emplace_back((void **)p, used);
+        used = (used + std::max<size_t>(n, 1) * sizeof(**p) + 255) & ~(size_t)255;
+    };
+    hold(&s->kf, (size_t)(hv ? 2 * Nh : d.N) * s->ldk);
+    hold(&s->ka, (size_t)(hv ? 2 : 1) * nk * s->ldu);
+    hold(&s->df, dft_f_len(d));
+    hold(&s->da, dft_a_len(d));
+    const size_t padded = used;  // arrays with columns past the last, which are zero
+    hold(&s->hz, (size_t)(2 * d.Nz - 1) * d.S);
+    hold(&s->cols, (size_t)2 * d.nb);
+    hold(&s->taps, input_len(d));
+    hold(&s->g, g_len(d));
+    hold(&s->t, rows * d.W * d.S);
+    hold(&s->part, (size_t)z_parts(d) * rows * d.N);
+    if (hv) hold(&s->eo, rows * 2 * s->ldu);
+    const size_t k_len = (size_t)d.N * nk;
+    const bool over_g = k_len * sizeof(double) <= g_len(d) * sizeof(float);
     double *K = nullptr;
     int rc = MPI_FFL_ERR_OOM;
-    const bool ok = zalloc(&s->kf, kf_len) && zalloc(&s->ka, ka_len) && zalloc(&K, (size_t)d.N * nk) &&
-              (!hv || zalloc(&s->eo, (size_t)d.M * d.Nz * 2 * s->ldu)) &&
-              zalloc(&s->hz, (size_t)(2 * d.Nz - 1) * d.S) && zalloc(&s->df, dft_f_len(d)) &&
-              zalloc(&s->da, dft_a_len(d)) && zalloc(&s->cols, (size_t)2 * d.nb) && zalloc(&s->g, g_len(d)) &&
-              zalloc(&s->t, (size_t)d.M * d.Nz * d.W * d.S) && zalloc(&unit_p, d.P) &&
-              zalloc(&s->part, (size_t)z_parts(d) * d.M * d.Nz * d.N) && zalloc(&s->taps, tap_len(d)) &&
-              zalloc(&s->drive, d.S);
-    if (ok) {
-        const double kPi = 3.14159265358979323846;
-        std::vector<double2> up(d.P);
-        for (int p = 0; p < d.P; ++p) up[p] = make_double2(std::cos(2.0 * kPi * p / d.P), std::sin(2.0 * kPi * p / d.P));
-        cudaMemcpy(unit_p, up.data(), up.size() * sizeof(double2), cudaMemcpyHostToDevice);
-        cudaMemset(s->kf, 0, kf_len * sizeof(float));  // the columns past the last
-        cudaMemset(s->ka, 0, ka_len * sizeof(float));
-        cudaMemset(s->df, 0, dft_f_len(d) * sizeof(float));
-        cudaMemset(s->da, 0, dft_a_len(d) * sizeof(float));
-        k_zfold_k<<<(nk + 127) / 128, 128>>>(unit_p, K, d, nk);
-        k_zfold_operands<<<608, 256>>>(K, s->kf, s->ka, d.N, nk, s->ldk, s->ldu, hv);
-        k_zfold_dft<<<dim3(64, d.hw + 1), 128>>>(h->t_dgam, s->df, s->da, s->cols, d);
-        rc = fold_h(h) ? MPI_FFL_OK : MPI_FFL_ERR_CUDA;
+    if (dev_malloc(&s->mem, used) != cudaSuccess) {
+        s->mem = nullptr;
+        cudaGetLastError();
+    } else if (!over_g && dev_malloc((void **)&K, k_len * sizeof(double)) != cudaSuccess) {
+        K = nullptr;
+        cudaGetLastError();
+    } else {
+        for (auto &p : place) *p.first = (char *)s->mem + p.second;
+        double *k64 = over_g ? reinterpret_cast<double *>(s->g) : K;
+        cudaMemsetAsync(s->mem, 0, padded, nullptr);
+        rc = MPI_FFL_ERR_CUDA;
+        if (fold_h(h, true)) {
+            k_zfold_k<<<(nk + 31) / 32, 32>>>(drive_of(s, d) + d.S, k64, d, nk);
+            k_zfold_operands<<<608, 256>>>(k64, s->kf, s->ka, d.N, nk, s->ldk, s->ldu, hv);
+            k_zfold_dft<<<dim3(64, d.hw + 1), 128>>>(h->t_dgam, s->df, s->da, s->cols, d);
+            if (cudaGetLastError() == cudaSuccess && tables_done(s)) rc = MPI_FFL_OK;
+        }
     }
-    if (unit_p) dev_free(unit_p);
     if (K) dev_free(K);
     if (rc != MPI_FFL_OK) {  // nothing of a failed build is kept
         zfold_release(h);
@@ -628,9 +660,9 @@ int zfold_ready(mpi_ffl_handle *h) {
 void zfold_psf_changed(mpi_ffl_handle *h) {
     ZFold *s = zs(h);
     if (!s || !s->ready) return;
-    s->stale = true;  // until fold_h has succeeded
+    s->stale = true;  // until the table is there
     try {
-        fold_h(h);
+        if (fold_h(h, false)) tables_done(s);
     } catch (...) {  // a host allocation
     }
 }
@@ -732,9 +764,7 @@ void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream
 void zfold_release(mpi_ffl_handle *h) {
     ZFold *s = zs(h);
     if (!s) return;
-    for (void *p : {(void *)s->kf, (void *)s->ka, (void *)s->hz, (void *)s->df, (void *)s->da, (void *)s->cols,
-                    (void *)s->g, (void *)s->t, (void *)s->part, (void *)s->eo, (void *)s->taps, (void *)s->drive})
-        if (p) dev_free(p);
+    if (s->mem) dev_free(s->mem);
     delete s;
     h->zfold_state = nullptr;
 }
