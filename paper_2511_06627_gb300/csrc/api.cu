@@ -17,6 +17,8 @@ using namespace mpiffl;
 
 // the z-drive scan (defined with its entry points below)
 void z_check(mpi_ffl_handle *h);
+bool use_zfold(mpi_ffl_handle *h);
+void ensure_z_sampled(mpi_ffl_handle *h);
 void z_line_forward(mpi_ffl_handle *h, const float *proj, float *b, cudaStream_t st);
 void z_line_adjoint(mpi_ffl_handle *h, const float *b, float *proj, cudaStream_t st);
 void adjoint_z_impl(mpi_ffl_handle *h, const float *b, float *x, cudaStream_t st);
@@ -1216,7 +1218,11 @@ extern "C" int mpi_ffl_set_scans(mpi_ffl_handle *h, int32_t scans) {
         }
         const Dims &d = h->d;
         CK(cudaDeviceSynchronize());
-        if (scans & MPI_FFL_SCAN_Z) z_check(h);
+        if (scans & MPI_FFL_SCAN_Z) {
+            // what the scan's first product would allocate: that product may be captured
+            z_check(h);
+            if (!use_zfold(h)) ensure_z_sampled(h);
+        }
         const int n = ((scans & MPI_FFL_SCAN_X) ? 1 : 0) + ((scans & MPI_FFL_SCAN_Z) ? 1 : 0);
         if (n == 2 && !h->w_scanproj) {
             // residual and power-iteration data of both scans, and the two line transposes

@@ -25,7 +25,8 @@ struct FoldState {
     // FP32 operands: B of the forward [n_par][N][ldf] of slot 0 (h) and 1 (d h / d fwhm), and of
     // the adjoint [n_par][2 n_b][lda] of slot 0
     float *f[2] = {nullptr, nullptr}, *a = nullptr;
-    bool stale[2] = {false, false};  // of another width: refolded on the next use
+    bool used[2] = {false, false};   // a call has applied the slot
+    bool ready[2] = {false, false};  // its operands are those of the handle's width
     int ldf = 0, lda = 0;
     int *rows = nullptr;  // lines of trajectory 0, then of trajectory 1
     int nrows[2] = {0, 0};
@@ -218,7 +219,14 @@ int fold_slots(mpi_ffl_handle *h, int first, int n, cudaStream_t st) {
     return MPI_FFL_OK;
 }
 
-// the operands of slots [first, first + n), whose buffers are there
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) cudaGetLastError();  // the legacy stream, which cannot be
+    return c == cudaStreamCaptureStatusActive;
+}
+
+// The operands of slots [first, first + n), whose buffers are there. Under capture the fold
+// becomes part of the graph, whose replays then fold too, and the slot does not count as ready.
 int refold(mpi_ffl_handle *h, int first, int n, cudaStream_t st) {
     const Dims &d = h->d;
     const int rc = fold_slots(h, first, n, st);
@@ -227,9 +235,10 @@ int refold(mpi_ffl_handle *h, int first, int n, cudaStream_t st) {
     const int R = 2 * d.nb, work = std::max(d.N * s->ldf, R * s->lda);
     k_fold_operands<<<dim3(std::min(608, (work + 255) / 256), d.n_par, n), 256, 0, st>>>(
         s->WH, s->f[first], s->f[1], first == 0 ? s->a : nullptr, R, d.N, s->ldf, s->lda);
+    if (capturing(st)) return MPI_FFL_OK;
     // another stream may use the operands next
     if (cudaStreamSynchronize(st) != cudaSuccess) return MPI_FFL_ERR_CUDA;
-    for (int k = first; k < first + n; ++k) s->stale[k] = false;
+    for (int k = first; k < first + n; ++k) s->ready[k] = s->used[k] = true;
     return MPI_FFL_OK;
 }
 
@@ -357,7 +366,7 @@ bool fold_fits(const Dims &d) {
 int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
     const Dims &d = h->d;
     FoldState *s = state(h);
-    if (s->f[slot] && !s->stale[slot]) return MPI_FFL_OK;
+    if (s->ready[slot]) return MPI_FFL_OK;
     const int R = 2 * d.nb;
     if (!s->rows) {
         std::vector<int> rows;
@@ -375,18 +384,17 @@ int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
     }
     s->ldf = (R + 3) / 4 * 4;
     s->lda = (d.N + 3) / 4 * 4;
+    // the buffers of both slots: the first gradient may be captured after a forward outside
     int rc = MPI_FFL_ERR_OOM;
-    if (falloc(&s->f[slot], (size_t)d.n_par * d.N * s->ldf) &&
-        (slot || falloc(&s->a, (size_t)d.n_par * R * s->lda)))
+    const size_t f_len = (size_t)d.n_par * d.N * s->ldf;
+    if (falloc(&s->f[0], f_len) && falloc(&s->f[1], f_len) && falloc(&s->a, (size_t)d.n_par * R * s->lda))
         rc = refold(h, slot, 1, st);
-    if (rc != MPI_FFL_OK) {  // no operands of a failed build are kept: the next call tries again
-        for (float **p : {&s->f[slot], slot ? nullptr : &s->a})
-            if (p && *p) {
+    if (rc != MPI_FFL_OK && !s->used[0] && !s->used[1])  // no operands of a failed build are kept
+        for (float **p : {&s->f[0], &s->f[1], &s->a})
+            if (*p) {
                 dev_free(*p);
                 *p = nullptr;
             }
-        s->stale[slot] = false;
-    }
     return rc;
 }
 
@@ -416,16 +424,16 @@ void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float
 }
 
 void fold_psf_changed(mpi_ffl_handle *h) {
-    if (FoldState *s = fs(h))
-        for (int slot = 0; slot < 2; ++slot) s->stale[slot] = s->f[slot] != nullptr;
+    if (FoldState *s = fs(h)) s->ready[0] = s->ready[1] = false;
 }
 
 void fold_refresh(mpi_ffl_handle *h) {
     const FoldState *s = fs(h);
-    if (!s || !(s->stale[0] || s->stale[1])) return;
+    if (!s) return;
+    const bool need[2] = {s->used[0] && !s->ready[0], s->used[1] && !s->ready[1]};
+    if (!need[0] && !need[1]) return;
     try {
-        const int first = s->stale[0] ? 0 : 1;
-        refold(h, first, s->stale[0] && s->stale[1] ? 2 : 1, nullptr);
+        refold(h, need[0] ? 0 : 1, need[0] && need[1] ? 2 : 1, nullptr);
     } catch (...) {  // a host allocation
     }
 }

@@ -26,8 +26,8 @@ bool fold_fits(const Dims &d);                  // the rule by sizes
 int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st);  // operands built on first use
 void fold_forward(mpi_ffl_handle *h, int slot, const float *proj, const float *gain, float *data, cudaStream_t st);
 void fold_adjoint(mpi_ffl_handle *h, const float *data, const float *gain, float *proj, cudaStream_t st);
-void fold_psf_changed(mpi_ffl_handle *h);       // marks the operands that were built as stale
-// Refolds the stale operands. Those it could not refold are left to their next use, which
+void fold_psf_changed(mpi_ffl_handle *h);       // marks the operands as stale
+// Refolds the stale operands of the slots that calls have used. Those it could not refold are left to their next use, which
 // tries again and reports.
 void fold_refresh(mpi_ffl_handle *h);
 void fold_release(mpi_ffl_handle *h);
