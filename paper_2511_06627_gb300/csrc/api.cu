@@ -1128,11 +1128,13 @@ static int set_path_impl(mpi_ffl_handle *h, int32_t path) {
             col_init(h);  // W and W H are built on first use
         } catch (...) {
             col_release(h);
+            fold_trim(h);
             h->err = "building the collapsed line operator failed";
             return MPI_FFL_ERR_OOM;
         }
         if (col_init_oom(h)) {  // nothing of a failed build is kept: the next call retries
             col_release(h);
+            fold_trim(h);
             h->err = "device allocation failed while building the collapsed line operator";
             return MPI_FFL_ERR_OOM;
         }
@@ -1172,9 +1174,14 @@ extern "C" int mpi_ffl_set_psf_model(mpi_ffl_handle *h, int32_t model) {
         }
         CK(cudaDeviceSynchronize());
         if (model == MPI_FFL_PSF_TENSOR && !ten_ready(h)) {
-            if (!h->col_state) col_init(h);
-            const int rc = ten_init(h);
+            const bool had = h->col_state != nullptr;
+            if (!had) col_init(h);
+            int rc = col_init_oom(h) ? MPI_FFL_ERR_OOM : ten_init(h);
             if (rc != MPI_FFL_OK) {
+                if (!had && rc == MPI_FFL_ERR_OOM) {  // nothing of a failed build is kept
+                    col_release(h);
+                    fold_trim(h);
+                }
                 h->err = rc == MPI_FFL_ERR_UNSUPPORTED
                              ? "the tensor PSF needs the collapsed line operator, which this shape does not support"
                              : "building the tensor-PSF operator failed";

@@ -363,11 +363,13 @@ bool fold_fits(const Dims &d) {
     return folded <= staged && (double)d.n_par * 2 * d.nb * d.Ne * sizeof(double) <= 512e6;
 }
 
-int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
+namespace {
+
+// the staged path's lines and buffers, of both slots: the first gradient may be captured after a
+// forward outside
+int staged_buffers(mpi_ffl_handle *h) {
     const Dims &d = h->d;
-    FoldState *s = state(h);
-    if (s->ready[slot]) return MPI_FFL_OK;
-    const int R = 2 * d.nb;
+    FoldState *s = fs(h);
     if (!s->rows) {
         std::vector<int> rows;
         for (int par = 0; par < d.n_par; ++par) {
@@ -382,20 +384,31 @@ int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
             return MPI_FFL_ERR_CUDA;
         }
     }
+    const int R = 2 * d.nb;
     s->ldf = (R + 3) / 4 * 4;
     s->lda = (d.N + 3) / 4 * 4;
-    // the buffers of both slots: the first gradient may be captured after a forward outside
-    int rc = MPI_FFL_ERR_OOM;
     const size_t f_len = (size_t)d.n_par * d.N * s->ldf;
-    if (falloc(&s->f[0], f_len) && falloc(&s->f[1], f_len) && falloc(&s->a, (size_t)d.n_par * R * s->lda))
-        rc = refold(h, slot, 1, st);
-    if (rc != MPI_FFL_OK && !s->used[0] && !s->used[1])  // no operands of a failed build are kept
-        for (float **p : {&s->f[0], &s->f[1], &s->a})
-            if (*p) {
-                dev_free(*p);
-                *p = nullptr;
-            }
+    return falloc(&s->f[0], f_len) && falloc(&s->f[1], f_len) && falloc(&s->a, (size_t)d.n_par * R * s->lda)
+               ? MPI_FFL_OK
+               : MPI_FFL_ERR_OOM;
+}
+
+}  // namespace
+
+int fold_ready(mpi_ffl_handle *h, int slot, cudaStream_t st) {
+    FoldState *s = state(h);
+    if (s->ready[slot]) return MPI_FFL_OK;
+    int rc = staged_buffers(h);
+    if (rc == MPI_FFL_OK) rc = refold(h, slot, 1, st);
+    if (rc != MPI_FFL_OK) fold_trim(h);
     return rc;
+}
+
+// Nothing of a failed build is kept: without operands of the staged path or of the collapsed
+// operator in use the next call builds all of it again.
+void fold_trim(mpi_ffl_handle *h) {
+    const FoldState *s = fs(h);
+    if (s && !s->used[0] && !s->used[1] && !col_supported(h)) fold_release(h);
 }
 
 void fold_forward(mpi_ffl_handle *h, int slot, const float *proj, const float *gain, float *data, cudaStream_t st) {

@@ -30,6 +30,7 @@ void fold_psf_changed(mpi_ffl_handle *h);       // marks the operands as stale
 // Refolds the stale operands of the slots that calls have used. Those it could not refold are left to their next use, which
 // tries again and reports.
 void fold_refresh(mpi_ffl_handle *h);
+void fold_trim(mpi_ffl_handle *h);              // after a failed build: releases what nothing uses
 void fold_release(mpi_ffl_handle *h);
 
 // C[crow[i]][ccol[n]] = scale[arow[i] / rdiv] sum_k A[arow[i]][acol[k]] B[k][n] in FP32
