@@ -150,7 +150,8 @@ typedef struct {
     int32_t n_bins;  /* (k_max - k_min + 1) * (2 half_width + 1)           */
     int32_t fine_len;/* N_e = (nx-1) Q + 2 ceil(A Q) + 1                  */
     int32_t line_len;/* L = S P                                           */
-    int64_t workspace_bytes; /* device memory the handle holds            */
+    int64_t workspace_bytes; /* device memory the handle holds at the time of the call: what it
+                                builds on first use is counted once it is there */
     int32_t fine_len_z; /* N_ez = (N_z - 1) Q + 2 D + 1: fine z grid of the z-drive scan */
 } mpi_ffl_sizes;
 

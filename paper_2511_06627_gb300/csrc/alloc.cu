@@ -48,6 +48,16 @@ cudaError_t dev_free(void *p) {
     return cudaFree(p);
 }
 
+int64_t dev_bytes(const BufferList &list) {
+    std::lock_guard<std::mutex> lock(g_mu);
+    int64_t sum = 0;
+    for (void *p : list) {
+        auto it = g_live.find(p);
+        if (it != g_live.end()) sum += (int64_t)it->second;
+    }
+    return sum;
+}
+
 }  // namespace mpiffl
 
 extern "C" int mpi_ffl_test_fail_alloc(int32_t nth) {

@@ -104,7 +104,6 @@ void dev_alloc(mpi_ffl_handle *h, T **p, size_t n) {
         set_err(h, "cudaMalloc of " + std::to_string(n * sizeof(T)) + " bytes failed: " + cudaGetErrorString(e));
         throw Fail{e == cudaErrorMemoryAllocation ? MPI_FFL_ERR_OOM : MPI_FFL_ERR_CUDA};
     }
-    h->bytes += (int64_t)(n * sizeof(T));
 }
 
 template <class T>
@@ -405,27 +404,30 @@ void group_table(mpi_ffl_handle *h) {
     upload(h, &h->t_groups, g);
 }
 
+// The handle's device allocations, those of its parts (tc.h, collapsed.h, fold.h) apart
+BufferList own_buffers(const mpi_ffl_handle *h) {
+    return {h->t_ang, h->t_gain, h->t_unit_gain, h->t_htab, h->t_dhtab, h->t_traj, h->t_csr_ptr,
+            h->t_csr, h->t_tw1, h->t_tw2_ro, h->t_tw2_qr, h->t_dgam, h->t_dgam_unit, h->t_groups, h->w_volT,
+            h->w_proj, h->w_fine, h->w_sig, h->w_data, h->w_vol2, h->w_red, h->w_scal, h->w_count,
+            h->s_xp, h->s_y, h->s_g, h->s_r, h->s_hist, h->s_flags, h->tc_twb, h->t_agroups,
+            h->t_tnf, h->t_vr, h->w_err, h->t_coil, h->w_projc, h->w_scanproj, h->w_volI,
+            h->t_ra_tile, h->t_ra_j, h->t_ra_w, h->t_twp, h->w_bins, h->hs_in[0], h->hs_in[1], h->hs_out,
+            h->tz_ua, h->tz_n0, h->tz_plo, h->tz_phi, h->tz_tap_ptr, h->tz_f0, h->tz_v, h->tz_taps, h->tz_optr,
+            h->tz_otap, h->w_zcoef, h->w_fine_z, h->w_projT, h->w_tz};
+}
+
+int64_t held_bytes(mpi_ffl_handle *h) {
+    return dev_bytes(own_buffers(h)) + dev_bytes(tc_buffers(h)) + dev_bytes(col_buffers(h)) +
+           dev_bytes(fold_buffers(h)) + dev_bytes(zfold_buffers(h)) + dev_bytes(ten_buffers(h));
+}
+
 void release(mpi_ffl_handle *h) {
-    void *ptrs[] = {h->t_ang, h->t_gain, h->t_unit_gain, h->t_htab, h->t_dhtab, h->t_traj, h->t_csr_ptr,
-                    h->t_csr, h->t_tw1, h->t_tw2_ro, h->t_tw2_qr, h->t_dgam, h->t_dgam_unit, h->t_groups, h->w_volT,
-                    h->w_proj, h->w_fine, h->w_sig, h->w_data, h->w_vol2, h->w_red, h->w_scal, h->w_count,
-                    h->s_xp, h->s_y, h->s_g, h->s_r, h->s_hist, h->s_flags, h->tc_twb, h->t_agroups,
-                    h->t_tnf, h->t_vr, h->w_err, h->t_coil, h->w_projc, h->w_scanproj, h->w_volI,
-                    h->t_ra_tile, h->t_ra_j, h->t_ra_w, h->t_twp, h->w_bins};
-    for (void *p : ptrs)
-        if (p) dev_free(p);
+    for (void *p : own_buffers(h)) dev_free(p);
     for (auto &r : h->prof_rec) {
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
     }
     for (auto e : h->ev_pool) cudaEventDestroy(e);
-    for (float *p : {h->hs_in[0], h->hs_in[1], h->hs_out})
-        if (p) dev_free(p);
-    for (void *p : {(void *)h->tz_ua, (void *)h->tz_n0, (void *)h->tz_plo, (void *)h->tz_phi, (void *)h->tz_tap_ptr,
-                    (void *)h->tz_f0, (void *)h->tz_v, (void *)h->tz_taps, (void *)h->tz_optr, (void *)h->tz_otap,
-                    (void *)h->w_zcoef, (void *)h->w_fine_z,
-                    (void *)h->w_projT, (void *)h->w_tz})
-        if (p) dev_free(p);
     for (int k = 0; k < 2; ++k) {
         if (h->hs_ready[k]) cudaEventDestroy(h->hs_ready[k]);
         if (h->hs_free[k]) cudaEventDestroy(h->hs_free[k]);
@@ -1013,7 +1015,6 @@ extern "C" int mpi_ffl_create(const mpi_ffl_geometry *geom, const mpi_ffl_trajec
             if (!make_il_maps(h->w_volI, d.N, d.Nz, &h->il_maps)) {  // the plain projector serves
                 dev_free(h->w_volI);
                 h->w_volI = nullptr;
-                h->bytes -= (int64_t)(il_len(d.N, d.Nz) * sizeof(float));
             }
         }
         dev_alloc(h, &h->w_proj, d.nproj);
@@ -1073,6 +1074,7 @@ extern "C" const char *mpi_ffl_last_error(const mpi_ffl_handle *h) {
 
 extern "C" int mpi_ffl_get_sizes(const mpi_ffl_handle *h, mpi_ffl_sizes *o) {
     if (!h || !o) return MPI_FFL_ERR_INVALID_ARG;
+    o->workspace_bytes = held_bytes(const_cast<mpi_ffl_handle *>(h));
     o->n_vox = h->d.nvox;
     o->n_data = h->d.ndata;
     o->n_proj = h->d.nproj;
@@ -1082,7 +1084,6 @@ extern "C" int mpi_ffl_get_sizes(const mpi_ffl_handle *h, mpi_ffl_sizes *o) {
     o->fine_len = h->d.Ne;
     o->line_len = h->d.L;
     o->fine_len_z = h->d.Nez;
-    o->workspace_bytes = h->bytes;
     return MPI_FFL_OK;
 }
 
@@ -1239,7 +1240,6 @@ extern "C" int mpi_ffl_set_scans(mpi_ffl_handle *h, int32_t scans) {
             dev_alloc(h, &h->w_scanproj, (size_t)2 * d.nproj);
             CK(dev_free(h->s_r));
             CK(dev_free(h->w_data));
-            h->bytes -= (int64_t)(2 * d.ndata * sizeof(float));
             h->s_r = r;
             h->w_data = w;
         }

@@ -773,18 +773,23 @@ void col_init(mpi_ffl_handle *h) {
     s->ok = true;
 }
 
+BufferList col_buffers(const mpi_ffl_handle *h) {
+    const ColState *s = cs(h);
+    if (!s) return {};
+    BufferList v{s->err};
+    for (int p = 0; p < 2; ++p) {
+        for (int f = 0; f < 2; ++f)
+            for (const Packed *pk : {&s->evf_f[f][p], &s->evf_a[f][p], &s->full_f[f][p], &s->full_a[f][p]})
+                v.add({pk->dev});
+        v.add({s->rows[p], s->apk[0][p], s->apk[1][p]});
+    }
+    return v;
+}
+
 void col_release(mpi_ffl_handle *h) {
     ColState *s = cs(h);
     if (!s) return;
-    for (int p = 0; p < 2; ++p) {
-        for (int f = 0; f < 2; ++f)
-            for (Packed *pk : {&s->evf_f[f][p], &s->evf_a[f][p], &s->full_f[f][p], &s->full_a[f][p]})
-                if (pk->dev) dev_free(pk->dev);
-        if (s->rows[p]) dev_free(s->rows[p]);
-        for (int dir = 0; dir < 2; ++dir)
-            if (s->apk[dir][p]) dev_free(s->apk[dir][p]);
-    }
-    if (s->err) dev_free(s->err);
+    for (void *p : col_buffers(h)) dev_free(p);
     delete s;
     h->col_state = nullptr;
 }

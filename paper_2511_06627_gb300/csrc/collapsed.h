@@ -7,6 +7,7 @@
 namespace mpiffl {
 
 void col_init(mpi_ffl_handle *h);        // splits W and W H (fold.h) into operands
+BufferList col_buffers(const mpi_ffl_handle *h);  // its device allocations
 void col_release(mpi_ffl_handle *h);
 bool col_supported(const mpi_ffl_handle *h);
 bool col_init_oom(const mpi_ffl_handle *h);  // col_init failed on a device allocation
@@ -39,6 +40,7 @@ void col_batch_init();
 // builds its tables for the handle's PSF width, ten_ready says whether they are there.
 int ten_init(mpi_ffl_handle *h);
 bool ten_ready(const mpi_ffl_handle *h);
+BufferList ten_buffers(const mpi_ffl_handle *h);
 void ten_release(mpi_ffl_handle *h);
 void ten_forward(mpi_ffl_handle *h, const float *proj, const float *coil, float *data, cudaStream_t st);
 void ten_adjoint(mpi_ffl_handle *h, const float *data, const float *coil, float *proj, cudaStream_t st);

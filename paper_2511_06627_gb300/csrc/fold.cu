@@ -451,12 +451,16 @@ void fold_refresh(mpi_ffl_handle *h) {
     }
 }
 
+BufferList fold_buffers(const mpi_ffl_handle *h) {
+    const FoldState *s = fs(h);
+    if (!s) return {};
+    return {s->W, s->taps, s->WH, s->f[0], s->f[1], s->a, s->rows};
+}
+
 void fold_release(mpi_ffl_handle *h) {
     FoldState *s = fs(h);
     if (!s) return;
-    for (void *p : {(void *)s->W, (void *)s->taps, (void *)s->WH, (void *)s->f[0], (void *)s->f[1], (void *)s->a,
-                    (void *)s->rows})
-        if (p) dev_free(p);
+    for (void *p : fold_buffers(h)) dev_free(p);
     delete s;
     h->fold_state = nullptr;
 }

@@ -31,6 +31,7 @@ void fold_psf_changed(mpi_ffl_handle *h);       // marks the operands as stale
 // tries again and reports.
 void fold_refresh(mpi_ffl_handle *h);
 void fold_trim(mpi_ffl_handle *h);              // after a failed build: releases what nothing uses
+BufferList fold_buffers(const mpi_ffl_handle *h);  // its device allocations
 void fold_release(mpi_ffl_handle *h);
 
 // C[crow[i]][ccol[n]] = scale[arow[i] / rdiv] sum_k A[arow[i]][acol[k]] B[k][n] in FP32
@@ -70,6 +71,7 @@ void zfold_forward(mpi_ffl_handle *h, const float *proj, float *data, cudaStream
 void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream_t st);
 // Rebuilds the table of the width, or leaves it to its next use, which tries again and reports.
 void zfold_psf_changed(mpi_ffl_handle *h);
+BufferList zfold_buffers(const mpi_ffl_handle *h);
 void zfold_release(mpi_ffl_handle *h);
 
 }  // namespace mpiffl

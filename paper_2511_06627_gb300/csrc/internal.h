@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -190,7 +191,6 @@ struct mpi_ffl_handle {
     void *col_state = nullptr;  // collapsed line operator (collapsed.cu)
     void *fold_state = nullptr; // its FP64 matrices and the staged path's FP32 operands (fold.cu)
     int path = 0;               // MPI_FFL_PATH_*
-    int64_t bytes = 0;
     // host buffers given to forward/adjoint: device staging, allocated on first use
     float *hs_in[2] = {nullptr, nullptr};  // copies of host inputs, alternating
     float *hs_out = nullptr;                // result before its copy to a host output
@@ -347,6 +347,18 @@ void set_thread_error(const std::string &msg);
 // of mpi_ffl_test_fail_alloc.
 cudaError_t dev_malloc(void **p, size_t bytes);
 cudaError_t dev_free(void *p);
+// Allocations of one owner (NULL among them is ignored). No heap: it also serves their release.
+struct BufferList {
+    void *p[80];
+    int n = 0;
+    BufferList(std::initializer_list<void *> v = {}) { add(v); }
+    void add(std::initializer_list<void *> v) {
+        for (void *q : v) p[n++] = q;
+    }
+    void *const *begin() const { return p; }
+    void *const *end() const { return p + n; }
+};
+int64_t dev_bytes(const BufferList &list);  // of the live ones
 
 // ---------------------------------------------------------------- launchers
 // Projector (k_projector.cu)

@@ -240,12 +240,16 @@ int ten_init(mpi_ffl_handle *h) {
 
 bool ten_ready(const mpi_ffl_handle *h) { return ts(h) && ts(h)->fwhm == h->fwhm; }
 
+BufferList ten_buffers(const mpi_ffl_handle *h) {
+    const TenState *t = ts(h);
+    if (!t) return {};
+    return {t->t, t->tp[0], t->tp[1], t->tt, t->vf, t->va, t->rows, t->ps, t->ds, t->pad};
+}
+
 void ten_release(mpi_ffl_handle *h) {
     TenState *t = ts(h);
     if (!t) return;
-    for (void *p : {(void *)t->t, (void *)t->tp[0], (void *)t->tp[1], (void *)t->tt, (void *)t->vf, (void *)t->va,
-                    (void *)t->rows, (void *)t->ps, (void *)t->ds, (void *)t->pad})
-        if (p) dev_free(p);
+    for (void *p : ten_buffers(h)) dev_free(p);
     delete t;
     h->ten_state = nullptr;
 }

@@ -761,6 +761,12 @@ void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream
     if (np > 1) launch_coil_pad(s->part, nullptr, proj, rows, d.Nz, d.N, d.N, st, np, rows * d.N);
 }
 
+BufferList zfold_buffers(const mpi_ffl_handle *h) {
+    const ZFold *s = zs(h);
+    if (!s) return {};
+    return {s->mem};
+}
+
 void zfold_release(mpi_ffl_handle *h) {
     ZFold *s = zs(h);
     if (!s) return;

@@ -793,12 +793,16 @@ bool tc_init_oom(const mpi_ffl_handle *h) {
     return s && s->oom;
 }
 
+BufferList tc_buffers(mpi_ffl_handle *h) {
+    const TcState *s = state(h);
+    if (!s) return {};
+    return {s->jobs_fwd, s->jobs_adj, s->twB, s->twA, s->tw2, s->err, s->wbase};
+}
+
 void tc_release(mpi_ffl_handle *h) {
     TcState *s = state(h);
     if (!s) return;
-    void *ptrs[] = {s->jobs_fwd, s->jobs_adj, s->twB, s->twA, s->tw2, s->err, s->wbase};
-    for (void *p : ptrs)
-        if (p) dev_free(p);
+    for (void *p : tc_buffers(h)) dev_free(p);
     delete s;
     h->tc_state = nullptr;
 }

@@ -7,6 +7,7 @@
 namespace mpiffl {
 
 void tc_init(mpi_ffl_handle *h);                 // builds the operand tables
+BufferList tc_buffers(mpi_ffl_handle *h);  // its device allocations
 void tc_release(mpi_ffl_handle *h);
 void tc_tables_changed(mpi_ffl_handle *h);      // PSF or gain tables were replaced
 bool tc_supported(const mpi_ffl_handle *h);     // shapes the kernels accept

@@ -107,7 +107,8 @@ def estimate_job_bytes(op):
 
 
 def estimate_request_bytes(geometry):
-    """Device bytes a request will hold (handle workspace + job state), from its sizes."""
+    """Device bytes a request will hold (handle workspace, collapsed line operator and job
+    state), from its sizes."""
     nx, nz, m = geometry["nx"], geometry["nz"], geometry["n_angles"]
     S, P, Q, A = geometry["S"], geometry["P"], geometry.get("Q", 8), geometry.get("A", 6.0)
     K = geometry["k_max"] - geometry["k_min"] + 1
@@ -115,6 +116,11 @@ def estimate_request_bytes(geometry):
     ne = (nx - 1) * Q + 2 * int(-(-A * Q // 1)) + 1
     nvox, nproj, nfine, ndata = nz * nx * nx, m * nz * nx, m * nz * ne, 2 * m * nz * nb
     handle = 4 * (3 * nvox + nproj + nfine + 2 * ndata) + 4 * (3 * nvox + max(nvox, nproj)) + 4 * 2 * S * P * 12 + (8 << 20)
+    # W and W H of both trajectories: 8 bytes a value (W H of two slots), split operands of 4 and 8
+    # bytes in both directions, in tiles; the split rows of the lines and of the data
+    par, rows = 1 + int(bool(geometry.get("zigzag", 1))), 2 * nb
+    handle += par * 8 * rows * (ne + 2 * nx) + par * 24 * (rows + 64) * (ne + nx + 128)
+    handle += 8 * (nproj + ndata) + 8 * 32 * 2 * m * nz + 16 * S * nb
     return handle + 4 * (4 * nvox + 2 * ndata)
 
 
