@@ -1568,7 +1568,6 @@ void z_line_forward(mpi_ffl_handle *h, const float *proj, float *b, cudaStream_t
     const Dims &d = h->d;
     if (use_zfold(h)) {
         TIMED(MPI_FFL_K_ZDRIVE, zfold_forward(h, proj, b, st));
-        h->launches += 2;  // a convolution and the band DFT's products in the same timed stage
         check_launch(h, "z-drive forward");
         return;
     }
@@ -1585,7 +1584,6 @@ void z_line_adjoint(mpi_ffl_handle *h, const float *b, float *proj, cudaStream_t
     const Dims &d = h->d;
     if (use_zfold(h)) {
         TIMED(MPI_FFL_K_ZDRIVE, zfold_adjoint(h, b, proj, st));
-        h->launches += 2;
     } else {
         ensure_z_sampled(h);
         TIMED(MPI_FFL_K_ZDRIVE, launch_zdft_adj(b, h->t_tw1, h->t_tw2_qr, h->t_dgam, z_tables(h), h->t_gain,
