@@ -94,10 +94,13 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
     }
     const bool vec = !g.acol && g.lda % 4 == 0 && (reinterpret_cast<uintptr_t>(gA) & 15) == 0;
     const int Kv = MODE == 2 ? g.half : g.K, th = (Kv + kSgK - 1) / kSgK;  // values and stages of a product
+    // first value of stage t: k0 + t kstep (a product in halves counts its own)
+    const int kstep = MODE != 2 && g.back ? -kSgK : kSgK, k0 = MODE != 2 && g.back ? (th - 1) * kSgK : 0;
+    auto stage_k = [&](int t) { return MODE == 2 ? (t >= th ? t - th : t) * kSgK : k0 + t * kstep; };
     auto copy_a = [&](int t) {
         float *st = smf + (t % kSgStages) * kStage + (tid / (kSgK / 4)) * kSgRow + ka;
         const bool second = MODE == 2 && t >= th;
-        const int k = (second ? t - th : t) * kSgK + ka, n = min(4, max(0, Kv - k));
+        const int k = stage_k(t) + ka, n = min(4, max(0, Kv - k));
         const int ks = min(k, (Kv - 1) & ~3) + (second ? g.ahalf : 0);
 #pragma unroll
         for (int u = 0; u < NA; ++u) {
@@ -125,7 +128,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
             if ((BN * kSgK / 4) % T && tid + u * T >= BN * kSgK / 4) break;
-            const int kk = (second ? t - th : t) * kSgK + kb0 + u * (T / (BN / 4));
+            const int kk = stage_k(t) + kb0 + u * (T / (BN / 4));
             cp_async16(st + 4 * u * T, bp + (int64_t)(min(kk, Kv - 1) + (second ? g.bhalf : 0)) * g.ldb,
                        kk < kvalid ? 16 : 0);
         }
