@@ -41,7 +41,7 @@ void fold_release(mpi_ffl_handle *h);
 // multiple of 4) and sC values apart. half > 0: two products E and O of half values of k
 // each, O's in columns ahalf (a multiple of 4) and rows bhalf further on; E + O goes to
 // column n, E - O to column c1 + n, or c1 - n when mirror is set (no acol and ccol, one batch).
-// back: k is summed from the last stage of 16 to the first (not with half).
+// back: k is summed from the last stage of 16 to the first (not with half). fine: in short runs.
 struct SgemmArgs {
     const float *A = nullptr;
     int64_t lda = 0;
@@ -60,7 +60,7 @@ struct SgemmArgs {
     int64_t sA = 0, sB = 0, sC = 0;
     int half = 0, ahalf = 0, bhalf = 0, c1 = 0;
     bool mirror = false;
-    bool back = false;
+    bool back = false, fine = false;
 };
 constexpr int kSgemmMax = 9;  // problems of one launch
 void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st);

@@ -529,6 +529,8 @@ int z_kper(const Dims &d) {
     SgemmArgs a{};
     a.M = d.M * d.Nz;
     a.N = halved(d) ? (d.N + 1) / 2 : d.N;
+    a.fine = true;
+    a.half = halved(d) ? 1 : 0;
     const int tiles = std::max(1, sgemm_tiles(a));
     if (halved(d)) {
         const int want = std::max(1, std::min(kSgemmMax, 3 * 152 / tiles));
@@ -748,6 +750,7 @@ void zfold_adjoint(mpi_ffl_handle *h, const float *data, float *proj, cudaStream
         g[i].C = np > 1 ? s->part + i * rows * d.N : proj;
         g[i].ldc = d.N;
         g[i].rdiv = 1;
+        g[i].fine = true;
         if (hv) {
             g[i].N = (d.N + 1) / 2;
             g[i].half = K;

@@ -38,12 +38,14 @@ __device__ __forceinline__ void cp_async_wait() {
 
 struct SgemmBatch {
     SgemmArgs g[kSgemmMax];
+    int run;                   // K of one run of sums
     int first[kSgemmMax + 1];  // first block of each problem
 };
 
-// K of one run of sums: longer products add their runs' sums, so that rounding errors grow
-// with the run and the number of runs, not with K
-constexpr int kSgRun = 320;
+// K of one run of sums (a multiple of kSgK): longer products add their runs' sums, so that rounding
+// errors grow with the run and the number of runs, not with K. The shorter run is that of fine
+// products in large tiles.
+constexpr int kSgRun = 320, kSgRunFine = 64;
 
 // One BM x BN tile per block. A warp covers 8 row groups x 4 column groups of TM x TN sums
 // each (a thread's rows are 8 apart, its columns come in runs of 4, BN / (TN / 4) apart). A
@@ -51,14 +53,15 @@ constexpr int kSgRun = 320;
 // loads here), four where they do not (B). KG: groups of threads that take their share of
 // each stage's K and add their sums at the end (more warps for products with few tiles).
 // MODE 1: K above kSgRun, the runs' sums are added in shared memory. MODE 2: two products of
-// half values of k each; the first one's sums wait there for the second's.
+// half values of k each; the first one's sums wait there for the second's. FINE: the sums of a
+// stage are formed apart and then added, which takes a second set of registers.
 __host__ __device__ constexpr int sgemm_stage_floats(int BM, int BN) { return BM * kSgRow + kSgK * BN; }
 __host__ __device__ constexpr int sgemm_ring_floats(int BM, int BN, int join, int stages) {
     const int ring = stages * sgemm_stage_floats(BM, BN);
     return ring > join ? ring : join;
 }
 
-template <int BM, int BN, int TM, int TN, int KG, int MODE>
+template <int BM, int BN, int TM, int TN, int KG, int MODE, bool FINE = false>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) * (BN / TN) * KG))
     k_sgemm(const __grid_constant__ SgemmBatch batch) {
     constexpr int TG = (BM / TM) * (BN / TN), T = TG * KG;
@@ -160,6 +163,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
         }
         cp_async_commit();
         const float *st = smf + (t % kSgStages) * kStage;
+        f32x2 part[FINE ? TM : 1][FINE ? TN / 2 : 1];  // sums of this stage
         const float *sa = st + tr * kSgRow + kg * KS, *sb = st + BM * kSgRow + kg * KS * BN + 4 * tc;
 #pragma unroll
         for (int kb = 0; kb < KS; kb += 4) {
@@ -180,10 +184,17 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
                 for (int i = 0; i < TM; ++i) {
                     const f32x2 a2 = dup2(q == 0 ? a4[i].x : q == 1 ? a4[i].y : q == 2 ? a4[i].z : a4[i].w);
 #pragma unroll
-                    for (int j = 0; j < TN / 2; ++j) acc[i][j] = fma2(a2, bv[j], acc[i][j]);
+                    for (int j = 0; j < TN / 2; ++j)
+                        if constexpr (FINE) part[i][j] = kb + q == 0 ? mul2(a2, bv[j]) : fma2(a2, bv[j], part[i][j]);
+                        else acc[i][j] = fma2(a2, bv[j], acc[i][j]);
                 }
             }
         }
+        if constexpr (FINE)
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN / 2; ++j) acc[i][j] = add2(acc[i][j], part[i][j]);
         if (MODE == 2 && t + 1 == th)  // a thread's own words
 #pragma unroll
             for (int i = 0; i < TM; ++i)
@@ -192,8 +203,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN) * KG, 384 / ((BM / TM) *
                     sum[(i * (TN / 2) + j) * T + tid] = unpack2(acc[i][j]);
                     acc[i][j] = 0;
                 }
-        if (MODE == 1 && ((t + 1) % (kSgRun * KG / kSgK) == 0 || t + 1 == nk)) {  // a thread's own words
-            const bool first = t < kSgRun * KG / kSgK;
+        if (MODE == 1 && ((t + 1) % (batch.run * KG / kSgK) == 0 || t + 1 == nk)) {  // a thread's own words
+            const bool first = t < batch.run * KG / kSgK;
 #pragma unroll
             for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -288,26 +299,40 @@ template <int BM, int BN, int TM, int TN, int KG>
 void run(const SgemmArgs *g, int n, cudaStream_t st) {
     constexpr int T = (BM / TM) * (BN / TN) * KG;
     SgemmBatch b{};
-    bool runs = false;  // of the products of one launch: all halved or none
+    const bool fine = g[0].fine;  // all products of one launch or none; the same for half
+    b.run = fine && KG == 1 ? kSgRunFine : kSgRun;
+    bool runs = false;
     for (int i = 0; i < kSgemmMax; ++i) {
         const int tiles = i < n ? (g[i].M + BM - 1) / BM * ((g[i].N + BN - 1) / BN) : 0;
         if (i < n) b.g[i] = g[i];
-        if (i < n && (g[i].half > 0 || g[i].K > kSgRun * KG)) runs = true;
+        if (i < n && (g[i].half > 0 || g[i].K > b.run * KG)) runs = true;
         b.first[i + 1] = b.first[i] + tiles * batches(g, i, n);
     }
     const int total = b.first[kSgemmMax];
     if (total == 0) return;
     const size_t smem = sizeof(float) * (sgemm_ring_floats(BM, BN, (KG - 1) * T / KG * TM * TN, sg_stages(runs)) + (runs ? TM * TN * T : 0));
-    auto kernel = runs ? k_sgemm<BM, BN, TM, TN, KG, 1> : k_sgemm<BM, BN, TM, TN, KG, 0>;
-    if constexpr (TM == 4 || KG == 1)
-        if (g[0].half > 0) kernel = k_sgemm<BM, BN, TM, TN, KG, 2>;
+    void (*kernel)(SgemmBatch);
+    if constexpr (TM == 6) {  // fine halves alone
+        kernel = k_sgemm<BM, BN, TM, TN, KG, 2, true>;
+    } else {
+        kernel = runs ? k_sgemm<BM, BN, TM, TN, KG, 1> : k_sgemm<BM, BN, TM, TN, KG, 0>;
+        if constexpr (TM == 4)
+            if (fine) kernel = runs ? k_sgemm<BM, BN, TM, TN, KG, 1, true> : k_sgemm<BM, BN, TM, TN, KG, 0, true>;
+        if constexpr (TM == 4 || KG == 1)
+            if (g[0].half > 0) kernel = k_sgemm<BM, BN, TM, TN, KG, 2>;
+    }
     if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     launch_dependent(kernel, dim3(total), dim3(T), smem, st, b);
 }
 
 }  // namespace
 
-int sgemm_tiles(const SgemmArgs &g) { return (g.M + 63) / 64 * ((g.N + 127) / 128); }
+constexpr int kFineRows = 48;  // of a tile of fine halves
+
+int sgemm_tiles(const SgemmArgs &g) {
+    const int rows = g.fine && g.half > 0 ? kFineRows : 64;
+    return (g.M + rows - 1) / rows * ((g.N + 127) / 128);
+}
 
 // 8 x 8 sums a thread (the fewest shared loads an FMA) where such tiles come to almost a wave
 // of three blocks an SM: 4608 x 2304 x 256 in 106 us, 68% of the FP32 FMA rate (4 x 8 sums in
@@ -315,6 +340,13 @@ int sgemm_tiles(const SgemmArgs &g) { return (g.M + 63) / 64 * ((g.N + 127) / 12
 // 4608 x 288 x 256 in 22 us (29 us with the large tiles), 1536 x 168 x 128 in 5.5 us (11 us).
 // Of the large tiles those of 56 rows where their waves are shorter: two halves of 4608 x 1152
 // x 128 in 59 us (two waves of 64 rows, the second a third full: 67 us).
+//
+// Fine products (the z-drive adjoint's last one, over n_par W S values without an order of size):
+// the small tiles have the registers for a stage's own sums, halves take them in tiles of 48 rows
+// (those of 64 or 56 spill: the z-drive adjoint at 256^2 x 128 and 36 angles 282 us, this way 275,
+// and 270 in plain sums), whole products in large tiles add runs of 64. The adjoint's error
+// against 64 bits at that size is 2.1e-7 (2.9e-7 in plain sums, 1.9e-7 sample by sample), at 64^2
+// x 32 and 12 angles 1.5e-7 (2.0e-7, 1.4e-7).
 //
 // Batches of products with few rows each (one per frequency or angle) take tiles of 64 columns
 // whose height fits the rows: the least padding, a tile's loads of B counted as 24 rows. 127
@@ -338,7 +370,8 @@ void launch_sgemm(const SgemmArgs *g, int n, cudaStream_t st) {
             tiles += (int64_t)g[i].nbatch * ((g[i].M + height - 1) / height) * ((g[i].N + 63) / 64);
         if (tiles < kWave) height = 32;
     }
-    if (height == 40) run<40, 64, 5, 8, 2>(g, n, st);
+    if (g[0].fine && g[0].half > 0) run<kFineRows, 128, 6, 8, 1>(g, n, st);
+    else if (height == 40) run<40, 64, 5, 8, 2>(g, n, st);
     else if (height == 56) run<56, 64, 7, 8, 2>(g, n, st);
     else if (height == 64) run<64, 64, 8, 8, 2>(g, n, st);
     else if (height == 72) run<72, 64, 9, 8, 2>(g, n, st);
