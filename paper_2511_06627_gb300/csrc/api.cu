@@ -1157,8 +1157,11 @@ static int set_path_impl(mpi_ffl_handle *h, int32_t path) {
 // The staged path's operands follow a width at once while that path is selected, or when it is
 // selected: its calls then find them built (a captured graph of theirs too).
 static int staged_selected(mpi_ffl_handle *h, int rc) {
-    if (rc == MPI_FFL_OK && h->path == MPI_FFL_PATH_STAGED) fold_refresh(h);
-    return rc;
+    if (rc != MPI_FFL_OK || h->path != MPI_FFL_PATH_STAGED) return rc;
+    return guarded(h, [&]() {  // on the handle's device
+        fold_refresh(h);
+        return MPI_FFL_OK;
+    });
 }
 
 extern "C" int mpi_ffl_set_precision(mpi_ffl_handle *h, int32_t precision) {

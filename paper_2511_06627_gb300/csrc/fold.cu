@@ -249,8 +249,10 @@ namespace {
 // W of a small scan (at most kHostW values) on the host, sample by sample: 3 to 6 ms on the
 // thread that prepares a request, beside the running batch, without the temporary device
 // memory of the device build, whose release waits for the batch. The device build takes 0.6
-// ms at these sizes; with it a tiny request is done 9 ms after its arrival, and requests 10 ms
-// apart no longer meet in the server, which tests/test_gpu_serving.py holds it to.
+// ms at these sizes. No measurement favours the host here: with the device build a tiny request
+// is done 9 ms after its arrival, and requests 10 ms apart no longer meet in the server, which
+// tests/test_gpu_serving.py holds it to (it failed in three of six runs). The line lies between
+// that test's largest scan (40082 values) and the next size in use (48080).
 constexpr size_t kHostW = 40960;
 
 std::vector<double> w_host(const mpi_ffl_handle *h) {

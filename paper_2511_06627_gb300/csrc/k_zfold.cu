@@ -642,12 +642,16 @@ int zfold_ready(mpi_ffl_handle *h) {
         for (auto &p : place) *p.first = (char *)s->mem + p.second;
         double *k64 = over_g ? reinterpret_cast<double *>(s->g) : K;
         cudaMemsetAsync(s->mem, 0, padded, nullptr);
-        rc = MPI_FFL_ERR_CUDA;
-        if (fold_h(h, true)) {
-            k_zfold_k<<<(nk + 31) / 32, 32>>>(drive_of(s, d) + d.S, k64, d, nk);
-            k_zfold_operands<<<608, 256>>>(k64, s->kf, s->ka, d.N, nk, s->ldk, s->ldu, hv);
-            k_zfold_dft<<<dim3(64, d.hw + 1), 128>>>(h->t_dgam, s->df, s->da, s->cols, d);
-            if (cudaGetLastError() == cudaSuccess && tables_done(s)) rc = MPI_FFL_OK;
+        try {
+            rc = MPI_FFL_ERR_CUDA;
+            if (fold_h(h, true)) {
+                k_zfold_k<<<(nk + 31) / 32, 32>>>(drive_of(s, d) + d.S, k64, d, nk);
+                k_zfold_operands<<<608, 256>>>(k64, s->kf, s->ka, d.N, nk, s->ldk, s->ldu, hv);
+                k_zfold_dft<<<dim3(64, d.hw + 1), 128>>>(h->t_dgam, s->df, s->da, s->cols, d);
+                if (cudaGetLastError() == cudaSuccess && tables_done(s)) rc = MPI_FFL_OK;
+            }
+        } catch (...) {
+            rc = MPI_FFL_ERR_OOM;  // a host allocation
         }
     }
     if (K) dev_free(K);
