@@ -1215,7 +1215,7 @@ extern "C" int mpi_ffl_set_coil_map(mpi_ffl_handle *h, const float *b_zu) {
             }
         if (!h->t_coil) dev_alloc(h, &h->t_coil, (size_t)d.Nz * d.N);
         if (!h->w_projc) dev_alloc(h, &h->w_projc, (size_t)d.M * d.Nz * d.N);
-        CK(cudaMemcpy(h->t_coil, b_zu, sizeof(float) * d.Nz * d.N, cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(h->t_coil, b_zu, sizeof(float) * d.Nz * d.N, cudaMemcpyHostToDevice, nullptr));
         uploads_done(h);
         return MPI_FFL_OK;
     });
@@ -1266,7 +1266,7 @@ extern "C" int mpi_ffl_set_gain(mpi_ffl_handle *h, const float *gain) {
         }
         for (int m = 0; m < h->d.M; ++m) h->gains[m] = gain[m];
         CK(cudaDeviceSynchronize());
-        CK(cudaMemcpy(h->t_gain, h->gains.data(), sizeof(float) * h->d.M, cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(h->t_gain, h->gains.data(), sizeof(float) * h->d.M, cudaMemcpyHostToDevice, nullptr));
         uploads_done(h);
         return MPI_FFL_OK;
     });
@@ -1288,8 +1288,8 @@ extern "C" int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm) {
         CK(cudaDeviceSynchronize());
         h->fwhm = fwhm;
         h->taps = std::move(taps);
-        CK(cudaMemcpy(h->t_htab, ht.data(), sizeof(float) * ht.size(), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(h->t_dhtab, dht.data(), sizeof(float) * dht.size(), cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(h->t_htab, ht.data(), sizeof(float) * ht.size(), cudaMemcpyHostToDevice, nullptr));
+        CK(cudaMemcpyAsync(h->t_dhtab, dht.data(), sizeof(float) * dht.size(), cudaMemcpyHostToDevice, nullptr));
         uploads_done(h);
         tc_tables_changed(h);
         fold_psf_changed(h);
