@@ -206,10 +206,10 @@ int mpi_ffl_set_psf_fwhm(mpi_ffl_handle *h, double fwhm_vox);
  * (L(xi)/xi) z^2/rho^2], xi = rho / a, rho^2 = u^2 + z^2, a from the FWHM along the drive
  * axis as for COLLINEAR (on z = 0 the two agree). Every line then reads every slice of
  * its projection, c[l][e] = sum_{z', i} p[z'][i] h_uu(u_lo + e/Q - i, l - z'), with full
- * support. It runs as one GEMM per line (forward) or per slice (adjoint) against
- * per-offset folded line operators W H_d, built on the device in FP64 when the model is
- * first selected (2 n_par (2 N_z - 1) 2 n_b N split operands, 4 bytes each, plus
- * n_par N_z 2 n_b N doubles) and again after set_psf_fwhm or a precision change. It
+ * support. It runs as FP32 products: a transform along z, one product per frequency and
+ * the transform back. The frequencies' matrices are built on the device in FP64 when the
+ * model is first selected and after set_psf_fwhm (n_par (N_z + 1) 2 n_b N doubles while
+ * they are built, kept as two FP32 copies); they do not depend on the precision. It
  * needs the collapsed line operator (the GEMM paths' tables) and applies whatever
  * the handle's path; MPI_FFL_ERR_UNSUPPORTED otherwise. Gradients of mpi_ffl_param_grad
  * and the batched jobs API use COLLINEAR only (MPI_FFL_ERR_UNSUPPORTED / the job runs
