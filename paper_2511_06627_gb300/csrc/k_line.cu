@@ -35,23 +35,34 @@ constexpr int kPsfTF = 9;
 // sixteen outputs per lane in the transpose: 16 FMA pairs per pair of shared loads
 constexpr int kPsfTA = 16;
 static_assert(kPsfTF <= kPsfT && kPsfTA <= kPsfT, "the tap table is padded for the windows");
-// Few lines (less than a warp of tasks a scheduler): the time is one thread's chain of packed
-// FMAs, so threads take fewer outputs, and a line's tasks are spread over blocks of one row
-// of the grid (blockIdx.y), four warps of them each. The sums and their order are the same.
-// Pairs of the line-GEMM path: 110 lines of 184 bins 142 -> 126 us (one line a thread: 133 us),
-// 297 lines of 48 bins 67 -> 64 us (66 us).
-constexpr int kPsfTFew = 5, kPsfTAFew = 8;
+// Few lines (less than two warps of tasks an SM in the transpose): the time is one thread's chain of
+// FMAs, so threads take fewer outputs, and a line's tasks are spread over blocks of one row of
+// the grid (blockIdx.y), four warps of them each. The sums and their order are the same. H^T of 297
+// lines of 48 bins takes 6.3 us so (9.4 in pairs, 8.3 one line at a time), of 110 lines of 184 bins
+// 14.4 us (16.5, 14.5); from there on the larger tiles are as fast or faster (242 lines of 236
+// bins: 26.7 us, 19.2 one line at a time).
+constexpr int kPsfTAFew = 8;
 constexpr int kPsfSMs = 152;
 // A pair of lines and the taps fit a block's shared memory for every x-drive scan that
 // mpi_ffl_create takes. Along z they may not (columns of 440 slices and more at Q = 32: a pair and
 // the taps need 264 KB, a line and the taps 199 KB): such columns go one at a time.
 constexpr int kPsfSmem = 227 * 1024;
 
+// Pairs or one line at a time: a pair's block takes some 1.75 times as long as one line's, and the
+// SM with the most blocks ends last. H^T of 1536 lines of 160 bins, 2 blocks of pairs on the
+// fullest SM or 3 of lines: 37.0 us, 30.8 one at a time; 2016 lines of 192 bins, 2 or 4: 41.1, 45.2.
+// H of 640 lines of 96 bins, 3 or 5: 10.3, 8.4; of 1536 lines of 160 bins, 6 or 11: 24.7, 26.7. H^T
+// also where pairs leave 3/7 of the SMs idle (630 lines of 200 bins: 32.9, 30.9).
+static bool psf_singly(int pair_blocks, int line_blocks) {
+    const int p = (pair_blocks + kPsfSMs - 1) / kPsfSMs, l = (line_blocks + kPsfSMs - 1) / kPsfSMs;
+    return 7 * p > 4 * l;
+}
+
 // Blocks that share the tasks of one block's lines: gx blocks with `warps` warps of tasks each
 static int psf_split(int gx, int warps) {
     return gx < kPsfSMs ? std::min((warps + 3) / 4, (2 * kPsfSMs + gx - 1) / gx) : 1;
 }
-static bool psf_few(int gx, int warps) { return (long long)gx * warps < 4 * kPsfSMs; }
+static bool psf_few(int gx, int warps) { return (long long)gx * warps < 2 * kPsfSMs; }
 
 // FP32-bound: 2.5 GFMA at 256^2 x 128 and 36 angles in 121 us (144 us one line at a
 // time), of 67 us at the FMA rate.
@@ -119,13 +130,10 @@ static void run_psf_fwd(const float *proj, const float *htab, float *fine, const
 }
 
 void launch_psf_fwd(const float *proj, const float *htab, float *fine, const Dims &d, cudaStream_t st) {
-    const int n_a = (d.Ne + d.Q - 1) / d.Q;
-    auto warps = [&](int t) { return (d.Q * ((n_a + t - 1) / t) + 31) / 32; };
-    if (sizeof(float) * (2 * (size_t)d.N + d.htab_len) > kPsfSmem)
-        run_psf_fwd<kPsfTFew, false>(proj, htab, fine, d, warps(kPsfTFew), st);
-    else if (psf_few((d.nseg + 1) / 2, warps(kPsfTF)))
-        run_psf_fwd<kPsfTFew, true>(proj, htab, fine, d, warps(kPsfTFew), st);
-    else run_psf_fwd<kPsfTF, true>(proj, htab, fine, d, warps(kPsfTF), st);
+    const int warps = (d.Q * (((d.Ne + d.Q - 1) / d.Q + kPsfTF - 1) / kPsfTF) + 31) / 32;
+    if (psf_singly((d.nseg + 1) / 2, d.nseg) || sizeof(float) * (2 * (size_t)d.N + d.htab_len) > kPsfSmem)
+        run_psf_fwd<kPsfTF, false>(proj, htab, fine, d, warps, st);
+    else run_psf_fwd<kPsfTF, true>(proj, htab, fine, d, warps, st);
 }
 
 // H^T: proj[i] = sum_e fine[e] h((e - D)/Q - i). Lanes of a warp are
@@ -206,16 +214,16 @@ __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restr
 
 // Line pairs of a block: 32 / Q of them fill a warp's lanes; fewer where the rows of so many do
 // not fit the shared memory beside the taps, at most two where the lines are few. Where not even
-// one pair fits, one line a block.
+// one pair fits, one line a block. One line at a time as many lines as pairs fill the lanes.
 template <int T, bool TWO>
 static void run_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, int pairs, cudaStream_t st) {
     // lanes = (line pair, phase); Q must be a power of two dividing 32 for the shuffle tree
-    const int stride = d.Ne + (((d.Q - d.Ne) % 16) + 16) % 16;  // stride = Q (mod 16)
-    constexpr int B = TWO ? 2 : 1;
+    constexpr int B = TWO ? 2 : 1, banks = 32 / B;
+    const int stride = d.Ne + (((d.Q - d.Ne) % banks) + banks) % banks;  // stride = Q (mod banks of B words)
     auto bytes = [&](int p) { return sizeof(float) * (d.htab_len + B * (size_t)p * stride); };
     while (pairs > 1 && bytes(pairs) > kPsfSmem) pairs /= 2;
     const size_t smem = bytes(pairs);
-    if (TWO && smem > kPsfSmem) return run_psf_adj<kPsfTAFew, false>(fine, htab, proj, d, 1, st);
+    if (TWO && smem > kPsfSmem) return run_psf_adj<kPsfTA, false>(fine, htab, proj, d, 1, st);
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(k_psf_adj<T, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPsfSmem);
     const int gx = (d.nseg + B * pairs - 1) / (B * pairs);
@@ -224,9 +232,11 @@ static void run_psf_adj(const float *fine, const float *htab, float *proj, const
 }
 
 void launch_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, cudaStream_t st) {
-    const int pairs = 32 / d.Q;
-    if (psf_few((d.nseg + 2 * pairs - 1) / (2 * pairs), (d.N + kPsfTA - 1) / kPsfTA))
+    const int pairs = 32 / d.Q, gx = (d.nseg + 2 * pairs - 1) / (2 * pairs);
+    if (psf_few(gx, (d.N + kPsfTA - 1) / kPsfTA))
         run_psf_adj<kPsfTAFew, true>(fine, htab, proj, d, std::min(pairs, 2), st);
+    else if (7 * gx <= 4 * kPsfSMs || psf_singly(gx, (d.nseg + pairs - 1) / pairs))  // (pairs on half of the SMs)
+        run_psf_adj<kPsfTA, false>(fine, htab, proj, d, pairs, st);
     else
         run_psf_adj<kPsfTA, true>(fine, htab, proj, d, pairs, st);
 }

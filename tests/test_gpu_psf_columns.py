@@ -1,5 +1,6 @@
-"""The PSF along z of columns so long that two of them do not fit a block's shared memory beside
-the taps: such columns go through H and its transpose one at a time."""
+"""H and its transpose where lines go one at a time and not in pairs: columns along z so long that
+two of them do not fit a block's shared memory beside the taps, and numbers of lines that pairs
+would spread unevenly."""
 
 import numpy as np
 import pytest
@@ -71,4 +72,22 @@ def test_a_column_of_ten_thousand_slices():
     e = np.unique(np.concatenate([rng.integers(0, zdrive.n_fine_z(st), 300), [0, zdrive.n_fine_z(st) - 1]]))
     h = psf.h((e[:, None] - st.D) / st.Q - np.arange(st.nz)[None, :], st.fwhm)
     assert rel_l2(got[:, e], (h @ proj[0].astype(np.float64)).T) < OP_TOL
+    op.close()
+
+
+# lines in pairs and one at a time, by the blocks on the fullest SM: H in pairs and H^T not, the
+# reverse, both singly, both in pairs; lines that are no multiple of a block's; other numbers of lanes
+@pytest.mark.parametrize("nx,nz,M,Q", [(40, 64, 24, 8), (33, 41, 13, 8), (64, 23, 9, 8), (35, 96, 21, 8),
+                                       (30, 61, 25, 4), (21, 51, 12, 16), (19, 70, 30, 2)])
+def test_lines_in_pairs_and_singly(nx, nz, M, Q):
+    from paper_2511_06627_gb300 import FFLOperator
+
+    geom = dict(GEOM, nx=nx, nz=nz, n_angles=M, S=16, P=20, Q=Q, k_max=4)
+    st, op = Setup(**geom), FFLOperator(**geom)
+    h = psf.h((np.arange(st.n_fine)[:, None] - st.D) / st.Q - np.arange(nx)[None, :], st.fwhm)
+    rng = np.random.default_rng(53)
+    p = rng.standard_normal((M, nz, nx)).astype(np.float32)
+    f = rng.standard_normal((M, nz, st.n_fine)).astype(np.float32)
+    assert rel_l2(op.apply_stage(1, _t(p)).cpu().numpy(), p @ h.T) < OP_TOL
+    assert rel_l2(op.apply_stage(1, _t(f), transpose=True).cpu().numpy(), f @ h) < OP_TOL
     op.close()
