@@ -22,7 +22,7 @@ namespace mpiffl {
 
 // ----------------------------------------------------------------------------- H
 
-// Both directions take lines two at a time: a thread's sums of the two lines are the halves of
+// Both directions take lines two at a time, unless psf_singly says otherwise: a thread's sums of the two lines are the halves of
 // an fma.rn.f32x2 with the same taps, so the issue slots that loads and tap duplication need
 // stay free beside the FMAs (one line at a time, an FMA was followed by a shared load or a
 // move in every fifth slot and a thread of 9 sums issued 11 instructions for 9 FMAs).
@@ -212,9 +212,9 @@ __global__ void __launch_bounds__(kPsfAdjThreads) k_psf_adj(const float *__restr
     }
 }
 
-// Line pairs of a block: 32 / Q of them fill a warp's lanes; fewer where the rows of so many do
-// not fit the shared memory beside the taps, at most two where the lines are few. Where not even
-// one pair fits, one line a block. One line at a time as many lines as pairs fill the lanes.
+// Line pairs (lines, where they go singly) of a block: 32 / Q of them fill a warp's lanes; fewer
+// where the rows of so many do not fit the shared memory beside the taps, at most two where the
+// lines are few. Where not even one pair fits, one line a block.
 template <int T, bool TWO>
 static void run_psf_adj(const float *fine, const float *htab, float *proj, const Dims &d, int pairs, cudaStream_t st) {
     // lanes = (line pair, phase); Q must be a power of two dividing 32 for the shuffle tree
